@@ -17,6 +17,7 @@
 // overflow, which bounded scores never do.  Every wait is bounded; on expiry the kernel
 // records kDevTimeoutAttention in the status word, releases its tensor memory and returns.
 #include "httm_internal.h"
+#include "httm_launch.cuh"
 #include "tc_sm100.cuh"
 
 #include <type_traits>
@@ -121,7 +122,7 @@ __device__ __noinline__ RedoneTile redo_score_tile(const __nv_bfloat16* q_row, c
     if (q_row) {
 #pragma unroll
         for (int i = 0; i < kHeadDim / 8; ++i) {
-            const uint4 u = __ldg(reinterpret_cast<const uint4*>(q_row) + i);
+            const uint4 u = ld_global(reinterpret_cast<const uint4*>(q_row) + i);
             const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -138,7 +139,7 @@ __device__ __noinline__ RedoneTile redo_score_tile(const __nv_bfloat16* q_row, c
         float a0 = 0.f, a1 = 0.f;
 #pragma unroll
         for (int i = 0; i < kHeadDim / 8; ++i) {
-            const uint4 u = __ldg(kr + i);
+            const uint4 u = ld_global(kr + i);
             const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -271,10 +272,10 @@ __device__ __forceinline__ RowTargets row_targets(const TcParams& p, int head, i
     }
     const int32_t* gs = p.group_start + (int64_t)head * (p.m_q + 1) + grow;
     const int32_t* member = p.group_member + (int64_t)head * p.n_tokens;
-    t.first = __ldg(gs);
-    t.count = __ldg(gs + 1) - t.first;
+    t.first = ld_global(gs);
+    t.count = ld_global(gs + 1) - t.first;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) t.token[i] = i < t.count ? __ldg(member + t.first + i) : 0;
+    for (int i = 0; i < 4; ++i) t.token[i] = i < t.count ? ld_global(member + t.first + i) : 0;
     return t;
 }
 // Every lane hands in its row (eight 16-byte pieces) and its targets.  The row is staged in shared memory and leaves as
@@ -299,7 +300,7 @@ __device__ __forceinline__ void store_rows(const TcParams& p, int head, const ui
 #pragma unroll
     for (int q = 0; q < 4; ++q)
         if (q < t.count) send(t.token[q]);
-    for (int q = 4; q < t.count; ++q) send(__ldg(member + q));
+    for (int q = 4; q < t.count; ++q) send(ld_global(member + q));
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
@@ -347,13 +348,15 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     int32_t* s_prefix = reinterpret_cast<int32_t*>(smem + (2 + 2 * KV_STAGES) * TILE_BYTES + 256 + 1024);   // [heads + 1]
     int32_t* s_mq = s_prefix + kTableHeads + 4;                                                               // [heads]
     const bool tables_on_chip = VAR && p.heads <= kTableHeads;
+    if (warp == 1) tc::tmem_alloc(tc::smem_addr(&bars->tmem_base), TMEM_COLS);
+    depend_wait();
+    dependents_launch();
     if (tables_on_chip) {
         for (int i = tid; i <= p.heads; i += NTHREADS) {
             s_prefix[i] = p.tile_prefix[i];
             if (i < p.heads) s_mq[i] = p.mq_head[i];
         }
     }
-    if (warp == 1) tc::tmem_alloc(tc::smem_addr(&bars->tmem_base), TMEM_COLS);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -751,14 +754,11 @@ cudaError_t launch_attention(const AttentionArgs& a, int sm_count, cudaStream_t 
                a.group_start, a.group_member, a.n_tokens, a.q.ptr, a.k.ptr, a.q.stride_head, a.q.stride_token, a.k.stride_head, a.k.stride_token};
     if (a.mq_head) {   // the tile table lives in device memory: full grid, CTAs without tiles leave at once
         if (a.group_start) return cudaErrorInvalidValue;   // (the member lists are built for equal query lengths only)
-        attention_tc_kernel<true, false><<<sm_count < 1 ? 1 : sm_count, NTHREADS, SMEM_BYTES, stream>>>(mq, mk, mv, p);
-        return cudaGetLastError();
+        return launch_kernel(attention_tc_kernel<true, false>, sm_count < 1 ? 1 : sm_count, NTHREADS, SMEM_BYTES, stream, mq, mk, mv, p);
     }
     if (a.group_start)
-        attention_tc_kernel<false, true><<<ctas, NTHREADS, SMEM_BYTES, stream>>>(mq, mk, mv, p);
-    else
-        attention_tc_kernel<false, false><<<ctas, NTHREADS, SMEM_BYTES, stream>>>(mq, mk, mv, p);
-    return cudaGetLastError();
+        return launch_kernel(attention_tc_kernel<false, true>, ctas, NTHREADS, SMEM_BYTES, stream, mq, mk, mv, p);
+    return launch_kernel(attention_tc_kernel<false, false>, ctas, NTHREADS, SMEM_BYTES, stream, mq, mk, mv, p);
 }
 
 }  // namespace httm

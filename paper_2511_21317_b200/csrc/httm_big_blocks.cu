@@ -12,6 +12,7 @@
 //                       gathers the members of a row in that order; writes merged Q / K / V and rank_q
 // All three read the reordered copies (a block is a contiguous run of rows there).
 #include "httm_internal.h"
+#include "httm_launch.cuh"
 #include "tc_sm100.cuh"
 
 namespace httm {
@@ -99,6 +100,8 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = bars->tmem_base;
+    depend_wait();
+    dependents_launch();
 
     // completions so far of every barrier (each role counts its own): they give the phase parities across chunks and items
     uint32_t n_tiles_done = 0;   // token tiles so far: tile k uses ring stage k % SC_STAGES and score buffer k & 1
@@ -143,8 +146,8 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     w[u] = 0.f;
                     if (dl < d_cnt) {
                         const int pos = dst_position(d_lo + dl, bi.n_rule, nd);
-                        v[u] = __ldg(reinterpret_cast<const uint4*>(x + (int64_t)pos * kHeadDim) + c16);
-                        w[u] = __ldg(inv + pos);
+                        v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)pos * kHeadDim) + c16);
+                        w[u] = ld_global(inv + pos);
                     }
                 }
 #pragma unroll
@@ -301,7 +304,7 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         }
                         const int p = it.row0 + i * TILE + row;   // token number inside the block
                         if (p < n) {
-                            const float w = __ldg(a.inv_norm[t] + head_row0 + p);
+                            const float w = ld_global(a.inv_norm[t] + head_row0 + p);
                             a.best_key[t][head_row0 + p] = score_key(best * w);
                             a.best_pos[t][head_row0 + p] = dst_position(arg, bi.n_rule, nd);
                         }
@@ -365,6 +368,8 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) big_select_kernel(const BigMat
     const BlockInfo bi = a.blocks[b];
     const int n = bi.n, r = t == 0 ? bi.r_q : bi.r_k, nd = t == 0 ? bi.nd_q : bi.nd_k;
     const int64_t base = (int64_t)h * a.n_tokens + bi.start;
+    depend_wait();
+    dependents_launch();
     int32_t* A = a.assign[t] + base;
     if (r == 0) {   // nothing merges: identity
         for (int j = tid; j < n; j += SEL_THREADS) A[j] = bi.start + j;
@@ -582,6 +587,8 @@ __global__ void __launch_bounds__(T, 1) big_merge_kernel(const MergeArgs a, int 
     int* seg = reinterpret_cast<int*>(mg_smem + (4 * T) * 6);                       // [n_kept + 1] first sorted index of every merged row
     int* warp_sum = seg + (4 * T) + 4;                                              // [32]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    depend_wait();
+    dependents_launch();
     const int n_block_ctas = 2 * a.heads * a.n_blocks;
     const int ch = lane & 7, sub = lane >> 3;   // 16-byte chunk of a row; which of four rows in flight
 
@@ -591,7 +598,7 @@ __global__ void __launch_bounds__(T, 1) big_merge_kernel(const MergeArgs a, int 
         if (row < a.n_special_total) {
             for (int t = 0; t < 3; ++t) {
                 const int m_len = t == 0 ? a.m_q : a.m_k;
-                const uint4 v = __ldg(reinterpret_cast<const uint4*>(a.xr[t] + ((int64_t)h * a.n_tokens + row) * kHeadDim) + (tid & 7));
+                const uint4 v = ld_global(reinterpret_cast<const uint4*>(a.xr[t] + ((int64_t)h * a.n_tokens + row) * kHeadDim) + (tid & 7));
                 reinterpret_cast<uint4*>(a.merged[t] + ((int64_t)h * m_len + row) * kHeadDim)[tid & 7] = v;
             }
         }
@@ -602,7 +609,7 @@ __global__ void __launch_bounds__(T, 1) big_merge_kernel(const MergeArgs a, int 
     const BlockInfo bi = a.blocks[b];
     const int n = bi.n, r = m == 0 ? bi.r_q : bi.r_k, m_len = m == 0 ? a.m_q : a.m_k;
     const bool variable = m == 0 && a.moff_q_var != nullptr;   // after outlier filtering the kept count of a block varies by head
-    const int moff = m == 0 ? (variable ? __ldg(a.moff_q_var + (int64_t)h * a.n_blocks + b) : bi.moff_q) : bi.moff_k;
+    const int moff = m == 0 ? (variable ? ld_global(a.moff_q_var + (int64_t)h * a.n_blocks + b) : bi.moff_q) : bi.moff_k;
     const int limit = variable ? n : n - r;                    // most kept tokens a valid map can have
     const int64_t base = (int64_t)h * a.n_tokens + bi.start;
     const int32_t* A = a.assign[m] + base;
@@ -627,7 +634,7 @@ __global__ void __launch_bounds__(T, 1) big_merge_kernel(const MergeArgs a, int 
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     v[u] = make_uint4(0u, 0u, 0u, 0u);
-                    if (i + u < i1) v[u] = __ldg(reinterpret_cast<const uint4*>(x + (int64_t)(keys[i + u] & 4095u) * kHeadDim) + ch);
+                    if (i + u < i1) v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)(keys[i + u] & 4095u) * kHeadDim) + ch);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -673,6 +680,8 @@ __global__ void __launch_bounds__(T, 1) big_deviation_kernel(const OutlierArgs a
     const BlockInfo bi = a.blocks[b];
     const int n = bi.n;
     const int64_t base = (int64_t)h * a.n_tokens + bi.start;
+    depend_wait();
+    dependents_launch();
     float* eps = a.eps + base;
     if (bi.r_q == 0) {   // nothing merged in this block (uniform)
         for (int j = tid; j < n; j += T) eps[j] = 0.f;
@@ -700,7 +709,7 @@ __global__ void __launch_bounds__(T, 1) big_deviation_kernel(const OutlierArgs a
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     v[u] = make_uint4(0u, 0u, 0u, 0u);
-                    if (i + u < i1) v[u] = __ldg(reinterpret_cast<const uint4*>(x + (int64_t)(keys[i + u] & 4095u) * st) + ch);
+                    if (i + u < i1) v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)(keys[i + u] & 4095u) * st) + ch);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -724,7 +733,7 @@ __global__ void __launch_bounds__(T, 1) big_deviation_kernel(const OutlierArgs a
             for (int u = 0; u < 4; ++u) {
                 pos[u] = i + u < i1 ? (int)(keys[i + u] & 4095u) : -1;
                 v[u] = make_uint4(0u, 0u, 0u, 0u);
-                if (cnt >= 2 && pos[u] >= 0) v[u] = __ldg(reinterpret_cast<const uint4*>(x + (int64_t)pos[u] * st) + ch);
+                if (cnt >= 2 && pos[u] >= 0) v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)pos[u] * st) + ch);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -764,6 +773,8 @@ __global__ void __launch_bounds__(T, 1) big_filter_kernel(const OutlierArgs a) {
     const int n = bi.n;
     const int64_t base = (int64_t)h * a.n_tokens + bi.start;
     const int32_t* A = a.assign_q + base;
+    depend_wait();
+    dependents_launch();
     int32_t* A_out = a.assign_q_out + base;
     if (bi.r_q == 0) {   // nothing merged, every deviation is 0: nothing to filter unless everything is an outlier, which changes nothing here
         for (int j = tid; j < n; j += T) A_out[j] = bi.start + j;
@@ -836,16 +847,14 @@ cudaError_t with_cta_size(int max_block, F&& f) {
 cudaError_t launch_big_deviation(const OutlierArgs& a, int max_block, cudaStream_t stream) {
     return with_cta_size(max_block, [&](auto t) {
         constexpr int T = decltype(t)::value;
-        big_deviation_kernel<T><<<a.heads * a.n_blocks, T, mg_smem_bytes(T), stream>>>(a);
-        return cudaGetLastError();
+        return launch_kernel(big_deviation_kernel<T>, a.heads * a.n_blocks, T, mg_smem_bytes(T), stream, a);
     });
 }
 
 cudaError_t launch_big_filter(const OutlierArgs& a, int max_block, cudaStream_t stream) {
     return with_cta_size(max_block, [&](auto t) {
         constexpr int T = decltype(t)::value;
-        big_filter_kernel<T><<<a.heads * a.n_blocks, T, of_smem_bytes(T), stream>>>(a);
-        return cudaGetLastError();
+        return launch_kernel(big_filter_kernel<T>, a.heads * a.n_blocks, T, of_smem_bytes(T), stream, a);
     });
 }
 
@@ -877,21 +886,18 @@ cudaError_t launch_big_scores(const BigMatchArgs& a, int sm_count, cudaStream_t 
     int ctas = sm_count < 1 ? 1 : sm_count;
     if (ctas > total) ctas = (int)total;
     if (ctas < 1) ctas = 1;
-    big_scores_kernel<<<ctas, SC_THREADS, SC_SMEM, stream>>>(mq, mk, a);
-    return cudaGetLastError();
+    return launch_kernel(big_scores_kernel, ctas, SC_THREADS, SC_SMEM, stream, mq, mk, a);
 }
 
 cudaError_t launch_big_select(const BigMatchArgs& a, cudaStream_t stream) {
-    big_select_kernel<<<2 * a.heads * a.n_blocks, SEL_THREADS, 0, stream>>>(a);
-    return cudaGetLastError();
+    return launch_kernel(big_select_kernel, 2 * a.heads * a.n_blocks, SEL_THREADS, 0, stream, a);
 }
 
 cudaError_t launch_big_merge(const MergeArgs& a, int max_block, cudaStream_t stream) {
     return with_cta_size(max_block, [&](auto t) {
         constexpr int T = decltype(t)::value;
         const int sp_chunks = (a.n_special_total + T / 8 - 1) / (T / 8);
-        big_merge_kernel<T><<<2 * a.heads * a.n_blocks + a.heads * sp_chunks, T, mg_smem_bytes(T), stream>>>(a, sp_chunks);
-        return cudaGetLastError();
+        return launch_kernel(big_merge_kernel<T>, 2 * a.heads * a.n_blocks + a.heads * sp_chunks, T, mg_smem_bytes(T), stream, a, sp_chunks);
     });
 }
 

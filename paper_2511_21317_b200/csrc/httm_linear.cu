@@ -9,6 +9,7 @@
 // DRAM once and the weights stay in L2.  Every wait is bounded; on expiry the status word is set and the kernel returns.
 #include "../../include/httm.h"
 #include "httm_internal.h"
+#include "httm_launch.cuh"
 #include "tc_sm100.cuh"
 
 namespace httm {
@@ -57,6 +58,8 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = bars->tmem_base;
+    depend_wait();
+    dependents_launch();
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer
@@ -170,8 +173,7 @@ cudaError_t launch_linear(const LinearArgs& a, int sm_count, cudaStream_t stream
     int ctas = sm_count < 1 ? 1 : sm_count;
     if (ctas > total) ctas = (int)total;
     if (ctas < 1) return cudaSuccess;   // nothing to do
-    linear_kernel<<<ctas, LIN_THREADS, LIN_SMEM, stream>>>(mx, mw, a.y, a.ldy, a.n_rows, a.out_features, k_blocks, n_tiles, total, a.status);
-    return cudaGetLastError();
+    return launch_kernel(linear_kernel, ctas, LIN_THREADS, LIN_SMEM, stream, mx, mw, a.y, a.ldy, a.n_rows, a.out_features, k_blocks, n_tiles, total, a.status);
 }
 
 }  // namespace httm

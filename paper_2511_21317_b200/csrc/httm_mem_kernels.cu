@@ -1,6 +1,7 @@
 // HBM-bound kernels of the HTTM path: temporal reorder (gather), per-(head, block)
 // cosine matching, mean merge, and unmerge + inverse reorder.  sm_100a only.
 #include "httm_internal.h"
+#include "httm_launch.cuh"
 #include "tc_sm100.cuh"   // mbarrier / TMA wrappers (device), tensor-map encoders (host)
 
 namespace httm {
@@ -54,11 +55,19 @@ __global__ void __launch_bounds__(kReorderThreads) reorder_kernel(const __grid_c
     const int64_t st = a.src[t].stride_token;
     __nv_bfloat16* dst = a.dst[t] + (int64_t)h * a.n_tokens * kHeadDim + chunk * 8;
     uint4 v[kReorderUnroll];
+    int row[kReorderUnroll];
+#pragma unroll
+    for (int u = 0; u < kReorderUnroll; ++u) {
+        const int p = base + u * (kReorderThreads / 8) + slot;
+        row[u] = p < a.n_tokens ? __ldg(a.pi + p) : 0;
+    }
+    depend_wait();
+    dependents_launch();
 #pragma unroll
     for (int u = 0; u < kReorderUnroll; ++u) {
         const int p = base + u * (kReorderThreads / 8) + slot;
         v[u] = make_uint4(0u, 0u, 0u, 0u);
-        if (p < a.n_tokens) v[u] = __ldg(reinterpret_cast<const uint4*>(src + (int64_t)__ldg(a.pi + p) * st));
+        if (p < a.n_tokens) v[u] = ld_global(reinterpret_cast<const uint4*>(src + (int64_t)row[u] * st));
     }
 #pragma unroll
     for (int u = 0; u < kReorderUnroll; ++u) {
@@ -81,10 +90,8 @@ __global__ void __launch_bounds__(kReorderThreads) reorder_kernel(const __grid_c
 cudaError_t launch_reorder(const ReorderArgs& a, cudaStream_t stream) {
     dim3 grid((a.n_tokens + kReorderTokensPerCta - 1) / kReorderTokensPerCta, a.heads, 3);
     if (a.inv_norm[0])
-        reorder_kernel<true><<<grid, kReorderThreads, 0, stream>>>(a);
-    else
-        reorder_kernel<false><<<grid, kReorderThreads, 0, stream>>>(a);
-    return cudaGetLastError();
+        return launch_kernel(reorder_kernel<true>, grid, kReorderThreads, 0, stream, a);
+    return launch_kernel(reorder_kernel<false>, grid, kReorderThreads, 0, stream, a);
 }
 
 // ------------------------------------------------------------------------------------
@@ -271,6 +278,8 @@ match_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
             tma_rows_load(stage0 + buf * STAGE_BYTES, c.t == 0 ? &map_q : &map_k, mb, start, c.h);
         }
     };
+    depend_wait();
+    dependents_launch();
     if (first < n_tasks && lane == 0) issue(nxt, 0);
     nxt.advance();
     if (STAGES == 2) {
@@ -541,10 +550,8 @@ static cudaError_t launch_match_t(const MatchArgs& a, int sm_count, cudaStream_t
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
     if (direct)
-        match_kernel<PASSES, true><<<(unsigned)grid, WARPS * 32, smem, stream>>>(mq, mk, a);
-    else
-        match_kernel<PASSES, false><<<(unsigned)grid, WARPS * 32, smem, stream>>>(mq, mk, a);
-    return cudaGetLastError();
+        return launch_kernel(match_kernel<PASSES, true>, (unsigned)grid, WARPS * 32, smem, stream, mq, mk, a);
+    return launch_kernel(match_kernel<PASSES, false>, (unsigned)grid, WARPS * 32, smem, stream, mq, mk, a);
 }
 
 // ------------------------------------------------------------------------------------
@@ -562,6 +569,8 @@ __host__ __device__ constexpr int anchor_smem_bytes(int nmax) { return nmax * (k
 __global__ void __launch_bounds__(kAnchorThreads) match_anchor_kernel(const MatchArgs a, const TensorView src_q, const TensorView src_k,
                                                                        const int32_t* __restrict__ pi, int n_anchor, int main_capacity, int nmax) {
     extern __shared__ __align__(16) unsigned char sm_anchor[];
+    depend_wait();
+    dependents_launch();
     const int task = blockIdx.x;
     const int b = task % n_anchor, h = (task / n_anchor) % a.heads, t = task / (n_anchor * a.heads);
     const BlockInfo bi = a.blocks[b];
@@ -576,7 +585,7 @@ __global__ void __launch_bounds__(kAnchorThreads) match_anchor_kernel(const Matc
     for (int q = threadIdx.x; q < n * 8; q += kAnchorThreads) {
         const int row = q >> 3, c = q & 7;
         const int64_t orig = pi ? __ldg(pi + bi.start + row) : bi.start + row;   // (no index: the tensors are the reordered copies)
-        *reinterpret_cast<uint4*>(rows + row * kAnchorPitch + c * 16) = __ldg(reinterpret_cast<const uint4*>(base + orig * sv.stride_token + c * 8));
+        *reinterpret_cast<uint4*>(rows + row * kAnchorPitch + c * 16) = ld_global(reinterpret_cast<const uint4*>(base + orig * sv.stride_token + c * 8));
     }
     __syncthreads();
     for (int j = threadIdx.x; j < n; j += kAnchorThreads) {
@@ -636,8 +645,7 @@ cudaError_t launch_match_anchor(const MatchArgs& a, const TensorView& src_q, con
                                 int main_capacity, int max_block_tokens, cudaStream_t stream) {
     if (n_anchor <= 0) return cudaSuccess;
     const int nmax = max_block_tokens < kMaxBlockTokens ? max_block_tokens : kMaxBlockTokens;
-    match_anchor_kernel<<<2 * a.heads * n_anchor, kAnchorThreads, anchor_smem_bytes(nmax), stream>>>(a, src_q, src_k, pi, n_anchor, main_capacity, nmax);
-    return cudaGetLastError();
+    return launch_kernel(match_anchor_kernel, 2 * a.heads * n_anchor, kAnchorThreads, anchor_smem_bytes(nmax), stream, a, src_q, src_k, pi, n_anchor, main_capacity, nmax);
 }
 
 cudaError_t launch_match(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
@@ -738,6 +746,8 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             tma_block_load(stage0 + buf * STAGE_BYTES, c.t == 0 ? &map_q : (c.t == 1 ? &map_k : &map_v), mb, bg.x0, bg.y0, bg.s0, c.h);
         }
     };
+    depend_wait();
+    dependents_launch();
     if (first < n_tasks && lane == 0) issue(nxt, 0);
     nxt.advance();
     if (first + stride < n_tasks && lane == 0) issue(nxt, 1);
@@ -767,7 +777,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             m.start = bi.start;
             m.n = bi.n;
             m.r = c.t == 0 ? bi.r_q : bi.r_k;
-            m.moff = c.t == 0 ? (a.moff_q_var ? __ldg(a.moff_q_var + (int64_t)c.h * a.n_blocks + c.u) : bi.moff_q) : bi.moff_k;
+            m.moff = c.t == 0 ? (a.moff_q_var ? ld_global(a.moff_q_var + (int64_t)c.h * a.n_blocks + c.u) : bi.moff_q) : bi.moff_k;
         }
         return m;
     };
@@ -778,7 +788,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     };
     auto load_target = [&](const Meta& m) {   // token this lane's token is merged into (number in the block), -1 if the lane holds none
         const int tok = token_of_lane(m);
-        return m.r > 0 && tok >= 0 ? __ldg(a.assign[m.t == 0 ? 0 : 1] + (int64_t)m.h * a.n_tokens + m.start + tok) - m.start : -1;
+        return m.r > 0 && tok >= 0 ? ld_global(a.assign[m.t == 0 ? 0 : 1] + (int64_t)m.h * a.n_tokens + m.start + tok) - m.start : -1;
     };
     Meta meta_next{};
     int target_next = -1;
@@ -962,10 +972,8 @@ static cudaError_t launch_merge_tc(const MergeArgs& a, int sm_count, cudaStream_
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
     if (direct)
-        merge_tc_kernel<true><<<(unsigned)grid, kMergeTcWarps * 32, kMergeTcSmem, stream>>>(m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
-    else
-        merge_tc_kernel<false><<<(unsigned)grid, kMergeTcWarps * 32, kMergeTcSmem, stream>>>(m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
-    return cudaGetLastError();
+        return launch_kernel(merge_tc_kernel<true>, (unsigned)grid, kMergeTcWarps * 32, kMergeTcSmem, stream, m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
+    return launch_kernel(merge_tc_kernel<false>, (unsigned)grid, kMergeTcWarps * 32, kMergeTcSmem, stream, m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
 }
 
 // ------------------------------------------------------------------------------------
@@ -1062,6 +1070,8 @@ merge_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             tma_block_load(stage0 + buf * STAGE_BYTES, c.t == 0 ? &map_q : (c.t == 1 ? &map_k : &map_v), mb, bg.x0, bg.y0, bg.s0, c.h);
         }
     };
+    depend_wait();
+    dependents_launch();
     if (first < n_tasks && lane == 0) issue(nxt, 0);
     nxt.advance();
     if (STAGES == 2) {
@@ -1110,7 +1120,7 @@ merge_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                                         : ((own_t[p] < bg.frames && own_y[p] < bg.rows && own_x[p] < bg.cols) ? (own_t[p] * bg.rows + own_y[p]) * bg.cols + own_x[p] : -1);
             rep[p] = -1;
             if (r > 0 && tok[p] >= 0) {
-                rep[p] = __ldg(a.assign[t == 0 ? 0 : 1] + (int64_t)h * a.n_tokens + start + tok[p]) - start;
+                rep[p] = ld_global(a.assign[t == 0 ? 0 : 1] + (int64_t)h * a.n_tokens + start + tok[p]) - start;
                 if (rep[p] < 0 || rep[p] >= n) {   // corrupt map: record, treat as kept
                     atomicCAS(a.status, kDevOk, kDevBadIndex);
                     rep[p] = tok[p];
@@ -1244,10 +1254,8 @@ static cudaError_t launch_merge_multi(const MergeArgs& a, int sm_count, cudaStre
     if (grid > sm_count) grid = sm_count;
     if (grid < 1) grid = 1;
     if (direct)
-        merge_multi_kernel<PASSES, true><<<(unsigned)grid, WARPS * 32, merge_multi_smem(NMAX), stream>>>(m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
-    else
-        merge_multi_kernel<PASSES, false><<<(unsigned)grid, WARPS * 32, merge_multi_smem(NMAX), stream>>>(m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
-    return cudaGetLastError();
+        return launch_kernel(merge_multi_kernel<PASSES, true>, (unsigned)grid, WARPS * 32, merge_multi_smem(NMAX), stream, m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
+    return launch_kernel(merge_multi_kernel<PASSES, false>, (unsigned)grid, WARPS * 32, merge_multi_smem(NMAX), stream, m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
 }
 
 cudaError_t launch_merge(const MergeArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
@@ -1316,6 +1324,8 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
         mbar_expect_tx(mb, (uint32_t)box_rows * kRowBytes);
         tma_block_load(stage0 + buf * STAGE_BYTES, &map_q, mb, bg.x0, bg.y0, bg.s0, c.h);
     };
+    depend_wait();
+    dependents_launch();
 #pragma unroll
     for (int st = 0; st < kDevStages; ++st) {
         if (first + st * stride < n_tasks && lane == 0) issue(nxt, st);
@@ -1336,7 +1346,7 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
         float* eps = a.eps + (int64_t)h * a.n_tokens + bi.start;
         int rep = -1;   // stage ROW of the token this lane's token was merged into
         if (r > 0 && tok >= 0) {
-            rep = __ldg(a.assign_q + (int64_t)h * a.n_tokens + bi.start + tok) - bi.start;
+            rep = ld_global(a.assign_q + (int64_t)h * a.n_tokens + bi.start + tok) - bi.start;
             if (rep < 0 || rep >= n) {
                 atomicCAS(a.status, kDevOk, kDevBadIndex);
                 rep = tok;
@@ -1498,16 +1508,16 @@ __device__ void select_level(const OutlierArgs& a, int level, int* hist) {
         }
         return;
     }
-    if (level > 0 && __ldcg(a.sel + kSelFinished)) return;
+    if (level > 0 && ld_global_cg(a.sel + kSelFinished)) return;
     const int nb = level == 2 ? 1024 : 2048, shift = level == 0 ? 21 : (level == 1 ? 10 : 0);
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) hist[i] = __ldcg(a.sel + kSelHist + level * 2048 + i);
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) hist[i] = ld_global_cg(a.sel + kSelHist + level * 2048 + i);
     __syncthreads();
     if (threadIdx.x < 32) {
-        const int rank = level == 0 ? (int)a.budget : __ldcg(a.sel + kSelRank + level - 1);
+        const int rank = level == 0 ? (int)a.budget : ld_global_cg(a.sel + kSelRank + level - 1);
         select_bin(hist, nb, rank, &s_bin, &s_rank);
         __syncwarp();
         if (threadIdx.x == 0) {
-            const uint32_t prefix = (level == 0 ? 0u : (uint32_t)__ldcg(a.sel + kSelPrefix + level - 1)) | ((uint32_t)s_bin << shift);
+            const uint32_t prefix = (level == 0 ? 0u : (uint32_t)ld_global_cg(a.sel + kSelPrefix + level - 1)) | ((uint32_t)s_bin << shift);
             if (level < 2) {
                 a.sel[kSelPrefix + level] = (int)prefix;
                 a.sel[kSelRank + level] = s_rank;
@@ -1536,6 +1546,8 @@ __device__ void finish_level(const OutlierArgs& a, int level, int* hist) {
 }
 __global__ void __launch_bounds__(256) select_level_kernel(const OutlierArgs a, int level) {
     __shared__ int hist[2048];
+    depend_wait();
+    dependents_launch();
     select_level(a, level, hist);
 }
 
@@ -1546,19 +1558,21 @@ constexpr int kRefineThreads = 256;
 template <int LEVEL>
 __global__ void __launch_bounds__(kRefineThreads) refine_kernel(const OutlierArgs a) {
     __shared__ int hist[2048];
-    if (__ldcg(a.sel + kSelFinished)) return;   // (same answer in every thread of every CTA)
+    depend_wait();
+    dependents_launch();
+    if (ld_global(a.sel + kSelFinished)) return;   // (same answer in every thread of every CTA)
     constexpr int NB = LEVEL == 2 ? 1024 : 2048, SHIFT = LEVEL == 0 ? 21 : (LEVEL == 1 ? 10 : 0);
     constexpr uint32_t MASK = LEVEL == 0 ? 0u : (LEVEL == 1 ? 0xffe00000u : 0xfffffc00u);
     for (int i = threadIdx.x; i < NB; i += kRefineThreads) hist[i] = 0;
     __syncthreads();
-    const uint32_t prefix = LEVEL == 0 ? 0u : (uint32_t)__ldcg(a.sel + kSelPrefix + (LEVEL > 0 ? LEVEL - 1 : 0));
+    const uint32_t prefix = LEVEL == 0 ? 0u : (uint32_t)ld_global_cg(a.sel + kSelPrefix + (LEVEL > 0 ? LEVEL - 1 : 0));
     const int64_t count = (int64_t)a.heads * a.n_tokens, quads = count >> 2;
     const uint4* bits4 = reinterpret_cast<const uint4*>(a.eps);   // (the array comes from cudaMalloc: 16-byte aligned)
     auto tally = [&](uint32_t b) {
         if ((b & MASK) == prefix) atomicAdd(&hist[(b >> SHIFT) & (NB - 1)], 1);
     };
     for (int64_t i = (int64_t)blockIdx.x * kRefineThreads + threadIdx.x; i < quads; i += (int64_t)gridDim.x * kRefineThreads) {
-        const uint4 b = __ldg(bits4 + i);
+        const uint4 b = ld_global(bits4 + i);
         tally(b.x);
         tally(b.y);
         tally(b.z);
@@ -1577,6 +1591,8 @@ __global__ void __launch_bounds__(kRefineThreads) refine_kernel(const OutlierArg
 // An outlier maps to itself; the other tokens of a group stay together, under their old representative if
 // that is not an outlier, else under the remaining member with the lowest position.
 __global__ void __launch_bounds__(256) filter_kernel(const OutlierArgs a) {
+    depend_wait();
+    dependents_launch();
     const int lane = threadIdx.x & 31;
     const int64_t task = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (task >= (int64_t)a.heads * a.n_blocks) return;
@@ -1616,6 +1632,8 @@ __global__ void __launch_bounds__(kOffsetsThreads, 1) offsets_kernel(const Outli
     __shared__ int warp_sum[32];
     __shared__ int s_last;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = blockIdx.x;
+    depend_wait();
+    dependents_launch();
     const int32_t* cnt = a.kept_cnt + (int64_t)h * a.n_blocks;
     int32_t* moff = a.moff_var + (int64_t)h * a.n_blocks;
     int running = a.n_special_total;
@@ -1655,7 +1673,7 @@ __global__ void __launch_bounds__(kOffsetsThreads, 1) offsets_kernel(const Outli
         int t = 0;
         for (int hh = 0; hh < a.heads; ++hh) {
             a.tile_prefix[hh] = t;
-            t += (__ldcg(a.mq_head + hh) + 127) / 128;
+            t += (ld_global_cg(a.mq_head + hh) + 127) / 128;
         }
         a.tile_prefix[a.heads] = t;
     }
@@ -1668,27 +1686,23 @@ cudaError_t launch_deviation(const OutlierArgs& a, int sm_count, cudaStream_t st
     int64_t grid = (n_tasks + kDevWarps - 1) / kDevWarps;
     if (grid > 2ll * sm_count) grid = 2ll * sm_count;
     if (grid < 1) grid = 1;
-    deviation_kernel<<<(unsigned)grid, kDevWarps * 32, kDevSmem, stream>>>(mq, a);
-    return cudaGetLastError();
+    return launch_kernel(deviation_kernel, (unsigned)grid, kDevWarps * 32, kDevSmem, stream, mq, a);
 }
 cudaError_t launch_threshold(const OutlierArgs& a, int sm_count, cudaStream_t stream) {
     const int64_t quads = ((int64_t)a.heads * a.n_tokens) >> 2;
     int64_t grid = (quads + kRefineThreads * 4 - 1) / (kRefineThreads * 4);   // about four 16-byte loads per thread
     if (grid > 2ll * sm_count) grid = 2ll * sm_count;
     if (grid < 1) grid = 1;
-    refine_kernel<1><<<(unsigned)grid, kRefineThreads, 0, stream>>>(a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(refine_kernel<1>, (unsigned)grid, kRefineThreads, 0, stream, a);
     if (e != cudaSuccess) return e;
-    refine_kernel<2><<<(unsigned)grid, kRefineThreads, 0, stream>>>(a);
-    return cudaGetLastError();
+    return launch_kernel(refine_kernel<2>, (unsigned)grid, kRefineThreads, 0, stream, a);
 }
 cudaError_t launch_threshold0(const OutlierArgs& a, int sm_count, cudaStream_t stream) {
     const int64_t quads = ((int64_t)a.heads * a.n_tokens) >> 2;
     int64_t grid = (quads + kRefineThreads * 4 - 1) / (kRefineThreads * 4);
     if (grid > 2ll * sm_count) grid = 2ll * sm_count;
     if (grid < 1) grid = 1;
-    refine_kernel<0><<<(unsigned)grid, kRefineThreads, 0, stream>>>(a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(refine_kernel<0>, (unsigned)grid, kRefineThreads, 0, stream, a);
     if (e != cudaSuccess) return e;
     return launch_threshold(a, sm_count, stream);
 }
@@ -1698,25 +1712,20 @@ cudaError_t launch_refine_level(const OutlierArgs& a, int level, int sm_count, c
     if (grid > 2ll * sm_count) grid = 2ll * sm_count;
     if (grid < 1) grid = 1;
     if (level == 0)
-        refine_kernel<0><<<(unsigned)grid, kRefineThreads, 0, stream>>>(a);
-    else if (level == 1)
-        refine_kernel<1><<<(unsigned)grid, kRefineThreads, 0, stream>>>(a);
-    else
-        refine_kernel<2><<<(unsigned)grid, kRefineThreads, 0, stream>>>(a);
-    return cudaGetLastError();
+        return launch_kernel(refine_kernel<0>, (unsigned)grid, kRefineThreads, 0, stream, a);
+    if (level == 1)
+        return launch_kernel(refine_kernel<1>, (unsigned)grid, kRefineThreads, 0, stream, a);
+    return launch_kernel(refine_kernel<2>, (unsigned)grid, kRefineThreads, 0, stream, a);
 }
 cudaError_t launch_select_level(const OutlierArgs& a, int level, cudaStream_t stream) {
-    select_level_kernel<<<1, 256, 0, stream>>>(a, level);
-    return cudaGetLastError();
+    return launch_kernel(select_level_kernel, 1, 256, 0, stream, a, level);
 }
 cudaError_t launch_offsets(const OutlierArgs& a, cudaStream_t stream) {
-    offsets_kernel<<<(unsigned)a.heads, kOffsetsThreads, 0, stream>>>(a);
-    return cudaGetLastError();
+    return launch_kernel(offsets_kernel, (unsigned)a.heads, kOffsetsThreads, 0, stream, a);
 }
 cudaError_t launch_filter(const OutlierArgs& a, cudaStream_t stream) {
     const int64_t threads = (int64_t)a.heads * a.n_blocks * 32;
-    filter_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(filter_kernel, (unsigned)((threads + 255) / 256), 256, 0, stream, a);
     if (e != cudaSuccess) return e;
     return launch_offsets(a, stream);
 }
@@ -1747,15 +1756,17 @@ __global__ void __launch_bounds__(kUnmergeThreads) unmerge_kernel(const __grid_c
         const int i = base + u * (kUnmergeThreads / 8) + slot;
         p[u] = i < a.n_tokens ? __ldg(a.pi_inv + i) : 0;
     }
+    depend_wait();
+    dependents_launch();
 #pragma unroll
-    for (int u = 0; u < kUnmergeUnroll; ++u) row[u] = __ldg(rank + p[u]);
+    for (int u = 0; u < kUnmergeUnroll; ++u) row[u] = ld_global(rank + p[u]);
 #pragma unroll
     for (int u = 0; u < kUnmergeUnroll; ++u) {
         if (row[u] < 0 || row[u] >= a.m_q) {   // corrupt map: record, copy row 0 instead of reading out of range
             atomicCAS(a.status, kDevOk, kDevBadIndex);
             row[u] = 0;
         }
-        v[u] = __ldg(om + (int64_t)row[u] * 8);
+        v[u] = ld_global(om + (int64_t)row[u] * 8);
     }
 #pragma unroll
     for (int u = 0; u < kUnmergeUnroll; ++u) {
@@ -1766,8 +1777,7 @@ __global__ void __launch_bounds__(kUnmergeThreads) unmerge_kernel(const __grid_c
 
 cudaError_t launch_unmerge(const UnmergeArgs& a, cudaStream_t stream) {
     dim3 grid((a.n_tokens + kUnmergeTokensPerCta - 1) / kUnmergeTokensPerCta, a.heads);
-    unmerge_kernel<<<grid, kUnmergeThreads, 0, stream>>>(a);
-    return cudaGetLastError();
+    return launch_kernel(unmerge_kernel, grid, kUnmergeThreads, 0, stream, a);
 }
 
 cudaError_t configure_kernels() {
