@@ -61,6 +61,19 @@ bool encode_patch_tensor_map(CUtensorMap* map, const void* base, int grid_w, int
     return r == CUDA_SUCCESS;
 }
 
+bool encode_matrix_tensor_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t stride_row, int box_rows, int box_cols) {
+    std::call_once(g_encode_once, resolve_encode);
+    if (!g_encode) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)stride_row * 2};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+    const cuuint32_t elem[2] = {1, 1};
+    CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, elem,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS;
+}
+
 bool encode_frame_tensor_map(CUtensorMap* map, const void* base, int64_t tokens_per_frame, int frames, int64_t heads,
                              int64_t stride_token, int64_t stride_head, int box_tokens) {
     std::call_once(g_encode_once, resolve_encode);

@@ -246,6 +246,9 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
 bool encode_rows_tensor_map(CUtensorMap* map, const void* base, int64_t rows, int64_t heads, int64_t stride_row,
                             int64_t stride_head, int box_rows);
 
+// Host: 2-D bf16 tensor map of a matrix {cols, rows} with a {box_cols, box_rows} box (box_cols * 2 bytes: one 128-byte swizzle row).
+bool encode_matrix_tensor_map(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t stride_row, int box_rows, int box_cols);
+
 // Host: 5-D bf16 tensor map over the patch tokens of an original [heads][tokens][64] tensor (any head / token
 // strides): dimensions {64 channels, grid_w, grid_h, frames, heads}, box {64, box_w, box_h, box_frames, 1},
 // 128-byte swizzle; `base` points at patch (0, 0) of frame 0.  A box is one merging block in (frame, row,

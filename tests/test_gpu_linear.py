@@ -46,6 +46,13 @@ def test_shapes_with_ragged_tiles(ctx, n, k, o):
     check(ctx, n, k, o, seed=n + k + o)
 
 
+@pytest.mark.parametrize("n,k,o", [(255, 64, 128), (256, 64, 264), (257, 128, 520), (385, 64, 72), (5003, 128, 1160), (20000, 64, 256)])
+def test_edges_of_the_pair_tiles(ctx, n, k, o):
+    """256 x 256 tiles of a CTA pair: rows and columns just before and behind a half tile and a tile, and more tiles than
+    pairs (a pair then works on several, with both accumulators and the ring in their later phases)."""
+    check(ctx, n, k, o, seed=n + k + o)
+
+
 def test_strided_rows_and_large_values(ctx):
     check(ctx, 260, 128, 520, seed=5, ldx=136, ldw=200, ldy=528)
     check(ctx, 260, 64, 256, seed=6, scale=100.0)
