@@ -459,11 +459,13 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) big_select_kernel(const BigMat
 
 // ------------------------------------------------------------------------------------------------ merging
 // One CTA per (map in {Q, K}, head, block) - the K map also merges V - plus CTAs that copy the special tokens.
-// The sorted-group kernels are templated on T, the threads of a CTA; a CTA holds one block of up to 4 T tokens (thread i
-// owns tokens 4 i .. 4 i + 3).  T is chosen from the largest block of the context: 1024 for blocks of 4096 tokens, 64 for
-// blocks of up to 256, so that small blocks get many small CTAs per SM.
-__host__ __device__ constexpr int mg_smem_bytes(int T) { return 4 * T * 4 /*keys*/ + 4 * T * 2 /*row of kept token*/ + (4 * T + 4) * 4 /*segments*/ + 256; }
-__host__ __device__ constexpr int of_smem_bytes(int T) { return mg_smem_bytes(T) + 4 * T * 2 /*position of every row's kept token*/ + 4 * T /*outlier flags*/ + 4 * T * 2 /*new representative of every row*/; }
+// The sorted-group kernels are templated on T, the threads of a CTA, and E, the tokens per thread: a CTA holds one block of up
+// to E T tokens, chosen from the largest block of the context: 64 threads for blocks of up to 256 tokens .. 512 for 4096.
+// They gather rows from DRAM and are bound by the loads in flight: several CTAs share an SM (1536 threads of at most 40
+// registers), so that one gathers while another sorts.
+constexpr int kSortedThreads = 1536;   // resident threads per SM the kernels are compiled for (40 registers)
+__host__ __device__ constexpr int mg_smem_bytes(int N) { return N * 4 /*keys*/ + N * 2 /*row of kept token*/ + (N + 4) * 4 /*segments*/ + 256; }   // N = E T tokens
+__host__ __device__ constexpr int of_smem_bytes(int N) { return mg_smem_bytes(N) + N * 2 /*position of every row's kept token*/ + N /*outlier flags*/ + N * 2 /*new representative of every row*/; }
 
 __device__ __forceinline__ void unpack8f(const uint4& raw, float* f) {
     const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
@@ -478,96 +480,142 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// One stable counting pass over the keys of a block by a six-bit digit of their row: warp w holds elements 32 (E w + s) + lane
+// (s = 0 .. E - 1), in this order, and hist[digit * (warps + 1) + warp] counts (the odd pitch spreads the digits over the banks).
+// Returns every element's place in the sorted order; elements without a key have digit kRadix.
+constexpr int kRadix = 64;
+template <int T, int E>
+__device__ __forceinline__ void radix_places(const int (&digit)[E], int (&place)[E], int* hist, int* warp_tot) {
+    constexpr int W = T / 32, PITCH = W + 1;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+#pragma unroll
+    for (int i = tid; i < kRadix * PITCH; i += T) hist[i] = 0;
+    __syncthreads();
+    const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+    for (int s = 0; s < E; ++s) {
+        const unsigned peers = __match_any_sync(0xffffffffu, digit[s]);
+        int* h = hist + (digit[s] & (kRadix - 1)) * PITCH + warp;
+        const int before = digit[s] < kRadix ? *h : 0;
+        place[s] = before + __popc(peers & below);
+        __syncwarp();
+        if (digit[s] < kRadix && (peers & below) == 0) *h = before + __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    // exclusive sum over the counters in (digit, warp) order, two per thread
+    const int e0 = 2 * tid, d0 = e0 / W, d1 = (e0 + 1) / W;
+    int* h0 = hist + d0 * PITCH + (e0 - d0 * W);
+    int* h1 = hist + d1 * PITCH + (e0 + 1 - d1 * W);
+    const int c0 = *h0, c1 = *h1;
+    int incl = c0 + c1;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += o;
+    }
+    if (lane == 31) warp_tot[warp] = incl;
+    __syncthreads();
+    int base = 0;   // totals of the warps before this one
+    {
+        const int w = lane < W ? warp_tot[lane] : 0;
+        int v = lane < warp ? w : 0;
+        base = __reduce_add_sync(0xffffffffu, v);
+    }
+    const int excl = base + incl - c0 - c1;
+    *h0 = excl;
+    *h1 = excl + c0;
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < E; ++s) place[s] += digit[s] < kRadix ? hist[digit[s] * PITCH + warp] : 0;
+}
+
 // The groups of one block from its map A (every thread of the T-thread CTA calls this): merged row of every kept token =
 // its rank among the kept tokens in position order (row_of; -1 for merged tokens); all tokens sorted by (merged row,
 // position) in keys[] = (row << 12) | position, so that the members of a row are one ascending run; seg[row] = first
 // sorted index of the row, seg[n_kept] = n.  rep_of_row (optional) gets the position of every row's kept token; rank_out
 // (optional) the merged row of every token plus moff.  Returns the number of kept tokens, at most `limit` (tokens whose
 // row would lie beyond it, or whose target is not a kept token, are recorded as a corrupt map and left out).
-template <int T>
+// The order comes from two stable counting passes over six bits of the row each (one if there are at most 64 rows), so
+// it does not depend on scheduling.  A bitonic sort of the keys took 28 us for 3840 tokens (78 rounds with a barrier each).
+// At 82 440 tokens x 16 heads in 3840-token blocks, one CTA of 1024 threads per SM: deviation 203 -> 153 us, filter 92 -> 40, merge
+// 310 -> 303; with three CTAs of 512 threads per SM, half of which gather while others sort: 144, 31 and 212 us.
+template <int T, int E>
 __device__ int build_groups(const int32_t* A, int block_start, int n, int limit, uint32_t* keys, int16_t* row_of, int* seg, int* warp_sum,
                             int16_t* rep_of_row, int32_t* status, int32_t* rank_out, int moff) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    int rep[4];
-    int kept = 0;
+    int* hist = seg;   // (the counters lie where the segments go: 64 (T / 32 + 1) <= E T + 4 words)
+    int rep[E];
+    unsigned kept[E];
+    int n_mine = 0;   // kept tokens of this warp
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int j = 4 * tid + e;
-        rep[e] = -1;
+    for (int s = 0; s < E; ++s) {
+        const int j = (warp * E + s) * 32 + lane;
+        rep[s] = -1;
         if (j < n) {
-            rep[e] = A[j] - block_start;
-            if (rep[e] < 0 || rep[e] >= n) {   // corrupt map: record, treat as kept
+            rep[s] = ld_global(A + j) - block_start;
+            if (rep[s] < 0 || rep[s] >= n) {   // corrupt map: record, treat as kept
                 atomicCAS(status, kDevOk, kDevBadIndex);
-                rep[e] = j;
+                rep[s] = j;
             }
-            kept += rep[e] == j ? 1 : 0;
         }
-    }
-    int incl = kept;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += o;
+        kept[s] = __ballot_sync(0xffffffffu, j < n && rep[s] == j);
+        n_mine += __popc(kept[s]);
     }
     __syncthreads();   // (the scratch arrays may still be in use by a previous call's readers)
-    if (lane == 31) warp_sum[warp] = incl;
+    if (lane == 0) warp_sum[warp] = n_mine;
     __syncthreads();
-    if (warp == 0) {
-        int w = lane < T / 32 ? warp_sum[lane] : 0;
+    const int w = lane < T / 32 ? warp_sum[lane] : 0;
+    const int n_kept = min(__reduce_add_sync(0xffffffffu, w), limit);
+    int next_row = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0);
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int o = __shfl_up_sync(0xffffffffu, w, off);
-            if (lane >= off) w += o;
+    for (int s = 0; s < E; ++s) {
+        const int j = (warp * E + s) * 32 + lane;
+        if (j < n) {
+            const bool is_kept = (kept[s] >> lane) & 1u;
+            const int row = next_row + __popc(kept[s] & ((1u << lane) - 1u));
+            row_of[j] = is_kept ? (int16_t)row : (int16_t)-1;
+            if (is_kept && rep_of_row && row < n_kept) rep_of_row[row] = (int16_t)j;
         }
-        if (lane < T / 32) warp_sum[lane] = w;
+        next_row += __popc(kept[s]);
     }
     __syncthreads();
-    const int n_kept = min(warp_sum[T / 32 - 1], limit);
-    int next_row = (warp > 0 ? warp_sum[warp - 1] : 0) + incl - kept;
+    uint32_t key[E];
+    int digit[E], place[E];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int j = 4 * tid + e;
+    for (int s = 0; s < E; ++s) {
+        const int j = (warp * E + s) * 32 + lane;
+        key[s] = 0xffffffffu;
+        digit[s] = kRadix;
         if (j < n) {
-            const bool is_kept = rep[e] == j;
-            row_of[j] = is_kept ? (int16_t)next_row : (int16_t)-1;
-            if (is_kept) {
-                if (rep_of_row && next_row < n_kept) rep_of_row[next_row] = (int16_t)j;
-                ++next_row;
-            }
-        }
-    }
-    __syncthreads();
-    int P = 32;
-    while (P < n) P <<= 1;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int j = 4 * tid + e;
-        uint32_t key = 0xffffffffu;
-        if (j < n) {
-            int row = row_of[rep[e]];
+            int row = row_of[rep[s]];
             if (row < 0 || row >= n_kept) {   // target is not a kept token, or more kept tokens than a valid map has
                 atomicCAS(status, kDevOk, kDevBadIndex);
-                row = 0xfffff;                // sorts behind every valid row, is never gathered
+                row = n_kept;                 // (at most 4095 then) sorts behind every valid row, is never gathered
             } else if (rank_out) {
                 rank_out[j] = moff + row;
             }
-            key = ((uint32_t)row << 12) | (uint32_t)j;
+            key[s] = ((uint32_t)row << 12) | (uint32_t)j;
+            digit[s] = row & (kRadix - 1);
         }
-        if (j < P) keys[j] = key;
     }
+    radix_places<T, E>(digit, place, hist, warp_sum + 32);
+#pragma unroll
+    for (int s = 0; s < E; ++s)
+        if (key[s] != 0xffffffffu) keys[place[s]] = key[s];
     __syncthreads();
-    for (int k = 2; k <= P; k <<= 1) {   // bitonic sort: the keys are distinct, so the order is unique
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-            for (int c = tid; c < (P >> 1); c += T) {   // comparator c of this stage: elements i and i + jj (bit jj of i clear)
-                const int i = ((c & ~(jj - 1)) << 1) | (c & (jj - 1));
-                const uint32_t x = keys[i], y = keys[i + jj];
-                if ((x > y) == ((i & k) == 0)) {
-                    keys[i] = y;
-                    keys[i + jj] = x;
-                }
-            }
-            __syncthreads();
+    if (n_kept >= kRadix) {   // (uniform; row n_kept may occur)
+#pragma unroll
+        for (int s = 0; s < E; ++s) {
+            const int j = (warp * E + s) * 32 + lane;
+            key[s] = j < n ? keys[j] : 0xffffffffu;
+            digit[s] = j < n ? (int)(key[s] >> 18) : kRadix;
         }
+        radix_places<T, E>(digit, place, hist, warp_sum + 32);   // (its barriers: every key has been read)
+#pragma unroll
+        for (int s = 0; s < E; ++s)
+            if (key[s] != 0xffffffffu) keys[place[s]] = key[s];
+        __syncthreads();
     }
     for (int i = tid; i <= n; i += T) {
         const int row = i < n ? (int)(keys[i] >> 12) : n_kept;
@@ -579,13 +627,13 @@ __device__ int build_groups(const int32_t* A, int block_start, int n, int limit,
     return n_kept;
 }
 
-template <int T>
-__global__ void __launch_bounds__(T, 1) big_merge_kernel(const MergeArgs a, int sp_chunks) {
+template <int T, int E>
+__global__ void __launch_bounds__(T, kSortedThreads / T) big_merge_kernel(const MergeArgs a, int sp_chunks) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
     uint32_t* keys = reinterpret_cast<uint32_t*>(mg_smem);                                     // [P] (merged row << 12) | position
-    int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (4 * T) * 4);            // [n] merged row of a kept token, -1
-    int* seg = reinterpret_cast<int*>(mg_smem + (4 * T) * 6);                       // [n_kept + 1] first sorted index of every merged row
-    int* warp_sum = seg + (4 * T) + 4;                                              // [32]
+    int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (E * T) * 4);            // [n] merged row of a kept token, -1
+    int* seg = reinterpret_cast<int*>(mg_smem + (E * T) * 6);                       // [n_kept + 1] first sorted index of every merged row
+    int* warp_sum = seg + (E * T) + 4;                                              // [32]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     depend_wait();
     dependents_launch();
@@ -605,7 +653,8 @@ __global__ void __launch_bounds__(T, 1) big_merge_kernel(const MergeArgs a, int 
         return;
     }
     const int per_map = a.heads * a.n_blocks;
-    const int m = blockIdx.x / per_map, h = (blockIdx.x % per_map) / a.n_blocks, b = blockIdx.x % a.n_blocks;
+    // (the K map, which also merges V, first: its CTAs take longer)
+    const int m = 1 - blockIdx.x / per_map, h = (blockIdx.x % per_map) / a.n_blocks, b = blockIdx.x % a.n_blocks;
     const BlockInfo bi = a.blocks[b];
     const int n = bi.n, r = m == 0 ? bi.r_q : bi.r_k, m_len = m == 0 ? a.m_q : a.m_k;
     const bool variable = m == 0 && a.moff_q_var != nullptr;   // after outlier filtering the kept count of a block varies by head
@@ -614,21 +663,18 @@ __global__ void __launch_bounds__(T, 1) big_merge_kernel(const MergeArgs a, int 
     const int64_t base = (int64_t)h * a.n_tokens + bi.start;
     const int32_t* A = a.assign[m] + base;
 
-    const int n_kept = build_groups<T>(A, bi.start, n, limit, keys, row_of, seg, warp_sum, nullptr, a.status, m == 0 ? a.rank_q + base : nullptr, moff);
+    const int n_kept = build_groups<T, E>(A, bi.start, n, limit, keys, row_of, seg, warp_sum, nullptr, a.status, m == 0 ? a.rank_q + base : nullptr, moff);
     // eight lanes per merged row (a lane owns one 16-byte chunk of the row), four rows per warp at a time, four
-    // members of a row in flight: the gather is bound by load latency, so it needs many loads in the air.  Member
-    // i of a row goes to accumulator i mod 4; the four are added in a fixed order: the result does not depend on
-    // scheduling.
+    // members of a row in flight: the gather is bound by load latency, so it needs many loads in the air.  The members are
+    // added in position order: the result does not depend on scheduling.
     for (int t = (m == 0 ? 0 : 1); t <= (m == 0 ? 0 : 2); ++t) {
         const __nv_bfloat16* x = a.xr[t] + base * kHeadDim;
         __nv_bfloat16* out = a.merged[t] + ((int64_t)h * m_len + moff) * kHeadDim;
         for (int row = warp * 4 + sub; row < n_kept; row += (T / 32) * 4) {
             const int i0 = seg[row], i1 = seg[row + 1];
-            float acc[4][8];
+            float acc[8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[u][e] = 0.f;
+            for (int e = 0; e < 8; ++e) acc[e] = 0.f;
             for (int i = i0; i < i1; i += 4) {
                 uint4 v[4];
 #pragma unroll
@@ -641,14 +687,14 @@ __global__ void __launch_bounds__(T, 1) big_merge_kernel(const MergeArgs a, int 
                     float f[8];
                     unpack8f(v[u], f);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[u][e] += f[e];
+                    for (int e = 0; e < 8; ++e) acc[e] += f[e];
                 }
             }
             if (i1 > i0) {
                 const float inv = 1.0f / (float)(i1 - i0);
                 float r8[8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) r8[e] = ((acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e])) * inv;
+                for (int e = 0; e < 8; ++e) r8[e] = acc[e] * inv;
                 uint4 o;
                 o.x = pack2(r8[0], r8[1]);
                 o.y = pack2(r8[2], r8[3]);
@@ -667,13 +713,13 @@ __global__ void __launch_bounds__(T, 1) big_merge_kernel(const MergeArgs a, int 
 // kernel.  One CTA per (head, block).
 
 // eps[h][p] = || q_p - mean of the group p was merged into ||_2 in fp32; 0 for a token on its own
-template <int T>
-__global__ void __launch_bounds__(T, 1) big_deviation_kernel(const OutlierArgs a) {
+template <int T, int E>
+__global__ void __launch_bounds__(T, kSortedThreads / T) big_deviation_kernel(const OutlierArgs a) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
     uint32_t* keys = reinterpret_cast<uint32_t*>(mg_smem);
-    int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (4 * T) * 4);
-    int* seg = reinterpret_cast<int*>(mg_smem + (4 * T) * 6);
-    int* warp_sum = seg + (4 * T) + 4;
+    int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (E * T) * 4);
+    int* seg = reinterpret_cast<int*>(mg_smem + (E * T) * 6);
+    int* warp_sum = seg + (E * T) + 4;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ch = lane & 7, sub = lane >> 3;
     const int h = blockIdx.x / a.n_blocks, b = blockIdx.x % a.n_blocks;
@@ -687,7 +733,7 @@ __global__ void __launch_bounds__(T, 1) big_deviation_kernel(const OutlierArgs a
         for (int j = tid; j < n; j += T) eps[j] = 0.f;
         return;
     }
-    const int n_kept = build_groups<T>(a.assign_q + base, bi.start, n, n, keys, row_of, seg, warp_sum, nullptr, a.status, nullptr, 0);
+    const int n_kept = build_groups<T, E>(a.assign_q + base, bi.start, n, n, keys, row_of, seg, warp_sum, nullptr, a.status, nullptr, 0);
     const __nv_bfloat16* x = a.src_q.ptr + (int64_t)h * a.src_q.stride_head + (int64_t)bi.start * a.src_q.stride_token;
     const int64_t st = a.src_q.stride_token;
     // eight lanes per group (a lane owns 8 of the 64 channels), four groups per warp at a time
@@ -699,11 +745,9 @@ __global__ void __launch_bounds__(T, 1) big_deviation_kernel(const OutlierArgs a
 #pragma unroll
         for (int e = 0; e < 8; ++e) mean[e] = 0.f;
         if (cnt >= 2) {
-            float acc[4][8];
+            float acc[8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) acc[u][e] = 0.f;
+            for (int e = 0; e < 8; ++e) acc[e] = 0.f;
             for (int i = i0; i < i1; i += 4) {
                 uint4 v[4];
 #pragma unroll
@@ -716,12 +760,12 @@ __global__ void __launch_bounds__(T, 1) big_deviation_kernel(const OutlierArgs a
                     float f[8];
                     unpack8f(v[u], f);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[u][e] += f[e];
+                    for (int e = 0; e < 8; ++e) acc[e] += f[e];
                 }
             }
             const float inv = 1.0f / (float)cnt;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) mean[e] = ((acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e])) * inv;   // kept in fp32
+            for (int e = 0; e < 8; ++e) mean[e] = acc[e] * inv;   // kept in fp32
         }
         // (the eight lanes of a group walk its members together: the trip count is the same in all of them); four members
         // at a time, so that four loads are in flight
@@ -756,16 +800,16 @@ __global__ void __launch_bounds__(T, 1) big_deviation_kernel(const OutlierArgs a
 
 // Outliers (eps > tau) leave their groups: an outlier maps to itself; the other tokens of a group stay together, under
 // their old representative if it is not an outlier, else under the remaining member with the lowest position.
-template <int T>
-__global__ void __launch_bounds__(T, 1) big_filter_kernel(const OutlierArgs a) {
+template <int T, int E>
+__global__ void __launch_bounds__(T, kSortedThreads / T) big_filter_kernel(const OutlierArgs a) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
     uint32_t* keys = reinterpret_cast<uint32_t*>(mg_smem);
-    int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (4 * T) * 4);
-    int* seg = reinterpret_cast<int*>(mg_smem + (4 * T) * 6);
-    int* warp_sum = seg + (4 * T) + 4;
-    int16_t* rep_of_row = reinterpret_cast<int16_t*>(mg_smem + mg_smem_bytes(T));
-    unsigned char* outl = mg_smem + mg_smem_bytes(T) + (4 * T) * 2;
-    int16_t* new_rep = reinterpret_cast<int16_t*>(mg_smem + mg_smem_bytes(T) + (4 * T) * 3);
+    int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (E * T) * 4);
+    int* seg = reinterpret_cast<int*>(mg_smem + (E * T) * 6);
+    int* warp_sum = seg + (E * T) + 4;
+    int16_t* rep_of_row = reinterpret_cast<int16_t*>(mg_smem + mg_smem_bytes(E * T));
+    unsigned char* outl = mg_smem + mg_smem_bytes(E * T) + (E * T) * 2;
+    int16_t* new_rep = reinterpret_cast<int16_t*>(mg_smem + mg_smem_bytes(E * T) + (E * T) * 3);
     __shared__ int s_kept, s_out;
     const int tid = threadIdx.x;
     const int h = blockIdx.x / a.n_blocks, b = blockIdx.x % a.n_blocks;
@@ -786,7 +830,7 @@ __global__ void __launch_bounds__(T, 1) big_filter_kernel(const OutlierArgs a) {
         s_out = 0;
     }
     const float tau = *a.tau;
-    const int n_kept = build_groups<T>(A, bi.start, n, n, keys, row_of, seg, warp_sum, rep_of_row, a.status, nullptr, 0);
+    const int n_kept = build_groups<T, E>(A, bi.start, n, n, keys, row_of, seg, warp_sum, rep_of_row, a.status, nullptr, 0);
     int n_out = 0;
     for (int j = tid; j < n; j += T) {
         const bool o = a.eps[base + j] > tau;
@@ -834,46 +878,47 @@ __global__ void __launch_bounds__(T, 1) big_filter_kernel(const OutlierArgs a) {
 
 }  // namespace
 
-// threads per CTA for blocks of up to max_block tokens
+// threads per CTA and tokens per thread for blocks of up to max_block tokens
 template <typename F>
 cudaError_t with_cta_size(int max_block, F&& f) {
-    if (max_block <= 256) return f(std::integral_constant<int, 64>{});
-    if (max_block <= 512) return f(std::integral_constant<int, 128>{});
-    if (max_block <= 1024) return f(std::integral_constant<int, 256>{});
-    if (max_block <= 2048) return f(std::integral_constant<int, 512>{});
-    return f(std::integral_constant<int, 1024>{});
+    using four = std::integral_constant<int, 4>;
+    if (max_block <= 256) return f(std::integral_constant<int, 64>{}, four{});
+    if (max_block <= 512) return f(std::integral_constant<int, 128>{}, four{});
+    if (max_block <= 1024) return f(std::integral_constant<int, 256>{}, four{});
+    if (max_block <= 2048) return f(std::integral_constant<int, 512>{}, four{});
+    return f(std::integral_constant<int, 512>{}, std::integral_constant<int, 8>{});
 }
 
 cudaError_t launch_big_deviation(const OutlierArgs& a, int max_block, cudaStream_t stream) {
-    return with_cta_size(max_block, [&](auto t) {
-        constexpr int T = decltype(t)::value;
-        return launch_kernel(big_deviation_kernel<T>, a.heads * a.n_blocks, T, mg_smem_bytes(T), stream, a);
+    return with_cta_size(max_block, [&](auto t, auto e) {
+        constexpr int T = decltype(t)::value, E = decltype(e)::value;
+        return launch_kernel(big_deviation_kernel<T, E>, a.heads * a.n_blocks, T, mg_smem_bytes(E * T), stream, a);
     });
 }
 
 cudaError_t launch_big_filter(const OutlierArgs& a, int max_block, cudaStream_t stream) {
-    return with_cta_size(max_block, [&](auto t) {
-        constexpr int T = decltype(t)::value;
-        return launch_kernel(big_filter_kernel<T>, a.heads * a.n_blocks, T, of_smem_bytes(T), stream, a);
+    return with_cta_size(max_block, [&](auto t, auto e) {
+        constexpr int T = decltype(t)::value, E = decltype(e)::value;
+        return launch_kernel(big_filter_kernel<T, E>, a.heads * a.n_blocks, T, of_smem_bytes(E * T), stream, a);
     });
 }
 
-template <int T>
+template <int T, int E>
 cudaError_t configure_sorted_group_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(big_merge_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, mg_smem_bytes(T));
+    cudaError_t e = cudaFuncSetAttribute(big_merge_kernel<T, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, mg_smem_bytes(E * T));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(big_deviation_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, mg_smem_bytes(T));
+    e = cudaFuncSetAttribute(big_deviation_kernel<T, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, mg_smem_bytes(E * T));
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(big_filter_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, of_smem_bytes(T));
+    return cudaFuncSetAttribute(big_filter_kernel<T, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, of_smem_bytes(E * T));
 }
 
 cudaError_t configure_big_blocks() {
     cudaError_t e = cudaFuncSetAttribute(big_scores_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM);
-    if (e == cudaSuccess) e = configure_sorted_group_kernels<64>();
-    if (e == cudaSuccess) e = configure_sorted_group_kernels<128>();
-    if (e == cudaSuccess) e = configure_sorted_group_kernels<256>();
-    if (e == cudaSuccess) e = configure_sorted_group_kernels<512>();
-    if (e == cudaSuccess) e = configure_sorted_group_kernels<1024>();
+    if (e == cudaSuccess) e = configure_sorted_group_kernels<64, 4>();
+    if (e == cudaSuccess) e = configure_sorted_group_kernels<128, 4>();
+    if (e == cudaSuccess) e = configure_sorted_group_kernels<256, 4>();
+    if (e == cudaSuccess) e = configure_sorted_group_kernels<512, 4>();
+    if (e == cudaSuccess) e = configure_sorted_group_kernels<512, 8>();
     return e;
 }
 
@@ -894,10 +939,10 @@ cudaError_t launch_big_select(const BigMatchArgs& a, cudaStream_t stream) {
 }
 
 cudaError_t launch_big_merge(const MergeArgs& a, int max_block, cudaStream_t stream) {
-    return with_cta_size(max_block, [&](auto t) {
-        constexpr int T = decltype(t)::value;
+    return with_cta_size(max_block, [&](auto t, auto e) {
+        constexpr int T = decltype(t)::value, E = decltype(e)::value;
         const int sp_chunks = (a.n_special_total + T / 8 - 1) / (T / 8);
-        return launch_kernel(big_merge_kernel<T>, 2 * a.heads * a.n_blocks + a.heads * sp_chunks, T, mg_smem_bytes(T), stream, a, sp_chunks);
+        return launch_kernel(big_merge_kernel<T, E>, 2 * a.heads * a.n_blocks + a.heads * sp_chunks, T, mg_smem_bytes(E * T), stream, a, sp_chunks);
     });
 }
 

@@ -95,3 +95,14 @@ def test_paper_block_regime_full_size_sampled():
     toks = np.unique(np.concatenate([rng.integers(0, wl.n_tokens, 24), [0, 4, 5, wl.n_tokens - 1]]))
     stats = run_big(wl, sample=toks)
     assert stats["out_err"] <= parity.OUT_TOL and stats["peaky_needed"] == 0
+
+
+@pytest.mark.parametrize("n", [511, 512, 513, 1023, 1025, 2047, 2048, 2049, 4095])
+def test_block_sizes_at_the_cta_size_limits(n):
+    """One block of n tokens per head: the sorted-group kernels take 4 tokens per thread of a 128 .. 512-thread CTA, 8 above
+    2048 tokens; many groups (two counting passes) for the queries, at most 64 (one pass) for the keys."""
+    wl = synth.Workload(f"one_block_{n}", 1, 1, n, 1, 1, n, 0.7, 1.0 - 60.0 / n, n_camera=0, n_register=2, heads=2, seed=n)
+    run_big(wl, peaky=True)
+    if n in (513, 2049):
+        from tests.test_gpu_outlier import run_filtered
+        run_filtered(wl, 0.1, peaky=True, launches=12)
