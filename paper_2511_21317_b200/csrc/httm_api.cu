@@ -52,6 +52,9 @@ struct httm_ctx {
     // path, so O_m does not hold its attention output (httm_export recomputes it on request).
     int32_t *d_group_start = nullptr, *d_group_member = nullptr;
     bool om_stale = false;
+    // query tiles of the merged attention that are split over CTAs (the last ones, where whole tiles would leave SMs idle)
+    float* d_partial = nullptr;
+    int32_t* d_part_count = nullptr;
     // first-frame anchoring: blocks of the first frame group (the first n_anchor blocks) with more dst tokens than the
     // match kernel holds (match_capacity) are matched by a kernel of their own, launched behind it
     int32_t n_anchor = 0, match_capacity = 0;
@@ -123,7 +126,7 @@ struct httm_ctx {
                         d_vr, d_qm,     d_km,       d_vm,       d_om,     hs[0].q,  hs[0].k,  hs[0].v, hs[0].out, hs[1].q, hs[1].k, hs[1].v, hs[1].out,
                         d_assign_qf, d_kept_cnt, d_moff_var, d_mq_head, d_tile_prefix, d_sel, d_eps, d_tau, d_qm_var, d_om_var,
                         d_big_items, d_inv_norm_q, d_inv_norm_k, d_best_key_q, d_best_key_k, d_best_pos_q, d_best_pos_k,
-                        d_group_start, d_group_member};
+                        d_group_start, d_group_member, d_partial, d_part_count};
         for (void* p : ptrs)
             if (p) cudaFree(p);
         for (HostSet& h : hs)
@@ -354,6 +357,8 @@ int stage_attention(httm_ctx* c, cudaStream_t s, const httm_tensor* final_out = 
     a.heads = c->cfg.heads;
     a.scale_log2 = scale_log2();
     a.status = c->d_status;
+    a.partial = c->d_partial;
+    a.part_count = c->d_part_count;
     c->launches++;
     return check_cuda(c, launch_attention(a, c->sm_count, s), "attention launch");
 }
@@ -616,6 +621,9 @@ int httm_create(const httm_config* cfg, httm_ctx** out) {
         (rc = c->alloc(&c->d_vm, H * c->m_k * kHeadDim)) || (rc = c->alloc(&c->d_om, H * c->m_q * kHeadDim)))
         return done(rc);
 
+    if ((rc = c->alloc(&c->d_partial, attention_partial_floats(c->sm_count))) || (rc = c->alloc(&c->d_part_count, attention_partial_counters(c->sm_count))))
+        return done(rc);
+    if ((rc = check_cuda(c, cudaMemset(c->d_part_count, 0, attention_partial_counters(c->sm_count) * 4), "workspace setup"))) return done(rc);
     if (c->max_block <= 32) {   // member lists of the merged query rows; entry M_q of every head is the constant N
         if ((rc = c->alloc(&c->d_group_start, H * (size_t)(c->m_q + 1))) || (rc = c->alloc(&c->d_group_member, H * N))) return done(rc);
         std::vector<int32_t> gs(H * (size_t)(c->m_q + 1), 0);

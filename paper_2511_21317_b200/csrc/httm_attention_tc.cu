@@ -51,6 +51,7 @@ struct Barriers {
     uint64_t x_full, x_done;         // single pass: tile B's (max, sum) published / tile A done reading O_B
     uint32_t tmem_base;
     int abort_flag;
+    int last_part;   // split tiles: this CTA's part was the tile's last to arrive
 };
 
 struct TcParams {
@@ -60,12 +61,15 @@ struct TcParams {
     float scale_log2;
     int32_t* status;
     int32_t tiles_per_head, total_tiles, rounds;  // query tiles per head and in all heads; rounds of pair passes
+    int32_t parts, singles;      // TailPlan (per-head query lengths: made on the device)
     const int32_t* mq_head;      // optional: per-head query length (then m_q is the row stride and tile_prefix the tile table)
     const int32_t* tile_prefix;
     int32_t heads;
     const int32_t* group_start;  // optional (UNMERGE): members of every merged query row, see AttentionArgs
     const int32_t* group_member;
     int32_t n_tokens;
+    float* partial;              // optional: partial results of query tiles that are split over CTAs, see TailPlan
+    int32_t* part_count;         // their arrivals, one counter per split tile, all zero between launches
     const __nv_bfloat16 *q, *k;  // the rows themselves, for the tile that is redone (element strides)
     int64_t q_stride_head, q_stride_token, k_stride_head, k_stride_token;
 };
@@ -81,31 +85,28 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
-// 2^t for two values without the special-function unit.  The arguments are clamped to [-125, 125] (an argument of
-// 125 or more gives 2^125, which the caller's test of the tile's row sum catches; without the clamps the exponent
-// arithmetic below would wrap).  Then round-to-nearest range reduction t = n + f, f in [-0.5, 0.5] (the integer lands
-// in the low mantissa bits of t + 1.5 * 2^23), a cubic minimax polynomial for 2^f (relative error < 1e-4, far below
-// the bf16 rounding of P) evaluated with packed fp32 FMAs, and n added to the exponent field.
-__device__ __forceinline__ float2 exp2_poly2(float2 t) {
-    const float kMagic = 12582912.0f;
-    t.x = fminf(fmaxf(t.x, -125.0f), 125.0f);
-    t.y = fminf(fmaxf(t.y, -125.0f), 125.0f);
-    const float2 tt = tc::fadd2(t, make_float2(kMagic, kMagic));
-    const float2 n = tc::fadd2(tt, make_float2(-kMagic, -kMagic));
-    const float2 f = tc::ffma2(n, make_float2(-1.0f, -1.0f), t);
+// 2^t for two values without the special-function unit.  The argument comes as u = (t + 125) / 250 clamped to [0, 1] by the
+// saturating multiply-add that scales the scores (an argument of 125 or more gives 2^125, which the caller's test of the
+// tile's row sum catches; without the clamp the exponent arithmetic below would wrap).  Then round-to-nearest range reduction
+// t = n + f, f in [-0.5, 0.5] (the integer lands in the low mantissa bits of t + 1.5 * 2^23), a cubic minimax polynomial for
+// 2^f (relative error < 1e-4, far below the bf16 rounding of P) evaluated with packed fp32 FMAs, and n added to the exponent
+// field.  16 cycles of the FMA pipe per pair and warp; min / max clamps took another 8 of the ALU.
+__device__ __forceinline__ float2 exp2_poly2(float2 u) {
+    const float kMagic = 12582912.0f - 125.0f;
+    const float2 magic = make_float2(kMagic, kMagic), width = make_float2(250.0f, 250.0f);
+    const float2 tt = tc::ffma2(u, width, magic);
+    const float2 f = tc::ffma2(u, width, tc::fsub2(magic, tt));
     float2 q = tc::ffma2(make_float2(0.055171460f, 0.055171460f), f, make_float2(0.24261086f, 0.24261086f));
     q = tc::ffma2(q, f, make_float2(0.69326097f, 0.69326097f));
     q = tc::ffma2(q, f, make_float2(0.99992812f, 0.99992812f));
     return make_float2(__int_as_float(__float_as_int(q.x) + (__float_as_int(tt.x) << 23)),
                        __int_as_float(__float_as_int(q.y) + (__float_as_int(tt.y) << 23)));
 }
-// Of every eight pairs of scores, the pairs whose bit is set here take the polynomial (FMA pipe), the
-// others ex2.approx (special-function unit, 16 results per clock per SM: with every exponential there,
-// the softmax of two query tiles needs 2048 cycles against 1056 of tensor-core work).  The polynomial
-// costs about ten issue slots per pair against two.  Measured at 10500 x 10500 x 16 heads with the
-// persistent kernel: 0/8: 545 us, 1/8: 510 us, 2/8: 481 us, 3/8: 497-504 us, 4/8: 570 us, 8/8: 790 us
-// (alternating 2/8 and 3/8 over the 16-column groups: 480 us).
-constexpr uint32_t kPolyPairs = 0x11;   // pairs 0 and 4 of 8
+// Of every sixteen pairs of scores, the pairs whose bit is set here take the polynomial (FMA pipe), the others ex2.approx
+// (special-function unit: 8 cycles per warp instruction and scheduler, so 1024 cycles for the 128 scores of a row against 528
+// of tensor-core work per tile).  Measured in the whole kernel, 10992 x 10992 x 16 heads: 4 of 16 with min / max clamps 520 us;
+// with the saturating form 4 of 16 515, 5 of 16 505 (other choices of five 511 .. 515), 6 of 16 529.
+constexpr uint32_t kPolyPairs = 0x9211;
 
 // A score tile whose weights overflowed with the stabiliser at hand is done again here, for one query row per thread:
 // its 128 scores are recomputed from the rows in global memory by plain fp32 FMAs (the tile in tensor memory is
@@ -173,29 +174,57 @@ __device__ __noinline__ RedoneTile redo_score_tile(const __nv_bfloat16* q_row, c
 
 // Work decomposition.  The query tiles of all heads form one list (head-major, T tiles).  With G CTAs
 // (one per SM), round r < R = T / (2 G) gives CTA c the two tiles 2 (r G + c), +1: a PAIR pass (tiles A and B
-// share the K/V stream) if they belong to the same head, else two single passes.  The remaining
-// T - 2 G R < 2 G tiles are one more partial round of pairs if there are more than G of them, else they are
-// dealt one per CTA as SINGLE passes: the same machinery with ONE query tile whose
-// even key tiles go to softmax group A / accumulator O_A and odd ones to group B / O_B (two partial
-// softmaxes over disjoint keys), combined in the epilogue; a single pass takes about half a pair pass.
-// Either way score tile k is handled by group k mod 2 in buffer k mod 3.  All CTAs work on neighbouring
-// tiles at any time (K/V of one or two heads stay in L2), and the SMs finish within half a pass of each
-// other, whereas a grid of 672 two-tile CTAs on 148 SMs runs 4.54 waves as 5.
+// share the K/V stream) if they belong to the same head, else two single passes.  A SINGLE pass is the same machinery with
+// ONE query tile whose even key tiles go to softmax group A / accumulator O_A and odd ones to group B / O_B (two partial
+// softmaxes over disjoint keys), combined in the epilogue; it takes about half a pair pass (1050 against 2094 cycles per key
+// tile).  Either way score tile k is handled by group k mod 2 in buffer k mod 3.
+// The remaining T - 2 G R < 2 G tiles are dealt by TailPlan.  All CTAs work on neighbouring tiles at any time (K/V of one
+// or two heads stay in L2).
+//
+// TailPlan: of the remaining tiles, G are dealt one per CTA as single passes if there are more than G; e < G are left.  Dealt
+// whole (one single pass on e of the CTAs) they take as long as one on every CTA.  Where e <= G / 2 each of them is split
+// into P = G / e parts of the keys, one per CTA: a part is a single pass over n / P key tiles that leaves its unnormalised
+// output, maxima and sums in a workspace, and the CTA whose part of a tile arrives last adds them up (nobody waits).  A part
+// costs about kPartCost key tiles besides its own, and single passes for all CTAs and then parts kPassCost more than a round
+// of pairs, hence the rule (3.03 tiles per SM of 28 key tiles: whole 127 us, split 143).  Where the tiles are not split and more than G remain they
+// go as one more (partial) round of pairs, which takes the same time as two rounds of single passes.
+// Measured (whole call, before / after): 9.19 tiles per SM of 83 key tiles 732 / 698 us, 14.05 of 195 3038 / 2922 us.
+constexpr int kPartCost = 14, kPassCost = 10, kMinPart = 8;
+constexpr int kPartFloats = BM * (kHeadDim + 2);   // one part: output [16][128 rows][4], then maxima [128], sums [128]
+struct TailPlan {
+    int parts;       // P, or 1
+    int singles;     // tiles dealt one per CTA ahead of the split ones: 0 or G
+    __host__ __device__ TailPlan(int tail, int n_tiles, int ctas) {
+        singles = tail > ctas ? ctas : 0;
+        const int e = tail - singles;
+        parts = 1;
+        if (e > 0 && 2 * e <= ctas) {
+            const int most = n_tiles / kMinPart, p = ctas / e < most ? ctas / e : most;
+            if (p > 1 && (n_tiles + p - 1) / p + kPartCost + (singles ? kPassCost : 0) < n_tiles) parts = p;
+        }
+        if (parts == 1) singles = 0;
+    }
+};
 struct Pass {
     int head, tile;   // tile = index of query tile A inside the head
+    int j0, n;        // its key tiles
+    int part;         // >= 0: index of this part (the P parts of a tile are consecutive); -1: the pass covers all keys
     bool pair;
 };
 template <bool VAR>   // VAR: the heads differ in query length (tile table in device memory)
 struct PassWalker {
     int r = 0, sub = 0;
-    int rounds, total, tiles_per_head;
+    int rounds, total, tiles_per_head, n_tiles, parts, singles;
     const int32_t* prefix;   // optional: first tile of every head (heads + 1 entries) when the heads differ in length
     int heads;
-    __device__ PassWalker(int rounds_, int total_, int tph, const int32_t* prefix_, int heads_)
-        : rounds(rounds_), total(total_), tiles_per_head(tph), prefix(prefix_), heads(heads_) {
+    __device__ PassWalker(const TcParams& p, const int32_t* prefix_, int n_tiles_)
+        : rounds(p.rounds), total(p.total_tiles), tiles_per_head(p.tiles_per_head), n_tiles(n_tiles_), parts(p.parts), singles(p.singles), prefix(prefix_), heads(p.heads) {
         if (VAR) {
             total = prefix[heads];
             rounds = total / (2 * (int)gridDim.x);
+            const TailPlan plan(total - 2 * (int)gridDim.x * rounds, n_tiles, gridDim.x);
+            parts = p.partial ? plan.parts : 1;
+            singles = p.partial ? plan.singles : 0;
         }
     }
     __device__ int head_of(int t) const {
@@ -214,6 +243,9 @@ struct PassWalker {
         ps->head = head_of(t);
         ps->tile = t - (VAR ? prefix[ps->head] : ps->head * tiles_per_head);
         ps->pair = pair;
+        ps->j0 = 0;
+        ps->n = n_tiles;
+        ps->part = -1;
     }
     __device__ bool same_head(int t) const {   // tiles t and t + 1
         if (!VAR) return t / tiles_per_head == (t + 1) / tiles_per_head;
@@ -222,7 +254,7 @@ struct PassWalker {
     __device__ bool next(Pass* ps) {
         const int G = gridDim.x, c = blockIdx.x;
         const int rem = total - 2 * G * rounds;               // tiles left after the full rounds, < 2 G
-        const int pair_rounds = rounds + (rem > G ? 1 : 0);   // more than G left: one more (partial) round of pairs
+        const int pair_rounds = rounds + (parts == 1 && rem > G ? 1 : 0);   // more than G left and not split: one more (partial) round of pairs
         if (r < pair_rounds) {
             const int t = 2 * (r * G + c);
             if (t + 1 < total && same_head(t)) {
@@ -239,17 +271,33 @@ struct PassWalker {
             r = pair_rounds + 1;
             return false;
         }
-        if (r > pair_rounds || rem > G) return false;
-        const int t = 2 * G * rounds + c;                     // at most G left: one single pass each
-        ++r;
-        if (t >= total) return false;
-        set(ps, t, false);
+        if (parts == 1) {
+            if (r > pair_rounds || rem > G) return false;
+            const int t = 2 * G * rounds + c;                     // at most G left: one single pass each
+            ++r;
+            if (t >= total) return false;
+            set(ps, t, false);
+            return true;
+        }
+        if (r == rounds && singles) {
+            ++r;
+            sub = 1;
+            set(ps, 2 * G * rounds + c, false);
+            return true;
+        }
+        if (r > rounds + sub || c >= (rem - singles) * parts) return false;
+        r = rounds + 2;
+        const int e = c / parts, i = c - e * parts;
+        set(ps, 2 * G * rounds + singles + e, false);
+        ps->j0 = n_tiles * i / parts;
+        ps->n = n_tiles * (i + 1) / parts - ps->j0;
+        ps->part = c;
         return true;
     }
 };
 // Completions a pass adds to each barrier family, so that every role can carry the phase parities from
 // pass to pass: stage st of the K/V ring completes once per key tile j with j mod 3 == st; score buffer b
-// once per score tile k with k mod 3 == b (2 n tiles in a pair pass, n in a single pass).
+// once per score tile k with k mod 3 == b (2 n tiles in a pair pass, n in a single pass), n key tiles in the pass.
 __device__ __forceinline__ int count_mod3(int n, int r) { return (n - r + 2) / 3; }
 
 // Where the 32 output rows of a softmax warp go.  UNMERGE (Eq. 5-7 folded into the epilogue): row `grow` is the attention
@@ -304,10 +352,90 @@ __device__ __forceinline__ void store_rows(const TcParams& p, int head, const ui
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
+// The end of a pass over part of the keys (group A's four warps, thread = row of the tile): the combined but unnormalised
+// output of both groups, the maximum and the sum go to the workspace.  The CTA that arrives last adds the parts of the tile
+// up, in the order of their keys, and sends the rows out.
+struct PartArgs {
+    int head, grow, mq_rows;          // this thread's row, rows of the head
+    int part, parts;                  // see TailPlan
+    uint32_t t_o, parity, x_parity;   // accumulator; phases of o_final and x_full
+    float m, l;                       // this row's stabiliser and sum of weights
+};
+template <bool UNMERGE>
+__device__ __noinline__ bool epilogue_part(const TcParams& p, const PartArgs& a, Barriers* bars, const float2* xch, unsigned char* stage, int row) {
+    volatile int* abort_flag = &bars->abort_flag;
+    const int lane = row & 31, part = a.part, parts = a.parts, first = part - part % parts;
+    if (!__all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->o_final), a.parity, abort_flag) &&
+                                     tc::mbar_wait(tc::smem_addr(&bars->x_full), a.x_parity, abort_flag)))
+        return false;
+    tc::fence_after_sync();
+    float* mine = p.partial + (int64_t)part * kPartFloats;
+    {
+        const float2 pb = *xch;
+        const float mm = fmaxf(a.m, pb.x);
+        const float fa = exp2f(a.m - mm), fb = exp2f(pb.x - mm);   // 2^(-inf) = 0 when group B had no key tile
+#pragma unroll 1
+        for (int c = 0; c < kHeadDim; c += 8) {
+            uint32_t oa[8], ob[8];
+            tc::tmem_ld8(a.t_o + c, oa);
+            tc::tmem_ld8(a.t_o + kHeadDim + c, ob);   // O_B sits right behind O_A; same TMEM lanes
+            tc::tmem_wait_ld();
+            float o[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o[i] = fmaf(__uint_as_float(oa[i]), fa, __uint_as_float(ob[i]) * fb);
+            __stcg(reinterpret_cast<float4*>(mine) + (c >> 2) * BM + row, make_float4(o[0], o[1], o[2], o[3]));
+            __stcg(reinterpret_cast<float4*>(mine) + (c >> 2) * BM + BM + row, make_float4(o[4], o[5], o[6], o[7]));
+        }
+        __stcg(mine + BM * kHeadDim + row, mm);
+        __stcg(mine + BM * (kHeadDim + 1) + row, a.l * fa + pb.y * fb);
+    }
+    tc::fence_before_sync();
+    tc::mbar_arrive(tc::smem_addr(&bars->x_done));
+    asm volatile("bar.sync 1, 128;" ::: "memory");   // every row of this part has been written
+    if (row == 0) {
+        int32_t* count = p.part_count + first / parts;
+        __threadfence();
+        const bool last = atomicAdd(count, 1) == parts - 1;
+        if (last) *count = 0;   // (as the next launch finds it)
+        __threadfence();
+        bars->last_part = last;
+    }
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (!bars->last_part) return true;   // (a CTA has one part: the flag is not written again)
+    const RowTargets targets = row_targets<UNMERGE>(p, a.head, a.grow, a.grow < a.mq_rows);
+    const float* other = p.partial + (int64_t)first * kPartFloats;
+    float top = -INFINITY, sum = 0.f, o[kHeadDim];
+#pragma unroll 4
+    for (int i = 0; i < parts; ++i) top = fmaxf(top, __ldcg(other + (int64_t)i * kPartFloats + BM * kHeadDim + row));
+#pragma unroll
+    for (int i = 0; i < kHeadDim; ++i) o[i] = 0.f;
+#pragma unroll 1
+    for (int i = 0; i < parts; ++i, other += kPartFloats) {
+        const float f = exp2f(__ldcg(other + BM * kHeadDim + row) - top);
+        sum = fmaf(__ldcg(other + BM * (kHeadDim + 1) + row), f, sum);
+#pragma unroll
+        for (int q = 0; q < kHeadDim / 4; ++q) {
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(other) + q * BM + row);
+            o[4 * q] = fmaf(v.x, f, o[4 * q]);
+            o[4 * q + 1] = fmaf(v.y, f, o[4 * q + 1]);
+            o[4 * q + 2] = fmaf(v.z, f, o[4 * q + 2]);
+            o[4 * q + 3] = fmaf(v.w, f, o[4 * q + 3]);
+        }
+    }
+    const float inv = 1.0f / sum;
+    uint4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        v[i] = make_uint4(pack_bf16(o[8 * i] * inv, o[8 * i + 1] * inv), pack_bf16(o[8 * i + 2] * inv, o[8 * i + 3] * inv),
+                          pack_bf16(o[8 * i + 4] * inv, o[8 * i + 5] * inv), pack_bf16(o[8 * i + 6] * inv, o[8 * i + 7] * inv));
+    store_rows<UNMERGE>(p, a.head, v, targets, stage, lane);
+    return true;
+}
+
 template <bool VAR, bool UNMERGE>
 __global__ void __launch_bounds__(NTHREADS, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                    const __grid_constant__ CUtensorMap map_v, const TcParams p) {
+                    const __grid_constant__ CUtensorMap map_v, const __grid_constant__ TcParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t s_q = tc::smem_addr(smem);                             // 2 tiles
@@ -318,7 +446,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n_tiles = (p.m_k + BN - 1) / BN;
-    const int kv_cnt[3] = {count_mod3(n_tiles, 0), count_mod3(n_tiles, 1), count_mod3(n_tiles, 2)};   // per pass
 
     if (tid == 0) {
         bars->abort_flag = 0;
@@ -363,7 +490,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     const uint32_t tmem = bars->tmem_base;
     // columns: score buffers [0,128) [128,256) [256,384); O_A [384,448)  O_B [448,512); P overlays the last 64 columns of its S
     const int32_t* mq_table = tables_on_chip ? s_mq : p.mq_head;
-    PassWalker<VAR> walker(p.rounds, p.total_tiles, p.tiles_per_head, tables_on_chip ? s_prefix : p.tile_prefix, p.heads);
+    PassWalker<VAR> walker(p, tables_on_chip ? s_prefix : p.tile_prefix, n_tiles);
     Pass ps;
 
     if (warp == 0) {
@@ -379,22 +506,22 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 tc::tma_load_3d(s_q, &map_q, qb, 0, ps.tile * BM, ps.head);
                 if (ps.pair) tc::tma_load_3d(s_q + TILE_BYTES, &map_q, qb, 0, (ps.tile + 1) * BM, ps.head);
                 bool ok = true;
-                for (int j = 0; j < n_tiles; ++j) {
+                for (int j = 0; j < ps.n; ++j) {
                     const int st = j % KV_STAGES;
                     const uint32_t fill = kv_base[st] + (uint32_t)(j / KV_STAGES);         // completion index of tile j in stage st
                     const uint32_t par = fill & 1u;
                     if (fill > 0 && !(ok = tc::mbar_wait(tc::smem_addr(&bars->k_empty[st]), par ^ 1u, abort_flag))) break;
                     const uint32_t kb = tc::smem_addr(&bars->k_full[st]);
                     tc::mbar_expect_tx(kb, TILE_BYTES);
-                    tc::tma_load_3d(s_k + st * TILE_BYTES, &map_k, kb, 0, j * BN, ps.head);
+                    tc::tma_load_3d(s_k + st * TILE_BYTES, &map_k, kb, 0, (ps.j0 + j) * BN, ps.head);
                     if (fill > 0 && !(ok = tc::mbar_wait(tc::smem_addr(&bars->v_empty[st]), par ^ 1u, abort_flag))) break;
                     const uint32_t vb = tc::smem_addr(&bars->v_full[st]);
                     tc::mbar_expect_tx(vb, TILE_BYTES);
-                    tc::tma_load_3d(s_v + st * TILE_BYTES, &map_v, vb, 0, j * BN, ps.head);
+                    tc::tma_load_3d(s_v + st * TILE_BYTES, &map_v, vb, 0, (ps.j0 + j) * BN, ps.head);
                 }
                 if (!ok) break;
 #pragma unroll
-                for (int st = 0; st < 3; ++st) kv_base[st] += (uint32_t)kv_cnt[st];
+                for (int st = 0; st < 3; ++st) kv_base[st] += (uint32_t)count_mod3(ps.n, st);
             }
         }
         __syncwarp();
@@ -449,7 +576,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
             };
             // SINGLE pass, score tile k = key tile k = k0 + C with k0 a multiple of 6: buffer and ring stage k mod 3,
             // softmax group and accumulator k mod 2.
-            auto step_single = [&](auto c_c, int k0) -> bool {
+            auto step_single = [&](auto c_c, int k0, int n_single) -> bool {
                 constexpr int C = decltype(c_c)::value;
                 constexpr int B = C % 3, X = C % 2;
                 constexpr uint32_t IDX = C / 3;   // completion index of this tile in its buffer / stage, modulo 2 (k0 / 3 is even)
@@ -460,12 +587,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 issue_pv(t_o, t_buf + kPColumn, dv0 + B * kStageStep);
                 tc::mma_commit(tc::smem_addr(&bars->o_done[X]));
                 tc::mma_commit(tc::smem_addr(&bars->v_empty[B]));
-                if (k0 + C + 3 < n_tiles) {
+                if (k0 + C + 3 < n_single) {
                     if (!tc::mbar_wait(tc::smem_addr(&bars->k_full[B]), (kv_base[B] + IDX + 1u) & 1u, abort_flag)) return false;
                     tc::fence_after_sync();
                     issue_qk(t_buf, dq0, dk0 + B * kStageStep, tc::smem_addr(&bars->s_full[B]));
                     tc::mma_commit(tc::smem_addr(&bars->k_empty[B]));
-                    if (k0 + C + 4 == n_tiles) tc::mma_commit(tc::smem_addr(&bars->q_free));   // that was the last S of the pass
+                    if (k0 + C + 4 == n_single) tc::mma_commit(tc::smem_addr(&bars->q_free));   // that was the last S of the pass
                 }
                 return true;
             };
@@ -477,7 +604,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 if (!ok) break;
                 tc::fence_after_sync();
                 if (ps.pair) {
-                    const int n_score = 2 * n_tiles;   // score tiles k = 2 j + x
+                    const int n_score = 2 * ps.n;   // score tiles k = 2 j + x
                     // prologue: S(0), S(1) from key tile 0, S(2) from key tile 1
                     issue_qk(tmem, dq0, dk0, tc::smem_addr(&bars->s_full[0]));
                     issue_qk(tmem + BN, dq0 + kStageStep, dk0, tc::smem_addr(&bars->s_full[1]));
@@ -500,36 +627,37 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 #pragma unroll
                     for (int b = 0; b < 3; ++b) sp_base[b] += (uint32_t)count_mod3(n_score, b);
                 } else {
+                    const int n_single = ps.n;
                     // prologue: S(0), S(1), S(2) from key tiles 0, 1, 2
                     issue_qk(tmem, dq0, dk0, tc::smem_addr(&bars->s_full[0]));
                     tc::mma_commit(tc::smem_addr(&bars->k_empty[0]));
-                    if (n_tiles > 1) {
+                    if (n_single > 1) {
                         if (!(ok = tc::mbar_wait(tc::smem_addr(&bars->k_full[1]), kv_base[1] & 1u, abort_flag))) break;
                         tc::fence_after_sync();
                         issue_qk(tmem + BN, dq0, dk0 + kStageStep, tc::smem_addr(&bars->s_full[1]));
                         tc::mma_commit(tc::smem_addr(&bars->k_empty[1]));
                     }
-                    if (n_tiles > 2) {
+                    if (n_single > 2) {
                         if (!(ok = tc::mbar_wait(tc::smem_addr(&bars->k_full[2]), kv_base[2] & 1u, abort_flag))) break;
                         tc::fence_after_sync();
                         issue_qk(tmem + 2 * BN, dq0, dk0 + 2 * kStageStep, tc::smem_addr(&bars->s_full[2]));
                         tc::mma_commit(tc::smem_addr(&bars->k_empty[2]));
                     }
-                    if (n_tiles <= 3) tc::mma_commit(tc::smem_addr(&bars->q_free));
-                    for (int k0 = 0; ok && k0 < n_tiles; k0 += 6) {
-                        ok = step_single(std::integral_constant<int, 0>{}, k0);
-                        if (ok && k0 + 1 < n_tiles) ok = step_single(std::integral_constant<int, 1>{}, k0);
-                        if (ok && k0 + 2 < n_tiles) ok = step_single(std::integral_constant<int, 2>{}, k0);
-                        if (ok && k0 + 3 < n_tiles) ok = step_single(std::integral_constant<int, 3>{}, k0);
-                        if (ok && k0 + 4 < n_tiles) ok = step_single(std::integral_constant<int, 4>{}, k0);
-                        if (ok && k0 + 5 < n_tiles) ok = step_single(std::integral_constant<int, 5>{}, k0);
+                    if (n_single <= 3) tc::mma_commit(tc::smem_addr(&bars->q_free));
+                    for (int k0 = 0; ok && k0 < n_single; k0 += 6) {
+                        ok = step_single(std::integral_constant<int, 0>{}, k0, n_single);
+                        if (ok && k0 + 1 < n_single) ok = step_single(std::integral_constant<int, 1>{}, k0, n_single);
+                        if (ok && k0 + 2 < n_single) ok = step_single(std::integral_constant<int, 2>{}, k0, n_single);
+                        if (ok && k0 + 3 < n_single) ok = step_single(std::integral_constant<int, 3>{}, k0, n_single);
+                        if (ok && k0 + 4 < n_single) ok = step_single(std::integral_constant<int, 4>{}, k0, n_single);
+                        if (ok && k0 + 5 < n_single) ok = step_single(std::integral_constant<int, 5>{}, k0, n_single);
                     }
 #pragma unroll
-                    for (int b = 0; b < 3; ++b) sp_base[b] += (uint32_t)count_mod3(n_tiles, b);
+                    for (int b = 0; b < 3; ++b) sp_base[b] += (uint32_t)count_mod3(n_single, b);
                 }
                 if (ok) tc::mma_commit(tc::smem_addr(&bars->o_final));
 #pragma unroll
-                for (int st = 0; st < 3; ++st) kv_base[st] += (uint32_t)kv_cnt[st];
+                for (int st = 0; st < 3; ++st) kv_base[st] += (uint32_t)count_mod3(ps.n, st);
             }
         }
         __syncwarp();
@@ -548,14 +676,12 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                                    (warp - 2) * 32 * kOutRowPitch;   // this warp's 32 output rows
         bool ok = true;
         for (int pass = 0; ok && walker.next(&ps); ++pass) {
-            const int n_score = ps.pair ? 2 * n_tiles : n_tiles;
+            const int n_score = ps.pair ? 2 * ps.n : ps.n;
             const int mq_rows = VAR ? mq_table[ps.head] : p.m_q;   // valid query rows of this head
             // this group's score tiles are k = 2 i + x; in a pair pass they come from key tile i, in a single pass from key tile k
-            const int n_own = ps.pair ? n_tiles : (n_tiles - x + 1) / 2;
+            const int n_own = ps.pair ? ps.n : (ps.n - x + 1) / 2;
             const int own_row = (ps.tile + (ps.pair ? x : 0)) * BM + row;   // this thread's query row inside the head
             const bool row_exists = own_row < mq_rows;
-            const __nv_bfloat16* q_row = row_exists ? p.q + (int64_t)ps.head * p.q_stride_head + (int64_t)own_row * p.q_stride_token : nullptr;
-            const __nv_bfloat16* k_head = p.k + (int64_t)ps.head * p.k_stride_head;
             {
                 float m = -INFINITY, l = 0.f;
                 {   // the accumulator O starts at zero: every PV step accumulates (ordered before the first p_full arrival)
@@ -568,11 +694,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 }
                 for (int j = 0; j < n_own; ++j) {
                     const int k = 2 * j + x, buf = k % 3;                      // score tile and its buffer
-                    const int key_tile = ps.pair ? j : k;
+                    const int key_tile = ps.j0 + (ps.pair ? j : k);
                     const uint32_t kpar = (sp_base[buf] + (uint32_t)(k / 3)) & 1u;
                     const uint32_t t_s = tmem + buf * BN + lane_addr;
                     const uint32_t sbar = tc::smem_addr(&bars->s_full[buf]), pbar = tc::smem_addr(&bars->p_full[buf]);
-                    if (!(ok = tc::mbar_wait(sbar, kpar, abort_flag))) break;
+                    if (!(ok = __all_sync(0xffffffffu, tc::mbar_wait(sbar, kpar, abort_flag)))) break;   // (the warp gives up together)
                     tc::fence_after_sync();
                     uint32_t s[BN];   // fp32 bit patterns of this row of S
 #pragma unroll
@@ -608,14 +734,21 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                     };
                     auto weights = [&]() {   // P = 2^(s c - m) as bf16 pairs over the LAST 64 columns of S; returns the row sum
                         const float2 c2 = make_float2(c, c), neg_m2 = make_float2(-m, -m);
+                        const float cu = c * (1.0f / 250.0f), mu = (125.0f - m) * (1.0f / 250.0f);
                         float2 sum0 = make_float2(0.f, 0.f), sum1 = sum0;
 #pragma unroll
                         for (int cc = 0; cc < 8; ++cc) {
                             uint32_t pk[8];
 #pragma unroll
                             for (int i = 0; i < 8; ++i) {
-                                const float2 t = tc::ffma2(make_float2(__uint_as_float(s[cc * 16 + 2 * i]), __uint_as_float(s[cc * 16 + 2 * i + 1])), c2, neg_m2);
-                                const float2 e = ((kPolyPairs >> i) & 1u) ? exp2_poly2(t) : make_float2(fast_exp2(t.x), fast_exp2(t.y));
+                                const float sx = __uint_as_float(s[cc * 16 + 2 * i]), sy = __uint_as_float(s[cc * 16 + 2 * i + 1]);
+                                float2 e;
+                                if ((kPolyPairs >> ((cc & 1) * 8 + i)) & 1u) {
+                                    e = exp2_poly2(make_float2(tc::ffma_sat(sx, cu, mu), tc::ffma_sat(sy, cu, mu)));
+                                } else {
+                                    const float2 t = tc::ffma2(make_float2(sx, sy), c2, neg_m2);
+                                    e = make_float2(fast_exp2(t.x), fast_exp2(t.y));
+                                }
                                 if (i & 1)
                                     sum1 = tc::fadd2(sum1, e);
                                 else
@@ -629,8 +762,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                     if (j == 0) m = row_max() * c;
                     float tile_sum = weights();
                     if (j > 0 && __any_sync(0xffffffffu, row_exists && !(tile_sum < kSumLimit))) {
-                        if (!(ok = tc::mbar_wait(obar, (od_base + (uint32_t)(j - 1)) & 1u, abort_flag))) break;
+                        if (!(ok = __all_sync(0xffffffffu, tc::mbar_wait(obar, (od_base + (uint32_t)(j - 1)) & 1u, abort_flag)))) break;
                         tc::fence_after_sync();
+                        const __nv_bfloat16* q_row = row_exists ? p.q + (int64_t)ps.head * p.q_stride_head + (int64_t)own_row * p.q_stride_token : nullptr;
+                        const __nv_bfloat16* k_head = p.k + (int64_t)ps.head * p.k_stride_head;
                         const RedoneTile redone = redo_score_tile(q_row, k_head + (int64_t)key_tile * BN * p.k_stride_token, p.k_stride_token,
                                                                   valid < BN ? valid : BN, c, m, t_s + kPColumn);
                         const float f = exp2f(m - redone.m);
@@ -678,6 +813,19 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                     xch[row] = make_float2(m, l);
                     tc::mbar_arrive(tc::smem_addr(&bars->x_full));
                     ok = tc::mbar_wait(tc::smem_addr(&bars->x_done), n_single & 1u, abort_flag);
+                } else if (ok && ps.part >= 0) {
+                    PartArgs pa;
+                    pa.head = ps.head;
+                    pa.grow = own_row;
+                    pa.mq_rows = mq_rows;
+                    pa.part = ps.part;
+                    pa.parts = walker.parts;
+                    pa.t_o = t_o;
+                    pa.parity = (uint32_t)pass & 1u;
+                    pa.x_parity = n_single & 1u;
+                    pa.m = m;
+                    pa.l = l;
+                    ok = epilogue_part<UNMERGE>(p, pa, bars, xch + row, out_stage, row);
                 } else if (ok) {
                     // single pass, group A: combine the two partial softmaxes over disjoint keys
                     //   out = (O_A 2^(m_A - m) + O_B 2^(m_B - m)) / (l_A 2^(m_A - m) + l_B 2^(m_B - m)),  m = max(m_A, m_B)
@@ -730,6 +878,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
 }  // namespace
 
+// at most one part per CTA, of at most half as many tiles
+size_t attention_partial_floats(int sm_count) { return (size_t)sm_count * kPartFloats; }
+size_t attention_partial_counters(int sm_count) { return (size_t)sm_count; }
+
 cudaError_t configure_attention() {
     cudaError_t e = cudaFuncSetAttribute(attention_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e != cudaSuccess) return e;
@@ -746,12 +898,16 @@ cudaError_t launch_attention(const AttentionArgs& a, int sm_count, cudaStream_t 
         !encode_rows_tensor_map(&mv, a.v.ptr, a.m_k, a.heads, a.v.stride_token, a.v.stride_head, BN))
         return cudaErrorInvalidValue;
     const int tiles_per_head = (a.m_q + BM - 1) / BM, total = tiles_per_head * a.heads;
-    // one CTA per SM (fewer when there are fewer tiles)
+    // one CTA per SM (fewer when there are fewer tiles, unless they are split)
     int ctas = sm_count < 1 ? 1 : sm_count;
-    if (ctas > total) ctas = total;
+    const int n_tiles = (a.m_k + BN - 1) / BN;
+    TailPlan plan(total - total / (2 * ctas) * 2 * ctas, n_tiles, ctas);
+    if (!a.partial) plan.parts = 1, plan.singles = 0;
+    if (ctas > total && plan.parts == 1) ctas = total;
     const int rounds = total / (2 * ctas);
-    TcParams p{a.out, a.out_stride_head, a.out_stride_token, a.m_q, a.m_k, a.scale_log2, a.status, tiles_per_head, total, rounds, a.mq_head, a.tile_prefix, a.heads,
-               a.group_start, a.group_member, a.n_tokens, a.q.ptr, a.k.ptr, a.q.stride_head, a.q.stride_token, a.k.stride_head, a.k.stride_token};
+    TcParams p{a.out, a.out_stride_head, a.out_stride_token, a.m_q, a.m_k, a.scale_log2, a.status, tiles_per_head, total, rounds, plan.parts, plan.singles,
+               a.mq_head, a.tile_prefix, a.heads, a.group_start, a.group_member, a.n_tokens, a.partial, a.part_count, a.q.ptr, a.k.ptr, a.q.stride_head,
+               a.q.stride_token, a.k.stride_head, a.k.stride_token};
     if (a.mq_head) {   // the tile table lives in device memory: full grid, CTAs without tiles leave at once
         if (a.group_start) return cudaErrorInvalidValue;   // (the member lists are built for equal query lengths only)
         return launch_kernel(attention_tc_kernel<true, false>, sm_count < 1 ? 1 : sm_count, NTHREADS, SMEM_BYTES, stream, mq, mk, mv, p);

@@ -174,6 +174,10 @@ struct AttentionArgs {
     const int32_t* group_start;
     const int32_t* group_member;
     int32_t n_tokens;
+    // optional: workspace for query tiles that are split over CTAs (attention_partial_floats / _counters; the counters are zero
+    // before the first launch and after every launch); null: tiles are dealt whole.  Launches that share it run in order.
+    float* partial;
+    int32_t* part_count;
 };
 
 struct LinearArgs {   // y[n_rows][out] = x[n_rows][in] . w[out][in]^T, leading dimensions in elements
@@ -210,6 +214,8 @@ cudaError_t launch_linear(const LinearArgs& a, int sm_count, cudaStream_t stream
 cudaError_t configure_linear();
 cudaError_t launch_attention(const AttentionArgs& a, int sm_count, cudaStream_t stream);   // tcgen05 / TMEM kernel
 cudaError_t configure_attention();
+size_t attention_partial_floats(int sm_count);
+size_t attention_partial_counters(int sm_count);
 cudaError_t configure_kernels();   // one-time function attributes (dynamic shared memory sizes)
 cudaError_t launch_wait_expiry(const void* tiles, float* scratch, int32_t* status, cudaStream_t stream);   // time-out path test, see httm_umma_selftest.cu
 
