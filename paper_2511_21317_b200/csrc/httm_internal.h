@@ -28,7 +28,7 @@ enum : int {
 // r_* = number of src tokens merged away, nd_* = number of dst tokens,
 // moff_* = merged row of the block's first kept token (closed form: the per-block kept
 // count n - r is the same for every head).
-struct BlockInfo {
+struct alignas(16) BlockInfo {   // (fetched as three 16-byte words)
     int32_t start, n;
     int32_t r_q, nd_q, moff_q;
     int32_t r_k, nd_k, moff_k;
@@ -41,8 +41,8 @@ struct BlockInfo {
 // Where a merging block sits in the original layout (used when the kernels read the blocks straight from
 // Q/K/V with tiled TMA loads instead of from the reordered copies): first frame, first patch row and
 // column, and the clipped extents.
-struct BlockGeom {
-    int16_t s0, y0, x0, frames, rows, cols;   // rows x cols patches over `frames` frames; 12 bytes
+struct alignas(16) BlockGeom {
+    int16_t s0, y0, x0, frames, rows, cols;   // rows x cols patches over `frames` frames; fetched as one 16-byte word
 };
 // Geometry of the original token layout: token (frame s, in-frame index p) is row s * tokens_per_frame + p;
 // patch (y, x) has p = n_special + y * grid_w + x.
@@ -196,6 +196,9 @@ cudaError_t launch_match(const MatchArgs& a, int max_block_tokens, int sm_count,
 cudaError_t launch_match_anchor(const MatchArgs& a, const TensorView& src_q, const TensorView& src_k, const int32_t* pi, int n_anchor,
                                 int main_capacity, int max_block_tokens, cudaStream_t stream);
 cudaError_t launch_merge(const MergeArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream);
+cudaError_t launch_match_small(const MatchArgs& a, int sm_count, cudaStream_t stream);   // blocks of at most 32 tokens
+cudaError_t launch_merge_small(const MergeArgs& a, int sm_count, cudaStream_t stream);
+cudaError_t configure_small_blocks();
 cudaError_t launch_unmerge(const UnmergeArgs& a, cudaStream_t stream);
 cudaError_t launch_deviation(const OutlierArgs& a, int sm_count, cudaStream_t stream);
 cudaError_t launch_threshold(const OutlierArgs& a, int sm_count, cudaStream_t stream);

@@ -2,41 +2,9 @@
 // cosine matching, mean merge, and unmerge + inverse reorder.  sm_100a only.
 #include "httm_internal.h"
 #include "httm_launch.cuh"
-#include "tc_sm100.cuh"   // mbarrier / TMA wrappers (device), tensor-map encoders (host)
+#include "httm_blocks.cuh"
 
 namespace httm {
-
-// ------------------------------------------------------------------------------------
-// small device helpers (mbarrier and address wrappers: tc_sm100.cuh)
-// ------------------------------------------------------------------------------------
-using tc::mbar_expect_tx;
-using tc::mbar_init;
-using tc::mbar_try_wait;
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return tc::smem_addr(p); }
-// Bounded wait of the warp-per-block kernels: gives up after about two seconds, records `code` in the
-// status word and returns false.  Never spins forever.
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t mbar, uint32_t parity, int32_t* status, int code) {
-    if (mbar_try_wait(mbar, parity)) return true;
-    const uint64_t t0 = tc::timer_ns();
-    for (;;) {
-        for (int i = 0; i < 64; ++i)
-            if (mbar_try_wait(mbar, parity)) return true;
-        if (tc::timer_ns() - t0 > 2000000000ull) {
-            atomicCAS(status, kDevOk, code);
-            return false;
-        }
-    }
-}
-__device__ __forceinline__ void unpack8(const uint4& raw, float* f) {
-    f[0] = __uint_as_float(raw.x << 16);
-    f[1] = __uint_as_float(raw.x & 0xffff0000u);
-    f[2] = __uint_as_float(raw.y << 16);
-    f[3] = __uint_as_float(raw.y & 0xffff0000u);
-    f[4] = __uint_as_float(raw.z << 16);
-    f[5] = __uint_as_float(raw.z & 0xffff0000u);
-    f[6] = __uint_as_float(raw.w << 16);
-    f[7] = __uint_as_float(raw.w & 0xffff0000u);
-}
 
 // ------------------------------------------------------------------------------------
 // a1. Temporal reorder (Sec. 3.3; Algorithm 1 "Reorder"): xr[h][p'] = x[h][pi[p']]
@@ -95,42 +63,6 @@ cudaError_t launch_reorder(const ReorderArgs& a, cudaStream_t stream) {
 }
 
 // ------------------------------------------------------------------------------------
-// Task cursor: (tensor t, head h, unit u) of a linear task index that advances by a fixed
-// stride, kept up to date with carries instead of 64-bit divisions in the loop.
-// ------------------------------------------------------------------------------------
-struct TaskCursor {
-    int t, h, u;
-    int st, sh, su;        // the stride, decomposed the same way
-    int heads, units;
-    __device__ void init(int64_t first, int64_t stride, int heads_, int units_) {
-        heads = heads_;
-        units = units_;
-        const int64_t per_tensor = (int64_t)heads * units;
-        t = (int)(first / per_tensor);
-        int64_t rem = first - t * per_tensor;
-        h = (int)(rem / units);
-        u = (int)(rem - (int64_t)h * units);
-        st = (int)(stride / per_tensor);
-        rem = stride - st * per_tensor;
-        sh = (int)(rem / units);
-        su = (int)(rem - (int64_t)sh * units);
-    }
-    __device__ __forceinline__ void advance() {
-        u += su;
-        if (u >= units) {
-            u -= units;
-            ++h;
-        }
-        h += sh;
-        if (h >= heads) {
-            h -= heads;
-            ++t;
-        }
-        t += st;
-    }
-};
-
-// ------------------------------------------------------------------------------------
 // a2. Block-wise bipartite matching (Eq. 1; Sec. 3.2 top-r rule), one warp per
 //     (tensor in {Q, K}, head, block).  The block (n x 64 bf16, contiguous after the
 //     reorder) is staged in shared memory by a tiled TMA load with the 128-byte swizzle,
@@ -156,65 +88,6 @@ __host__ __device__ constexpr int match_stages(int nmax) { return nmax <= 32 ? 2
 __host__ __device__ constexpr int match_aux_bytes(int nmax) { return nmax * 4 + 16; }   // inverse norms + 2 mbarriers
 __host__ __device__ constexpr int match_smem_bytes(int nmax) {
     return match_warps_per_cta(nmax) * (match_stages(nmax) * nmax * kRowBytes + match_aux_bytes(nmax)) + 1024 /*alignment slack*/;
-}
-
-// tiled TMA load {64 channels, rows, heads} -> this CTA's shared memory; the channel coordinate is 0
-__device__ __forceinline__ void tma_rows_load(uint32_t dst_smem, const CUtensorMap* map, uint32_t mbar, int row, int head) {
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(
-                     dst_smem),
-                 "l"(reinterpret_cast<uint64_t>(map)), "r"(mbar), "r"(0), "r"(row), "r"(head)
-                 : "memory");
-}
-__device__ __forceinline__ void ldmatrix_x4(uint32_t* r, uint32_t saddr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(saddr)
-                 : "memory");
-}
-// c (16x8 fp32) += a (16x16 bf16, row) * b (16x8 bf16, col)
-__device__ __forceinline__ void mma_bf16_16816(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// tiled TMA load of one merging block straight from an original tensor: {64 channels, x, y, frame, head}
-__device__ __forceinline__ void tma_block_load(uint32_t dst_smem, const CUtensorMap* map, uint32_t mbar, int x0, int y0, int s0, int head) {
-    asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(dst_smem),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(mbar), "r"(0), "r"(x0), "r"(y0), "r"(s0), "r"(head)
-        : "memory");
-}
-// Direct mode: a block arrives as the box [box_frames][box_h][box_w] of 128-byte rows (zero rows where the block
-// is clipped by the grid edge or the last frame); its tokens are numbered in the same (frame, row, column)
-// order without the holes.  For a block that is not clipped both numberings coincide.
-struct BoxMap {
-    int box_h, box_w;          // rows and columns of the box
-    int rows, cols;            // of this block
-    uint32_t m_plane, m_cols;  // multipliers for floor(j / (rows * cols)) and floor(j / cols), j < 256
-    bool clipped;
-    __device__ void set(int box_frames, int bh, int bw, int frames, int r, int c) {
-        box_h = bh;
-        box_w = bw;
-        rows = r;
-        cols = c;
-        clipped = frames != box_frames || r != bh || c != bw;
-        if (clipped) {
-            m_plane = 65536u / (uint32_t)(r * c) + 1u;
-            m_cols = 65536u / (uint32_t)c + 1u;
-        }
-    }
-    // token number -> box row
-    __device__ __forceinline__ int row_of_token(int j) const {
-        if (!clipped) return j;
-        const int t = (int)(((uint32_t)j * m_plane) >> 16), rem = j - t * rows * cols;
-        const int y = (int)(((uint32_t)rem * m_cols) >> 16), x = rem - y * cols;
-        return (t * box_h + y) * box_w + x;
-    }
-};
-// monotone map float -> uint32 (larger float <-> larger key); every real score maps to a key >= 1
-__device__ __forceinline__ uint32_t score_key(float s) {
-    const uint32_t b = __float_as_uint(s);
-    return b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u);
 }
 
 template <int PASSES, bool DIRECT>
@@ -520,14 +393,6 @@ match_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
     }
 }
 
-// 5-D map of the patch tokens of an original tensor with one merging block as the box
-static bool encode_block_map(CUtensorMap* map, const TensorView& t, const SourceLayout& L, int heads) {
-    const int bw = L.blk_w < L.grid_w ? L.blk_w : L.grid_w, bh = L.blk_h < L.grid_h ? L.blk_h : L.grid_h,
-              bf = L.blk_frames < L.frames ? L.blk_frames : L.frames;
-    return encode_patch_tensor_map(map, t.ptr + (int64_t)L.n_special * t.stride_token, L.grid_w, L.grid_h, L.frames, heads, t.stride_token,
-                                   L.tokens_per_frame, t.stride_head, bw, bh, bf);
-}
-
 template <int PASSES>
 static cudaError_t launch_match_t(const MatchArgs& a, int sm_count, cudaStream_t stream) {
     constexpr int NMAX = 32 * PASSES;
@@ -649,331 +514,10 @@ cudaError_t launch_match_anchor(const MatchArgs& a, const TensorView& src_q, con
 }
 
 cudaError_t launch_match(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
-    if (max_block_tokens <= 32) return launch_match_t<1>(a, sm_count, stream);
+    if (max_block_tokens <= 32) return launch_match_small(a, sm_count, stream);
     if (max_block_tokens <= 64) return launch_match_t<2>(a, sm_count, stream);
     if (max_block_tokens <= 128) return launch_match_t<4>(a, sm_count, stream);
     return launch_match_t<8>(a, sm_count, stream);
-}
-
-// ------------------------------------------------------------------------------------
-// a3 (blocks of at most 32 tokens).  The group sums of a block are one small dense
-//     contraction: merged_sum[kept row][channel] = sum_token W[row][token] x[token][channel]
-//     with the 0/1 assignment matrix W.  It runs on the tensor cores (m16n8k16, bf16 inputs,
-//     fp32 accumulation: W is exact in bf16, the products are exact, and the measured
-//     accumulation error is below that of an fp32 add chain).  W is built in registers from
-//     the map; x comes from the swizzled TMA stage through ldmatrix.trans (conflict free).
-//     The mean is the sum times the reciprocal of the group size, rounded once to bf16.
-//     One warp per (tensor, head, block); kept tokens are compacted in reordered order.
-// ------------------------------------------------------------------------------------
-constexpr int kMergeTcWarps = 8;
-constexpr int kMergeTcAux = 32 * 4 + 16 + 32 * 4;   // reciprocal group sizes per kept row + 2 mbarriers + group sizes / starts
-constexpr int kMergeTcSmem = kMergeTcWarps * (2 * 32 * kRowBytes + kMergeTcAux) + 1024 /*alignment slack*/;
-
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t* r, uint32_t saddr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(saddr)
-                 : "memory");
-}
-
-// DIRECT: the blocks come straight from the original tensors (5-D block maps), the special tokens frame by
-// frame (4-D frame maps sq, sk, sv); otherwise from the reordered copies, specials in chunks of 32.
-template <bool DIRECT>
-__global__ void __launch_bounds__(kMergeTcWarps * 32, 2)
-merge_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_sq,
-                const __grid_constant__ CUtensorMap map_sk, const __grid_constant__ CUtensorMap map_sv, const MergeArgs a) {
-    constexpr uint32_t STAGE_BYTES = 32 * kRowBytes;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 2, tq = lane & 3;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
-    unsigned char* stage = smem + (size_t)warp * 2 * STAGE_BYTES;                       // [2][32][128], 1024-aligned, swizzled
-    unsigned char* aux = smem + (size_t)kMergeTcWarps * 2 * STAGE_BYTES + (size_t)warp * kMergeTcAux;
-    float* rcnt = reinterpret_cast<float*>(aux);                                        // [32] 1 / group size of kept row
-    const uint32_t mbar0 = smem_u32(aux + 32 * 4), stage0 = smem_u32(stage);
-    int* gsz = reinterpret_cast<int*>(aux + 32 * 4 + 16);                               // [32] size, then first member, of kept row
-
-    if (lane == 0) {
-        mbar_init(mbar0, 1);
-        mbar_init(mbar0 + 8, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncwarp();
-
-    // task -> (tensor t, head h, unit u); units 0 .. n_blocks-1 are merging blocks, the rest are
-    // chunks of 32 special tokens (never merged: rows 0 .. n_special_total-1 are copied)
-    const int sp_chunks = DIRECT ? (a.layout.n_special > 0 ? a.layout.frames : 0) : (a.n_special_total + 31) / 32;
-    const int per_head = a.n_blocks + sp_chunks;
-    const int box_f = DIRECT ? min(a.layout.blk_frames, a.layout.frames) : 1, box_h = DIRECT ? min(a.layout.blk_h, a.layout.grid_h) : 1,
-              box_w = DIRECT ? min(a.layout.blk_w, a.layout.grid_w) : 1;
-    const int box_rows = box_f * box_h * box_w;
-    const int own_t = DIRECT ? lane / (box_h * box_w) : 0, own_y = DIRECT ? (lane / box_w) % box_h : 0, own_x = DIRECT ? lane % box_w : 0;
-    if (DIRECT) {   // stage rows that no block load writes enter the MMAs with weight 0: they must hold finite values
-        for (int q = box_rows * 8 + lane; q < 32 * 8; q += 32) {   // (a load of special tokens may overwrite some of them later)
-            *reinterpret_cast<uint4*>(stage + q * 16) = make_uint4(0u, 0u, 0u, 0u);
-            *reinterpret_cast<uint4*>(stage + STAGE_BYTES + q * 16) = make_uint4(0u, 0u, 0u, 0u);
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-    }
-    BoxMap bm;
-    bm.clipped = false;
-    const int64_t n_tasks = 3ll * a.heads * per_head;
-    const int64_t stride = (int64_t)gridDim.x * kMergeTcWarps;
-    const int64_t first = (int64_t)blockIdx.x * kMergeTcWarps + warp;
-    TaskCursor cur, nxt;   // the task being processed; the task whose load is issued next
-    cur.init(first, stride, a.heads, per_head);
-    nxt = cur;
-
-    auto unit_start = [&](const TaskCursor& c) { return c.u >= a.n_blocks ? (c.u - a.n_blocks) * 32 : __ldg(&a.blocks[c.u].start); };
-    auto issue = [&](const TaskCursor& c, int buf) {   // lane 0 only; the whole 32-row box is transferred (rows past the head's end are zero filled)
-        const uint32_t mb = mbar0 + 8 * buf;
-        if (!DIRECT) {
-            mbar_expect_tx(mb, STAGE_BYTES);
-            tma_rows_load(stage0 + buf * STAGE_BYTES, c.t == 0 ? &map_q : (c.t == 1 ? &map_k : &map_v), mb, unit_start(c), c.h);
-        } else if (c.u >= a.n_blocks) {   // the special tokens of frame u - n_blocks
-            mbar_expect_tx(mb, (uint32_t)a.layout.n_special * kRowBytes);
-            const CUtensorMap* m = c.t == 0 ? &map_sq : (c.t == 1 ? &map_sk : &map_sv);
-            asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(
-                             stage0 + buf * STAGE_BYTES),
-                         "l"(reinterpret_cast<uint64_t>(m)), "r"(mb), "r"(0), "r"(0), "r"(c.u - a.n_blocks), "r"(c.h)
-                         : "memory");
-        } else {
-            const BlockGeom bg = a.geom[c.u];
-            mbar_expect_tx(mb, (uint32_t)box_rows * kRowBytes);
-            tma_block_load(stage0 + buf * STAGE_BYTES, c.t == 0 ? &map_q : (c.t == 1 ? &map_k : &map_v), mb, bg.x0, bg.y0, bg.s0, c.h);
-        }
-    };
-    depend_wait();
-    dependents_launch();
-    if (first < n_tasks && lane == 0) issue(nxt, 0);
-    nxt.advance();
-    if (first + stride < n_tasks && lane == 0) issue(nxt, 1);
-    nxt.advance();
-
-    // Everything a task needs besides the staged rows: its place in the tables, and this lane's map entry.
-    // Both are fetched one task ahead (table entry at the start of the previous task, map entry behind its
-    // MMAs), so that their global-memory latency is not paid between waiting for a stage and using it.
-    struct Meta {
-        int t, h, start, n, r, moff;
-        bool special;
-        BlockGeom bg;
-    };
-    auto load_meta = [&](const TaskCursor& c) {
-        Meta m{};
-        m.t = c.t;
-        m.h = c.h;
-        m.special = c.u >= a.n_blocks;
-        if (m.special) {
-            m.start = DIRECT ? (c.u - a.n_blocks) * a.layout.n_special : (c.u - a.n_blocks) * 32;
-            m.n = DIRECT ? a.layout.n_special : min(32, a.n_special_total - m.start);
-            m.r = 0;
-            m.moff = m.start;
-        } else {
-            if (DIRECT) m.bg = a.geom[c.u];
-            const BlockInfo bi = a.blocks[c.u];
-            m.start = bi.start;
-            m.n = bi.n;
-            m.r = c.t == 0 ? bi.r_q : bi.r_k;
-            m.moff = c.t == 0 ? (a.moff_q_var ? ld_global(a.moff_q_var + (int64_t)c.h * a.n_blocks + c.u) : bi.moff_q) : bi.moff_k;
-        }
-        return m;
-    };
-    // lane = row of the stage; number of the token it holds in the block (-1: none)
-    auto token_of_lane = [&](const Meta& m) {
-        return !DIRECT || m.special ? (lane < m.n ? lane : -1)
-                                    : ((own_t < m.bg.frames && own_y < m.bg.rows && own_x < m.bg.cols) ? (own_t * m.bg.rows + own_y) * m.bg.cols + own_x : -1);
-    };
-    auto load_target = [&](const Meta& m) {   // token this lane's token is merged into (number in the block), -1 if the lane holds none
-        const int tok = token_of_lane(m);
-        return m.r > 0 && tok >= 0 ? ld_global(a.assign[m.t == 0 ? 0 : 1] + (int64_t)m.h * a.n_tokens + m.start + tok) - m.start : -1;
-    };
-    Meta meta_next{};
-    int target_next = -1;
-    if (first < n_tasks) {
-        meta_next = load_meta(cur);
-        target_next = load_target(meta_next);
-    }
-    TaskCursor ahead = cur;   // the task after the current one
-    ahead.advance();
-
-    int it = 0;
-    bool failed = false;
-    for (int64_t task = first; task < n_tasks; task += stride, ++it, cur.advance(), nxt.advance(), ahead.advance()) {
-        const int buf = it & 1;
-        const uint32_t parity = (it >> 1) & 1;
-        const bool more = task + 2 * stride < n_tasks, has_next = task + stride < n_tasks;
-        const Meta meta = meta_next;
-        int rep = target_next;
-        if (has_next) meta_next = load_meta(ahead);   // in flight while this task is processed
-        const int t = meta.t, h = meta.h, start = meta.start, n = meta.n, r = meta.r, moff = meta.moff;
-        const bool special = meta.special;
-        const BlockGeom bg = meta.bg;
-        if (DIRECT && !special) bm.set(box_f, box_h, box_w, bg.frames, bg.rows, bg.cols);
-        if (special) bm.clipped = false;
-        const int m_len = t == 0 ? a.m_q : a.m_k;
-        uint32_t* out = reinterpret_cast<uint32_t*>(a.merged[t] + ((int64_t)h * m_len + moff) * kHeadDim);   // 32 words per row
-        const uint32_t blk = stage0 + buf * STAGE_BYTES;
-        const int tok = token_of_lane(meta);
-        // rep = ROW of the stage holding the token this lane's token is merged into
-        if (r > 0 && tok >= 0) {
-            if (rep < 0 || rep >= n) {   // corrupt map: record, treat as kept
-                atomicCAS(a.status, kDevOk, kDevBadIndex);
-                rep = tok;
-            }
-            if (DIRECT) rep = bm.row_of_token(rep);
-        } else {
-            rep = -1;
-        }
-        if (!mbar_wait_bounded(mbar0 + 8 * buf, parity, a.status, kDevTimeoutMatchLoad)) {
-            failed = true;
-            break;
-        }
-        if (r == 0) {   // nothing merges here: copy the rows, 16 bytes per lane (chunk c of row j sits at c ^ (j & 7))
-            const unsigned char* sb = stage + buf * STAGE_BYTES;
-            uint4* o4 = reinterpret_cast<uint4*>(out);
-            for (int q = lane; q < n * 8; q += 32) {
-                const int row = DIRECT ? bm.row_of_token(q >> 3) : q >> 3, ch = q & 7;
-                o4[q] = *reinterpret_cast<const uint4*>(sb + row * kRowBytes + ((ch ^ (row & 7)) << 4));
-            }
-            if (t == 0 && !special && lane < n) a.rank_q[(int64_t)h * a.n_tokens + start + lane] = moff + lane;
-            if (t == 0 && a.group_start && lane < n) {   // every token is a group of its own
-                a.group_start[(int64_t)h * (a.m_q + 1) + moff + lane] = start + lane;
-                a.group_member[(int64_t)h * a.n_tokens + start + lane] = __ldg(a.pi + start + lane);
-            }
-            if (has_next) target_next = load_target(meta_next);
-        } else {
-            // merged row of every token: rank of its representative among the kept tokens
-            const unsigned kept = __ballot_sync(0xffffffffu, rep == lane);   // rep == -1 for lanes >= n
-            const int n_kept = __popc(kept);
-            const int row_of = rep >= 0 ? __popc(kept & ((1u << rep) - 1u)) : -1;
-            if (t == 0 && tok >= 0) a.rank_q[(int64_t)h * a.n_tokens + start + tok] = moff + row_of;
-            const unsigned group = __match_any_sync(0xffffffffu, row_of);
-            if (rep == lane) rcnt[row_of] = 1.0f / (float)__popc(group);
-            if (t == 0 && a.group_start) {
-                // member lists of the merged rows: the block's tokens group by group, kept rows in rank order
-                // (first member of row k = tokens of the rows before it: a warp scan over the group sizes)
-                if (rep == lane) gsz[row_of] = __popc(group);
-                __syncwarp();
-                const int sz = lane < n_kept ? gsz[lane] : 0;
-                int incl = sz;
-#pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int v = __shfl_up_sync(0xffffffffu, incl, off);
-                    if (lane >= off) incl += v;
-                }
-                __syncwarp();   // every size has been read
-                if (lane < n_kept) {
-                    gsz[lane] = incl - sz;
-                    a.group_start[(int64_t)h * (a.m_q + 1) + moff + lane] = start + incl - sz;
-                }
-                __syncwarp();
-                if (tok >= 0) {   // the token's number in the original order: from the block's place in the scene, or through the reorder index
-                    const int orig = DIRECT ? (bg.s0 + own_t) * a.layout.tokens_per_frame + a.layout.n_special + (bg.y0 + own_y) * a.layout.grid_w + bg.x0 + own_x
-                                            : __ldg(a.pi + start + tok);
-                    a.group_member[(int64_t)h * a.n_tokens + start + gsz[row_of] + __popc(group & ((1u << lane) - 1u))] = orig;
-                }
-            }
-            // x fragments: for k step ks (16 tokens) and channel tile pair np, one ldmatrix.x4.trans gives
-            // b0, b1 of channel tile 2 np and b0, b1 of channel tile 2 np + 1
-            uint32_t bf[2][4][4];
-            const int n_ks = (DIRECT ? box_rows : n) > 16 ? 2 : 1;   // rows of the stage that may hold tokens
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-                if (ks < n_ks) {
-                    const int tok = 16 * ks + (lane & 7) + ((lane >> 3) & 1) * 8;
-                    const uint32_t rowaddr = blk + tok * kRowBytes;
-#pragma unroll
-                    for (int np = 0; np < 4; ++np) ldmatrix_x4_trans(bf[ks][np], rowaddr + (((2 * np + (lane >> 4)) ^ (tok & 7)) << 4));
-                }
-            }
-            // W fragments need the rows of tokens 16 ks + {2 tq, 2 tq + 1, 2 tq + 8, 2 tq + 9}
-            int rw[2][4];
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-                rw[ks][0] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq);
-                rw[ks][1] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 1);
-                rw[ks][2] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 8);
-                rw[ks][3] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 9);
-            }
-            __syncwarp();   // reciprocal group sizes visible; every lane has its fragments: the stage can be refilled
-            if (more && lane == 0) issue(nxt, buf);
-            const int n_mt = n_kept > 16 ? 2 : 1;
-#pragma unroll 1
-            for (int mt = 0; mt < n_mt; ++mt) {
-                const int r0 = 16 * mt + g, r1 = r0 + 8;   // this lane's two accumulator rows
-                float c[8][4];
-#pragma unroll
-                for (int nt = 0; nt < 8; ++nt) c[nt][0] = c[nt][1] = c[nt][2] = c[nt][3] = 0.f;
-#pragma unroll
-                for (int ks = 0; ks < 2; ++ks) {
-                    if (ks < n_ks) {
-                        uint32_t af[4];   // bf16 1.0 = 0x3f80
-                        af[0] = (rw[ks][0] == r0 ? 0x3f80u : 0u) | (rw[ks][1] == r0 ? 0x3f800000u : 0u);
-                        af[1] = (rw[ks][0] == r1 ? 0x3f80u : 0u) | (rw[ks][1] == r1 ? 0x3f800000u : 0u);
-                        af[2] = (rw[ks][2] == r0 ? 0x3f80u : 0u) | (rw[ks][3] == r0 ? 0x3f800000u : 0u);
-                        af[3] = (rw[ks][2] == r1 ? 0x3f80u : 0u) | (rw[ks][3] == r1 ? 0x3f800000u : 0u);
-#pragma unroll
-                        for (int nt = 0; nt < 8; ++nt)
-                            mma_bf16_16816(c[nt], af, bf[ks][nt >> 1][2 * (nt & 1)], bf[ks][nt >> 1][2 * (nt & 1) + 1]);
-                    }
-                }
-                if (mt == 0 && has_next) target_next = load_target(meta_next);   // behind this task's MMAs
-                const int cap = t == 0 && a.moff_q_var ? n : n - r;   // (a corrupt map cannot overrun; after outlier filtering more than n - r may be kept)
-                const bool w0 = r0 < n_kept && r0 < cap, w1 = r1 < n_kept && r1 < cap;
-                const float i0 = w0 ? rcnt[r0] : 0.f, i1 = w1 ? rcnt[r1] : 0.f;
-#pragma unroll
-                for (int nt = 0; nt < 8; ++nt) {
-                    if (w0) {
-                        const __nv_bfloat162 o = __floats2bfloat162_rn(c[nt][0] * i0, c[nt][1] * i0);
-                        out[r0 * 32 + nt * 4 + tq] = *reinterpret_cast<const uint32_t*>(&o);
-                    }
-                    if (w1) {
-                        const __nv_bfloat162 o = __floats2bfloat162_rn(c[nt][2] * i1, c[nt][3] * i1);
-                        out[r1 * 32 + nt * 4 + tq] = *reinterpret_cast<const uint32_t*>(&o);
-                    }
-                }
-            }
-            __syncwarp();   // every lane is done with the reciprocals before the next task rewrites them
-            continue;
-        }
-        __syncwarp();   // every lane is done reading this stage buffer
-        if (more && lane == 0) issue(nxt, buf);
-    }
-    if (failed) {
-        mbar_wait_bounded(mbar0, (it >> 1) & 1, a.status, kDevTimeoutMatchLoad);
-        mbar_wait_bounded(mbar0 + 8, (it >> 1) & 1, a.status, kDevTimeoutMatchLoad);
-    }
-}
-
-static cudaError_t launch_merge_tc(const MergeArgs& a, int sm_count, cudaStream_t stream) {
-    CUtensorMap m[3], sp[3];
-    const int64_t N = a.n_tokens;
-    const bool direct = a.geom != nullptr;
-    const int sp_units = direct ? (a.layout.n_special > 0 ? a.layout.frames : 0) : (a.n_special_total + 31) / 32;
-    for (int t = 0; t < 3; ++t) {
-        if (direct) {
-            if (!encode_block_map(&m[t], a.src[t], a.layout, a.heads)) return cudaErrorInvalidValue;
-            if (a.layout.n_special > 0 &&
-                !encode_frame_tensor_map(&sp[t], a.src[t].ptr, a.layout.tokens_per_frame, a.layout.frames, a.heads, a.src[t].stride_token,
-                                         a.src[t].stride_head, a.layout.n_special))
-                return cudaErrorInvalidValue;
-            if (a.layout.n_special <= 0) sp[t] = m[t];   // never used
-        } else {
-            if (!encode_rows_tensor_map(&m[t], a.xr[t], N, a.heads, kHeadDim, N * kHeadDim, 32)) return cudaErrorInvalidValue;
-            sp[t] = m[t];   // not used
-        }
-    }
-    const int64_t n_tasks = 3ll * a.heads * (a.n_blocks + sp_units);
-    int64_t grid = (n_tasks + kMergeTcWarps - 1) / kMergeTcWarps;
-    const int64_t cap = (int64_t)sm_count * 2;
-    if (grid > cap) grid = cap;
-    if (grid < 1) grid = 1;
-    if (direct)
-        return launch_kernel(merge_tc_kernel<true>, (unsigned)grid, kMergeTcWarps * 32, kMergeTcSmem, stream, m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
-    return launch_kernel(merge_tc_kernel<false>, (unsigned)grid, kMergeTcWarps * 32, kMergeTcSmem, stream, m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
 }
 
 // ------------------------------------------------------------------------------------
@@ -1259,7 +803,7 @@ static cudaError_t launch_merge_multi(const MergeArgs& a, int sm_count, cudaStre
 }
 
 cudaError_t launch_merge(const MergeArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
-    if (max_block_tokens <= 32) return launch_merge_tc(a, sm_count, stream);
+    if (max_block_tokens <= 32) return launch_merge_small(a, sm_count, stream);
     if (max_block_tokens <= 64) return launch_merge_multi<2>(a, sm_count, stream);
     if (max_block_tokens <= 128) return launch_merge_multi<4>(a, sm_count, stream);
     return launch_merge_multi<8>(a, sm_count, stream);
@@ -1785,8 +1329,6 @@ cudaError_t configure_kernels() {
 #define HTTM_SET_SMEM(kern, bytes)                                                                      \
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bytes));          \
     if (e != cudaSuccess) return e;
-    HTTM_SET_SMEM((match_kernel<1, false>), match_smem_bytes(32));
-    HTTM_SET_SMEM((match_kernel<1, true>), match_smem_bytes(32));
     HTTM_SET_SMEM((match_kernel<2, false>), match_smem_bytes(64));
     HTTM_SET_SMEM((match_kernel<2, true>), match_smem_bytes(64));
     HTTM_SET_SMEM((match_kernel<4, true>), match_smem_bytes(128));
@@ -1794,8 +1336,6 @@ cudaError_t configure_kernels() {
     HTTM_SET_SMEM((match_kernel<4, false>), match_smem_bytes(128));
     HTTM_SET_SMEM((match_kernel<8, false>), match_smem_bytes(256));
     HTTM_SET_SMEM(deviation_kernel, kDevSmem);
-    HTTM_SET_SMEM(merge_tc_kernel<false>, kMergeTcSmem);
-    HTTM_SET_SMEM(merge_tc_kernel<true>, kMergeTcSmem);
     HTTM_SET_SMEM((merge_multi_kernel<2, false>), merge_multi_smem(64));
     HTTM_SET_SMEM((merge_multi_kernel<4, false>), merge_multi_smem(128));
     HTTM_SET_SMEM((merge_multi_kernel<8, false>), merge_multi_smem(256));
@@ -1803,6 +1343,7 @@ cudaError_t configure_kernels() {
     HTTM_SET_SMEM((merge_multi_kernel<4, true>), merge_multi_smem(128));
     HTTM_SET_SMEM((merge_multi_kernel<8, true>), merge_multi_smem(256));
 #undef HTTM_SET_SMEM
+    if ((e = configure_small_blocks()) != cudaSuccess) return e;
     return configure_attention();
 }
 

@@ -1,0 +1,699 @@
+// Matching and merging for merging blocks of at most 32 tokens (Eq. 1, Sec. 3.2), one warp per UNIT = one (head, block) with all
+// its tensors: the match kernel works off Q and K of a block, the merge kernel Q, K and V (V follows K's map).
+//
+// A block is 4 KB and 5 KFLOP per tensor, so what bounds these kernels is not the arithmetic but the instructions around it:
+// table entries, block geometry, dst positions, the next load.  With one task per (tensor, head, block) the match kernel
+// issued 697 warp instructions per task and the merge kernel 575, at 50 - 56 % of the issue slots with 16 warps per SM.  Here
+//   - table entry, geometry and cursor are taken once per unit, one unit ahead;
+//   - what a lane needs to know about a block's shape (which rows hold its dst tokens, which tokens it owns) is kept from block
+//     to block and recomputed when the shape changes (clipped blocks at the edges of the grid);
+//   - K's groups serve V, and the maps are read once per unit;
+//   - results leave through the stage as whole rows instead of 4 bytes per lane.
+// Measured at 32 976 tokens x 16 heads, 32-token blocks: match 53 -> 39.6 us, merge 69.6 -> 66.4 us (both
+// with the interval between two events).
+#include "httm_blocks.cuh"
+#include "httm_launch.cuh"
+
+namespace httm {
+
+namespace {
+
+constexpr int kWarps = 8;
+constexpr uint32_t kStage = 32 * kRowBytes;   // one block of one tensor, 128-byte swizzle
+
+// (head, unit of the head) of a linear index that advances by a fixed stride
+struct UnitCursor {
+    int h, u, sh, su, units;
+    __device__ void init(int first, int stride, int units_) {
+        units = units_;
+        h = first / units;
+        u = first - h * units;
+        sh = stride / units;
+        su = stride - sh * units;
+    }
+    __device__ __forceinline__ void advance() {
+        h += sh;
+        u += su;
+        if (u >= units) {
+            u -= units;
+            ++h;
+        }
+    }
+};
+
+struct Geometry {   // BlockGeom in registers
+    int s0, y0, x0, frames, rows, cols;
+};
+__device__ __forceinline__ int4 load_geometry(const BlockGeom* geom, int u) { return __ldg(reinterpret_cast<const int4*>(geom + u)); }
+__device__ __forceinline__ Geometry unpack_geometry(const int4& v) {
+    Geometry g;
+    g.s0 = (int16_t)(v.x & 0xffff);
+    g.y0 = v.x >> 16;
+    g.x0 = (int16_t)(v.y & 0xffff);
+    g.frames = v.y >> 16;
+    g.rows = (int16_t)(v.z & 0xffff);
+    g.cols = v.z >> 16;
+    return g;
+}
+// d (16x8 fp32) = a (16x16 bf16, row) * b (16x8 bf16, col): the first step of a sum
+__device__ __forceinline__ void mma_first(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
+}
+// floor(x / d) for 0 <= x < 2048, 1 <= d <= 64: (x + 0.5) / d is at least 1 / 128 away from an integer, far more than the error of the
+// approximate quotient
+__device__ __forceinline__ int small_div(int x, int d) { return (int)__fdividef((float)x + 0.5f, (float)d); }
+struct Box {   // extents of a block's TMA box (the block shape, clipped to the scene)
+    int frames, h, w, rows;
+    __device__ void set(const SourceLayout& L) {
+        frames = min(L.blk_frames, L.frames);
+        h = min(L.blk_h, L.grid_h);
+        w = min(L.blk_w, L.grid_w);
+        rows = frames * h * w;
+    }
+};
+// stage row of token j of a block
+__device__ __forceinline__ int row_of_token(const Box& box, const Geometry& g, int j) {
+    if (g.rows == box.h && g.cols == box.w) return j;   // (frames come last: clipping them leaves the numbering alone)
+    const int plane = g.rows * g.cols, t = small_div(j, plane), rem = j - t * plane, y = small_div(rem, g.cols);
+    return (t * box.h + y) * box.w + rem - y * g.cols;
+}
+// token number of stage row rho, -1 if the row holds none
+__device__ __forceinline__ int token_of_row(const Box& box, const Geometry& g, int rho) {
+    const int line = small_div(rho, box.w), t = small_div(line, box.h), y = line - t * box.h, x = rho - line * box.w;
+    return t < g.frames && y < g.rows && x < g.cols ? (t * g.rows + y) * g.cols + x : -1;
+}
+
+// ------------------------------------------------------------------------------------ match
+// Per tensor: cosine of every token with every dst token (at most 8), best dst per src token, the r best src tokens
+// merge; ties go to the lowest dst and the lowest src position.  The dot products and the squared norms (diagonals of a tile
+// against itself) are m16n8k16 MMAs on ldmatrix fragments of the swizzled stage; the dst rows are gathered by giving
+// ldmatrix their addresses.  Products of bf16 values are exact in fp32.
+// Row rho of the stage is owned, from the arg-max on, by lane (rho & 7) * 4 + ((rho >> 3) & 1), slot rho >> 4.
+constexpr int kMatchSmem = kWarps * (2 * (int)kStage + 16) + 1024 /*alignment slack*/;
+
+__device__ __forceinline__ float inv_norm(float square) {   // 1 / max(|x|, 1e-12), within 2 ulp
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(square));
+    return fminf(r, 1e12f);
+}
+
+// SPLIT: fewer units than warps: a warp has one tensor of one unit
+template <bool DIRECT, bool SPLIT>
+__global__ void __launch_bounds__(kWarps * 32, 3)
+match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ MatchArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = lane >> 2, tq = lane & 3, odd = tq & 1;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
+    const uint32_t stage0 = smem_u32(smem + (size_t)warp * 2 * kStage);
+    const uint32_t bar0 = smem_u32(smem + (size_t)kWarps * 2 * kStage + warp * 16);
+    if (lane == 0) {
+        mbar_init(bar0, 1);
+        mbar_init(bar0 + 8, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+
+    Box box{};
+    if (DIRECT) box.set(a.layout);
+    const int64_t n_units = (int64_t)a.heads * a.n_blocks;
+    int stride = gridDim.x * kWarps, first = blockIdx.x * kWarps + warp, t_first = 0, t_last = 1;
+    if (SPLIT) {
+        t_first = t_last = first >= n_units ? 1 : 0;
+        first = (int)min(n_units, first - t_first * n_units);
+        stride = (int)n_units;
+    }
+    UnitCursor next;   // the unit whose loads are issued next
+    next.init(first, stride, a.n_blocks);
+    auto issue = [&](int t, const int4& geom, int start, int h) {   // lane 0 only
+        const Geometry bg = unpack_geometry(geom);
+        const uint32_t mb = bar0 + 8 * t;
+        const CUtensorMap* m = t == 0 ? &map_q : &map_k;
+        if (DIRECT) {
+            mbar_expect_tx(mb, (uint32_t)box.rows * kRowBytes);
+            tma_block_load(stage0 + t * kStage, m, mb, bg.x0, bg.y0, bg.s0, h);
+        } else {
+            mbar_expect_tx(mb, kStage);
+            tma_rows_load(stage0 + t * kStage, m, mb, start, h);
+        }
+    };
+    BlockInfo bi_next{};
+    int4 bg_next{};
+    int h_next = 0;
+    auto fetch = [&]() {
+        bi_next = a.blocks[next.u];
+        if (DIRECT) bg_next = load_geometry(a.geom, next.u);
+        h_next = next.h;
+    };
+    if (first < n_units) fetch();
+    depend_wait();
+    dependents_launch();
+    if (first < n_units && lane == 0)
+        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t) issue(t, bg_next, bi_next.start, h_next);
+
+    // ldmatrix offsets of a 16-row tile: rows 0-7 / 8-15 (lane bit 3), k chunk 2 ks / 2 ks + 1 (lane bit 4); chunk c of row j sits at c ^ (j & 7)
+    uint32_t a_off[4];
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) a_off[ks] = ((lane & 7) + ((lane >> 3) & 1) * 8) * kRowBytes + (((2 * ks + (lane >> 4)) ^ (lane & 7)) << 4);
+    // what this lane knows about the shape of the blocks at hand
+    int shape_a = -1, shape_b = -1;
+    uint32_t d_off[2] = {0, 0};   // ldmatrix offsets of dst row lane & 7
+    int d_pos = 0;                // token number of dst lane & 7
+    int tok[2] = {-1, -1};        // tokens owned (-1: none)
+    bool is_src[2] = {false, false};
+
+    int it = 0;
+    bool failed = false;
+    for (int64_t unit = first; unit < n_units; unit += stride, ++it) {
+        const BlockInfo bi = bi_next;
+        const int4 geom = bg_next;
+        const int h = h_next, n = bi.n;
+        const bool more = unit + stride < n_units;
+        if (more) {
+            next.advance();
+            fetch();   // in flight while this unit is worked off
+        }
+#pragma unroll 1
+        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t) {
+            const int r = t == 0 ? bi.r_q : bi.r_k, nd = t == 0 ? bi.nd_q : bi.nd_k;
+            int32_t* A = a.assign[t] + (int64_t)h * a.n_tokens + bi.start;
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8 * t, it & 1, a.status, kDevTimeoutMatchLoad))) {
+                failed = true;
+                break;
+            }
+            if (r == 0 || nd > 8) {   // nothing merges, or an anchored block with more dst tokens (match_anchor_kernel)
+                if (r == 0 && lane < n) A[lane] = bi.start + lane;
+                __syncwarp();
+                if (more && lane == 0) issue(t, bg_next, bi_next.start, h_next);
+                continue;
+            }
+            const int n_rows = DIRECT ? box.rows : n;   // rows of the stage that may hold tokens
+            {
+                const int sa = n | (nd << 8) | (bi.n_rule << 16), sb = DIRECT ? geom.z + (geom.y & 0xffff0000) : 0;   // frames, rows, cols
+                if (sa != shape_a || sb != shape_b) {
+                    const Geometry bg = unpack_geometry(geom);
+                    shape_a = sa;
+                    shape_b = sb;
+                    const int n_rule = bi.n_rule;   // n (evenly spaced dst tokens) or n_dst (the first n_dst tokens: first-frame anchoring)
+                    d_pos = small_div((min(lane & 7, nd - 1) + 1) * n_rule + nd - 1, nd) - 1;
+                    const int row = DIRECT ? row_of_token(box, bg, d_pos) : d_pos;
+#pragma unroll
+                    for (int kp = 0; kp < 2; ++kp) d_off[kp] = row * kRowBytes + (((4 * kp + (lane >> 3)) ^ (row & 7)) << 4);
+#pragma unroll
+                    for (int mt = 0; mt < 2; ++mt) {
+                        const int rho = mt * 16 + odd * 8 + g;
+                        const int j = DIRECT ? token_of_row(box, bg, rho) : (rho < n ? rho : -1);
+                        tok[mt] = tq < 2 ? j : -1;
+                        is_src[mt] = tok[mt] >= 0 && !(j < n_rule && small_div((j + 1) * nd, n_rule) > small_div(j * nd, n_rule));
+                    }
+                }
+            }
+            const uint32_t blk = stage0 + t * kStage;
+            // ---- dst fragments (k steps 2 kp, 2 kp + 1 per ldmatrix.x4) and their norms: lane 9 tq holds that of dst 2 tq, 9 tq + 4 of 2 tq + 1
+            uint32_t bf[4][2];
+#pragma unroll
+            for (int kp = 0; kp < 2; ++kp) {
+                uint32_t rr[4];
+                ldmatrix_x4(rr, blk + d_off[kp]);
+                bf[2 * kp][0] = rr[0];
+                bf[2 * kp][1] = rr[1];
+                bf[2 * kp + 1][0] = rr[2];
+                bf[2 * kp + 1][1] = rr[3];
+            }
+            float dn[4];
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+                const uint32_t ad[4] = {bf[ks][0], bf[ks][0], bf[ks][1], bf[ks][1]};
+                if (ks == 0)
+                    mma_first(dn, ad, bf[ks][0], bf[ks][1]);
+                else
+                    mma_bf16_16816(dn, ad, bf[ks][0], bf[ks][1]);
+            }
+            const float dsel = (g & 1) ? dn[1] : dn[0];
+            const float w0 = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq)), w1 = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq + 4));
+            const bool has0 = 2 * tq < nd, has1 = 2 * tq + 1 < nd;
+            // ---- best dst of every row
+            uint32_t key[2] = {0u, 0u};
+            int best[2] = {0, 0};
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                if (mt * 16 < n_rows) {   // warp-uniform
+                    float c[4], lo[4], hi[4];
+#pragma unroll
+                    for (int ks = 0; ks < 4; ++ks) {
+                        uint32_t af[4];
+                        ldmatrix_x4(af, blk + mt * 16 * kRowBytes + a_off[ks]);
+                        if (ks == 0) {
+                            mma_first(c, af, bf[ks][0], bf[ks][1]);
+                            mma_first(lo, af, af[0], af[2]);   // against rows 0-7 of the tile
+                            mma_first(hi, af, af[1], af[3]);   // against rows 8-15
+                        } else {
+                            mma_bf16_16816(c, af, bf[ks][0], bf[ks][1]);
+                            mma_bf16_16816(lo, af, af[0], af[2]);
+                            mma_bf16_16816(hi, af, af[1], af[3]);
+                        }
+                    }
+                    // rows g and g + 8, this lane's two dst tokens (ties: the lower one)
+                    const float s00 = has0 ? c[0] * w0 : -INFINITY, s01 = has1 ? c[1] * w1 : -INFINITY;
+                    const float s10 = has0 ? c[2] * w0 : -INFINITY, s11 = has1 ? c[3] * w1 : -INFINITY;
+                    const float t0 = fmaxf(s00, s01), t1 = fmaxf(s10, s11);
+                    const int d0 = 2 * tq + (s01 > s00 ? 1 : 0), d1 = 2 * tq + (s11 > s10 ? 1 : 0);
+                    // lanes 0, 1 of a row's four split the two rows, then meet lanes 2, 3
+                    float top = odd ? t1 : t0;
+                    int arg = odd ? d1 : d0;
+                    {
+                        const float ov = __shfl_xor_sync(0xffffffffu, odd ? t0 : t1, 1);
+                        const int oa = __shfl_xor_sync(0xffffffffu, odd ? d0 : d1, 1);
+                        if (ov > top || (ov == top && oa < arg)) {
+                            top = ov;
+                            arg = oa;
+                        }
+                    }
+                    {
+                        const float ov = __shfl_xor_sync(0xffffffffu, top, 2);
+                        const int oa = __shfl_xor_sync(0xffffffffu, arg, 2);
+                        if (ov > top || (ov == top && oa < arg)) {
+                            top = ov;
+                            arg = oa;
+                        }
+                    }
+                    const int diag = 4 * g + (g >> 1);   // the lane that holds the squared norms of rows g and g + 8
+                    const float nl = __shfl_sync(0xffffffffu, (g & 1) ? lo[1] : lo[0], diag), nh = __shfl_sync(0xffffffffu, (g & 1) ? hi[3] : hi[2], diag);
+                    key[mt] = score_key(top * inv_norm(odd ? nh : nl));
+                    best[mt] = arg;
+                }
+            }
+            __syncwarp();   // every lane has read the stage
+            if (more && lane == 0) issue(t, bg_next, bi_next.start, h_next);
+
+            // ---- the r src with the best scores merge (ties: lowest position first)
+            const int n_out = n - nd - r;
+            bool merged[2];
+            const int rho0 = odd * 8 + g, rho1 = rho0 + 16;
+            if (r <= n_out) {
+                merged[0] = merged[1] = false;
+                for (int round = 0; round < r; ++round) {
+                    const uint32_t k0 = is_src[0] && !merged[0] ? key[0] : 0u, k1 = is_src[1] && !merged[1] ? key[1] : 0u;
+                    const uint32_t m = __reduce_max_sync(0xffffffffu, max(k0, k1));
+                    const int win = __reduce_min_sync(0xffffffffu, k0 == m ? rho0 : (k1 == m ? rho1 : 0x7fffffff));   // lowest position holding it
+                    merged[0] = merged[0] || (is_src[0] && win == rho0);
+                    merged[1] = merged[1] || (is_src[1] && win == rho1);
+                }
+            } else {
+                merged[0] = is_src[0];
+                merged[1] = is_src[1];
+                for (int round = 0; round < n_out; ++round) {
+                    const uint32_t k0 = merged[0] ? key[0] : 0xffffffffu, k1 = merged[1] ? key[1] : 0xffffffffu;
+                    const uint32_t m = __reduce_min_sync(0xffffffffu, min(k0, k1));
+                    const int win = __reduce_max_sync(0xffffffffu, merged[1] && k1 == m ? rho1 : (merged[0] && k0 == m ? rho0 : -1));   // highest position
+                    if (win == rho0) merged[0] = merged[0] && tq >= 2;
+                    if (win == rho1) merged[1] = merged[1] && tq >= 2;
+                }
+            }
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                const int target = __shfl_sync(0xffffffffu, d_pos, best[mt]);
+                if (tok[mt] >= 0) A[tok[mt]] = bi.start + (merged[mt] ? target : tok[mt]);
+            }
+        }
+        if (failed) break;
+    }
+    if (failed) {   // give copies that may still be in flight a bounded chance to land before the shared memory is released
+        for (int t = SPLIT ? t_first : 0; t <= t_last; ++t) mbar_wait_bounded(bar0 + 8 * t, it & 1, a.status, kDevTimeoutMatchLoad);
+    }
+}
+
+// ------------------------------------------------------------------------------------ merge
+// The group sums of a block are one small dense contraction: merged_sum[kept row][channel] = sum_token W[row][token] x[token][channel]
+// with the 0/1 assignment matrix W (exact in bf16, built in registers from the map), fp32 accumulation, times the reciprocal
+// of the group size, one rounding to bf16.  Kept tokens are compacted in reordered order.  The rows go through the stage they came
+// from (its fragments are in registers by then) and leave 16 bytes per lane, whole rows; then the stage is refilled.
+constexpr int kMergeAux = 32 * 4 + 32 * 4 + 32;   // reciprocal group sizes, group sizes / first members, 3 mbarriers
+constexpr int kMergeSmem = kWarps * (3 * (int)kStage + kMergeAux) + 1024 /*alignment slack*/;
+
+__device__ __forceinline__ void stmatrix_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
+}
+// fragment of W (16 merged rows x 16 tokens): rw = merged rows of this lane's four tokens, r0 its first row; bf16 1.0 = 0x3f80
+__device__ __forceinline__ void w_fragment(uint32_t* af, const int* rw, int r0) {
+    const int r1 = r0 + 8;
+    af[0] = (rw[0] == r0 ? 0x3f80u : 0u) | (rw[1] == r0 ? 0x3f800000u : 0u);
+    af[1] = (rw[0] == r1 ? 0x3f80u : 0u) | (rw[1] == r1 ? 0x3f800000u : 0u);
+    af[2] = (rw[2] == r0 ? 0x3f80u : 0u) | (rw[3] == r0 ? 0x3f800000u : 0u);
+    af[3] = (rw[2] == r1 ? 0x3f80u : 0u) | (rw[3] == r1 ? 0x3f800000u : 0u);
+}
+__device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// DIRECT: the blocks come straight from the original tensors (5-D block maps), the special tokens frame by
+// frame (4-D frame maps); otherwise from the reordered copies, specials in chunks of 32.
+struct MergeMaps {
+    CUtensorMap block[3], special[3];
+};
+
+template <bool DIRECT, bool SPLIT>
+__global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __grid_constant__ MergeMaps maps, const __grid_constant__ MergeArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = lane >> 2, tq = lane & 3;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
+    unsigned char* stage = smem + (size_t)warp * 3 * kStage;
+    unsigned char* aux = smem + (size_t)kWarps * 3 * kStage + (size_t)warp * kMergeAux;
+    float* rcnt = reinterpret_cast<float*>(aux);             // [32] 1 / group size of kept row
+    int* gsz = reinterpret_cast<int*>(aux + 32 * 4);         // [32] size, then first member, of kept row
+    const uint32_t stage0 = smem_u32(stage), bar0 = smem_u32(aux + 2 * 32 * 4);
+    if (lane == 0) {
+#pragma unroll
+        for (int t = 0; t < 3; ++t) mbar_init(bar0 + 8 * t, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    Box box{};
+    if (DIRECT) box.set(a.layout);
+    const int own_t = DIRECT ? lane / (box.h * box.w) : 0, own_y = DIRECT ? (lane / box.w) % box.h : 0, own_x = DIRECT ? lane % box.w : 0;
+    if (DIRECT)   // stage rows that no block load writes enter the MMAs with weight 0: they must hold finite values
+        for (int q = box.rows * 8 + lane; q < 32 * 8; q += 32)
+#pragma unroll
+            for (int t = 0; t < 3; ++t) *reinterpret_cast<uint4*>(stage + t * kStage + q * 16) = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+
+    // units 0 .. n_blocks - 1 of a head are merging blocks, the rest special tokens (never merged: copied)
+    const int sp_units = DIRECT ? (a.layout.n_special > 0 ? a.layout.frames : 0) : (a.n_special_total + 31) / 32;
+    const int per_head = a.n_blocks + sp_units;
+    const int64_t n_units = (int64_t)a.heads * per_head;
+    int stride = gridDim.x * kWarps, first = blockIdx.x * kWarps + warp, t_first = 0, t_last = 2;
+    if (SPLIT) {
+        t_first = t_last = (int)min((int64_t)2, first / n_units);
+        first = (int)min(n_units, first - t_first * n_units);
+        stride = (int)n_units;
+    }
+    struct Meta {
+        int h, start, sizes, moff_q, moff_k;   // sizes: n | r_q << 8 | r_k << 16, bit 24: special tokens
+        int4 geom;                             // (of special tokens: .w = their frame)
+        __device__ int n() const { return sizes & 0xff; }
+        __device__ int r(int t) const { return (sizes >> (t == 0 ? 8 : 16)) & 0xff; }
+        __device__ bool special() const { return sizes >> 24; }
+    };
+    UnitCursor next;
+    next.init(first, stride, per_head);
+    auto fetch = [&]() {
+        Meta m{};
+        m.h = next.h;
+        if (next.u >= a.n_blocks) {
+            m.geom.w = next.u - a.n_blocks;
+            m.start = m.geom.w * (DIRECT ? a.layout.n_special : 32);
+            m.sizes = (1 << 24) | (DIRECT ? a.layout.n_special : min(32, a.n_special_total - m.start));
+            m.moff_q = m.moff_k = m.start;
+        } else {
+            if (DIRECT) m.geom = load_geometry(a.geom, next.u);
+            const BlockInfo bi = a.blocks[next.u];
+            m.start = bi.start;
+            m.sizes = bi.n | (bi.r_q << 8) | (bi.r_k << 16);
+            m.moff_q = a.moff_q_var ? ld_global(a.moff_q_var + (int64_t)m.h * a.n_blocks + next.u) : bi.moff_q;
+            m.moff_k = bi.moff_k;
+        }
+        return m;
+    };
+    auto issue = [&](int t, const Meta& m) {   // lane 0 only
+        const uint32_t mb = bar0 + 8 * t, dst = stage0 + t * kStage;
+        if (!DIRECT) {
+            mbar_expect_tx(mb, kStage);   // (rows past the head's end are zero filled)
+            tma_rows_load(dst, &maps.block[t], mb, m.start, m.h);
+        } else if (m.special()) {
+            mbar_expect_tx(mb, (uint32_t)m.n() * kRowBytes);
+            asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
+                         "l"(reinterpret_cast<uint64_t>(&maps.special[t])), "r"(mb), "r"(0), "r"(0), "r"(m.geom.w), "r"(m.h)
+                         : "memory");
+        } else {
+            const Geometry bg = unpack_geometry(m.geom);
+            mbar_expect_tx(mb, (uint32_t)box.rows * kRowBytes);
+            tma_block_load(dst, &maps.block[t], mb, bg.x0, bg.y0, bg.s0, m.h);
+        }
+    };
+    // lane = row of the stage; number of the token it holds in the block (-1: none)
+    auto token_of_lane = [&](const Meta& m) {
+        if (!DIRECT || m.special()) return lane < m.n() ? lane : -1;
+        const Geometry bg = unpack_geometry(m.geom);
+        return own_t < bg.frames && own_y < bg.rows && own_x < bg.cols ? (own_t * bg.rows + own_y) * bg.cols + own_x : -1;
+    };
+    auto load_target = [&](const Meta& m, int map) {   // token this lane's token is merged into (number in the block)
+        const int tok = token_of_lane(m);
+        return m.r(map) > 0 && tok >= 0 ? ld_global(a.assign[map] + (int64_t)m.h * a.n_tokens + m.start + tok) - m.start : -1;
+    };
+    depend_wait();
+    dependents_launch();
+    Meta meta_next{};
+    int target_next[2] = {-1, -1};
+    if (first < n_units) {
+        meta_next = fetch();
+        if (lane == 0)
+#pragma unroll
+            for (int t = 0; t < 3; ++t)
+                if (!SPLIT || t == t_first) issue(t, meta_next);
+        if (t_first == 0) target_next[0] = load_target(meta_next, 0);
+        if (t_last > 0) target_next[1] = load_target(meta_next, 1);
+    }
+
+    const float recip = 1.0f / (float)(lane + 1);   // lane i holds 1 / (i + 1)
+
+    int it = 0;
+    bool failed = false;
+    for (int64_t unit = first; unit < n_units; unit += stride, ++it) {
+        const Meta m = meta_next;
+        const int target[2] = {target_next[0], target_next[1]};
+        const bool more = unit + stride < n_units;
+        if (more) {
+            next.advance();
+            meta_next = fetch();   // in flight while this unit is worked off
+        }
+        const int tok = token_of_lane(m), n = m.n();
+        uint32_t af0[2][4];   // W fragments of the first 16 merged rows (K's serve V)
+        const int n_ks = (DIRECT ? box.rows : n) > 16 ? 2 : 1;   // 16-row steps of the stage that may hold tokens
+        int row_of = -1, n_kept = 0;
+        int rw[2][4];
+#pragma unroll 1
+        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 2); ++t) {
+            const int r = m.r(t), moff = t == 0 ? m.moff_q : m.moff_k, m_len = t == 0 ? a.m_q : a.m_k;
+            uint4* out = reinterpret_cast<uint4*>(a.merged[t] + ((int64_t)m.h * m_len + moff) * kHeadDim);
+            const uint32_t blk = stage0 + t * kStage;
+            const unsigned char* rows = stage + t * kStage;
+            int n_out = n;   // rows that leave
+            if (r > 0 && (SPLIT || t < 2)) {   // the groups of this map (V follows K)
+                int rep = t == 0 ? target[0] : target[1];
+                if (tok >= 0) {
+                    if (rep < 0 || rep >= n) {   // corrupt map: record, treat as kept
+                        atomicCAS(a.status, kDevOk, kDevBadIndex);
+                        rep = tok;
+                    }
+                    if (DIRECT) rep = row_of_token(box, unpack_geometry(m.geom), rep);   // ROW of the stage holding the token it is merged into
+                } else {
+                    rep = -1;
+                }
+                // merged row of every token: rank of its representative among the kept tokens
+                const unsigned kept = __ballot_sync(0xffffffffu, rep == lane);
+                n_kept = __popc(kept);
+                row_of = rep >= 0 ? __popc(kept & ((1u << rep) - 1u)) : -1;
+                gsz[lane] = 0;
+                __syncwarp();
+                const int slot = row_of >= 0 ? atomicAdd(&gsz[row_of], 1) : 0;   // (the order of a row's members does not matter)
+                __syncwarp();
+                const int sz = gsz[lane];
+                rcnt[lane] = __shfl_sync(0xffffffffu, recip, (sz - 1) & 31);
+                __syncwarp();
+                if (t == 0) {
+                    if (tok >= 0) a.rank_q[(int64_t)m.h * a.n_tokens + m.start + tok] = moff + row_of;
+                    if (a.group_start) {
+                        // member lists of the merged rows: the block's tokens group by group, kept rows in rank order
+                        // (first member of row k = tokens of the rows before it: a warp scan over the group sizes)
+                        int incl = sz;
+#pragma unroll
+                        for (int off = 1; off < 32; off <<= 1) {
+                            const int v = __shfl_up_sync(0xffffffffu, incl, off);
+                            if (lane >= off) incl += v;
+                        }
+                        if (lane < min(n_kept, n - r)) a.group_start[(int64_t)m.h * (a.m_q + 1) + moff + lane] = m.start + incl - sz;
+                        const int begin = __shfl_sync(0xffffffffu, incl - sz, row_of & 31);
+                        if (tok >= 0) {   // the token's number in the original order: from the block's place in the scene, or through the reorder index
+                            const Geometry bg = unpack_geometry(m.geom);
+                            const int orig = DIRECT ? (bg.s0 + own_t) * a.layout.tokens_per_frame + a.layout.n_special + (bg.y0 + own_y) * a.layout.grid_w + bg.x0 + own_x
+                                                    : __ldg(a.pi + m.start + tok);
+                            a.group_member[(int64_t)m.h * a.n_tokens + m.start + begin + slot] = orig;
+                        }
+                    }
+                }
+                // W fragments need the rows of tokens 16 ks + {2 tq, 2 tq + 1, 2 tq + 8, 2 tq + 9}
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) {
+                    rw[ks][0] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq);
+                    rw[ks][1] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 1);
+                    rw[ks][2] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 8);
+                    rw[ks][3] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 9);
+                    w_fragment(af0[ks], rw[ks], g);
+                }
+            }
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8 * t, it & 1, a.status, kDevTimeoutMatchLoad))) {
+                failed = true;
+                break;
+            }
+            if (r == 0) {   // nothing merges here: the rows leave as they are
+                if (t == 0 && lane < n) {
+                    if (!m.special()) a.rank_q[(int64_t)m.h * a.n_tokens + m.start + lane] = moff + lane;
+                    if (a.group_start) {   // every token is a group of its own
+                        a.group_start[(int64_t)m.h * (a.m_q + 1) + moff + lane] = m.start + lane;
+                        a.group_member[(int64_t)m.h * a.n_tokens + m.start + lane] = __ldg(a.pi + m.start + lane);
+                    }
+                }
+            } else {
+                // x fragments: for k step ks (16 tokens) and channel tile pair np, one ldmatrix.x4.trans gives
+                // b0, b1 of channel tile 2 np and b0, b1 of channel tile 2 np + 1
+                uint32_t bf[2][4][4];
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) {
+                    if (ks < n_ks) {
+                        const int j = 16 * ks + (lane & 15);
+#pragma unroll
+                        for (int np = 0; np < 4; ++np) ldmatrix_x4_trans(bf[ks][np], blk + j * kRowBytes + (((2 * np + (lane >> 4)) ^ (j & 7)) << 4));
+                    }
+                }
+                __syncwarp();   // every lane has its fragments: the stage takes the merged rows
+                const int n_mt = n_kept > 16 ? 2 : 1;
+#pragma unroll 1
+                for (int mt = 0; mt < n_mt; ++mt) {
+                    const int r0 = 16 * mt + g, r1 = r0 + 8;   // this lane's two accumulator rows
+                    if (n_mt == 2) {   // (with one tile the fragments stay as they are)
+                        w_fragment(af0[0], rw[0], r0);
+                        w_fragment(af0[1], rw[1], r0);
+                    }
+                    float c[8][4];
+#pragma unroll
+                    for (int ks = 0; ks < 2; ++ks) {
+                        if (ks < n_ks) {
+                            uint32_t* af = af0[ks];
+#pragma unroll
+                            for (int nt = 0; nt < 8; ++nt) {
+                                if (ks == 0)
+                                    mma_first(c[nt], af, bf[ks][nt >> 1][2 * (nt & 1)], bf[ks][nt >> 1][2 * (nt & 1) + 1]);
+                                else
+                                    mma_bf16_16816(c[nt], af, bf[ks][nt >> 1][2 * (nt & 1)], bf[ks][nt >> 1][2 * (nt & 1) + 1]);
+                            }
+                        }
+                    }
+                    // rows past the last kept one become zeros (not 0 x something: the stage must stay finite)
+                    const bool w0 = r0 < n_kept, w1 = r1 < n_kept;
+                    const float i0 = w0 ? rcnt[r0] : 0.f, i1 = w1 ? rcnt[r1] : 0.f;
+                    const int j = 16 * mt + (lane & 7) + ((lane >> 4) << 3);   // row whose address this lane gives (matrices: rows 0-7 x two tiles, rows 8-15 x two)
+#pragma unroll
+                    for (int np = 0; np < 4; ++np) {
+                        const float(*p)[4] = &c[2 * np];
+                        stmatrix_x4(blk + j * kRowBytes + (((2 * np + ((lane >> 3) & 1)) ^ (j & 7)) << 4), w0 ? pack2_bf16(p[0][0] * i0, p[0][1] * i0) : 0u,
+                                    w0 ? pack2_bf16(p[1][0] * i0, p[1][1] * i0) : 0u, w1 ? pack2_bf16(p[0][2] * i1, p[0][3] * i1) : 0u,
+                                    w1 ? pack2_bf16(p[1][2] * i1, p[1][3] * i1) : 0u);
+                    }
+                }
+                __syncwarp();
+                n_out = min(n_kept, t == 0 && a.moff_q_var ? n : n - r);   // (a corrupt map cannot overrun; after outlier filtering more than n - r may be kept)
+            }
+            if (t == 0 && more) target_next[0] = load_target(meta_next, 0);   // (in flight during the stores and the next tensors)
+            if (t == 1 && more) target_next[1] = load_target(meta_next, 1);
+            if (DIRECT && r == 0 && !m.special()) {   // (the tokens of a clipped block are not consecutive rows)
+                const Geometry bg = unpack_geometry(m.geom);
+                for (int q = lane; q < n_out * 8; q += 32) {
+                    const int row = row_of_token(box, bg, q >> 3);
+                    out[q] = *reinterpret_cast<const uint4*>(rows + row * kRowBytes + (((q & 7) ^ (row & 7)) << 4));
+                }
+            } else {   // chunk c of row j sits at c ^ (j & 7); a lane's rows are 4 apart: two offsets serve all of them
+                const int j0 = lane >> 3, ch = lane & 7;
+                const unsigned char* even = rows + j0 * kRowBytes + ((ch ^ j0) << 4);
+                const unsigned char* odds = rows + j0 * kRowBytes + ((ch ^ (j0 + 4)) << 4);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (4 * i >= n_out) break;   // (uniform)
+                    if (4 * i + j0 < n_out) out[32 * i + lane] = *reinterpret_cast<const uint4*>(((i & 1) ? odds : even) + i * 4 * kRowBytes);
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the merged rows were written by ordinary stores, the refill is not
+            __syncwarp();
+            if (more && lane == 0) issue(t, meta_next);
+        }
+        if (failed) break;
+    }
+    if (failed) {
+        for (int t = SPLIT ? t_first : 0; t <= t_last; ++t) mbar_wait_bounded(bar0 + 8 * t, it & 1, a.status, kDevTimeoutMatchLoad);
+    }
+}
+
+int small_grid(int64_t units, int sm_count, int ctas_per_sm) {
+    const int64_t grid = (units + kWarps - 1) / kWarps, cap = (int64_t)(sm_count < 1 ? 1 : sm_count) * ctas_per_sm;
+    return (int)(grid > cap ? cap : (grid < 1 ? 1 : grid));
+}
+
+}  // namespace
+
+cudaError_t launch_match_small(const MatchArgs& a, int sm_count, cudaStream_t stream) {
+    CUtensorMap mq, mk;
+    const int64_t N = a.n_tokens;
+    const bool direct = a.geom != nullptr;
+    if (direct) {
+        if (!encode_block_map(&mq, a.src[0], a.layout, a.heads) || !encode_block_map(&mk, a.src[1], a.layout, a.heads)) return cudaErrorInvalidValue;
+    } else if (!encode_rows_tensor_map(&mq, a.xr[0], N, a.heads, kHeadDim, N * kHeadDim, 32) ||
+               !encode_rows_tensor_map(&mk, a.xr[1], N, a.heads, kHeadDim, N * kHeadDim, 32)) {
+        return cudaErrorInvalidValue;
+    }
+    // With no more than one tensor per warp the tensors of a unit go to different warps: the call then waits for one, not two
+    // (512 units: 11.3 -> 9.4 us, in the merge kernel below 13.1 -> 9.0).
+    const int64_t units = (int64_t)a.heads * a.n_blocks;
+    const int parts = 2 * units <= 3ll * kWarps * sm_count ? 2 : 1, grid = small_grid(units * parts, sm_count, 3);
+    const bool split = parts > 1;
+    auto kernel = direct ? (split ? match_small_kernel<true, true> : match_small_kernel<true, false>)
+                         : (split ? match_small_kernel<false, true> : match_small_kernel<false, false>);
+    return launch_kernel(kernel, grid, kWarps * 32, kMatchSmem, stream, mq, mk, a);
+}
+
+cudaError_t launch_merge_small(const MergeArgs& a, int sm_count, cudaStream_t stream) {
+    MergeMaps m;
+    const int64_t N = a.n_tokens;
+    const bool direct = a.geom != nullptr;
+    for (int t = 0; t < 3; ++t) {
+        if (direct) {
+            if (!encode_block_map(&m.block[t], a.src[t], a.layout, a.heads)) return cudaErrorInvalidValue;
+            m.special[t] = m.block[t];
+            if (a.layout.n_special > 0 &&
+                !encode_frame_tensor_map(&m.special[t], a.src[t].ptr, a.layout.tokens_per_frame, a.layout.frames, a.heads, a.src[t].stride_token,
+                                         a.src[t].stride_head, a.layout.n_special))
+                return cudaErrorInvalidValue;
+        } else {
+            if (!encode_rows_tensor_map(&m.block[t], a.xr[t], N, a.heads, kHeadDim, N * kHeadDim, 32)) return cudaErrorInvalidValue;
+            m.special[t] = m.block[t];   // not used
+        }
+    }
+    const int sp_units = direct ? (a.layout.n_special > 0 ? a.layout.frames : 0) : (a.n_special_total + 31) / 32;
+    const int64_t units = (int64_t)a.heads * (a.n_blocks + sp_units);
+    const int parts = 3 * units <= 2ll * kWarps * sm_count ? 3 : 1, grid = small_grid(units * parts, sm_count, 2);
+    const bool split = parts > 1;
+    auto kernel = direct ? (split ? merge_small_kernel<true, true> : merge_small_kernel<true, false>)
+                         : (split ? merge_small_kernel<false, true> : merge_small_kernel<false, false>);
+    return launch_kernel(kernel, grid, kWarps * 32, kMergeSmem, stream, m, a);
+}
+
+cudaError_t configure_small_blocks() {
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto kernel, int bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    set(match_small_kernel<false, false>, kMatchSmem);
+    set(match_small_kernel<false, true>, kMatchSmem);
+    set(match_small_kernel<true, false>, kMatchSmem);
+    set(match_small_kernel<true, true>, kMatchSmem);
+    set(merge_small_kernel<false, false>, kMergeSmem);
+    set(merge_small_kernel<false, true>, kMergeSmem);
+    set(merge_small_kernel<true, false>, kMergeSmem);
+    set(merge_small_kernel<true, true>, kMergeSmem);
+    return e;
+}
+
+}  // namespace httm
