@@ -1,5 +1,5 @@
-// HBM-bound kernels of the HTTM path: temporal reorder (gather), per-(head, block)
-// cosine matching, mean merge, and unmerge + inverse reorder.  sm_100a only.
+// HBM-bound kernels of the HTTM path: temporal reorder (gather), matching of first-frame blocks, outlier filtering, unmerge +
+// inverse reorder, and the choice of the matching and merging kernels by block size.  sm_100a only.
 #include "httm_internal.h"
 #include "httm_launch.cuh"
 #include "httm_blocks.cuh"
@@ -63,365 +63,8 @@ cudaError_t launch_reorder(const ReorderArgs& a, cudaStream_t stream) {
 }
 
 // ------------------------------------------------------------------------------------
-// a2. Block-wise bipartite matching (Eq. 1; Sec. 3.2 top-r rule), one warp per
-//     (tensor in {Q, K}, head, block).  The block (n x 64 bf16, contiguous after the
-//     reorder) is staged in shared memory by a tiled TMA load with the 128-byte swizzle,
-//     double buffered per warp.  The dot products of every token with every dst token are
-//     a small dense contraction (n x n_dst x 64): they run on the tensor cores as
-//     m16n8k16 bf16 MMAs with fp32 accumulation, operands fetched with ldmatrix straight
-//     from the swizzled stage (conflict free); the dst rows are gathered by giving
-//     ldmatrix their row addresses.  Products of bf16 values are exact in fp32, and the
-//     accumulation error measured on this hardware is below that of an fp32 FMA chain.
-//     Squared norms are the diagonal of the same kind of MMA (a tile of rows against
-//     itself).  Similarity = dot * inv_norm(src) * inv_norm(dst).
-//     argmax ties -> lowest dst; top-r ties -> lowest src.  The r merged src are found by
-//     min(r, n_src - r) rounds of a warp-wide max (or min) extraction.
-//     Token j of a block is owned, for the selection, by lane (j & 7) * 4 + ((j >> 3) & 1),
-//     slot j >> 4: the lane where the MMA accumulator layout leaves row j's results.
-// ------------------------------------------------------------------------------------
-// warps per CTA (one CTA per SM): as many as the shared memory takes at two stages per warp; a warp works alone on its
-// blocks, so the number of warps per scheduler is what hides its instruction latencies
-__host__ __device__ constexpr int match_warps_per_cta(int nmax) { return nmax <= 32 ? 8 : (nmax <= 64 ? 16 : (nmax <= 128 ? 12 : 6)); }
-// stages per warp: blocks of more than 64 tokens keep a warp busy for many microseconds, far longer than a load takes; one
-// stage there buys twice the warps for the same shared memory
-__host__ __device__ constexpr int match_stages(int nmax) { return nmax <= 32 ? 2 : 1; }
-__host__ __device__ constexpr int match_aux_bytes(int nmax) { return nmax * 4 + 16; }   // inverse norms + 2 mbarriers
-__host__ __device__ constexpr int match_smem_bytes(int nmax) {
-    return match_warps_per_cta(nmax) * (match_stages(nmax) * nmax * kRowBytes + match_aux_bytes(nmax)) + 1024 /*alignment slack*/;
-}
-
-template <int PASSES, bool DIRECT>
-__global__ void __launch_bounds__(match_warps_per_cta(32 * PASSES) * 32, PASSES == 1 ? 2 : 1)   // 3 CTAs/SM would need 80 registers: spills cost more than the third CTA gains
-match_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const MatchArgs a) {
-    constexpr int NMAX = 32 * PASSES;
-    constexpr int WARPS = match_warps_per_cta(NMAX);
-    constexpr int MT = NMAX / 16;        // 16-token row tiles
-    constexpr int NT = NMAX / 32;        // 8-dst column tiles (n_dst <= NMAX / 4)
-    constexpr bool KEEP_A = PASSES == 1; // row-tile fragments stay in registers between the two passes
-    constexpr int STAGES = match_stages(NMAX);
-    constexpr uint32_t STAGE_BYTES = NMAX * kRowBytes;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 2, tq = lane & 3;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
-    unsigned char* aux = smem + (size_t)WARPS * STAGES * STAGE_BYTES + (size_t)warp * match_aux_bytes(NMAX);
-    float* invn = reinterpret_cast<float*>(aux);                                   // [NMAX]
-    const uint32_t mbar0 = smem_u32(aux + NMAX * 4);                               // 2 mbarriers (one used with a single stage)
-    const uint32_t stage0 = smem_u32(smem + (size_t)warp * STAGES * STAGE_BYTES);  // [STAGES][NMAX][128], 1024-aligned
-
-    if (lane == 0) {
-        mbar_init(mbar0, 1);
-        mbar_init(mbar0 + 8, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncwarp();
-
-    const int64_t n_tasks = 2ll * a.heads * a.n_blocks;
-    const int64_t stride = (int64_t)gridDim.x * WARPS;
-    const int64_t first = (int64_t)blockIdx.x * WARPS + warp;
-    TaskCursor cur, nxt;   // the task being processed; the task whose load is issued next
-    cur.init(first, stride, a.heads, a.n_blocks);
-    nxt = cur;
-
-    // direct mode: box extents (clipped to the scene once) and the box coordinates of the rows this lane owns
-    const int box_f = DIRECT ? min(a.layout.blk_frames, a.layout.frames) : 1, box_h = DIRECT ? min(a.layout.blk_h, a.layout.grid_h) : 1,
-              box_w = DIRECT ? min(a.layout.blk_w, a.layout.grid_w) : 1;
-    const int box_rows = box_f * box_h * box_w;
-    const uint32_t box_bytes = (uint32_t)box_rows * kRowBytes;
-    int own_t[MT], own_y[MT], own_x[MT];
-#pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
-        const int rho = mt * 16 + (tq & 1) * 8 + g;
-        own_t[mt] = DIRECT ? rho / (box_h * box_w) : 0;
-        own_y[mt] = DIRECT ? (rho / box_w) % box_h : 0;
-        own_x[mt] = DIRECT ? rho % box_w : 0;
-    }
-    BoxMap bm;
-    bm.clipped = false;
-    auto issue = [&](const TaskCursor& c, int buf) {   // lane 0 only; the whole box is transferred (rows past the head's end are zero filled)
-        const uint32_t mb = mbar0 + 8 * buf;
-        if (DIRECT) {
-            const BlockGeom bg = a.geom[c.u];
-            mbar_expect_tx(mb, box_bytes);
-            tma_block_load(stage0 + buf * STAGE_BYTES, c.t == 0 ? &map_q : &map_k, mb, bg.x0, bg.y0, bg.s0, c.h);
-        } else {
-            const int start = __ldg(&a.blocks[c.u].start);
-            mbar_expect_tx(mb, STAGE_BYTES);
-            tma_rows_load(stage0 + buf * STAGE_BYTES, c.t == 0 ? &map_q : &map_k, mb, start, c.h);
-        }
-    };
-    depend_wait();
-    dependents_launch();
-    if (first < n_tasks && lane == 0) issue(nxt, 0);
-    nxt.advance();
-    if (STAGES == 2) {
-        if (first + stride < n_tasks && lane == 0) issue(nxt, 1);
-        nxt.advance();
-    }
-
-    int cached_n = -1, cached_nd = -1;
-    uint32_t magic_n = 0, magic_nd = 0;
-
-    int it = 0;
-    bool failed = false;
-    for (int64_t task = first; task < n_tasks; task += stride, ++it, cur.advance(), nxt.advance()) {
-        const int buf = STAGES == 2 ? (it & 1) : 0;
-        const uint32_t parity = STAGES == 2 ? ((it >> 1) & 1) : (it & 1);
-        const bool more = task + STAGES * stride < n_tasks;
-        const BlockInfo bi = a.blocks[cur.u];
-        const int n = bi.n, r = cur.t == 0 ? bi.r_q : bi.r_k, nd = cur.t == 0 ? bi.nd_q : bi.nd_k;
-        int32_t* A = a.assign[cur.t] + (int64_t)cur.h * a.n_tokens + bi.start;
-        if (!mbar_wait_bounded(mbar0 + 8 * buf, parity, a.status, kDevTimeoutMatchLoad)) {
-            failed = true;
-            break;
-        }
-        if (r == 0) {
-#pragma unroll
-            for (int p = 0; p < PASSES; ++p) {
-                const int j = lane + 32 * p;
-                if (j < n) A[j] = bi.start + j;
-            }
-            __syncwarp();
-            if (more && lane == 0) issue(nxt, buf);
-            continue;
-        }
-        if (nd > NT * 8) {   // first-frame anchoring with more dst tokens than a quarter of the largest block: match_anchor_kernel
-            __syncwarp();
-            if (more && lane == 0) issue(nxt, buf);
-            continue;
-        }
-        // floor(x / n) and floor(x / n_dst) by multiplication: exact for the operand ranges below (n <= 256, n_dst <= 64)
-        const int n_rule = bi.n_rule;   // n (evenly spaced dst tokens) or n_dst (the first n_dst tokens: first-frame anchoring)
-        if (n_rule != cached_n || nd != cached_nd) {
-            cached_n = n_rule;
-            cached_nd = nd;
-            magic_n = (1u << 23) / (uint32_t)n_rule + 1u;
-            magic_nd = (1u << 23) / (uint32_t)nd + 1u;
-        }
-        BlockGeom bg{};
-        if (DIRECT) {
-            bg = a.geom[cur.u];
-            bm.set(box_f, box_h, box_w, bg.frames, bg.rows, bg.cols);
-        }
-        const int n_rows = DIRECT ? box_rows : n;   // rows of the stage that may hold tokens
-        auto div_n = [&](int x) { return (int)(((uint32_t)x * magic_n) >> 23); };          // floor(x / n_rule), x < (n_rule + 1) * n_dst
-        auto pos_of = [&](int d) { return (int)(((uint32_t)((d + 1) * n_rule + nd - 1) * magic_nd) >> 23) - 1; };   // position of dst d
-        const uint32_t blk = stage0 + buf * STAGE_BYTES;
-        // ldmatrix address of 16-byte chunk `chunk` of row `row` (chunk c of row j sits at c ^ (j & 7))
-        auto chunk_addr = [&](int row, int chunk) { return blk + row * kRowBytes + ((chunk ^ (row & 7)) << 4); };
-
-        // ---- pass 1: squared norms of every token = diagonal of (row tile) x (row tile)^T
-        uint32_t af[KEEP_A ? MT : 1][4][4];   // [tile][k step][a0..a3]
-        auto load_a = [&](int mt, uint32_t (*dstf)[4]) {
-            // matrices of one ldmatrix.x4: rows 0-7 / 8-15 of the tile (lane bit 3), k chunk 2 ks / 2 ks + 1 (lane bit 4)
-            const int row = mt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks) ldmatrix_x4(dstf[ks], chunk_addr(row, 2 * ks + (lane >> 4)));
-        };
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-            if (mt * 16 < n_rows) {   // warp-uniform
-                uint32_t(*fr)[4] = af[KEEP_A ? mt : 0];
-                load_a(mt, fr);
-                float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int ks = 0; ks < 4; ++ks) {
-                    mma_bf16_16816(lo, fr[ks], fr[ks][0], fr[ks][2]);   // against rows 0-7 of the tile
-                    mma_bf16_16816(hi, fr[ks], fr[ks][1], fr[ks][3]);   // against rows 8-15
-                }
-                if (tq == (g >> 1)) {   // this lane holds the diagonal entries of rows g and g + 8
-                    const float s_lo = (g & 1) ? lo[1] : lo[0], s_hi = (g & 1) ? hi[3] : hi[2];
-                    // 1 / max(|x|, 1e-12): rsqrt.approx is within 2 ulp, far inside the 1e-5 margin rule
-                    invn[mt * 16 + g] = fminf(rsqrtf(s_lo), 1e12f);
-                    invn[mt * 16 + 8 + g] = fminf(rsqrtf(s_hi), 1e12f);
-                }
-            }
-        }
-        // ---- dst fragments: column tile nt holds dst 8 nt .. 8 nt + 7, gathered by row address
-        uint32_t bf[NT][4][2];   // [tile][k step][b0, b1]
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            if (nt * 8 < nd) {
-                const int d = min(nt * 8 + (lane & 7), nd - 1);
-                const int row = DIRECT ? bm.row_of_token(pos_of(d)) : pos_of(d);
-#pragma unroll
-                for (int kp = 0; kp < 2; ++kp) {   // one ldmatrix.x4 = k steps 2 kp and 2 kp + 1
-                    uint32_t rr[4];
-                    ldmatrix_x4(rr, chunk_addr(row, 4 * kp + (lane >> 3)));
-                    bf[nt][2 * kp][0] = rr[0];
-                    bf[nt][2 * kp][1] = rr[1];
-                    bf[nt][2 * kp + 1][0] = rr[2];
-                    bf[nt][2 * kp + 1][1] = rr[3];
-                }
-            }
-        }
-        __syncwarp();   // inverse norms visible; with one pass, every fragment is now in registers
-        if (KEEP_A) {
-            if (more && lane == 0) issue(nxt, buf);
-        }
-
-        // ---- pass 2: similarities, best dst of every token (kept by the owner lane of the token)
-        float wd[NT][2];   // inverse norms of this lane's dst columns
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int d = nt * 8 + 2 * tq + e;
-                wd[nt][e] = d < nd ? invn[DIRECT ? bm.row_of_token(pos_of(d)) : pos_of(d)] : 0.f;
-            }
-        uint32_t key[MT];
-        int best[MT], tok[MT];   // tok: number of the owned token in the block, -1 if the row holds none
-        bool is_src[MT];
-        const int own_half = tq & 1;   // owner of rows g (tq == 0) or g + 8 (tq == 1); lanes with tq >= 2 own nothing
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-            key[mt] = 0;
-            best[mt] = 0;
-            tok[mt] = -1;
-            is_src[mt] = false;
-            if (mt * 16 < n_rows) {
-                uint32_t(*fr)[4] = af[KEEP_A ? mt : 0];
-                if (!KEEP_A) load_a(mt, fr);
-                float top[2] = {-INFINITY, -INFINITY};   // rows g, g + 8
-                int arg[2] = {0, 0};
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt) {
-                    if (nt * 8 < nd) {
-                        float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                        for (int ks = 0; ks < 4; ++ks) mma_bf16_16816(c, fr[ks], bf[nt][ks][0], bf[nt][ks][1]);
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int d = nt * 8 + 2 * tq + e;
-                            if (d < nd) {
-                                const float w = wd[nt][e];
-                                const float s0 = c[e] * w, s1 = c[2 + e] * w;
-                                if (s0 > top[0]) {
-                                    top[0] = s0;
-                                    arg[0] = d;
-                                }
-                                if (s1 > top[1]) {
-                                    top[1] = s1;
-                                    arg[1] = d;
-                                }
-                            }
-                        }
-                    }
-                }
-                // combine the four lanes of a row (ties: lowest dst)
-#pragma unroll
-                for (int hrow = 0; hrow < 2; ++hrow) {
-#pragma unroll
-                    for (int off = 1; off <= 2; off <<= 1) {
-                        const float ov = __shfl_xor_sync(0xffffffffu, top[hrow], off);
-                        const int oa = __shfl_xor_sync(0xffffffffu, arg[hrow], off);
-                        if (ov > top[hrow] || (ov == top[hrow] && oa < arg[hrow])) {
-                            top[hrow] = ov;
-                            arg[hrow] = oa;
-                        }
-                    }
-                }
-                const int rho = mt * 16 + own_half * 8 + g;   // row of the stage; j: number of the token in the block
-                const bool valid = DIRECT ? (own_t[mt] < bg.frames && own_y[mt] < bg.rows && own_x[mt] < bg.cols) : rho < n;
-                const int j = DIRECT ? (own_t[mt] * bg.rows + own_y[mt]) * bg.cols + own_x[mt] : rho;
-                tok[mt] = valid ? j : -1;
-                if (tq < 2 && valid) {
-                    const int jr = min(j, n_rule);   // (positions from n_rule on are src tokens; the clamp keeps the operand in range)
-                    const int dj = div_n(jr * nd);
-                    if (!(j < n_rule && div_n((jr + 1) * nd) > dj)) {   // not a dst position: a src token
-                        is_src[mt] = true;
-                        key[mt] = score_key((own_half ? top[1] : top[0]) * invn[rho]);
-                        best[mt] = pos_of(own_half ? arg[1] : arg[0]);
-                    }
-                }
-            }
-        }
-
-        // ---- the r src with the best scores merge (ties: lowest position first)
-        const int n_src = n - nd, n_out = n_src - r;
-        bool merged[MT];
-        if (r <= n_out) {
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) merged[mt] = false;
-            for (int round = 0; round < r; ++round) {
-                uint32_t loc = 0;
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt) loc = max(loc, (is_src[mt] && !merged[mt]) ? key[mt] : 0u);
-                const uint32_t m = __reduce_max_sync(0xffffffffu, loc);
-                int cand = 0x7fffffff;   // lowest own position holding the maximum
-#pragma unroll
-                for (int mt = MT - 1; mt >= 0; --mt)
-                    if (is_src[mt] && !merged[mt] && key[mt] == m) cand = mt * 16 + own_half * 8 + g;
-                const int win = __reduce_min_sync(0xffffffffu, cand);
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-                    if (is_src[mt] && win == mt * 16 + own_half * 8 + g) merged[mt] = true;
-            }
-        } else {
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) merged[mt] = is_src[mt];
-            for (int round = 0; round < n_out; ++round) {
-                uint32_t loc = 0xffffffffu;
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt) loc = min(loc, merged[mt] ? key[mt] : 0xffffffffu);
-                const uint32_t m = __reduce_min_sync(0xffffffffu, loc);
-                int cand = -1;           // highest own position holding the minimum
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-                    if (merged[mt] && key[mt] == m) cand = mt * 16 + own_half * 8 + g;
-                const int win = __reduce_max_sync(0xffffffffu, cand);
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-                    if (merged[mt] && win == mt * 16 + own_half * 8 + g) merged[mt] = false;
-            }
-        }
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-            if (tq < 2 && tok[mt] >= 0) A[tok[mt]] = bi.start + (merged[mt] ? best[mt] : tok[mt]);
-        }
-        __syncwarp();   // every lane is done with the inverse norms (and, with several passes, the stage buffer)
-        if (!KEEP_A) {
-            if (more && lane == 0) issue(nxt, buf);
-        }
-    }
-    if (failed) {
-        // give copies that may still be in flight a bounded chance to land before the CTA's
-        // shared memory is released
-        mbar_wait_bounded(mbar0, STAGES == 2 ? ((it >> 1) & 1) : (it & 1), a.status, kDevTimeoutMatchLoad);
-        if (STAGES == 2) mbar_wait_bounded(mbar0 + 8, (it >> 1) & 1, a.status, kDevTimeoutMatchLoad);
-    }
-}
-
-template <int PASSES>
-static cudaError_t launch_match_t(const MatchArgs& a, int sm_count, cudaStream_t stream) {
-    constexpr int NMAX = 32 * PASSES;
-    constexpr int WARPS = match_warps_per_cta(NMAX);
-    const size_t smem = match_smem_bytes(NMAX);
-    const bool direct = a.geom != nullptr;
-    CUtensorMap mq, mk;
-    const int64_t N = a.n_tokens;
-    if (direct) {
-        if (!encode_block_map(&mq, a.src[0], a.layout, a.heads) || !encode_block_map(&mk, a.src[1], a.layout, a.heads)) return cudaErrorInvalidValue;
-    } else if (!encode_rows_tensor_map(&mq, a.xr[0], N, a.heads, kHeadDim, N * kHeadDim, NMAX) ||
-               !encode_rows_tensor_map(&mk, a.xr[1], N, a.heads, kHeadDim, N * kHeadDim, NMAX)) {
-        return cudaErrorInvalidValue;
-    }
-    const int64_t n_tasks = 2ll * a.heads * a.n_blocks;
-    int ctas_per_sm = (int)((224 * 1024) / (smem + 1024));
-    ctas_per_sm = ctas_per_sm < 1 ? 1 : (ctas_per_sm > 16 / WARPS ? (16 / WARPS < 1 ? 1 : 16 / WARPS) : ctas_per_sm);
-    int64_t grid = (n_tasks + WARPS - 1) / WARPS;
-    const int64_t cap = (int64_t)sm_count * ctas_per_sm;
-    if (grid > cap) grid = cap;
-    if (grid < 1) grid = 1;
-    if (direct)
-        return launch_kernel(match_kernel<PASSES, true>, (unsigned)grid, WARPS * 32, smem, stream, mq, mk, a);
-    return launch_kernel(match_kernel<PASSES, false>, (unsigned)grid, WARPS * 32, smem, stream, mq, mk, a);
-}
-
-// ------------------------------------------------------------------------------------
 // a2 under first-frame anchoring (the paper's appendix on error mitigation: all tokens of frame 0 are dst tokens), for the
-//     blocks of the first frame group whose dst tokens exceed what match_kernel holds (a quarter of the largest block:
+//     blocks of the first frame group whose dst tokens exceed what match_team_kernel holds (a quarter of the largest block:
 //     blocks of two or three frames).  Same rule, plain formulation: one CTA per (tensor, head, block), the block's rows
 //     gathered through the reorder index into shared memory, inverse norms, for every src token the dot products with
 //     the dst tokens (the block's first n_dst tokens) by fp32 FMAs on exact bf16 products, best dst (ties: lowest),
@@ -440,7 +83,7 @@ __global__ void __launch_bounds__(kAnchorThreads) match_anchor_kernel(const Matc
     const int b = task % n_anchor, h = (task / n_anchor) % a.heads, t = task / (n_anchor * a.heads);
     const BlockInfo bi = a.blocks[b];
     const int n = bi.n, nd = t == 0 ? bi.nd_q : bi.nd_k, r = t == 0 ? bi.r_q : bi.r_k;
-    if (bi.n_rule == n || nd <= main_capacity || r == 0 || n > nmax) return;   // match_kernel has written this block's map
+    if (bi.n_rule == n || nd <= main_capacity || r == 0 || n > nmax) return;   // the match kernel has written this block's map
     unsigned char* rows = sm_anchor;
     float* inv = reinterpret_cast<float*>(sm_anchor + (size_t)nmax * kAnchorPitch);
     float* score = inv + nmax;
@@ -514,299 +157,10 @@ cudaError_t launch_match_anchor(const MatchArgs& a, const TensorView& src_q, con
 }
 
 cudaError_t launch_match(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
-    if (max_block_tokens <= 32) return launch_match_small(a, sm_count, stream);
-    if (max_block_tokens <= 64) return launch_match_t<2>(a, sm_count, stream);
-    if (max_block_tokens <= 128) return launch_match_t<4>(a, sm_count, stream);
-    return launch_match_t<8>(a, sm_count, stream);
+    return max_block_tokens <= 32 ? launch_match_small(a, sm_count, stream) : launch_match_mid(a, max_block_tokens, sm_count, stream);
 }
-
-// ------------------------------------------------------------------------------------
-// a3 (blocks of 33 to 256 tokens).  The same contraction as above, merged_sum = W x, for blocks that
-//     take several 32-token passes: lane l holds the map entries of tokens l, l + 32, ...; the kept rows
-//     are walked in tiles of 16, the tokens in steps of 16, and the x fragments are fetched per
-//     (row tile, token step) with ldmatrix.trans from the swizzled TMA stage (blocks come from the
-//     reordered copies).  Group sizes are counted with shared-memory atomics.
-// ------------------------------------------------------------------------------------
-__host__ __device__ constexpr int merge_multi_warps(int nmax) { return nmax <= 64 ? 16 : (nmax <= 128 ? 12 : 6); }   // as for the match kernel
-__host__ __device__ constexpr int merge_multi_stages(int nmax) { return nmax <= 32 ? 2 : 1; }                          // (see match_stages)
-__host__ __device__ constexpr int merge_multi_aux(int nmax) { return nmax * 8 + 16; }   // counts, reciprocals, 2 mbarriers
-__host__ __device__ constexpr int merge_multi_smem(int nmax) {
-    return merge_multi_warps(nmax) * (merge_multi_stages(nmax) * nmax * kRowBytes + merge_multi_aux(nmax)) + 1024 /*alignment slack*/;
-}
-
-template <int PASSES, bool DIRECT>
-__global__ void __launch_bounds__(merge_multi_warps(32 * PASSES) * 32, 1)
-merge_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                   const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_sq,
-                   const __grid_constant__ CUtensorMap map_sk, const __grid_constant__ CUtensorMap map_sv, const MergeArgs a) {
-    constexpr int NMAX = 32 * PASSES;
-    constexpr int WARPS = merge_multi_warps(NMAX);
-    constexpr int STAGES = merge_multi_stages(NMAX);
-    constexpr int KS = NMAX / 16;   // token steps
-    constexpr uint32_t STAGE_BYTES = NMAX * kRowBytes;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 2, tq = lane & 3;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
-    unsigned char* stage = smem + (size_t)warp * STAGES * STAGE_BYTES;                  // [STAGES][NMAX][128], 1024-aligned, swizzled
-    unsigned char* aux = smem + (size_t)WARPS * STAGES * STAGE_BYTES + (size_t)warp * merge_multi_aux(NMAX);
-    int* cnt = reinterpret_cast<int*>(aux);                                             // [NMAX] group size of kept row
-    float* rcnt = reinterpret_cast<float*>(aux + NMAX * 4);                             // [NMAX] its reciprocal
-    const uint32_t mbar0 = smem_u32(aux + NMAX * 8), stage0 = smem_u32(stage);
-
-    if (lane == 0) {
-        mbar_init(mbar0, 1);
-        mbar_init(mbar0 + 8, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    __syncwarp();
-
-    // task -> (tensor t, head h, unit u); units 0 .. n_blocks-1 are merging blocks, the rest are
-    // chunks of 32 special tokens (never merged: rows 0 .. n_special_total-1 are copied)
-    const int sp_chunks = DIRECT ? (a.layout.n_special > 0 ? a.layout.frames : 0) : (a.n_special_total + 31) / 32;
-    const int per_head = a.n_blocks + sp_chunks;
-    // direct mode: box extents and the box coordinates of the stage rows lane + 32 p
-    const int box_f = DIRECT ? min(a.layout.blk_frames, a.layout.frames) : 1, box_h = DIRECT ? min(a.layout.blk_h, a.layout.grid_h) : 1,
-              box_w = DIRECT ? min(a.layout.blk_w, a.layout.grid_w) : 1;
-    const int box_rows = box_f * box_h * box_w;
-    int own_t[PASSES], own_y[PASSES], own_x[PASSES];
-#pragma unroll
-    for (int p = 0; p < PASSES; ++p) {
-        const int rho = lane + 32 * p;
-        own_t[p] = DIRECT ? rho / (box_h * box_w) : 0;
-        own_y[p] = DIRECT ? (rho / box_w) % box_h : 0;
-        own_x[p] = DIRECT ? rho % box_w : 0;
-    }
-    if (DIRECT) {   // stage rows that no block load writes enter the MMAs with weight 0: they must hold finite values
-        for (int q = box_rows * 8 + lane; q < NMAX * 8; q += 32) {   // (a load of special tokens may overwrite some of them later)
-            *reinterpret_cast<uint4*>(stage + q * 16) = make_uint4(0u, 0u, 0u, 0u);
-            if (STAGES == 2) *reinterpret_cast<uint4*>(stage + STAGE_BYTES + q * 16) = make_uint4(0u, 0u, 0u, 0u);   // (one stage: there is no second buffer)
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-    }
-    BoxMap bm;
-    bm.clipped = false;
-    const int64_t n_tasks = 3ll * a.heads * per_head;
-    const int64_t stride = (int64_t)gridDim.x * WARPS;
-    const int64_t first = (int64_t)blockIdx.x * WARPS + warp;
-    TaskCursor cur, nxt;   // the task being processed; the task whose load is issued next
-    cur.init(first, stride, a.heads, per_head);
-    nxt = cur;
-
-    auto issue = [&](const TaskCursor& c, int buf) {   // lane 0 only; the whole NMAX-row box is transferred (rows past the head's end are zero filled)
-        const uint32_t mb = mbar0 + 8 * buf;
-        if (!DIRECT) {
-            const int start = c.u >= a.n_blocks ? (c.u - a.n_blocks) * 32 : __ldg(&a.blocks[c.u].start);
-            mbar_expect_tx(mb, STAGE_BYTES);
-            tma_rows_load(stage0 + buf * STAGE_BYTES, c.t == 0 ? &map_q : (c.t == 1 ? &map_k : &map_v), mb, start, c.h);
-        } else if (c.u >= a.n_blocks) {   // the special tokens of frame u - n_blocks
-            mbar_expect_tx(mb, (uint32_t)a.layout.n_special * kRowBytes);
-            const CUtensorMap* m = c.t == 0 ? &map_sq : (c.t == 1 ? &map_sk : &map_sv);
-            asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(
-                             stage0 + buf * STAGE_BYTES),
-                         "l"(reinterpret_cast<uint64_t>(m)), "r"(mb), "r"(0), "r"(0), "r"(c.u - a.n_blocks), "r"(c.h)
-                         : "memory");
-        } else {
-            const BlockGeom bg = a.geom[c.u];
-            mbar_expect_tx(mb, (uint32_t)box_rows * kRowBytes);
-            tma_block_load(stage0 + buf * STAGE_BYTES, c.t == 0 ? &map_q : (c.t == 1 ? &map_k : &map_v), mb, bg.x0, bg.y0, bg.s0, c.h);
-        }
-    };
-    depend_wait();
-    dependents_launch();
-    if (first < n_tasks && lane == 0) issue(nxt, 0);
-    nxt.advance();
-    if (STAGES == 2) {
-        if (first + stride < n_tasks && lane == 0) issue(nxt, 1);
-        nxt.advance();
-    }
-
-    int it = 0;
-    bool failed = false;
-    for (int64_t task = first; task < n_tasks; task += stride, ++it, cur.advance(), nxt.advance()) {
-        const int buf = STAGES == 2 ? (it & 1) : 0;
-        const uint32_t parity = STAGES == 2 ? ((it >> 1) & 1) : (it & 1);
-        const bool more = task + STAGES * stride < n_tasks;
-        const int t = cur.t, h = cur.h;
-        const bool special = cur.u >= a.n_blocks;
-        int start, n, r, moff;
-        BlockGeom bg{};
-        bm.clipped = false;
-        if (special) {
-            start = DIRECT ? (cur.u - a.n_blocks) * a.layout.n_special : (cur.u - a.n_blocks) * 32;
-            n = DIRECT ? a.layout.n_special : min(32, a.n_special_total - start);
-            r = 0;
-            moff = start;
-        } else {
-            if (DIRECT) {
-                bg = a.geom[cur.u];
-                bm.set(box_f, box_h, box_w, bg.frames, bg.rows, bg.cols);
-            }
-            const BlockInfo bi = a.blocks[cur.u];
-            start = bi.start;
-            n = bi.n;
-            r = t == 0 ? bi.r_q : bi.r_k;
-            moff = t == 0 ? bi.moff_q : bi.moff_k;
-        }
-        const int m_len = t == 0 ? a.m_q : a.m_k;
-        uint32_t* out = reinterpret_cast<uint32_t*>(a.merged[t] + ((int64_t)h * m_len + moff) * kHeadDim);   // 32 words per row
-        const uint32_t blk = stage0 + buf * STAGE_BYTES;
-
-        // the map entries do not depend on the staged rows: fetch them before waiting
-        // stage row lane + 32 p holds token tok[p] of the block (-1: none), merged into the token in stage ROW rep[p]
-        int rep[PASSES], tok[PASSES];
-#pragma unroll
-        for (int p = 0; p < PASSES; ++p) {
-            const int rho = lane + 32 * p;
-            tok[p] = !DIRECT || special ? (rho < n ? rho : -1)
-                                        : ((own_t[p] < bg.frames && own_y[p] < bg.rows && own_x[p] < bg.cols) ? (own_t[p] * bg.rows + own_y[p]) * bg.cols + own_x[p] : -1);
-            rep[p] = -1;
-            if (r > 0 && tok[p] >= 0) {
-                rep[p] = ld_global(a.assign[t == 0 ? 0 : 1] + (int64_t)h * a.n_tokens + start + tok[p]) - start;
-                if (rep[p] < 0 || rep[p] >= n) {   // corrupt map: record, treat as kept
-                    atomicCAS(a.status, kDevOk, kDevBadIndex);
-                    rep[p] = tok[p];
-                }
-                if (DIRECT) rep[p] = bm.row_of_token(rep[p]);
-            }
-        }
-        if (!mbar_wait_bounded(mbar0 + 8 * buf, parity, a.status, kDevTimeoutMatchLoad)) {
-            failed = true;
-            break;
-        }
-        if (r == 0) {   // nothing merges here: copy the rows, 16 bytes per lane (chunk c of row j sits at c ^ (j & 7))
-            const unsigned char* sb = stage + buf * STAGE_BYTES;
-            uint4* o4 = reinterpret_cast<uint4*>(out);
-            for (int q = lane; q < n * 8; q += 32) {
-                const int row = DIRECT ? bm.row_of_token(q >> 3) : q >> 3, ch = q & 7;
-                o4[q] = *reinterpret_cast<const uint4*>(sb + row * kRowBytes + ((ch ^ (row & 7)) << 4));
-            }
-            if (t == 0 && !special)
-                for (int j = lane; j < n; j += 32) a.rank_q[(int64_t)h * a.n_tokens + start + j] = moff + j;
-        } else {
-            // merged row of every token: rank of its representative among the kept tokens
-            unsigned kept[PASSES];
-            int kept_before[PASSES], n_kept = 0;
-#pragma unroll
-            for (int p = 0; p < PASSES; ++p) {
-                kept[p] = __ballot_sync(0xffffffffu, rep[p] == lane + 32 * p);   // rep == -1 for positions >= n
-                kept_before[p] = n_kept;
-                n_kept += __popc(kept[p]);
-                cnt[lane + 32 * p] = 0;
-            }
-            __syncwarp();
-            int row_of[PASSES];
-#pragma unroll
-            for (int p = 0; p < PASSES; ++p) {
-                row_of[p] = -1;
-                if (rep[p] >= 0) {
-#pragma unroll
-                    for (int pp = 0; pp < PASSES; ++pp)
-                        if ((rep[p] >> 5) == pp) row_of[p] = kept_before[pp] + __popc(kept[pp] & ((1u << (rep[p] & 31)) - 1u));
-                    atomicAdd(&cnt[row_of[p]], 1);
-                    if (t == 0) a.rank_q[(int64_t)h * a.n_tokens + start + tok[p]] = moff + row_of[p];
-                }
-            }
-            __syncwarp();
-#pragma unroll
-            for (int p = 0; p < PASSES; ++p)
-                if (lane + 32 * p < n_kept) rcnt[lane + 32 * p] = 1.0f / (float)cnt[lane + 32 * p];
-            __syncwarp();
-            const int n_ks = ((DIRECT ? box_rows : n) + 15) >> 4, n_mt = (n_kept + 15) >> 4;   // stage rows that may hold tokens
-            const int n_out = min(n_kept, n - r);   // (a corrupt map cannot overrun)
-#pragma unroll 1
-            for (int mt = 0; mt < n_mt; ++mt) {
-                const int r0 = 16 * mt + g, r1 = r0 + 8;   // this lane's two accumulator rows
-                float c[8][4];
-#pragma unroll
-                for (int nt = 0; nt < 8; ++nt) c[nt][0] = c[nt][1] = c[nt][2] = c[nt][3] = 0.f;
-#pragma unroll
-                for (int ks = 0; ks < KS; ++ks) {
-                    if (ks < n_ks) {   // warp-uniform
-                        // W fragment: rows of tokens 16 ks + {2 tq, 2 tq + 1, 2 tq + 8, 2 tq + 9} (held by pass ks / 2, lane 16 (ks & 1) + ..)
-                        const int src = 16 * (ks & 1) + 2 * tq;
-                        const int w0 = __shfl_sync(0xffffffffu, row_of[ks >> 1], src), w1 = __shfl_sync(0xffffffffu, row_of[ks >> 1], src + 1);
-                        const int w2 = __shfl_sync(0xffffffffu, row_of[ks >> 1], src + 8), w3 = __shfl_sync(0xffffffffu, row_of[ks >> 1], src + 9);
-                        uint32_t af[4];   // bf16 1.0 = 0x3f80
-                        af[0] = (w0 == r0 ? 0x3f80u : 0u) | (w1 == r0 ? 0x3f800000u : 0u);
-                        af[1] = (w0 == r1 ? 0x3f80u : 0u) | (w1 == r1 ? 0x3f800000u : 0u);
-                        af[2] = (w2 == r0 ? 0x3f80u : 0u) | (w3 == r0 ? 0x3f800000u : 0u);
-                        af[3] = (w2 == r1 ? 0x3f80u : 0u) | (w3 == r1 ? 0x3f800000u : 0u);
-                        if (__any_sync(0xffffffffu, (af[0] | af[1] | af[2] | af[3]) != 0u)) {   // no token of this step belongs to this row tile: skip
-                            const int tok = 16 * ks + (lane & 7) + ((lane >> 3) & 1) * 8;
-                            const uint32_t rowaddr = blk + tok * kRowBytes;
-#pragma unroll
-                            for (int np = 0; np < 4; ++np) {
-                                uint32_t bf[4];
-                                ldmatrix_x4_trans(bf, rowaddr + (((2 * np + (lane >> 4)) ^ (tok & 7)) << 4));
-                                mma_bf16_16816(c[2 * np], af, bf[0], bf[1]);
-                                mma_bf16_16816(c[2 * np + 1], af, bf[2], bf[3]);
-                            }
-                        }
-                    }
-                }
-                const bool s0 = r0 < n_out, s1 = r1 < n_out;
-                const float i0 = s0 ? rcnt[r0] : 0.f, i1 = s1 ? rcnt[r1] : 0.f;
-#pragma unroll
-                for (int nt = 0; nt < 8; ++nt) {
-                    if (s0) {
-                        const __nv_bfloat162 o = __floats2bfloat162_rn(c[nt][0] * i0, c[nt][1] * i0);
-                        out[r0 * 32 + nt * 4 + tq] = *reinterpret_cast<const uint32_t*>(&o);
-                    }
-                    if (s1) {
-                        const __nv_bfloat162 o = __floats2bfloat162_rn(c[nt][2] * i1, c[nt][3] * i1);
-                        out[r1 * 32 + nt * 4 + tq] = *reinterpret_cast<const uint32_t*>(&o);
-                    }
-                }
-            }
-        }
-        __syncwarp();   // every lane is done reading this stage buffer and the per-row tables
-        if (more && lane == 0) issue(nxt, buf);
-    }
-    if (failed) {
-        mbar_wait_bounded(mbar0, STAGES == 2 ? ((it >> 1) & 1) : (it & 1), a.status, kDevTimeoutMatchLoad);
-        if (STAGES == 2) mbar_wait_bounded(mbar0 + 8, (it >> 1) & 1, a.status, kDevTimeoutMatchLoad);
-    }
-}
-
-template <int PASSES>
-static cudaError_t launch_merge_multi(const MergeArgs& a, int sm_count, cudaStream_t stream) {
-    constexpr int NMAX = 32 * PASSES;
-    constexpr int WARPS = merge_multi_warps(NMAX);
-    constexpr int STAGES = merge_multi_stages(NMAX);
-    CUtensorMap m[3], sp[3];
-    const int64_t N = a.n_tokens;
-    const bool direct = a.geom != nullptr;
-    for (int t = 0; t < 3; ++t) {
-        if (direct) {
-            if (!encode_block_map(&m[t], a.src[t], a.layout, a.heads)) return cudaErrorInvalidValue;
-            if (a.layout.n_special > 0 &&
-                !encode_frame_tensor_map(&sp[t], a.src[t].ptr, a.layout.tokens_per_frame, a.layout.frames, a.heads, a.src[t].stride_token,
-                                         a.src[t].stride_head, a.layout.n_special))
-                return cudaErrorInvalidValue;
-            if (a.layout.n_special <= 0) sp[t] = m[t];   // never used
-        } else {
-            if (!encode_rows_tensor_map(&m[t], a.xr[t], N, a.heads, kHeadDim, N * kHeadDim, NMAX)) return cudaErrorInvalidValue;
-            sp[t] = m[t];   // not used
-        }
-    }
-    const int sp_units = direct ? (a.layout.n_special > 0 ? a.layout.frames : 0) : (a.n_special_total + 31) / 32;
-    const int64_t n_tasks = 3ll * a.heads * (a.n_blocks + sp_units);
-    int64_t grid = (n_tasks + WARPS - 1) / WARPS;
-    if (grid > sm_count) grid = sm_count;
-    if (grid < 1) grid = 1;
-    if (direct)
-        return launch_kernel(merge_multi_kernel<PASSES, true>, (unsigned)grid, WARPS * 32, merge_multi_smem(NMAX), stream, m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
-    return launch_kernel(merge_multi_kernel<PASSES, false>, (unsigned)grid, WARPS * 32, merge_multi_smem(NMAX), stream, m[0], m[1], m[2], sp[0], sp[1], sp[2], a);
-}
-
 cudaError_t launch_merge(const MergeArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
-    if (max_block_tokens <= 32) return launch_merge_small(a, sm_count, stream);
-    if (max_block_tokens <= 64) return launch_merge_multi<2>(a, sm_count, stream);
-    if (max_block_tokens <= 128) return launch_merge_multi<4>(a, sm_count, stream);
-    return launch_merge_multi<8>(a, sm_count, stream);
+    return max_block_tokens <= 32 ? launch_merge_small(a, sm_count, stream) : launch_merge_mid(a, max_block_tokens, sm_count, stream);
 }
 
 // ------------------------------------------------------------------------------------
@@ -829,7 +183,7 @@ __global__ void __launch_bounds__(kDevWarps * 32, 2)
 deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a) {
     constexpr uint32_t STAGE_BYTES = 32 * kRowBytes;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char* smem = smem_raw + align_pad(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tq = lane & 3;   // MMA accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
     unsigned char* stage = smem + (size_t)warp * kDevStages * STAGE_BYTES;
@@ -911,7 +265,7 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
             const unsigned multi = __ballot_sync(0xffffffffu, rep == lane && group_size >= 2);
             const int row_of = group_size >= 2 ? __popc(multi & ((1u << rep) - 1u)) : -1;
             if (rep == lane && group_size >= 2) rcnt[row_of] = 1.0f / (float)group_size;
-            // group sums = W x on the tensor cores, as in merge_tc_kernel: W [16 means][32 tokens] of zeros and ones
+            // group sums = W x on the tensor cores, as in merge_small_kernel: W [16 means][32 tokens] of zeros and ones
             uint32_t bf[2][4][4];
             const int n_ks = box_rows > 16 ? 2 : 1;
 #pragma unroll
@@ -1329,21 +683,9 @@ cudaError_t configure_kernels() {
 #define HTTM_SET_SMEM(kern, bytes)                                                                      \
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bytes));          \
     if (e != cudaSuccess) return e;
-    HTTM_SET_SMEM((match_kernel<2, false>), match_smem_bytes(64));
-    HTTM_SET_SMEM((match_kernel<2, true>), match_smem_bytes(64));
-    HTTM_SET_SMEM((match_kernel<4, true>), match_smem_bytes(128));
-    HTTM_SET_SMEM((match_kernel<8, true>), match_smem_bytes(256));
-    HTTM_SET_SMEM((match_kernel<4, false>), match_smem_bytes(128));
-    HTTM_SET_SMEM((match_kernel<8, false>), match_smem_bytes(256));
     HTTM_SET_SMEM(deviation_kernel, kDevSmem);
-    HTTM_SET_SMEM((merge_multi_kernel<2, false>), merge_multi_smem(64));
-    HTTM_SET_SMEM((merge_multi_kernel<4, false>), merge_multi_smem(128));
-    HTTM_SET_SMEM((merge_multi_kernel<8, false>), merge_multi_smem(256));
-    HTTM_SET_SMEM((merge_multi_kernel<2, true>), merge_multi_smem(64));
-    HTTM_SET_SMEM((merge_multi_kernel<4, true>), merge_multi_smem(128));
-    HTTM_SET_SMEM((merge_multi_kernel<8, true>), merge_multi_smem(256));
 #undef HTTM_SET_SMEM
-    if ((e = configure_small_blocks()) != cudaSuccess) return e;
+    if ((e = configure_small_blocks()) != cudaSuccess || (e = configure_mid_blocks()) != cudaSuccess) return e;
     return configure_attention();
 }
 

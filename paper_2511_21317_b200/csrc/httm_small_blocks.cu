@@ -21,70 +21,6 @@ namespace {
 constexpr int kWarps = 8;
 constexpr uint32_t kStage = 32 * kRowBytes;   // one block of one tensor, 128-byte swizzle
 
-// (head, unit of the head) of a linear index that advances by a fixed stride
-struct UnitCursor {
-    int h, u, sh, su, units;
-    __device__ void init(int first, int stride, int units_) {
-        units = units_;
-        h = first / units;
-        u = first - h * units;
-        sh = stride / units;
-        su = stride - sh * units;
-    }
-    __device__ __forceinline__ void advance() {
-        h += sh;
-        u += su;
-        if (u >= units) {
-            u -= units;
-            ++h;
-        }
-    }
-};
-
-struct Geometry {   // BlockGeom in registers
-    int s0, y0, x0, frames, rows, cols;
-};
-__device__ __forceinline__ int4 load_geometry(const BlockGeom* geom, int u) { return __ldg(reinterpret_cast<const int4*>(geom + u)); }
-__device__ __forceinline__ Geometry unpack_geometry(const int4& v) {
-    Geometry g;
-    g.s0 = (int16_t)(v.x & 0xffff);
-    g.y0 = v.x >> 16;
-    g.x0 = (int16_t)(v.y & 0xffff);
-    g.frames = v.y >> 16;
-    g.rows = (int16_t)(v.z & 0xffff);
-    g.cols = v.z >> 16;
-    return g;
-}
-// d (16x8 fp32) = a (16x16 bf16, row) * b (16x8 bf16, col): the first step of a sum
-__device__ __forceinline__ void mma_first(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
-                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
-}
-// floor(x / d) for 0 <= x < 2048, 1 <= d <= 64: (x + 0.5) / d is at least 1 / 128 away from an integer, far more than the error of the
-// approximate quotient
-__device__ __forceinline__ int small_div(int x, int d) { return (int)__fdividef((float)x + 0.5f, (float)d); }
-struct Box {   // extents of a block's TMA box (the block shape, clipped to the scene)
-    int frames, h, w, rows;
-    __device__ void set(const SourceLayout& L) {
-        frames = min(L.blk_frames, L.frames);
-        h = min(L.blk_h, L.grid_h);
-        w = min(L.blk_w, L.grid_w);
-        rows = frames * h * w;
-    }
-};
-// stage row of token j of a block
-__device__ __forceinline__ int row_of_token(const Box& box, const Geometry& g, int j) {
-    if (g.rows == box.h && g.cols == box.w) return j;   // (frames come last: clipping them leaves the numbering alone)
-    const int plane = g.rows * g.cols, t = small_div(j, plane), rem = j - t * plane, y = small_div(rem, g.cols);
-    return (t * box.h + y) * box.w + rem - y * g.cols;
-}
-// token number of stage row rho, -1 if the row holds none
-__device__ __forceinline__ int token_of_row(const Box& box, const Geometry& g, int rho) {
-    const int line = small_div(rho, box.w), t = small_div(line, box.h), y = line - t * box.h, x = rho - line * box.w;
-    return t < g.frames && y < g.rows && x < g.cols ? (t * g.rows + y) * g.cols + x : -1;
-}
-
 // ------------------------------------------------------------------------------------ match
 // Per tensor: cosine of every token with every dst token (at most 8), best dst per src token, the r best src tokens
 // merge; ties go to the lowest dst and the lowest src position.  The dot products and the squared norms (diagonals of a tile
@@ -93,18 +29,12 @@ __device__ __forceinline__ int token_of_row(const Box& box, const Geometry& g, i
 // Row rho of the stage is owned, from the arg-max on, by lane (rho & 7) * 4 + ((rho >> 3) & 1), slot rho >> 4.
 constexpr int kMatchSmem = kWarps * (2 * (int)kStage + 16) + 1024 /*alignment slack*/;
 
-__device__ __forceinline__ float inv_norm(float square) {   // 1 / max(|x|, 1e-12), within 2 ulp
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(square));
-    return fminf(r, 1e12f);
-}
-
 // SPLIT: fewer units than warps: a warp has one tensor of one unit
 template <bool DIRECT, bool SPLIT>
 __global__ void __launch_bounds__(kWarps * 32, 3)
 match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ MatchArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char* smem = smem_raw + align_pad(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tq = lane & 3, odd = tq & 1;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
     const uint32_t stage0 = smem_u32(smem + (size_t)warp * 2 * kStage);
@@ -337,29 +267,10 @@ constexpr int kMergeSmem = kWarps * (3 * (int)kStage + kMergeAux) + 1024 /*align
 __device__ __forceinline__ void stmatrix_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
     asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
 }
-// fragment of W (16 merged rows x 16 tokens): rw = merged rows of this lane's four tokens, r0 its first row; bf16 1.0 = 0x3f80
-__device__ __forceinline__ void w_fragment(uint32_t* af, const int* rw, int r0) {
-    const int r1 = r0 + 8;
-    af[0] = (rw[0] == r0 ? 0x3f80u : 0u) | (rw[1] == r0 ? 0x3f800000u : 0u);
-    af[1] = (rw[0] == r1 ? 0x3f80u : 0u) | (rw[1] == r1 ? 0x3f800000u : 0u);
-    af[2] = (rw[2] == r0 ? 0x3f80u : 0u) | (rw[3] == r0 ? 0x3f800000u : 0u);
-    af[3] = (rw[2] == r1 ? 0x3f80u : 0u) | (rw[3] == r1 ? 0x3f800000u : 0u);
-}
-__device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t*>(&v);
-}
-
-// DIRECT: the blocks come straight from the original tensors (5-D block maps), the special tokens frame by
-// frame (4-D frame maps); otherwise from the reordered copies, specials in chunks of 32.
-struct MergeMaps {
-    CUtensorMap block[3], special[3];
-};
-
 template <bool DIRECT, bool SPLIT>
 __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __grid_constant__ MergeMaps maps, const __grid_constant__ MergeArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    unsigned char* smem = smem_raw + align_pad(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tq = lane & 3;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
     unsigned char* stage = smem + (size_t)warp * 3 * kStage;
@@ -656,21 +567,8 @@ cudaError_t launch_match_small(const MatchArgs& a, int sm_count, cudaStream_t st
 
 cudaError_t launch_merge_small(const MergeArgs& a, int sm_count, cudaStream_t stream) {
     MergeMaps m;
-    const int64_t N = a.n_tokens;
     const bool direct = a.geom != nullptr;
-    for (int t = 0; t < 3; ++t) {
-        if (direct) {
-            if (!encode_block_map(&m.block[t], a.src[t], a.layout, a.heads)) return cudaErrorInvalidValue;
-            m.special[t] = m.block[t];
-            if (a.layout.n_special > 0 &&
-                !encode_frame_tensor_map(&m.special[t], a.src[t].ptr, a.layout.tokens_per_frame, a.layout.frames, a.heads, a.src[t].stride_token,
-                                         a.src[t].stride_head, a.layout.n_special))
-                return cudaErrorInvalidValue;
-        } else {
-            if (!encode_rows_tensor_map(&m.block[t], a.xr[t], N, a.heads, kHeadDim, N * kHeadDim, 32)) return cudaErrorInvalidValue;
-            m.special[t] = m.block[t];   // not used
-        }
-    }
+    if (!encode_merge_maps(&m, a, 32)) return cudaErrorInvalidValue;
     const int sp_units = direct ? (a.layout.n_special > 0 ? a.layout.frames : 0) : (a.n_special_total + 31) / 32;
     const int64_t units = (int64_t)a.heads * (a.n_blocks + sp_units);
     const int parts = 3 * units <= 2ll * kWarps * sm_count ? 3 : 1, grid = small_grid(units * parts, sm_count, 2);

@@ -1,0 +1,35 @@
+"""Blocks of 33 .. 256 tokens at the limits of the teams that work them off, against the oracle; and many blocks per team, where loads,
+tables and groups run one block ahead, against the same head alone, bit for bit."""
+import numpy as np
+import pytest
+
+from paper_2511_21317_b200 import binding as hb
+from paper_2511_21317_b200 import synth
+from tests.test_gpu_parity import report_peaky, run_case
+from tests.test_gpu_small_blocks import ITEMS, run
+
+pytestmark = pytest.mark.gpu
+
+
+# (block, ratio_q, ratio_kv): few merge (picked one by one), half, nearly all; block sizes around 32, 64, 128 and 256
+@pytest.mark.parametrize("blk,ratio_q,ratio_kv", [((1, 3, 11), 0.1, 0.9), ((4, 4, 4), 0.375, 0.2), ((1, 5, 13), 0.1, 0.7), ((2, 8, 8), 0.4, 0.0),
+                                                  ((3, 1, 43), 0.3, 0.95), ((4, 8, 8), 0.1, 0.5), ((3, 5, 17), 0.7, 0.99)],
+                         ids=["33", "64", "65", "128", "129", "256", "255"])
+def test_limits_of_the_teams(blk, ratio_q, ratio_kv):
+    wl = synth.Workload("limits", 4, blk[1] + 4, 2 * blk[2] + 1, *blk, ratio_q, ratio_kv, n_camera=1, n_register=4, heads=2, seed=5)
+    report_peaky("limits", run_case(wl, peaky=True))
+    x = synth.make_identical_block_tokens(wl, seed=6)   # all similarities of a block are ties: the order of the positions decides
+    _, k, v = synth.make_qkv(wl)
+    report_peaky("ties", run_case(wl, x, x, v, peaky=True))
+
+
+@pytest.mark.parametrize("blk,frames,specials", [((4, 4, 4), 34, 4), ((2, 8, 8), 41, 4), ((4, 8, 8), 42, 4), ((4, 4, 4), 34, 70)],
+                         ids=["64", "128", "256", "over_reordered_copies"])
+def test_many_blocks_per_team(blk, frames, specials):
+    wl = synth.Workload("many", frames, 21, 26, *blk, 0.6, 0.8, n_camera=1, n_register=specials, heads=24, seed=2)
+    q, k, v = (hb.bf16_from_bits(x, "cuda:0") for x in synth.make_qkv(wl))
+    whole = run(hb.HttmConfig.of(wl), (q, k, v))
+    for h in (0, 13, 23):
+        one = run(hb.HttmConfig.of(wl.replace(heads=1)), (q[h:h + 1], k[h:h + 1], v[h:h + 1]))
+        for name in ITEMS:
+            assert np.array_equal(whole[name][h], one[name][0]), (name, h)
