@@ -182,7 +182,8 @@ TensorView view(const __nv_bfloat16* p, int64_t rows) { return TensorView{p, row
 
 float scale_log2() { return 1.4426950408889634f / std::sqrt((float)kHeadDim); }
 
-int stage_reorder(httm_ctx* c, const httm_tensor& q, const httm_tensor& k, const httm_tensor& v, cudaStream_t s) {
+// clear: the selection state of the outlier filter is set to zero for the stages behind this one
+int stage_reorder(httm_ctx* c, const httm_tensor& q, const httm_tensor& k, const httm_tensor& v, cudaStream_t s, bool clear = false) {
     ReorderArgs a{};
     a.src[0] = view(q);
     a.src[1] = view(k);
@@ -195,6 +196,10 @@ int stage_reorder(httm_ctx* c, const httm_tensor& q, const httm_tensor& k, const
     a.heads = c->cfg.heads;
     a.inv_norm[0] = c->d_inv_norm_q;   // (null unless the context has large blocks)
     a.inv_norm[1] = c->d_inv_norm_k;
+    if (clear) {
+        a.clear = c->d_sel;
+        a.n_clear = kSelWords;
+    }
     c->launches++;
     return check_cuda(c, launch_reorder(a, s), "reorder launch");
 }
@@ -260,7 +265,7 @@ int stage_big_select(httm_ctx* c, cudaStream_t s) {
 }
 
 // src: the original Q, K, V (direct mode) or nullptr (blocks come from the reordered copies)
-int stage_match(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr) {
+int stage_match(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr, bool clear = false) {
     if (c->big()) return c->fail(HTTM_ERR_UNSUPPORTED, "blocks of more than 256 tokens are matched by the large-block stages");
     MatchArgs a{};
     if (src) {
@@ -278,6 +283,10 @@ int stage_match(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr) {
     a.n_tokens = c->n_tokens;
     a.heads = c->cfg.heads;
     a.status = c->d_status;
+    if (clear) {
+        a.clear = c->d_sel;
+        a.n_clear = kSelWords;
+    }
     c->launches++;
     int rc = check_cuda(c, launch_match(a, c->max_block, c->sm_count, s), "match launch");
     if (rc || c->n_anchor == 0) return rc;
@@ -288,7 +297,8 @@ int stage_match(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr) {
                       "anchor match launch");
 }
 
-int stage_merge(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr) {
+// chained: inside a call, behind the stages that come before it (see httm_launch.cuh)
+int stage_merge(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr, bool chained = false) {
     if ((c->big() || sorted_filter(c)) && src)
         return c->fail(HTTM_ERR_UNSUPPORTED, "this context merges from the reordered copies (blocks of more than 256 tokens, or outlier filtering with blocks of more than 32)");
     MergeArgs a{};
@@ -322,6 +332,7 @@ int stage_merge(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr) {
     a.m_q = c->q_rows();
     a.m_k = c->m_k;
     a.status = c->d_status;
+    a.early = chained;
     c->launches++;
     if (c->big() || sorted_filter(c)) return check_cuda(c, launch_big_merge(a, c->max_block, s), "sorted-group merge launch");
     return check_cuda(c, launch_merge(a, c->max_block, c->sm_count, s), "merge launch");
@@ -363,7 +374,7 @@ int stage_attention(httm_ctx* c, cudaStream_t s, const httm_tensor* final_out = 
     return check_cuda(c, launch_attention(a, c->sm_count, s), "attention launch");
 }
 
-int stage_unmerge(httm_ctx* c, const httm_tensor& out, cudaStream_t s) {
+int stage_unmerge(httm_ctx* c, const httm_tensor& out, cudaStream_t s, bool chained = false) {
     if (c->om_stale) return c->fail(HTTM_ERR_INVALID_ARG, "the merged output is not there: the last attention launch unmerged in its epilogue (run HTTM_STAGE_ATTENTION first)");
     UnmergeArgs a{};
     a.o_m = c->filtering() ? c->d_om_var : c->d_om;
@@ -376,12 +387,14 @@ int stage_unmerge(httm_ctx* c, const httm_tensor& out, cudaStream_t s) {
     a.heads = c->cfg.heads;
     a.m_q = c->q_rows();
     a.status = c->d_status;
+    a.early = chained;
     c->launches++;
     return check_cuda(c, launch_unmerge(a, s), "unmerge launch");
 }
 
 // Sec. 3.4 / Algorithm 2 between match and merge: deviations, global threshold, map update, per-head offsets
-int stage_outlier(httm_ctx* c, const httm_tensor& q, cudaStream_t s) {
+// chained: inside a call, whose first kernel has cleared the selection state
+int stage_outlier(httm_ctx* c, const httm_tensor& q, cudaStream_t s, bool chained = false) {
     OutlierArgs a{};
     a.geom = c->d_geom;
     a.blocks = c->d_blocks;
@@ -405,8 +418,9 @@ int stage_outlier(httm_ctx* c, const httm_tensor& q, cudaStream_t s) {
     a.heads = c->cfg.heads;
     a.n_special_total = c->cfg.frames * c->n_special;
     a.status = c->d_status;
+    a.early = chained;
     int rc;
-    if ((rc = check_cuda(c, cudaMemsetAsync(c->d_sel, 0, kSelWords * sizeof(int32_t), s), "selection state reset"))) return rc;
+    if (!chained && (rc = check_cuda(c, cudaMemsetAsync(c->d_sel, 0, kSelWords * sizeof(int32_t), s), "selection state reset"))) return rc;
     if (c->exchange) {
         // Head-sharded layer: the threshold is one for all heads, so every level's histogram is summed over the shards
         // (the caller's exchange, in stream order) before its bin is chosen.  Nine kernels (ten over the reordered copies).
@@ -484,36 +498,36 @@ int global_impl(httm_ctx* c, const httm_tensor& q, const httm_tensor& k, const h
     };
     int rc;
     if (c->big()) {   // six kernels: reorder (+ norms), scores, select, merge, attention, unmerge
-        if ((rc = part(stage_reorder(c, q, k, v, s), "reorder"))) return rc;
+        if ((rc = part(stage_reorder(c, q, k, v, s, c->filtering()), "reorder"))) return rc;
         if ((rc = part(stage_big_scores(c, s), "big_scores"))) return rc;
         if ((rc = part(stage_big_select(c, s), "big_select"))) return rc;
-        if (c->filtering() && (rc = part(stage_outlier(c, q, s), "outlier_filter"))) return rc;
-        if ((rc = part(stage_merge(c, s), "merge"))) return rc;
+        if (c->filtering() && (rc = part(stage_outlier(c, q, s, true), "outlier_filter"))) return rc;
+        if ((rc = part(stage_merge(c, s, nullptr, true), "merge"))) return rc;
         if ((rc = part(stage_attention(c, s), "attention"))) return rc;
-        return part(stage_unmerge(c, out, s), "unmerge");
+        return part(stage_unmerge(c, out, s, true), "unmerge");
     }
     if (sorted_filter(c)) {   // outlier filtering with blocks of 33 .. 256 tokens: everything from the reordered copies
-        if ((rc = part(stage_reorder(c, q, k, v, s), "reorder"))) return rc;
+        if ((rc = part(stage_reorder(c, q, k, v, s, c->filtering()), "reorder"))) return rc;
         if ((rc = part(stage_match(c, s), "match"))) return rc;
-        if ((rc = part(stage_outlier(c, q, s), "outlier_filter"))) return rc;
-        if ((rc = part(stage_merge(c, s), "merge"))) return rc;
+        if ((rc = part(stage_outlier(c, q, s, true), "outlier_filter"))) return rc;
+        if ((rc = part(stage_merge(c, s, nullptr, true), "merge"))) return rc;
         if ((rc = part(stage_attention(c, s), "attention"))) return rc;
-        return part(stage_unmerge(c, out, s), "unmerge");
+        return part(stage_unmerge(c, out, s, true), "unmerge");
     }
     if (direct_mode(c)) {   // the temporal reorder is folded into the block loads of match and merge
         const httm_tensor src[3] = {q, k, v};
-        if ((rc = part(stage_match(c, s, src), "match_direct"))) return rc;
-        if (c->filtering() && (rc = part(stage_outlier(c, q, s), "outlier_filter"))) return rc;
-        if ((rc = part(stage_merge(c, s, src), "merge_direct"))) return rc;
+        if ((rc = part(stage_match(c, s, src, c->filtering()), "match_direct"))) return rc;
+        if (c->filtering() && (rc = part(stage_outlier(c, q, s, true), "outlier_filter"))) return rc;
+        if ((rc = part(stage_merge(c, s, src, true), "merge_direct"))) return rc;
     } else {
-        if ((rc = part(stage_reorder(c, q, k, v, s), "reorder"))) return rc;
+        if ((rc = part(stage_reorder(c, q, k, v, s, c->filtering()), "reorder"))) return rc;
         if ((rc = part(stage_match(c, s), "match"))) return rc;
-        if ((rc = part(stage_merge(c, s), "merge"))) return rc;
+        if ((rc = part(stage_merge(c, s, nullptr, true), "merge"))) return rc;
     }
     // ... and the unmerge into the attention epilogue: three kernels
     if (fused_unmerge(c)) return part(stage_attention(c, s, &out), "attention_unmerge");
     if ((rc = part(stage_attention(c, s), "attention"))) return rc;
-    return part(stage_unmerge(c, out, s), "unmerge");
+    return part(stage_unmerge(c, out, s, true), "unmerge");
 }
 
 int device_status(httm_ctx* c, int32_t* value) {

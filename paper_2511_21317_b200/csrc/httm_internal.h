@@ -62,6 +62,8 @@ struct ReorderArgs {
     const int32_t* pi;       // [N]
     int32_t n_tokens, heads;
     float* inv_norm[2];      // optional, [H][N] each: 1 / max(|x|, 1e-12) of the reordered Q and K tokens (large-block path)
+    int32_t* clear;   // optional: words to set to zero for the kernels behind this one
+    int32_t n_clear;
 };
 
 // Large-block path (blocks of 257 .. 4096 tokens; Sec. 4.1's 128 x 30 regime): matching as a dense contraction.
@@ -90,6 +92,8 @@ struct MatchArgs {
     const BlockInfo* blocks;
     int32_t n_blocks, n_tokens, heads;
     int32_t* status;
+    int32_t* clear;   // optional: words to set to zero for the kernels behind this one
+    int32_t n_clear;
 };
 
 struct MergeArgs {
@@ -110,6 +114,7 @@ struct MergeArgs {
     const BlockInfo* blocks;
     int32_t n_blocks, n_tokens, heads, n_special_total, m_q, m_k;
     int32_t* status;
+    bool early;   // launched behind the match kernel of the same tensors: they may be read ahead of depend_wait (httm_launch.cuh)
 };
 
 // Query outlier filtering (Sec. 3.4): deviations, global threshold, map rewrite, per-head merged offsets.
@@ -146,6 +151,7 @@ struct OutlierArgs {
     // histograms, the bin is chosen by a kernel of its own once the histograms of all shards have been summed
     int64_t total_count;
     int32_t defer_select;
+    bool early;   // launched behind the match kernel of the same tensors, which may be read ahead of depend_wait (httm_launch.cuh)
 };
 
 struct UnmergeArgs {
@@ -156,6 +162,7 @@ struct UnmergeArgs {
     int64_t out_stride_head, out_stride_token;
     int32_t n_tokens, heads, m_q;
     int32_t* status;
+    bool early;   // launched behind the attention kernel of the call that wrote rank_q, which may be read ahead of depend_wait (httm_launch.cuh)
 };
 
 struct AttentionArgs {

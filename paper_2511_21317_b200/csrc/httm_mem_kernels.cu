@@ -31,6 +31,7 @@ __global__ void __launch_bounds__(kReorderThreads) reorder_kernel(const __grid_c
     }
     depend_wait();
     dependents_launch();
+    if (t == 0 && h == 0) clear_words(a.clear, a.n_clear, blockIdx.x, gridDim.x);
 #pragma unroll
     for (int u = 0; u < kReorderUnroll; ++u) {
         const int p = base + u * (kReorderThreads / 8) + slot;
@@ -222,13 +223,14 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
         mbar_expect_tx(mb, (uint32_t)box_rows * kRowBytes);
         tma_block_load(stage0 + buf * STAGE_BYTES, &map_q, mb, bg.x0, bg.y0, bg.s0, c.h);
     };
-    depend_wait();
-    dependents_launch();
+    if (!a.early) depend_wait();
 #pragma unroll
     for (int st = 0; st < kDevStages; ++st) {
         if (first + st * stride < n_tasks && lane == 0) issue(nxt, st);
         nxt.advance();
     }
+    if (a.early) depend_wait();
+    dependents_launch();
 
     int buf = 0;
     uint32_t parity = 0;
@@ -654,10 +656,11 @@ __global__ void __launch_bounds__(kUnmergeThreads) unmerge_kernel(const __grid_c
         const int i = base + u * (kUnmergeThreads / 8) + slot;
         p[u] = i < a.n_tokens ? __ldg(a.pi_inv + i) : 0;
     }
-    depend_wait();
-    dependents_launch();
+    if (!a.early) depend_wait();
 #pragma unroll
-    for (int u = 0; u < kUnmergeUnroll; ++u) row[u] = ld_global(rank + p[u]);
+    for (int u = 0; u < kUnmergeUnroll; ++u) row[u] = ld_global_cg(rank + p[u]);
+    if (a.early) depend_wait();
+    dependents_launch();
 #pragma unroll
     for (int u = 0; u < kUnmergeUnroll; ++u) {
         if (row[u] < 0 || row[u] >= a.m_q) {   // corrupt map: record, copy row 0 instead of reading out of range

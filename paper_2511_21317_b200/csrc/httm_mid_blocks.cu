@@ -134,6 +134,7 @@ match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     if (blockIdx.x < n_units) fetch();
     depend_wait();
     dependents_launch();
+    clear_words(a.clear, a.n_clear, blockIdx.x, gridDim.x);
     if (blockIdx.x < n_units && tid == 0) {
         issue(0, geom_next, bi_next.start, h_next);
         issue(1, geom_next, bi_next.start, h_next);
@@ -526,16 +527,20 @@ __global__ void __launch_bounds__(32 * W, team_ctas(W, P)) merge_team_kernel(con
             }
         }
     };
-    depend_wait();
-    dependents_launch();
     Meta m{}, meta_next{};
-    int n_kept[2] = {0, 0};
-    if (blockIdx.x < n_units) {
-        m = fetch();
-        if (tid == 0) {
+    if (blockIdx.x < n_units) m = fetch();
+    auto issue_first = [&]() {
+        if (blockIdx.x < n_units && tid == 0) {
             issue(0, 0, m);
             issue(1, 1, m);
         }
+    };
+    if (a.early) issue_first();
+    depend_wait();
+    dependents_launch();
+    if (!a.early) issue_first();
+    int n_kept[2] = {0, 0};
+    if (blockIdx.x < n_units) {
         Targets x = load_targets(m);
         find_kept(m, x, 0);
         team_sync<W>();

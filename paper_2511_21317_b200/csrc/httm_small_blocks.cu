@@ -81,6 +81,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     if (first < n_units) fetch();
     depend_wait();
     dependents_launch();
+    clear_words(a.clear, a.n_clear, blockIdx.x, gridDim.x);
     if (first < n_units && lane == 0)
         for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t) issue(t, bg_next, bi_next.start, h_next);
 
@@ -325,10 +326,13 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
             const BlockInfo bi = a.blocks[next.u];
             m.start = bi.start;
             m.sizes = bi.n | (bi.r_q << 8) | (bi.r_k << 16);
-            m.moff_q = a.moff_q_var ? ld_global(a.moff_q_var + (int64_t)m.h * a.n_blocks + next.u) : bi.moff_q;
+            m.moff_q = bi.moff_q;
             m.moff_k = bi.moff_k;
         }
         return m;
+    };
+    auto fetch_offset = [&](Meta* m) {   // with outlier filtering the heads' rows start elsewhere
+        if (a.moff_q_var && next.u < a.n_blocks) m->moff_q = ld_global(a.moff_q_var + (int64_t)m->h * a.n_blocks + next.u);
     };
     auto issue = [&](int t, const Meta& m) {   // lane 0 only
         const uint32_t mb = bar0 + 8 * t, dst = stage0 + t * kStage;
@@ -356,16 +360,21 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
         const int tok = token_of_lane(m);
         return m.r(map) > 0 && tok >= 0 ? ld_global(a.assign[map] + (int64_t)m.h * a.n_tokens + m.start + tok) - m.start : -1;
     };
-    depend_wait();
-    dependents_launch();
     Meta meta_next{};
-    int target_next[2] = {-1, -1};
-    if (first < n_units) {
-        meta_next = fetch();
-        if (lane == 0)
+    if (first < n_units) meta_next = fetch();
+    auto issue_first = [&]() {
+        if (first < n_units && lane == 0)
 #pragma unroll
             for (int t = 0; t < 3; ++t)
                 if (!SPLIT || t == t_first) issue(t, meta_next);
+    };
+    if (a.early) issue_first();
+    depend_wait();
+    dependents_launch();
+    if (!a.early) issue_first();
+    int target_next[2] = {-1, -1};
+    if (first < n_units) {
+        fetch_offset(&meta_next);
         if (t_first == 0) target_next[0] = load_target(meta_next, 0);
         if (t_last > 0) target_next[1] = load_target(meta_next, 1);
     }
@@ -381,6 +390,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
         if (more) {
             next.advance();
             meta_next = fetch();   // in flight while this unit is worked off
+            fetch_offset(&meta_next);
         }
         const int tok = token_of_lane(m), n = m.n();
         uint32_t af0[2][4];   // W fragments of the first 16 merged rows (K's serve V)

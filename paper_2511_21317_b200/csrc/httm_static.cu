@@ -209,7 +209,7 @@ extern "C" int httm_global_attention_static(const httm_config* cfg, httm_tensor 
     ga.xr[0] = d_qr; ga.xr[1] = d_kr; ga.xr[2] = d_vr; ga.assign[0] = d_aq; ga.assign[1] = d_ak;
     ga.merged[0] = d_qm; ga.merged[1] = d_km; ga.merged[2] = d_vm; ga.rank_q = d_rq;
     ga.blocks = d_blocks; ga.n_blocks = pl.n_blocks; ga.n_tokens = pl.n_tokens; ga.heads = cfg->heads;
-    ga.n_special_total = n_special_total; ga.m_q = pl.m_q; ga.m_k = pl.m_k; ga.status = d_status;
+    ga.n_special_total = n_special_total; ga.m_q = pl.m_q; ga.m_k = pl.m_k; ga.status = d_status; ga.early = true;
     if ((e = launch_merge(ga, pl.max_block, ds.sm_count, s)) != cudaSuccess) return cuda_fail(e, "merge launch");
 
     AttentionArgs aa{};
@@ -225,7 +225,7 @@ extern "C" int httm_global_attention_static(const httm_config* cfg, httm_tensor 
     UnmergeArgs ua{};
     ua.o_m = d_om; ua.rank_q = d_rq; ua.pi_inv = d_pi_inv; ua.out = reinterpret_cast<__nv_bfloat16*>(out.ptr);
     ua.out_stride_head = out.stride_head; ua.out_stride_token = out.stride_token;
-    ua.n_tokens = pl.n_tokens; ua.heads = cfg->heads; ua.m_q = pl.m_q; ua.status = d_status;
+    ua.n_tokens = pl.n_tokens; ua.heads = cfg->heads; ua.m_q = pl.m_q; ua.status = d_status; ua.early = true;
     if ((e = launch_unmerge(ua, s)) != cudaSuccess) return cuda_fail(e, "unmerge launch");
     return HTTM_OK;
 }

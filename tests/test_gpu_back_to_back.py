@@ -43,3 +43,42 @@ def test_alternating_inputs_without_waits(name):
         assert ctx.query(hb.Q_DEVICE_STATUS) == 0
         for i, out in enumerate(outs):
             assert torch.equal(out, alone[i & 1]), i
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", ["blocks_32", "blocks_32_filtered", "blocks_64", "blocks_480_filtered"])
+def test_inputs_written_right_before_the_call(name):
+    """Merge, deviation and unmerge kernels read data of kernels further back while their predecessor still runs: the projection that
+    writes Q, K and V in front of a call (it lets its successor start early, too) must be complete all the same."""
+    geometry, fraction = CASES[name]
+    wl = synth.WORKLOADS["tiny"].replace(frames=7, grid_h=13, grid_w=18, **geometry)
+    n, dim = wl.n_tokens, wl.heads * 64
+    gen = torch.Generator(device="cuda:0").manual_seed(3)
+    xs = [torch.randn(n, dim, device="cuda:0", generator=gen).bfloat16() for _ in range(2)]
+    w = (torch.randn(3 * dim, dim, device="cuda:0", generator=gen) / dim ** 0.5).bfloat16()
+    qkv = torch.empty(n, 3 * dim, dtype=torch.bfloat16, device="cuda:0")
+    views = [qkv[:, i * dim:(i + 1) * dim].view(n, wl.heads, 64).transpose(0, 1) for i in range(3)]
+    with hb.Httm(hb.HttmConfig.of(wl)) as ctx:
+        ctx.set_outlier_fraction(fraction)
+        alone, merged = [], []
+        for x in xs:
+            ctx.linear(x, w, qkv)
+            torch.cuda.synchronize()
+            alone.append(ctx.global_attention(*views))
+            torch.cuda.synchronize()
+            merged.append(ctx.export(hb.X_K_MERGED))
+        outs = [ctx.new_output() for _ in range(12)]
+        for i, out in enumerate(outs):
+            ctx.linear(xs[i & 1], w, qkv)
+            ctx.global_attention(*views, out)
+        torch.cuda.synchronize()
+        assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+        for i, out in enumerate(outs):
+            assert torch.equal(out, alone[i & 1]), i
+        if name == "blocks_32":   # a stage on its own waits for whatever is in front of it (maps: those of the last call)
+            for _ in range(4):
+                ctx.linear(xs[0], w, qkv)
+                ctx.linear(xs[1], w, qkv)
+                ctx.launch_stage(hb.STAGE_MERGE_DIRECT, *views)
+                torch.cuda.synchronize()
+                assert (ctx.export(hb.X_K_MERGED) == merged[1]).all()
