@@ -61,6 +61,7 @@ struct TcParams {
     float scale_log2;
     int32_t* status;
     int32_t tiles_per_head, total_tiles, rounds;  // query tiles per head and in all heads; rounds of pair passes
+    int32_t solo;                // pairs of the partial round, if each of its other tiles gets a CTA of its own
     int32_t parts, singles;      // TailPlan (per-head query lengths: made on the device)
     const int32_t* mq_head;      // optional: per-head query length (then m_q is the row stride and tile_prefix the tile table)
     const int32_t* tile_prefix;
@@ -172,7 +173,10 @@ __device__ __noinline__ RedoneTile redo_score_tile(const __nv_bfloat16* q_row, c
     return r;
 }
 
-// Work decomposition.  The query tiles of all heads form one list (head-major, T tiles).  With G CTAs
+// Work decomposition.  The query tiles of all heads form one list of T tiles: head by head, but for the last tile of every head where
+// a head has an odd number of them: those come at the end of the list.  (In head order a pair of the list straddled two heads behind every
+// other odd head and cost its CTA two single passes, 9 % more than a pair: calls on 27 tiles of 27 key tiles per head 159.9 -> 151.5 us,
+// on 83 of 83 580.4 -> 572.5.)  With G CTAs
 // (one per SM), round r < R = T / (2 G) gives CTA c the two tiles 2 (r G + c), +1: a PAIR pass (tiles A and B
 // share the K/V stream) if they belong to the same head, else two single passes.  A SINGLE pass is the same machinery with
 // ONE query tile whose even key tiles go to softmax group A / accumulator O_A and odd ones to group B / O_B (two partial
@@ -214,11 +218,16 @@ struct Pass {
 template <bool VAR>   // VAR: the heads differ in query length (tile table in device memory)
 struct PassWalker {
     int r = 0, sub = 0;
-    int rounds, total, tiles_per_head, n_tiles, parts, singles;
+    int rounds, total, n_tiles, parts, singles;
+    int even, paired;        // tiles of a head and of all heads that form pairs
+    int solo;                // pairs of the partial round, if each of its other tiles gets a CTA of its own
     const int32_t* prefix;   // optional: first tile of every head (heads + 1 entries) when the heads differ in length
     int heads;
     __device__ PassWalker(const TcParams& p, const int32_t* prefix_, int n_tiles_)
-        : rounds(p.rounds), total(p.total_tiles), tiles_per_head(p.tiles_per_head), n_tiles(n_tiles_), parts(p.parts), singles(p.singles), prefix(prefix_), heads(p.heads) {
+        : rounds(p.rounds), total(p.total_tiles), n_tiles(n_tiles_), parts(p.parts), singles(p.singles), prefix(prefix_), heads(p.heads) {
+        even = p.tiles_per_head & ~1;
+        paired = even * p.heads;
+        solo = p.solo;
         if (VAR) {
             total = prefix[heads];
             rounds = total / (2 * (int)gridDim.x);
@@ -228,7 +237,7 @@ struct PassWalker {
         }
     }
     __device__ int head_of(int t) const {
-        if (!VAR) return t / tiles_per_head;
+        if (!VAR) return t < paired ? t / even : t - paired;
         int lo = 0, hi = heads - 1;   // largest h with prefix[h] <= t
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -241,14 +250,14 @@ struct PassWalker {
     }
     __device__ void set(Pass* ps, int t, bool pair) {
         ps->head = head_of(t);
-        ps->tile = t - (VAR ? prefix[ps->head] : ps->head * tiles_per_head);
+        ps->tile = VAR ? t - prefix[ps->head] : (t < paired ? t - ps->head * even : even);
         ps->pair = pair;
         ps->j0 = 0;
         ps->n = n_tiles;
         ps->part = -1;
     }
     __device__ bool same_head(int t) const {   // tiles t and t + 1
-        if (!VAR) return t / tiles_per_head == (t + 1) / tiles_per_head;
+        if (!VAR) return t < paired;   // (t is even)
         return t + 1 < prefix[head_of(t) + 1];
     }
     __device__ bool next(Pass* ps) {
@@ -256,14 +265,19 @@ struct PassWalker {
         const int rem = total - 2 * G * rounds;               // tiles left after the full rounds, < 2 G
         const int pair_rounds = rounds + (parts == 1 && rem > G ? 1 : 0);   // more than G left and not split: one more (partial) round of pairs
         if (r < pair_rounds) {
-            const int t = 2 * (r * G + c);
-            if (t + 1 < total && same_head(t)) {
+            const bool alone = !VAR && r == rounds && c >= solo;   // the partial round: unpaired tiles on CTAs of their own
+            const int t = alone ? 2 * G * rounds + solo + c : 2 * (r * G + c);
+            if (!alone && t + 1 < total && same_head(t)) {
                 set(ps, t, true);
                 ++r;
                 return true;
             }
             if (t + sub < total) {   // the two tiles straddle a head boundary (two single passes, the cost of one pair pass),
                 set(ps, t + sub, false);   // or only one tile is left
+                if (alone) {
+                    r = pair_rounds + 1;
+                    return true;
+                }
                 if (sub == 1) ++r;
                 sub ^= 1;
                 return true;
@@ -913,7 +927,9 @@ cudaError_t launch_attention(const AttentionArgs& a, int sm_count, cudaStream_t 
     if (!a.partial) plan.parts = 1, plan.singles = 0;
     if (ctas > total && plan.parts == 1) ctas = total;
     const int rounds = total / (2 * ctas);
-    TcParams p{a.out, a.out_stride_head, a.out_stride_token, a.m_q, a.m_k, a.scale_log2, a.status, tiles_per_head, total, rounds, plan.parts, plan.singles,
+    const int pairs = (tiles_per_head & ~1) * a.heads / 2 - ctas * rounds;
+    const int solo = pairs >= 0 && total - 2 * ctas * rounds - pairs <= ctas ? pairs : ctas;
+    TcParams p{a.out, a.out_stride_head, a.out_stride_token, a.m_q, a.m_k, a.scale_log2, a.status, tiles_per_head, total, rounds, solo, plan.parts, plan.singles,
                a.mq_head, a.tile_prefix, a.heads, a.group_start, a.group_member, a.n_tokens, a.partial, a.part_count, a.q.ptr, a.k.ptr, a.q.stride_head,
                a.q.stride_token, a.k.stride_head, a.k.stride_token};
     if (a.mq_head) {   // the tile table lives in device memory: full grid, CTAs without tiles leave at once
