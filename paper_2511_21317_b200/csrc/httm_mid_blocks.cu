@@ -368,13 +368,6 @@ match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 // skipping steps without a member of the tile's rows.  K's groups serve V.  Tensor i of the CTA's sequence Q K V Q K V .. lies
 // in stage i & 1.  The next unit's groups are made between the tensors of this one (who is kept beside K, merged rows and
 // counts beside V), so that the barrier behind each tensor is the only one.
-// The rows of W come from the merged rows of the tokens kept as bf16 numbers (whole numbers up to 256 are exact): comparing two
-// of them at a time with the fragment's row IS the fragment, 1.0 where equal (4 instructions instead of 16).
-__device__ __forceinline__ uint32_t equal_rows(uint32_t rows, uint32_t row) {   // two bf16 each: 1.0 where equal, else 0
-    const __nv_bfloat162 e = __heq2(*reinterpret_cast<const __nv_bfloat162*>(&rows), *reinterpret_cast<const __nv_bfloat162*>(&row));
-    return *reinterpret_cast<const uint32_t*>(&e);
-}
-
 template <int W, int P, bool DIRECT>
 __global__ void __launch_bounds__(32 * W, team_ctas(W, P)) merge_team_kernel(const __grid_constant__ MergeMaps maps, const __grid_constant__ MergeArgs a) {
     constexpr int NMAX = team_tokens(W, P), T = 32 * W;
@@ -497,7 +490,7 @@ __global__ void __launch_bounds__(32 * W, team_ctas(W, P)) merge_team_kernel(con
     };
     // second half (a barrier later): merged row of every token = rank of its representative among the kept tokens
     auto rank_kept = [&](const Meta& m, const Targets& x, int par, int* n_kept) {
-        const int at = (own & ~15) + 4 * ((own & 7) >> 1) + 2 * ((own >> 3) & 1) + (own & 1);   // fragment order: 2 q, 2 q + 1, 2 q + 8, 2 q + 9
+        const int at = fragment_order(own);
 #pragma unroll
         for (int map = 0; map < 2; ++map) {
             int row[P], total = 0;
@@ -585,7 +578,7 @@ __global__ void __launch_bounds__(32 * W, team_ctas(W, P)) merge_team_kernel(con
 #pragma unroll 1
                 for (int mt = W == 8 ? warp >> 2 : 0; mt < n_mt; mt += W == 8 ? 2 : 1) {
                     const int r0 = 16 * mt + g, r1 = r0 + 8;   // this lane's two accumulator rows
-                    const uint32_t b0 = pack2_bf16((float)r0, (float)r0), b1 = pack2_bf16((float)r1, (float)r1);
+                    const uint32_t b0 = row_pair(r0), b1 = row_pair(r1);
                     float c[NP][2][4];
 #pragma unroll
                     for (int i = 0; i < NP; ++i)
@@ -594,7 +587,8 @@ __global__ void __launch_bounds__(32 * W, team_ctas(W, P)) merge_team_kernel(con
 #pragma unroll 2
                     for (int ks = 0; ks < n_ks; ++ks) {
                         const uint2 rw = *reinterpret_cast<const uint2*>(row_of + 16 * ks + 4 * tq);
-                        const uint32_t af[4] = {equal_rows(rw.x, b0), equal_rows(rw.x, b1), equal_rows(rw.y, b0), equal_rows(rw.y, b1)};
+                        uint32_t af[4];
+                        w_fragment(af, rw, b0, b1);
                         if (!__any_sync(0xffffffffu, (af[0] | af[1] | af[2] | af[3]) != 0u)) continue;   // no token of this step belongs to this tile
                         const int j = 16 * ks + (lane & 15);
 #pragma unroll

@@ -9,7 +9,7 @@
 //     to block and recomputed when the shape changes (clipped blocks at the edges of the grid);
 //   - K's groups serve V, and the maps are read once per unit;
 //   - results leave through the stage as whole rows instead of 4 bytes per lane.
-// Measured at 32 976 tokens x 16 heads, 32-token blocks: match 53 -> 39.6 us, merge 69.6 -> 66.4 us (both
+// Measured at 32 976 tokens x 16 heads, 32-token blocks: match 53 -> 39.6 us, merge 69.6 -> 62.4 us (both
 // with the interval between two events).
 #include "httm_blocks.cuh"
 #include "httm_launch.cuh"
@@ -262,7 +262,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 // with the 0/1 assignment matrix W (exact in bf16, built in registers from the map), fp32 accumulation, times the reciprocal
 // of the group size, one rounding to bf16.  Kept tokens are compacted in reordered order.  The rows go through the stage they came
 // from (its fragments are in registers by then) and leave 16 bytes per lane, whole rows; then the stage is refilled.
-constexpr int kMergeAux = 32 * 4 + 32 * 4 + 32;   // reciprocal group sizes, group sizes / first members, 3 mbarriers
+constexpr int kMergeAux = 32 * 4 + 32 * 4 + 32 + 64;   // reciprocal group sizes, group sizes, 3 mbarriers, merged rows of the tokens
 constexpr int kMergeSmem = kWarps * (3 * (int)kStage + kMergeAux) + 1024 /*alignment slack*/;
 
 __device__ __forceinline__ void stmatrix_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
@@ -277,8 +277,9 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
     unsigned char* stage = smem + (size_t)warp * 3 * kStage;
     unsigned char* aux = smem + (size_t)kWarps * 3 * kStage + (size_t)warp * kMergeAux;
     float* rcnt = reinterpret_cast<float*>(aux);             // [32] 1 / group size of kept row
-    int* gsz = reinterpret_cast<int*>(aux + 32 * 4);         // [32] size, then first member, of kept row
+    int* gsz = reinterpret_cast<int*>(aux + 32 * 4);         // [32] size of kept row
     const uint32_t stage0 = smem_u32(stage), bar0 = smem_u32(aux + 2 * 32 * 4);
+    __nv_bfloat16* rows_of = reinterpret_cast<__nv_bfloat16*>(aux + 2 * 32 * 4 + 32);   // [32] merged rows of the tokens, in fragment order
     if (lane == 0) {
 #pragma unroll
         for (int t = 0; t < 3; ++t) mbar_init(bar0 + 8 * t, 1);
@@ -396,7 +397,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
         uint32_t af0[2][4];   // W fragments of the first 16 merged rows (K's serve V)
         const int n_ks = (DIRECT ? box.rows : n) > 16 ? 2 : 1;   // 16-row steps of the stage that may hold tokens
         int row_of = -1, n_kept = 0;
-        int rw[2][4];
+        uint2 rw[2];
 #pragma unroll 1
         for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 2); ++t) {
             const int r = m.r(t), moff = t == 0 ? m.moff_q : m.moff_k, m_len = t == 0 ? a.m_q : a.m_k;
@@ -421,6 +422,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
                 row_of = rep >= 0 ? __popc(kept & ((1u << rep) - 1u)) : -1;
                 gsz[lane] = 0;
                 __syncwarp();
+                rows_of[fragment_order(lane)] = __float2bfloat16_rn((float)row_of);
                 const int slot = row_of >= 0 ? atomicAdd(&gsz[row_of], 1) : 0;   // (the order of a row's members does not matter)
                 __syncwarp();
                 const int sz = gsz[lane];
@@ -447,14 +449,10 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
                         }
                     }
                 }
-                // W fragments need the rows of tokens 16 ks + {2 tq, 2 tq + 1, 2 tq + 8, 2 tq + 9}
 #pragma unroll
                 for (int ks = 0; ks < 2; ++ks) {
-                    rw[ks][0] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq);
-                    rw[ks][1] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 1);
-                    rw[ks][2] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 8);
-                    rw[ks][3] = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 9);
-                    w_fragment(af0[ks], rw[ks], g);
+                    rw[ks] = *reinterpret_cast<const uint2*>(rows_of + 16 * ks + 4 * tq);
+                    w_fragment(af0[ks], rw[ks], row_pair(g), row_pair(g + 8));
                 }
             }
             if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8 * t, it & 1, a.status, kDevTimeoutMatchLoad))) {
@@ -487,8 +485,8 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
                 for (int mt = 0; mt < n_mt; ++mt) {
                     const int r0 = 16 * mt + g, r1 = r0 + 8;   // this lane's two accumulator rows
                     if (n_mt == 2) {   // (with one tile the fragments stay as they are)
-                        w_fragment(af0[0], rw[0], r0);
-                        w_fragment(af0[1], rw[1], r0);
+                        w_fragment(af0[0], rw[0], row_pair(r0), row_pair(r1));
+                        w_fragment(af0[1], rw[1], row_pair(r0), row_pair(r1));
                     }
                     float c[8][4];
 #pragma unroll
