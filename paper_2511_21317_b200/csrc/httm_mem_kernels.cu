@@ -174,10 +174,12 @@ cudaError_t launch_merge(const MergeArgs& a, int max_block_tokens, int sm_count,
 //                      merged length, and the head's first 128-row query tile (for the attention kernel)
 // ------------------------------------------------------------------------------------
 __device__ void finish_level(const OutlierArgs& a, int level, int* hist);   // (threshold selection, below)
-constexpr int kDevWarps = 6;     // 6 x 16.2 KB of shared memory: two CTAs per SM
-constexpr int kDevStages = 3;    // block loads in flight per warp (the kernel is bound by bytes in flight)
-constexpr int kCentStride = 65;  // floats per mean: odd, so that reads of different means spread over the banks
-constexpr int kDevAux = 16 * kCentStride * 4 + 16 * 4 + 32;   // means of the groups of two or more (at most 16 in 32 tokens), reciprocal sizes, mbarriers
+// Latency of the warps' instruction streams and bytes in flight bound the deviation kernel: 16 warps per SM with two stages each rather than
+// 12 with three, and the means read back 16 bytes at a time (32 976 tokens: all five kernels of the filter 72 -> 65.5 us, the call 685 -> 679 us).
+constexpr int kDevWarps = 8;     // 8 x 12.6 KB of shared memory: two CTAs per SM
+constexpr int kDevStages = 2;    // block loads in flight per warp
+constexpr int kCentStride = 68;  // floats per mean: 16-byte reads of eight different means fall on distinct banks
+constexpr int kDevAux = 16 * kCentStride * 4 + 16 * 4 + 32 + 64;   // means of the groups of two or more (at most 16 in 32 tokens), reciprocal sizes, mbarriers, rows
 constexpr int kDevSmem = kDevWarps * (kDevStages * 32 * kRowBytes + kDevAux) + 2048 * 4 /*histogram*/ + 1024 /*alignment slack*/;
 
 __global__ void __launch_bounds__(kDevWarps * 32, 2)
@@ -189,12 +191,13 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
     const int g = lane >> 2, tq = lane & 3;   // MMA accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
     unsigned char* stage = smem + (size_t)warp * kDevStages * STAGE_BYTES;
     unsigned char* aux = smem + (size_t)kDevWarps * kDevStages * STAGE_BYTES + (size_t)warp * kDevAux;
-    float* cent = reinterpret_cast<float*>(aux);                   // [16][65] group means
+    float* cent = reinterpret_cast<float*>(aux);                   // [16][68] group means
     float* rcnt = cent + 16 * kCentStride;                         // [16] 1 / group size
     int* hist = reinterpret_cast<int*>(smem + (size_t)kDevWarps * (kDevStages * STAGE_BYTES + kDevAux));   // [2048] bits 31-21 of this CTA's deviations
     for (int i = threadIdx.x; i < 2048; i += kDevWarps * 32) hist[i] = 0;
     __syncthreads();
     const uint32_t mbar0 = smem_u32(aux + 16 * kCentStride * 4 + 16 * 4), stage0 = smem_u32(stage);
+    __nv_bfloat16* rows_of = reinterpret_cast<__nv_bfloat16*>(aux + 16 * kCentStride * 4 + 16 * 4 + 32);   // [32] mean of each token, in fragment order
     if (lane == 0) {
         for (int st = 0; st < kDevStages; ++st) mbar_init(mbar0 + 8 * st, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -267,6 +270,7 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
             const unsigned multi = __ballot_sync(0xffffffffu, rep == lane && group_size >= 2);
             const int row_of = group_size >= 2 ? __popc(multi & ((1u << rep) - 1u)) : -1;
             if (rep == lane && group_size >= 2) rcnt[row_of] = 1.0f / (float)group_size;
+            rows_of[fragment_order(lane)] = __float2bfloat16_rn((float)row_of);
             // group sums = W x on the tensor cores, as in merge_small_kernel: W [16 means][32 tokens] of zeros and ones
             uint32_t bf[2][4][4];
             const int n_ks = box_rows > 16 ? 2 : 1;
@@ -279,37 +283,29 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
                     for (int np = 0; np < 4; ++np) ldmatrix_x4_trans(bf[ks][np], rowaddr + (((2 * np + (lane >> 4)) ^ (row & 7)) << 4));
                 }
             }
+            __syncwarp();   // rows and reciprocal group sizes visible
             float c[8][4];
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt) c[nt][0] = c[nt][1] = c[nt][2] = c[nt][3] = 0.f;
             const int r0 = g, r1 = g + 8;
 #pragma unroll
             for (int ks = 0; ks < 2; ++ks) {
                 if (ks < n_ks) {
-                    const int w0 = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq), w1 = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 1);
-                    const int w2 = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 8), w3 = __shfl_sync(0xffffffffu, row_of, 16 * ks + 2 * tq + 9);
                     uint32_t af[4];
-                    af[0] = (w0 == r0 ? 0x3f80u : 0u) | (w1 == r0 ? 0x3f800000u : 0u);
-                    af[1] = (w0 == r1 ? 0x3f80u : 0u) | (w1 == r1 ? 0x3f800000u : 0u);
-                    af[2] = (w2 == r0 ? 0x3f80u : 0u) | (w3 == r0 ? 0x3f800000u : 0u);
-                    af[3] = (w2 == r1 ? 0x3f80u : 0u) | (w3 == r1 ? 0x3f800000u : 0u);
+                    w_fragment(af, *reinterpret_cast<const uint2*>(rows_of + 16 * ks + 4 * tq), row_pair(r0), row_pair(r1));
 #pragma unroll
-                    for (int nt = 0; nt < 8; ++nt) mma_bf16_16816(c[nt], af, bf[ks][nt >> 1][2 * (nt & 1)], bf[ks][nt >> 1][2 * (nt & 1) + 1]);
+                    for (int nt = 0; nt < 8; ++nt) {
+                        if (ks == 0)
+                            mma_first(c[nt], af, bf[ks][nt >> 1][2 * (nt & 1)], bf[ks][nt >> 1][2 * (nt & 1) + 1]);
+                        else
+                            mma_bf16_16816(c[nt], af, bf[ks][nt >> 1][2 * (nt & 1)], bf[ks][nt >> 1][2 * (nt & 1) + 1]);
+                    }
                 }
             }
-            __syncwarp();   // reciprocal group sizes visible
             const int n_cent = __popc(multi);
             const float i0 = r0 < n_cent ? rcnt[r0] : 0.f, i1 = r1 < n_cent ? rcnt[r1] : 0.f;
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {   // the means stay in fp32 (no rounding to bf16 before the distance)
-                if (r0 < n_cent) {
-                    cent[r0 * kCentStride + nt * 8 + 2 * tq] = c[nt][0] * i0;
-                    cent[r0 * kCentStride + nt * 8 + 2 * tq + 1] = c[nt][1] * i0;
-                }
-                if (r1 < n_cent) {
-                    cent[r1 * kCentStride + nt * 8 + 2 * tq] = c[nt][2] * i1;
-                    cent[r1 * kCentStride + nt * 8 + 2 * tq + 1] = c[nt][3] * i1;
-                }
+                if (r0 < n_cent) *reinterpret_cast<float2*>(cent + r0 * kCentStride + nt * 8 + 2 * tq) = make_float2(c[nt][0] * i0, c[nt][1] * i0);
+                if (r1 < n_cent) *reinterpret_cast<float2*>(cent + r1 * kCentStride + nt * 8 + 2 * tq) = make_float2(c[nt][2] * i1, c[nt][3] * i1);
             }
             __syncwarp();   // means visible
             float dev = 0.f;
@@ -322,9 +318,11 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
                     for (int ch = 0; ch < 8; ++ch) {
                         float x[8];
                         unpack8(*reinterpret_cast<const uint4*>(row + ((ch ^ (lane & 7)) << 4)), x);
+                        const float4 lo = *reinterpret_cast<const float4*>(cr + ch * 8), hi = *reinterpret_cast<const float4*>(cr + ch * 8 + 4);
+                        const float m[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
 #pragma unroll
                         for (int e = 0; e < 8; ++e) {
-                            const float d = x[e] - cr[ch * 8 + e];
+                            const float d = x[e] - m[e];
                             d2 = fmaf(d, d, d2);
                         }
                     }
