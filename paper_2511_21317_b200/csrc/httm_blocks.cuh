@@ -188,6 +188,9 @@ __device__ __forceinline__ Geometry unpack_geometry(const int4& v) {
     g.cols = v.z >> 16;
     return g;
 }
+// frames, rows and columns of a block in bits of their own (each is at most 256).  What the match kernels keep from block to block holds for
+// one shape, so the key has to tell all shapes apart: blocks clipped in time and in width, (1, 4, 4) and (4, 4, 1), have equally many tokens.
+__device__ __forceinline__ int shape_key(const int4& v) { return (v.z & 0x3ff) | (v.z >> 16) << 10 | (v.y >> 16) << 20; }
 // d (16x8 fp32) = a (16x16 bf16, row) * b (16x8 bf16, col): the first step of a sum
 __device__ __forceinline__ void mma_first(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"

@@ -176,7 +176,7 @@ match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
             const int n_rows = DIRECT ? box.rows : n;   // rows of the stage that may hold tokens
             {
-                const int sa = n | (nd << 10) | (bi.n_rule << 20), sb = DIRECT ? geom.z + (geom.y & 0xffff0000) : 0;   // frames, rows, cols
+                const int sa = n | (nd << 10) | (bi.n_rule << 20), sb = DIRECT ? shape_key(geom) : 0;
                 if (sa != shape_a || sb != shape_b) {   // (uniform)
                     team_sync<W>();   // the tables may still be read for the previous tensor
                     shape_a = sa;

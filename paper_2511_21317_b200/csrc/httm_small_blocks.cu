@@ -123,7 +123,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
             const int n_rows = DIRECT ? box.rows : n;   // rows of the stage that may hold tokens
             {
-                const int sa = n | (nd << 8) | (bi.n_rule << 16), sb = DIRECT ? geom.z + (geom.y & 0xffff0000) : 0;   // frames, rows, cols
+                const int sa = n | (nd << 8) | (bi.n_rule << 16), sb = DIRECT ? shape_key(geom) : 0;
                 if (sa != shape_a || sb != shape_b) {
                     const Geometry bg = unpack_geometry(geom);
                     shape_a = sa;

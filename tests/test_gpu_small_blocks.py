@@ -21,8 +21,8 @@ def run(cfg, qkv):
 
 
 @pytest.mark.parametrize("blk,ratio,specials,frames", [((2, 4, 4), 0.7, 4, 12), ((1, 3, 5), 0.5, 0, 12), ((3, 3, 3), 0.9, 2, 13), ((2, 4, 4), 0.6, 40, 12),
-                                                       ((2, 2, 8), 0.0, 1, 12)],
-                         ids=["32_tokens", "15_tokens", "27_tokens", "over_reordered_copies", "keys_only"])
+                                                       ((2, 2, 8), 0.0, 1, 12), ((3, 3, 3), 0.7, 2, 13)],
+                         ids=["32_tokens", "15_tokens", "27_tokens", "over_reordered_copies", "keys_only", "equal_ratios"])
 def test_whole_units_and_split_units_agree(blk, ratio, specials, frames):
     """24 heads have more units than the chip has warps for, one head has fewer."""
     wl = synth.Workload("units", frames, 22, 25, *blk, ratio, 0.7, n_camera=1, n_register=specials, heads=24, seed=2)
