@@ -263,7 +263,7 @@ match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                                 const float s0 = c[2 * hrow] * w0, s1 = c[2 * hrow + 1] * w1, m = fmaxf(s0, s1);
                                 if (m > top[mt][hrow]) {
                                     top[mt][hrow] = m;
-                                    arg[mt][hrow] = da + (s1 > s0 ? 1 : 0);
+                                    arg[mt][hrow] = da + (s0 != m ? 1 : 0);   // (also where s0 is not a number)
                                 }
                             }
                         }
