@@ -627,6 +627,34 @@ __device__ int build_groups(const int32_t* A, int block_start, int n, int limit,
     return n_kept;
 }
 
+// Sum of the rows keys[i0 .. i1) (positions in the low 12 bits), eight channels from x on.  Four members are in flight: the gather is
+// bound by load latency.  They are added in pairs of pairs, to one of two sums in turn: n / 8 + 4 roundings for n members.  (Added
+// one after the other they took n: with one member 2^17 times the others, 2 048 of them left the mean half a step of bf16 off.)
+__device__ __forceinline__ void sum_members(const __nv_bfloat16* x, int64_t stride, const uint32_t* keys, int i0, int i1, float (&sum)[8]) {
+    float other[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) sum[e] = other[e] = 0.f;
+    auto add_four = [&](int i, float (&to)[8]) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            v[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (i + u < i1) v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)(keys[i + u] & 4095u) * stride));
+        }
+        float f[4][8];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) unpack8f(v[u], f[u]);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) to[e] += (f[0][e] + f[1][e]) + (f[2][e] + f[3][e]);
+    };
+    for (int i = i0; i < i1; i += 8) {
+        add_four(i, sum);
+        if (i + 4 < i1) add_four(i + 4, other);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) sum[e] += other[e];
+}
+
 template <int T, int E>
 __global__ void __launch_bounds__(T, kSortedThreads / T) big_merge_kernel(const MergeArgs a, int sp_chunks) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
@@ -664,32 +692,15 @@ __global__ void __launch_bounds__(T, kSortedThreads / T) big_merge_kernel(const 
     const int32_t* A = a.assign[m] + base;
 
     const int n_kept = build_groups<T, E>(A, bi.start, n, limit, keys, row_of, seg, warp_sum, nullptr, a.status, m == 0 ? a.rank_q + base : nullptr, moff);
-    // eight lanes per merged row (a lane owns one 16-byte chunk of the row), four rows per warp at a time, four
-    // members of a row in flight: the gather is bound by load latency, so it needs many loads in the air.  The members are
-    // added in position order: the result does not depend on scheduling.
+    // eight lanes per merged row (a lane owns one 16-byte chunk of the row), four rows per warp at a time.  The members are
+    // taken in position order: the result does not depend on scheduling.
     for (int t = (m == 0 ? 0 : 1); t <= (m == 0 ? 0 : 2); ++t) {
         const __nv_bfloat16* x = a.xr[t] + base * kHeadDim;
         __nv_bfloat16* out = a.merged[t] + ((int64_t)h * m_len + moff) * kHeadDim;
         for (int row = warp * 4 + sub; row < n_kept; row += (T / 32) * 4) {
             const int i0 = seg[row], i1 = seg[row + 1];
             float acc[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-            for (int i = i0; i < i1; i += 4) {
-                uint4 v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    v[u] = make_uint4(0u, 0u, 0u, 0u);
-                    if (i + u < i1) v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)(keys[i + u] & 4095u) * kHeadDim) + ch);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    float f[8];
-                    unpack8f(v[u], f);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[e] += f[e];
-                }
-            }
+            sum_members(x + 8 * ch, kHeadDim, keys, i0, i1, acc);
             if (i1 > i0) {
                 const float inv = 1.0f / (float)(i1 - i0);
                 float r8[8];
@@ -746,23 +757,7 @@ __global__ void __launch_bounds__(T, kSortedThreads / T) big_deviation_kernel(co
         for (int e = 0; e < 8; ++e) mean[e] = 0.f;
         if (cnt >= 2) {
             float acc[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-            for (int i = i0; i < i1; i += 4) {
-                uint4 v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    v[u] = make_uint4(0u, 0u, 0u, 0u);
-                    if (i + u < i1) v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)(keys[i + u] & 4095u) * st) + ch);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    float f[8];
-                    unpack8f(v[u], f);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[e] += f[e];
-                }
-            }
+            sum_members(x + 8 * ch, st, keys, i0, i1, acc);
             const float inv = 1.0f / (float)cnt;
 #pragma unroll
             for (int e = 0; e < 8; ++e) mean[e] = acc[e] * inv;   // kept in fp32

@@ -106,3 +106,41 @@ def test_block_sizes_at_the_cta_size_limits(n):
     if n in (513, 2049):
         from tests.test_gpu_outlier import run_filtered
         run_filtered(wl, 0.1, peaky=True, launches=12)
+
+
+def test_sums_of_many_members_with_one_far_larger_member():
+    """2 048 tokens in one block, multiples of one vector (every cosine a tie: nearly all of them merge into the first dst token), one of
+    them 2^17 times the others.  In fp32 every small member added to a running sum of that size is rounded in the same direction, so a
+    sum in position order is off by up to half a unit in the last place per member.  The bound is that of four running sums of every fourth
+    member each, (n / 4 + 2) roundings of at most 2^-24 of the sum of magnitudes."""
+    n, heads = 2048, 4
+    wl = synth.Workload("large_member", 1, 1, n, 1, 1, n, 0.99, 0.99, n_camera=0, n_register=1, heads=heads, seed=0)
+    gen = np.random.default_rng(5)
+    u = (1.0 + gen.integers(0, 128, (heads, 1, 64)) / 128.0) * gen.choice([-1.0, 1.0], (heads, 1, 64))
+    x = np.repeat(u, n + 1, axis=1)
+    x[:, 1] *= 2.0 ** 17
+    t = torch.from_numpy(x).bfloat16().to(DEV)
+    assert (t.double().cpu().numpy() == x).all()
+    with hb.Httm(hb.HttmConfig.of(wl)) as ctx:
+        ctx.set_outlier_fraction(1e-4)
+        ctx.global_attention(t, t, t)
+        torch.cuda.synchronize()
+        assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+        aq, ak = ctx.export(hb.X_ASSIGN_Q_INITIAL), ctx.export(hb.X_ASSIGN_K)
+        eps = ctx.export(hb.X_DEVIATION).astype(np.float64)
+        k_m, v_m = (parity.bits_to_f64(ctx.export(w)) for w in (hb.X_K_MERGED, hb.X_V_MERGED))
+    roundings = (n / 4 + 2) * 2.0 ** -24
+    for h in range(heads):
+        members = np.flatnonzero(aq[h] == aq[h][1])
+        assert len(members) > 0.98 * n and members[0] == 1
+        mean, size = x[h][members].mean(0), np.abs(x[h][members]).mean(0)
+        want = np.linalg.norm(x[h][members] - mean, axis=1)
+        bound = np.linalg.norm(roundings * size) + (64 + 4) * 2.0 ** -24 * want      # the mean, then differences, 64 squares and the root
+        assert (np.abs(eps[h][members] - want) <= bound).all(), (h, np.abs(eps[h][members] - want).max(), bound.max())
+        kept = np.flatnonzero(ak[h] == np.arange(n + 1))
+        members = np.flatnonzero(ak[h] == ak[h][1])
+        mean, size = x[h][members].mean(0), np.abs(x[h][members]).mean(0)
+        row = np.flatnonzero(kept == ak[h][1])[0]
+        for got in (k_m[h][row], v_m[h][row]):   # within half a bf16 step of the mean, up to the same bound
+            step = 2.0 ** (np.floor(np.log2(np.abs(mean))) - 7)
+            assert (np.abs(got - mean) <= step / 2 + roundings * size).all(), (h, (np.abs(got - mean) / step).max())
