@@ -255,9 +255,10 @@ cudaError_t launch_linear(const LinearArgs& a, int sm_count, cudaStream_t stream
     CUtensorMap mx, mw, my;
     // a matrix [rows][in] as {64 channels, rows, in / 64 blocks of 64 channels}: the block index is the third coordinate
     const int k_blocks = a.in_features / BK;
+    const int64_t ldy = a.n_rows == 1 ? a.out_features : a.ldy;   // (not used then: it need not be a stride that a tensor map can hold)
     if (!encode_rows_tensor_map(&mx, a.x, a.n_rows, k_blocks, a.ldx, BK, BM) ||
         !encode_rows_tensor_map(&mw, a.w, a.out_features, k_blocks, a.ldw, BK, BN / 2) ||
-        !encode_matrix_tensor_map(&my, a.y, a.n_rows, a.out_features, a.ldy, OUT_ROWS, OUT_COLS))
+        !encode_matrix_tensor_map(&my, a.y, a.n_rows, a.out_features, ldy, OUT_ROWS, OUT_COLS))
         return cudaErrorInvalidValue;
     const int n_tiles = (a.out_features + BN - 1) / BN;
     const int64_t total = ((a.n_rows + 2 * BM - 1) / (2 * BM)) * n_tiles;

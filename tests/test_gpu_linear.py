@@ -82,3 +82,15 @@ def test_stack_with_own_projections_matches_the_library_projections():
     finally:
         a.close()
         b.close()
+
+
+def test_one_row_with_any_leading_dimension(ctx):
+    """The leading dimension of a matrix of one row is not used: any multiple of 8 is taken."""
+    gen = torch.Generator(device="cuda:0").manual_seed(1)
+    x, w = (torch.randn(n, 128, device="cuda:0", generator=gen).bfloat16() for n in (1, 72))
+    want = ctx.linear(x, w)
+    for ld in (1 << 39, 1 << 45):
+        y = torch.zeros(72, dtype=torch.bfloat16, device="cuda:0").as_strided((1, 72), (ld, 1))
+        ctx.linear(x, w, y)
+        torch.cuda.synchronize()
+        assert torch.equal(y, want), ld
