@@ -51,7 +51,6 @@ struct Barriers {
     uint64_t x_full, x_done;         // single pass: tile B's (max, sum) published / tile A done reading O_B
     uint32_t tmem_base;
     int abort_flag;
-    int last_part;   // split tiles: this CTA's part was the tile's last to arrive
 };
 
 struct TcParams {
@@ -70,7 +69,7 @@ struct TcParams {
     const int32_t* group_member;
     int32_t n_tokens;
     float* partial;              // optional: partial results of query tiles that are split over CTAs, see TailPlan
-    int32_t* part_count;         // their arrivals, one counter per split tile, all zero between launches
+    int32_t* part_count;         // their arrivals, four counters (32 rows each) per split tile, all zero between launches
     const __nv_bfloat16 *q, *k;  // the rows themselves, for the tile that is redone (element strides)
     int64_t q_stride_head, q_stride_token, k_stride_head, k_stride_token;
 };
@@ -188,7 +187,7 @@ __device__ __noinline__ RedoneTile redo_score_tile(const __nv_bfloat16* q_row, c
 // TailPlan: of the remaining tiles, G are dealt one per CTA as single passes if there are more than G; e < G are left.  Dealt
 // whole (one single pass on e of the CTAs) they take as long as one on every CTA.  Where e <= G / 2 each of them is split
 // into P = G / e parts of the keys, one per CTA: a part is a single pass over n / P key tiles that leaves its unnormalised
-// output, maxima and sums in a workspace, and the CTA whose part of a tile arrives last adds them up (nobody waits).  A part
+// output, maxima and sums in a workspace, and the warp whose part of its rows arrives last adds them up (nobody waits).  A part
 // costs about kPartCost key tiles besides its own, and single passes for all CTAs and then parts kPassCost more than a round
 // of pairs, hence the rule (3.03 tiles per SM of 28 key tiles: whole 127 us, split 143).  Where the tiles are not split and more than G remain they
 // go as one more (partial) round of pairs, which takes the same time as two rounds of single passes.
@@ -375,8 +374,8 @@ __device__ __forceinline__ void store_rows(const TcParams& p, int head, const ui
 }
 
 // The end of a pass over part of the keys (group A's four warps, thread = row of the tile): the combined but unnormalised
-// output of both groups, the maximum and the sum go to the workspace.  The CTA that arrives last adds the parts of the tile
-// up, in the order of their keys, and sends the rows out.
+// output of both groups, the maximum and the sum go to the workspace.  Of the warps with the same 32 rows the one that arrives
+// last adds the parts up, in the order of their keys, and sends the rows out.
 struct PartArgs {
     int head, grow, mq_rows;          // this thread's row, rows of the head
     int part, parts;                  // see TailPlan
@@ -413,17 +412,18 @@ __device__ __noinline__ bool epilogue_part(const TcParams& p, const PartArgs& a,
     }
     tc::fence_before_sync();
     tc::mbar_arrive(tc::smem_addr(&bars->x_done));
-    asm volatile("bar.sync 1, 128;" ::: "memory");   // every row of this part has been written
-    if (row == 0) {
-        int32_t* count = p.part_count + first / parts;
+    // A warp adds up the 32 rows that the same warp of the tile's other parts has written, so arrivals are counted warp by warp and the
+    // warps of a CTA need not wait for one another: one that gives up leaves nobody behind.
+    bool last = false;
+    __syncwarp();
+    if (lane == 0) {
+        int32_t* count = p.part_count + 4 * (first / parts) + (row >> 5);
         __threadfence();
-        const bool last = atomicAdd(count, 1) == parts - 1;
+        last = atomicAdd(count, 1) == parts - 1;
         if (last) *count = 0;   // (as the next launch finds it)
         __threadfence();
-        bars->last_part = last;
     }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    if (!bars->last_part) return true;   // (a CTA has one part: the flag is not written again)
+    if (!__shfl_sync(0xffffffffu, last, 0)) return true;
     const RowTargets targets = row_targets<UNMERGE>(p, a.head, a.grow, a.grow < a.mq_rows);
     const float* other = p.partial + (int64_t)first * kPartFloats;
     float top = -INFINITY, sum = 0.f, o[kHeadDim];
@@ -900,9 +900,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
 }  // namespace
 
-// at most one part per CTA, of at most half as many tiles
+// at most one part per CTA, of at most half as many tiles (four counters each)
 size_t attention_partial_floats(int sm_count) { return (size_t)sm_count * kPartFloats; }
-size_t attention_partial_counters(int sm_count) { return (size_t)sm_count; }
+size_t attention_partial_counters(int sm_count) { return 2 * (size_t)sm_count; }
 
 cudaError_t configure_attention() {
     cudaError_t e = cudaFuncSetAttribute(attention_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
