@@ -329,10 +329,13 @@ int httm_call_times(httm_ctx* ctx, float* ms, const char** names, int32_t capaci
  *     barrier expects, so that the kernel's bounded wait runs out (about two seconds): it records the time-out in the
  *     context's status word, releases its tensor memory and returns.  The next httm_query(HTTM_Q_DEVICE_STATUS) /
  *     httm_export then reports HTTM_ERR_TIMEOUT; the context stays usable (the status word keeps the first error).
+ *   httm_leave_parts_unfinished(ctx, stream): leaves the arrival counters of split query tiles non-zero, as an attention kernel
+ *     does in which one part of a tile gave up.  The next call must not notice.
  * Errors: INVALID_ARG, UNSUPPORTED (a context with fewer than 384 token-heads), CUDA.
  */
 int httm_fail_nth_allocation(int32_t n);
 int httm_expire_a_wait(httm_ctx* ctx, void* cuda_stream);
+int httm_leave_parts_unfinished(httm_ctx* ctx, void* cuda_stream);
 
 /*
  * Diagnostic: one 128-row tile through the tensor-core building blocks of the attention kernel

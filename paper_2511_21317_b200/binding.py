@@ -34,7 +34,7 @@ EXPORTED_SYMBOLS = (
     "httm_create", "httm_global_attention", "httm_dense_attention", "httm_attention_host", "httm_launch_stage",
     "httm_query", "httm_export", "httm_last_error", "httm_launch_count", "httm_destroy",
     "httm_global_attention_static", "httm_selftest_tensor_core", "httm_set_outlier_fraction", "httm_linear",
-    "httm_set_head_shard", "httm_fail_nth_allocation", "httm_expire_a_wait", "httm_set_call_timing", "httm_call_times",
+    "httm_set_head_shard", "httm_fail_nth_allocation", "httm_expire_a_wait", "httm_leave_parts_unfinished", "httm_set_call_timing", "httm_call_times",
 )
 _EXCHANGE_FN = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p)
 
@@ -75,6 +75,7 @@ def load_library() -> ctypes.CDLL:
     L.httm_set_head_shard.argtypes = [vp, ctypes.c_int32, _EXCHANGE_FN, vp]
     L.httm_fail_nth_allocation.argtypes = [ctypes.c_int32]
     L.httm_expire_a_wait.argtypes = [vp, vp]
+    L.httm_leave_parts_unfinished.argtypes = [vp, vp]
     L.httm_linear.argtypes = [vp, vp, i64, vp, i64, vp, i64, i64, ctypes.c_int32, ctypes.c_int32, vp]
     L.httm_attention_host.argtypes = [vp, vp, vp, vp, vp, ctypes.c_int, vp]
     L.httm_launch_stage.argtypes = [vp, ctypes.c_int, _Tensor, _Tensor, _Tensor, _Tensor, vp]
@@ -235,6 +236,10 @@ class Httm:
     def expire_a_wait(self, stream=None):
         """Error-path test aid: a kernel whose bounded wait runs out (see httm_expire_a_wait)."""
         self._check(self._lib.httm_expire_a_wait(self._h, self._stream(stream)))
+
+    def leave_parts_unfinished(self, stream=None):
+        """Error-path test aid: the state an attention kernel that gave up leaves behind (see httm_leave_parts_unfinished)."""
+        self._check(self._lib.httm_leave_parts_unfinished(self._h, self._stream(stream)))
 
     def set_head_shard(self, total_heads: int, exchange=None):
         """This context holds some of the heads of a layer with `total_heads` heads (see httm_set_head_shard).

@@ -182,8 +182,14 @@ TensorView view(const __nv_bfloat16* p, int64_t rows) { return TensorView{p, row
 
 float scale_log2() { return 1.4426950408889634f / std::sqrt((float)kHeadDim); }
 
-// clear: the selection state of the outlier filter is set to zero for the stages behind this one
-int stage_reorder(httm_ctx* c, const httm_tensor& q, const httm_tensor& k, const httm_tensor& v, cudaStream_t s, bool clear = false) {
+// What the first kernel of a call sets to zero for the kernels behind it
+void clear_state(httm_ctx* c, ClearRange (&clear)[2]) {
+    clear[0] = ClearRange{c->d_part_count, (int32_t)attention_partial_counters(c->sm_count)};
+    if (c->filtering()) clear[1] = ClearRange{c->d_sel, kSelWords};
+}
+
+// first: the call's first kernel, which clears the state of the stages behind it
+int stage_reorder(httm_ctx* c, const httm_tensor& q, const httm_tensor& k, const httm_tensor& v, cudaStream_t s, bool first = false) {
     ReorderArgs a{};
     a.src[0] = view(q);
     a.src[1] = view(k);
@@ -196,10 +202,7 @@ int stage_reorder(httm_ctx* c, const httm_tensor& q, const httm_tensor& k, const
     a.heads = c->cfg.heads;
     a.inv_norm[0] = c->d_inv_norm_q;   // (null unless the context has large blocks)
     a.inv_norm[1] = c->d_inv_norm_k;
-    if (clear) {
-        a.clear = c->d_sel;
-        a.n_clear = kSelWords;
-    }
+    if (first) clear_state(c, a.clear);
     c->launches++;
     return check_cuda(c, launch_reorder(a, s), "reorder launch");
 }
@@ -265,7 +268,7 @@ int stage_big_select(httm_ctx* c, cudaStream_t s) {
 }
 
 // src: the original Q, K, V (direct mode) or nullptr (blocks come from the reordered copies)
-int stage_match(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr, bool clear = false) {
+int stage_match(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr, bool first = false) {
     if (c->big()) return c->fail(HTTM_ERR_UNSUPPORTED, "blocks of more than 256 tokens are matched by the large-block stages");
     MatchArgs a{};
     if (src) {
@@ -283,10 +286,7 @@ int stage_match(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr, b
     a.n_tokens = c->n_tokens;
     a.heads = c->cfg.heads;
     a.status = c->d_status;
-    if (clear) {
-        a.clear = c->d_sel;
-        a.n_clear = kSelWords;
-    }
+    if (first) clear_state(c, a.clear);
     c->launches++;
     int rc = check_cuda(c, launch_match(a, c->max_block, c->sm_count, s), "match launch");
     if (rc || c->n_anchor == 0) return rc;
@@ -339,8 +339,9 @@ int stage_merge(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr, b
 }
 
 // final_out: null = the merged output O_m is written (unmerged by the next stage); else the epilogue writes every merged row
-// to its member tokens in the caller's output tensor (needs fused_unmerge)
-int stage_attention(httm_ctx* c, cudaStream_t s, const httm_tensor* final_out = nullptr) {
+// to its member tokens in the caller's output tensor (needs fused_unmerge).  chained: inside a call, whose first kernel has cleared the
+// arrivals of split tiles
+int stage_attention(httm_ctx* c, cudaStream_t s, const httm_tensor* final_out = nullptr, bool chained = false) {
     AttentionArgs a{};
     a.q = view(c->filtering() ? c->d_qm_var : c->d_qm, c->q_rows());
     a.k = view(c->d_km, c->m_k);
@@ -370,6 +371,10 @@ int stage_attention(httm_ctx* c, cudaStream_t s, const httm_tensor* final_out = 
     a.status = c->d_status;
     a.partial = c->d_partial;
     a.part_count = c->d_part_count;
+    if (!chained) {
+        const int rc = check_cuda(c, cudaMemsetAsync(c->d_part_count, 0, attention_partial_counters(c->sm_count) * sizeof(int32_t), s), "part counters");
+        if (rc) return rc;
+    }
     c->launches++;
     return check_cuda(c, launch_attention(a, c->sm_count, s), "attention launch");
 }
@@ -498,35 +503,35 @@ int global_impl(httm_ctx* c, const httm_tensor& q, const httm_tensor& k, const h
     };
     int rc;
     if (c->big()) {   // six kernels: reorder (+ norms), scores, select, merge, attention, unmerge
-        if ((rc = part(stage_reorder(c, q, k, v, s, c->filtering()), "reorder"))) return rc;
+        if ((rc = part(stage_reorder(c, q, k, v, s, true), "reorder"))) return rc;
         if ((rc = part(stage_big_scores(c, s), "big_scores"))) return rc;
         if ((rc = part(stage_big_select(c, s), "big_select"))) return rc;
         if (c->filtering() && (rc = part(stage_outlier(c, q, s, true), "outlier_filter"))) return rc;
         if ((rc = part(stage_merge(c, s, nullptr, true), "merge"))) return rc;
-        if ((rc = part(stage_attention(c, s), "attention"))) return rc;
+        if ((rc = part(stage_attention(c, s, nullptr, true), "attention"))) return rc;
         return part(stage_unmerge(c, out, s, true), "unmerge");
     }
     if (sorted_filter(c)) {   // outlier filtering with blocks of 33 .. 256 tokens: everything from the reordered copies
-        if ((rc = part(stage_reorder(c, q, k, v, s, c->filtering()), "reorder"))) return rc;
+        if ((rc = part(stage_reorder(c, q, k, v, s, true), "reorder"))) return rc;
         if ((rc = part(stage_match(c, s), "match"))) return rc;
         if ((rc = part(stage_outlier(c, q, s, true), "outlier_filter"))) return rc;
         if ((rc = part(stage_merge(c, s, nullptr, true), "merge"))) return rc;
-        if ((rc = part(stage_attention(c, s), "attention"))) return rc;
+        if ((rc = part(stage_attention(c, s, nullptr, true), "attention"))) return rc;
         return part(stage_unmerge(c, out, s, true), "unmerge");
     }
     if (direct_mode(c)) {   // the temporal reorder is folded into the block loads of match and merge
         const httm_tensor src[3] = {q, k, v};
-        if ((rc = part(stage_match(c, s, src, c->filtering()), "match_direct"))) return rc;
+        if ((rc = part(stage_match(c, s, src, true), "match_direct"))) return rc;
         if (c->filtering() && (rc = part(stage_outlier(c, q, s, true), "outlier_filter"))) return rc;
         if ((rc = part(stage_merge(c, s, src, true), "merge_direct"))) return rc;
     } else {
-        if ((rc = part(stage_reorder(c, q, k, v, s, c->filtering()), "reorder"))) return rc;
+        if ((rc = part(stage_reorder(c, q, k, v, s, true), "reorder"))) return rc;
         if ((rc = part(stage_match(c, s), "match"))) return rc;
         if ((rc = part(stage_merge(c, s, nullptr, true), "merge"))) return rc;
     }
     // ... and the unmerge into the attention epilogue: three kernels
-    if (fused_unmerge(c)) return part(stage_attention(c, s, &out), "attention_unmerge");
-    if ((rc = part(stage_attention(c, s), "attention"))) return rc;
+    if (fused_unmerge(c)) return part(stage_attention(c, s, &out, true), "attention_unmerge");
+    if ((rc = part(stage_attention(c, s, nullptr, true), "attention"))) return rc;
     return part(stage_unmerge(c, out, s, true), "unmerge");
 }
 
@@ -637,7 +642,6 @@ int httm_create(const httm_config* cfg, httm_ctx** out) {
 
     if ((rc = c->alloc(&c->d_partial, attention_partial_floats(c->sm_count))) || (rc = c->alloc(&c->d_part_count, attention_partial_counters(c->sm_count))))
         return done(rc);
-    if ((rc = check_cuda(c, cudaMemset(c->d_part_count, 0, attention_partial_counters(c->sm_count) * 4), "workspace setup"))) return done(rc);
     if (c->max_block <= 32) {   // member lists of the merged query rows; entry M_q of every head is the constant N
         if ((rc = c->alloc(&c->d_group_start, H * (size_t)(c->m_q + 1))) || (rc = c->alloc(&c->d_group_member, H * N))) return done(rc);
         std::vector<int32_t> gs(H * (size_t)(c->m_q + 1), 0);
@@ -769,6 +773,14 @@ int httm_expire_a_wait(httm_ctx* c, void* cuda_stream) {
     c->launches++;
     return check_cuda(c, launch_wait_expiry(c->d_qr, reinterpret_cast<float*>(c->d_kr), c->d_status, static_cast<cudaStream_t>(cuda_stream)),
                       "wait-expiry launch");
+}
+
+int httm_leave_parts_unfinished(httm_ctx* c, void* cuda_stream) {
+    if (!c) return HTTM_ERR_INVALID_ARG;
+    DeviceGuard guard(c->cfg.device);
+    if (!guard.ok) return c->fail(HTTM_ERR_CUDA, "cudaSetDevice failed");
+    return check_cuda(c, cudaMemsetAsync(c->d_part_count, 1, attention_partial_counters(c->sm_count) * sizeof(int32_t), static_cast<cudaStream_t>(cuda_stream)),
+                      "part counters");
 }
 
 int httm_set_head_shard(httm_ctx* c, int32_t total_heads, httm_exchange_fn exchange, void* user) {

@@ -69,7 +69,7 @@ struct TcParams {
     const int32_t* group_member;
     int32_t n_tokens;
     float* partial;              // optional: partial results of query tiles that are split over CTAs, see TailPlan
-    int32_t* part_count;         // their arrivals, four counters (32 rows each) per split tile, all zero between launches
+    int32_t* part_count;         // their arrivals, four counters (32 rows each) per split tile, all zero before the launch
     const __nv_bfloat16 *q, *k;  // the rows themselves, for the tile that is redone (element strides)
     int64_t q_stride_head, q_stride_token, k_stride_head, k_stride_token;
 };
@@ -420,7 +420,6 @@ __device__ __noinline__ bool epilogue_part(const TcParams& p, const PartArgs& a,
         int32_t* count = p.part_count + 4 * (first / parts) + (row >> 5);
         __threadfence();
         last = atomicAdd(count, 1) == parts - 1;
-        if (last) *count = 0;   // (as the next launch finds it)
         __threadfence();
     }
     if (!__shfl_sync(0xffffffffu, last, 0)) return true;

@@ -56,14 +56,20 @@ struct TensorView {          // bf16, element strides
     int64_t stride_head, stride_token;
 };
 
+// Words that a call's first kernel sets to zero for the kernels behind it: the state of the outlier filter, the arrivals of split query
+// tiles.  Neither is trusted to be as an earlier call left it: one whose bounded wait ran out may have stopped anywhere.
+struct ClearRange {
+    int32_t* words;   // may be null
+    int32_t n;
+};
+
 struct ReorderArgs {
     TensorView src[3];
     __nv_bfloat16* dst[3];   // [H][N][64] contiguous
     const int32_t* pi;       // [N]
     int32_t n_tokens, heads;
     float* inv_norm[2];      // optional, [H][N] each: 1 / max(|x|, 1e-12) of the reordered Q and K tokens (large-block path)
-    int32_t* clear;   // optional: words to set to zero for the kernels behind this one
-    int32_t n_clear;
+    ClearRange clear[2];     // optional: set to zero for the kernels behind this one
 };
 
 // Large-block path (blocks of 257 .. 4096 tokens; Sec. 4.1's 128 x 30 regime): matching as a dense contraction.
@@ -92,8 +98,7 @@ struct MatchArgs {
     const BlockInfo* blocks;
     int32_t n_blocks, n_tokens, heads;
     int32_t* status;
-    int32_t* clear;   // optional: words to set to zero for the kernels behind this one
-    int32_t n_clear;
+    ClearRange clear[2];     // optional: set to zero for the kernels behind this one
 };
 
 struct MergeArgs {
@@ -182,7 +187,7 @@ struct AttentionArgs {
     const int32_t* group_member;
     int32_t n_tokens;
     // optional: workspace for query tiles that are split over CTAs (attention_partial_floats / _counters; the counters are zero
-    // before the first launch and after every launch); null: tiles are dealt whole.  Launches that share it run in order.
+    // before every launch); null: tiles are dealt whole.  Launches that share it run in order.
     float* partial;
     int32_t* part_count;
 };

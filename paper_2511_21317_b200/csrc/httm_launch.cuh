@@ -27,6 +27,8 @@
 
 #include <utility>
 
+#include "httm_internal.h"
+
 namespace httm {
 
 __device__ __forceinline__ void depend_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -44,9 +46,11 @@ __device__ __forceinline__ int32_t ld_global_cg(const int32_t* p) {   // from L2
 }
 // zeros for the kernels behind this one (counters and histograms), spread over the CTAs: a memset of its own between two kernels would
 // cost its launch and both overlaps
-__device__ __forceinline__ void clear_words(int32_t* words, int n, int cta, int ctas) {
-    if (words)
-        for (int i = cta * (int)blockDim.x + (int)threadIdx.x; i < n; i += ctas * (int)blockDim.x) words[i] = 0;
+__device__ __forceinline__ void clear_words(const ClearRange (&clear)[2], int cta, int ctas) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (clear[k].words)
+            for (int i = cta * (int)blockDim.x + (int)threadIdx.x; i < clear[k].n; i += ctas * (int)blockDim.x) clear[k].words[i] = 0;
 }
 __device__ __forceinline__ float ld_global(const float* p) {
     float v;

@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(kReorderThreads) reorder_kernel(const __grid_c
     }
     depend_wait();
     dependents_launch();
-    if (t == 0 && h == 0) clear_words(a.clear, a.n_clear, blockIdx.x, gridDim.x);
+    if (t == 0 && h == 0) clear_words(a.clear, blockIdx.x, gridDim.x);
 #pragma unroll
     for (int u = 0; u < kReorderUnroll; ++u) {
         const int p = base + u * (kReorderThreads / 8) + slot;

@@ -134,7 +134,7 @@ match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     if (blockIdx.x < n_units) fetch();
     depend_wait();
     dependents_launch();
-    clear_words(a.clear, a.n_clear, blockIdx.x, gridDim.x);
+    clear_words(a.clear, blockIdx.x, gridDim.x);
     if (blockIdx.x < n_units && tid == 0) {
         issue(0, geom_next, bi_next.start, h_next);
         issue(1, geom_next, bi_next.start, h_next);

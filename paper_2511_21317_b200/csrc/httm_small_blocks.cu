@@ -81,7 +81,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     if (first < n_units) fetch();
     depend_wait();
     dependents_launch();
-    clear_words(a.clear, a.n_clear, blockIdx.x, gridDim.x);
+    clear_words(a.clear, blockIdx.x, gridDim.x);
     if (first < n_units && lane == 0)
         for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t) issue(t, bg_next, bi_next.start, h_next);
 
