@@ -811,7 +811,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 if (ok && ps.pair) {
                     const int grow = (ps.tile + x) * BM + row;
                     const RowTargets targets = row_targets<UNMERGE>(p, ps.head, grow, grow < mq_rows);   // (in flight during the wait)
-                    if ((ok = tc::mbar_wait(tc::smem_addr(&bars->o_final), (uint32_t)pass & 1u, abort_flag))) {
+                    if ((ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->o_final), (uint32_t)pass & 1u, abort_flag)))) {
                         tc::fence_after_sync();
                         const float inv = 1.0f / l;
                         uint32_t o[64];
@@ -833,7 +833,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                     // Do not touch O_B again (next pass's zero fill) before group A has read it.
                     xch[row] = make_float2(m, l);
                     tc::mbar_arrive(tc::smem_addr(&bars->x_full));
-                    ok = tc::mbar_wait(tc::smem_addr(&bars->x_done), n_single & 1u, abort_flag);
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->x_done), n_single & 1u, abort_flag));
                 } else if (ok && ps.part >= 0) {
                     PartArgs pa;
                     pa.head = ps.head;
@@ -852,8 +852,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                     //   out = (O_A 2^(m_A - m) + O_B 2^(m_B - m)) / (l_A 2^(m_A - m) + l_B 2^(m_B - m)),  m = max(m_A, m_B)
                     const int grow = ps.tile * BM + row;
                     const RowTargets targets = row_targets<UNMERGE>(p, ps.head, grow, grow < mq_rows);   // (in flight during the waits)
-                    ok = tc::mbar_wait(tc::smem_addr(&bars->o_final), (uint32_t)pass & 1u, abort_flag) &&
-                         tc::mbar_wait(tc::smem_addr(&bars->x_full), n_single & 1u, abort_flag);
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->o_final), (uint32_t)pass & 1u, abort_flag) &&
+                                                     tc::mbar_wait(tc::smem_addr(&bars->x_full), n_single & 1u, abort_flag));
                     if (ok) {
                         tc::fence_after_sync();
                         const float2 pb = xch[row];

@@ -235,7 +235,7 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         best = best_s[mine];
                         arg = arg_s[mine];
                     }
-                    ok = tc::mbar_wait(tc::smem_addr(&bars->s_full[b]), (k >> 1) & 1u, abort_flag);
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->s_full[b]), (k >> 1) & 1u, abort_flag));   // (a warp gives up together)
                     if (!ok) break;
                     tc::fence_after_sync();
 #pragma unroll
@@ -288,12 +288,12 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     // the two column halves of a token meet: half 1 hands (best, arg) over, half 0 decides (ties: lowest dst)
                     const int slot = i & 1;
                     if (half == 1) {
-                        ok = tc::mbar_wait(tc::smem_addr(&bars->x_done[slot]), (n_x[slot] & 1u) ^ 1u, abort_flag);
+                        ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->x_done[slot]), (n_x[slot] & 1u) ^ 1u, abort_flag));
                         if (!ok) break;
                         xch[slot * TILE + row] = make_float2(best, __int_as_float(arg));
                         tc::mbar_arrive(tc::smem_addr(&bars->x_full[slot]));
                     } else {
-                        ok = tc::mbar_wait(tc::smem_addr(&bars->x_full[slot]), n_x[slot] & 1u, abort_flag);
+                        ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->x_full[slot]), n_x[slot] & 1u, abort_flag));
                         if (!ok) break;
                         const float2 o = xch[slot * TILE + row];
                         tc::mbar_arrive(tc::smem_addr(&bars->x_done[slot]));

@@ -256,7 +256,7 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
             }
             rep = bm.row_of_token(rep);
         }
-        if (!mbar_wait_bounded(mbar0 + 8 * buf, parity, a.status, kDevTimeoutMatchLoad)) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(mbar0 + 8 * buf, parity, a.status, kDevTimeoutMatchLoad))) {
             failed = true;
             break;
         }
