@@ -14,6 +14,8 @@
 #include "httm_blocks.cuh"
 #include "httm_launch.cuh"
 
+#include <math_constants.h>
+
 namespace httm {
 
 namespace {
@@ -164,8 +166,9 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     mma_bf16_16816(dn, ad, bf[ks][0], bf[ks][1]);
             }
             const float dsel = (g & 1) ? dn[1] : dn[0];
-            const float w0 = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq)), w1 = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq + 4));
-            const bool has0 = 2 * tq < nd, has1 = 2 * tq + 1 < nd;
+            float w0 = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq)), w1 = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq + 4));
+            if (2 * tq >= nd) w0 = CUDART_NAN_F;
+            if (2 * tq + 1 >= nd) w1 = CUDART_NAN_F;
             // ---- best dst of every row
             uint32_t key[2] = {0u, 0u};
             int best[2] = {0, 0};
@@ -188,11 +191,11 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         }
                     }
                     // rows g and g + 8, this lane's two dst tokens (ties: the lower one)
-                    const float s00 = has0 ? c[0] * w0 : -INFINITY, s01 = has1 ? c[1] * w1 : -INFINITY;
-                    const float s10 = has0 ? c[2] * w0 : -INFINITY, s11 = has1 ? c[3] * w1 : -INFINITY;
-                    // (the product of an overflowing dot product and a norm that overflows is not a number and never the best)
-                    const float t0 = tc::fmax3(s00, s01, -INFINITY), t1 = tc::fmax3(s10, s11, -INFINITY);
-                    const int d0 = 2 * tq + (s01 == t0 && s00 != t0 ? 1 : 0), d1 = 2 * tq + (s11 == t1 && s10 != t1 ? 1 : 0);
+                    // (the maximum with -infinity drops what is not a number: a place without a dst token, tokens whose norm overflows)
+                    const float s00 = fmaxf(c[0] * w0, -INFINITY), s01 = fmaxf(c[1] * w1, -INFINITY);
+                    const float s10 = fmaxf(c[2] * w0, -INFINITY), s11 = fmaxf(c[3] * w1, -INFINITY);
+                    const float t0 = fmaxf(s00, s01), t1 = fmaxf(s10, s11);
+                    const int d0 = 2 * tq + (s01 > s00 ? 1 : 0), d1 = 2 * tq + (s11 > s10 ? 1 : 0);
                     // lanes 0, 1 of a row's four split the two rows, then meet lanes 2, 3
                     float top = odd ? t1 : t0;
                     int arg = odd ? d1 : d0;
