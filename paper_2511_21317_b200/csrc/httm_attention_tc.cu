@@ -85,15 +85,18 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
-// 2^t for two values without the special-function unit.  The argument comes as u = (t + 125) / 250 clamped to [0, 1] by the
-// saturating multiply-add that scales the scores (an argument of 125 or more gives 2^125, which the caller's test of the
-// tile's row sum catches; without the clamp the exponent arithmetic below would wrap).  Then round-to-nearest range reduction
+// 2^t for two values without the special-function unit.  The argument is clamped to [-125, 125] (an argument of 125 or more gives
+// 2^125, which the caller's test of the tile's row sum catches; without the clamp the exponent arithmetic below would wrap) by a saturating
+// multiply-add, u = t / 250 + 1 / 2: min / max clamps took another 8 cycles of the ALU.  Then round-to-nearest range reduction
 // t = n + f, f in [-0.5, 0.5] (the integer lands in the low mantissa bits of t + 1.5 * 2^23), a cubic minimax polynomial for
 // 2^f (relative error < 1e-4, far below the bf16 rounding of P) evaluated with packed fp32 FMAs, and n added to the exponent
-// field.  16 cycles of the FMA pipe per pair and warp; min / max clamps took another 8 of the ALU.
-__device__ __forceinline__ float2 exp2_poly2(float2 u) {
+// field.  t itself is s c - m in one rounding, as the other exponentials take it: u straight from the score, s (c / 250) +
+// (125 - m) / 250, rounds two constants in proportion to m, which weighed these keys against the others by 1e-3 at scores of
+// 3e4 (error of the output against 64 bits 5.65e-3 instead of 5.61e-3 there, 7.28e-2 instead of 7.14e-2 at 5e5).
+__device__ __forceinline__ float2 exp2_poly2(float2 t) {
     const float kMagic = 12582912.0f - 125.0f;
     const float2 magic = make_float2(kMagic, kMagic), width = make_float2(250.0f, 250.0f);
+    const float2 u = make_float2(tc::ffma_sat(t.x, 1.0f / 250.0f, 0.5f), tc::ffma_sat(t.y, 1.0f / 250.0f, 0.5f));
     const float2 tt = tc::ffma2(u, width, magic);
     const float2 f = tc::ffma2(u, width, tc::fsub2(magic, tt));
     float2 q = tc::ffma2(make_float2(0.055171460f, 0.055171460f), f, make_float2(0.24261086f, 0.24261086f));
@@ -102,11 +105,11 @@ __device__ __forceinline__ float2 exp2_poly2(float2 u) {
     return make_float2(__int_as_float(__float_as_int(q.x) + (__float_as_int(tt.x) << 23)),
                        __int_as_float(__float_as_int(q.y) + (__float_as_int(tt.y) << 23)));
 }
-// Of every sixteen pairs of scores, the pairs whose bit is set here take the polynomial (FMA pipe), the others ex2.approx
+// Of every eight pairs of scores, the pairs whose bit is set here take the polynomial (FMA pipe), the others ex2.approx
 // (special-function unit: 8 cycles per warp instruction and scheduler, so 1024 cycles for the 128 scores of a row against 528
-// of tensor-core work per tile).  Measured in the whole kernel, 10992 x 10992 x 16 heads: 4 of 16 with min / max clamps 520 us;
-// with the saturating form 4 of 16 515, 5 of 16 505 (other choices of five 511 .. 515), 6 of 16 529.
-constexpr uint32_t kPolyPairs = 0x9211;
+// of tensor-core work per tile).  Measured in the whole kernel, 32 976 x 32 976 x 16 heads: two of eight 4 870 us, five of sixteen
+// 4 960, two of eight at other places (over sixteen pairs) 4 930 .. 5 000.
+constexpr uint32_t kPolyPairs = 0x11;   // pairs 0 and 4
 
 // A score tile whose weights overflowed with the stabiliser at hand is done again here, for one query row per thread:
 // its 128 scores are recomputed from the rows in global memory by plain fp32 FMAs (the tile in tensor memory is
@@ -755,7 +758,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                     };
                     auto weights = [&]() {   // P = 2^(s c - m) as bf16 pairs over the LAST 64 columns of S; returns the row sum
                         const float2 c2 = make_float2(c, c), neg_m2 = make_float2(-m, -m);
-                        const float cu = c * (1.0f / 250.0f), mu = (125.0f - m) * (1.0f / 250.0f);
                         float2 sum0 = make_float2(0.f, 0.f), sum1 = sum0;
 #pragma unroll
                         for (int cc = 0; cc < 8; ++cc) {
@@ -764,12 +766,11 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                             for (int i = 0; i < 8; ++i) {
                                 const float sx = __uint_as_float(s[cc * 16 + 2 * i]), sy = __uint_as_float(s[cc * 16 + 2 * i + 1]);
                                 float2 e;
-                                if ((kPolyPairs >> ((cc & 1) * 8 + i)) & 1u) {
-                                    e = exp2_poly2(make_float2(tc::ffma_sat(sx, cu, mu), tc::ffma_sat(sy, cu, mu)));
-                                } else {
-                                    const float2 t = tc::ffma2(make_float2(sx, sy), c2, neg_m2);
+                                const float2 t = tc::ffma2(make_float2(sx, sy), c2, neg_m2);
+                                if ((kPolyPairs >> i) & 1u)
+                                    e = exp2_poly2(t);
+                                else
                                     e = make_float2(fast_exp2(t.x), fast_exp2(t.y));
-                                }
                                 if (i & 1)
                                     sum1 = tc::fadd2(sum1, e);
                                 else

@@ -156,6 +156,24 @@ def test_scores_far_above_those_of_the_first_key_tile(heads):
             report_peaky(f"growing scores, {name}", stats)
 
 
+@pytest.mark.parametrize("size", [512, 1280, 2560, 3072])
+def test_equal_scores_of_any_size_weigh_the_same(size):
+    """All queries and all keys alike, with scores of size^2 / 8 (3e4 .. 1e6): every key has the same weight, whichever unit took its
+    exponential.  Key j has V = 1 in channel j mod 64, so every channel of the output is 1 / 64, up to half a step of the weights
+    in bf16 (2^-8 relative) and of the output (2^-9)."""
+    heads, n = 2, 1024
+    x = torch.zeros(heads, n, 64, device=DEV)
+    x[..., 0] = size
+    v = torch.eye(64, device=DEV).repeat(n // 64, 1).expand(heads, n, 64).contiguous()
+    with hb.Httm(hb.HttmConfig(frames=1, n_camera=0, n_register=0, grid_h=1, grid_w=n, heads=heads, head_dim=64, blk_frames=1, blk_h=1, blk_w=2,
+                               ratio_q=0.5, ratio_kv=0.5)) as ctx:
+        out = ctx.dense_attention(x.bfloat16(), x.bfloat16(), v.bfloat16()).double()
+        torch.cuda.synchronize()
+        assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+    err = (out * 64 - 1).abs().max().item()
+    assert err <= 2.0 ** -8 + 2.0 ** -9, err
+
+
 def test_dense_attention_small_config_sampled():
     wl = synth.WORKLOADS["small"].replace(heads=4)
     q, k, v = synth.make_qkv(wl)
