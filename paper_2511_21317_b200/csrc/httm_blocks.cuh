@@ -76,8 +76,8 @@ struct TaskCursor {
 };
 
 // bytes to the next multiple of 1024.  Added to the shared array's own name, so that the compiler still knows the address space:
-// behind a pointer rounded up as an integer every access was a generic one (LD instead of LDS; a call on
-// 11 016 tokens 121.0 -> 119.7 us, outlier filtering of 32 976 tokens 77.8 -> 72.1 us).
+// behind a pointer rounded up as an integer every access was a generic one (a call on 11 016 tokens 121.0 -> 119.7 us, outlier
+// filtering of 32 976 tokens 77.8 -> 72.1 us).
 __device__ __forceinline__ uint32_t align_pad(const void* shared) { return (0u - smem_u32(shared)) & 1023u; }
 
 // tiled TMA load {64 channels, rows, heads} -> this CTA's shared memory; the channel coordinate is 0

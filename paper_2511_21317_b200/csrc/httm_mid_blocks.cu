@@ -373,7 +373,8 @@ __global__ void __launch_bounds__(32 * W, team_ctas(W, P)) merge_team_kernel(con
     constexpr int NMAX = team_tokens(W, P), T = 32 * W;
     constexpr uint32_t STAGE = NMAX * kRowBytes;
     constexpr MergeAux X = merge_aux(NMAX);
-    constexpr int NP = W == 1 ? 4 : (W == 2 ? 2 : 1);   // pairs of 8-channel tiles per warp
+    static_assert(W == 1 || W == 4 || W == 8, "how the channels are dealt to the warps");
+    constexpr int NP = W == 1 ? 4 : 1;   // pairs of 8-channel tiles per warp
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + align_pad(smem_raw);
     unsigned char* aux = smem + 2 * STAGE;
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(32 * W, team_ctas(W, P)) merge_team_kernel(con
                 const int* members = cnt + (2 * par + map) * NMAX;
                 const int k = t == 0 ? n_kept[0] : n_kept[1];
                 const int n_mt = (k + 15) >> 4, n_out = min(k, m.n - r);   // (a corrupt map cannot overrun)
-                const int np0 = W == 1 ? 0 : (W == 2 ? 2 * warp : (warp & 3));
+                const int np0 = W == 1 ? 0 : (warp & 3);
 #pragma unroll 1
                 for (int mt = W == 8 ? warp >> 2 : 0; mt < n_mt; mt += W == 8 ? 2 : 1) {
                     const int r0 = 16 * mt + g, r1 = r0 + 8;   // this lane's two accumulator rows

@@ -1,5 +1,5 @@
 """Attention with query tiles that are split over CTAs: where a few 128-row query tiles are left after whole tiles have been dealt,
-each of them is worked off in parts of its keys by several CTAs and the part that arrives last adds the partial softmaxes up."""
+each of them is worked off in parts of its keys by several CTAs; of the warps with the same rows the one that arrives last adds the partial softmaxes up."""
 import pytest
 import torch
 
@@ -13,9 +13,9 @@ DEV = "cuda:0"
 # (heads, frames, blocks, ratio_q, ratio_kv, outlier fraction): tiles left, and parts, on 148 SMs
 CASES = {
     "few_tiles": (2, 4, (2, 4, 4), 0.9, 0.0, 0.0),            # 12 tiles in 5 parts of 8 or 9 key tiles, unmerge in the epilogue
-    "one_head_many_parts": (1, 11, (4, 4, 4), 0.9, 0.0, 0.0),  # 11 .. 12 tiles in 12 parts, plain rows
+    "one_head_many_parts": (1, 11, (4, 4, 4), 0.9, 0.0, 0.0),  # 14 tiles in 10 parts of 11 or 12, plain rows
     "two_parts": (12, 4, (2, 4, 4), 0.9, 0.0, 0.0),            # 72 tiles in 2 parts of 21 or 22
-    "singles_then_parts": (16, 8, (2, 4, 4), 0.7, 0.4, 0.0),   # 448 tiles: a round of pairs, one of single tiles, 4 tiles in parts
+    "singles_then_parts": (16, 8, (2, 4, 4), 0.7, 0.4, 0.0),   # 448 tiles: a round of pairs, one of single tiles, 4 tiles in 6 parts
     "per_head_lengths": (2, 8, (2, 4, 4), 0.8, 0.2, 0.03),     # the plan is made on the device
 }
 
