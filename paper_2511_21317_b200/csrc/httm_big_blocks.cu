@@ -629,7 +629,8 @@ __device__ int build_groups(const int32_t* A, int block_start, int n, int limit,
 
 // Sum of the rows keys[i0 .. i1) (positions in the low 12 bits), eight channels from x on.  Four members are in flight: the gather is
 // bound by load latency.  They are added in pairs of pairs, to one of two sums in turn: n / 8 + 4 roundings for n members.  (Added
-// one after the other they took n: with one member 2^17 times the others, 2 048 of them left the mean half a step of bf16 off.)
+// one after the other they took n: with one member 2^17 times the others, 2 048 of them left the mean half a step of bf16 off; that
+// was a little faster, at 82 440 tokens x 16 heads in 3840-token blocks filter 216 / 221 us, merge 224 / 237 us.)
 __device__ __forceinline__ void sum_members(const __nv_bfloat16* x, int64_t stride, const uint32_t* keys, int i0, int i1, float (&sum)[8]) {
     float other[8];
 #pragma unroll
