@@ -5,6 +5,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <numeric>
 #include <string>
 #include <vector>
 
@@ -70,8 +71,8 @@ struct httm_ctx {
     float *d_eps = nullptr, *d_tau = nullptr;
     __nv_bfloat16 *d_qm_var = nullptr, *d_om_var = nullptr;
     // large merging blocks (257 .. 4096 tokens, Sec. 4.1): matching as a tensor-core contraction, see httm_big_blocks.cu
-    std::vector<BigItem> big_items;
-    BigItem* d_big_items = nullptr;
+    std::vector<int32_t> big_order;   // blocks from the longest to the shortest
+    int32_t* d_big_order = nullptr;
     float *d_inv_norm_q = nullptr, *d_inv_norm_k = nullptr;
     uint32_t *d_best_key_q = nullptr, *d_best_key_k = nullptr;
     int32_t *d_best_pos_q = nullptr, *d_best_pos_k = nullptr;
@@ -125,7 +126,7 @@ struct httm_ctx {
         void* ptrs[] = {d_geom, d_pi, d_pi_inv, d_assign_q, d_assign_k, d_rank_q, d_status, d_blocks, d_qr, d_kr,
                         d_vr, d_qm,     d_km,       d_vm,       d_om,     hs[0].q,  hs[0].k,  hs[0].v, hs[0].out, hs[1].q, hs[1].k, hs[1].v, hs[1].out,
                         d_assign_qf, d_kept_cnt, d_moff_var, d_mq_head, d_tile_prefix, d_sel, d_eps, d_tau, d_qm_var, d_om_var,
-                        d_big_items, d_inv_norm_q, d_inv_norm_k, d_best_key_q, d_best_key_k, d_best_pos_q, d_best_pos_k,
+                        d_big_order, d_inv_norm_q, d_inv_norm_k, d_best_key_q, d_best_key_k, d_best_pos_q, d_best_pos_k,
                         d_group_start, d_group_member, d_partial, d_part_count};
         for (void* p : ptrs)
             if (p) cudaFree(p);
@@ -182,9 +183,11 @@ TensorView view(const __nv_bfloat16* p, int64_t rows) { return TensorView{p, row
 
 float scale_log2() { return 1.4426950408889634f / std::sqrt((float)kHeadDim); }
 
+// The counter of the large-block score kernel's work items lies behind the arrivals of split query tiles.
+int32_t* item_counter(httm_ctx* c) { return c->d_part_count + attention_partial_counters(c->sm_count); }
 // What the first kernel of a call sets to zero for the kernels behind it
 void clear_state(httm_ctx* c, ClearRange (&clear)[2]) {
-    clear[0] = ClearRange{c->d_part_count, (int32_t)attention_partial_counters(c->sm_count)};
+    clear[0] = ClearRange{c->d_part_count, (int32_t)attention_partial_counters(c->sm_count) + 1};
     if (c->filtering()) clear[1] = ClearRange{c->d_sel, kSelWords};
 }
 
@@ -250,15 +253,19 @@ BigMatchArgs big_match_args(httm_ctx* c) {
     a.assign[0] = c->d_assign_q;
     a.assign[1] = c->d_assign_k;
     a.blocks = c->d_blocks;
-    a.items = c->d_big_items;
-    a.n_items = (int32_t)c->big_items.size();
+    a.order = c->d_big_order;
+    a.counter = item_counter(c);
     a.n_blocks = c->n_blocks;
     a.n_tokens = c->n_tokens;
     a.heads = c->cfg.heads;
     a.status = c->d_status;
     return a;
 }
-int stage_big_scores(httm_ctx* c, cudaStream_t s) {
+int stage_big_scores(httm_ctx* c, cudaStream_t s, bool chained = false) {   // chained: inside a call, whose first kernel has cleared the counter
+    if (!chained) {
+        const int rc = check_cuda(c, cudaMemsetAsync(item_counter(c), 0, sizeof(int32_t), s), "item counter reset");
+        if (rc) return rc;
+    }
     c->launches++;
     return check_cuda(c, launch_big_scores(big_match_args(c), c->sm_count, s), "large-block score launch");
 }
@@ -504,7 +511,7 @@ int global_impl(httm_ctx* c, const httm_tensor& q, const httm_tensor& k, const h
     int rc;
     if (c->big()) {   // six kernels: reorder (+ norms), scores, select, merge, attention, unmerge
         if ((rc = part(stage_reorder(c, q, k, v, s, true), "reorder"))) return rc;
-        if ((rc = part(stage_big_scores(c, s), "big_scores"))) return rc;
+        if ((rc = part(stage_big_scores(c, s, true), "big_scores"))) return rc;
         if ((rc = part(stage_big_select(c, s), "big_select"))) return rc;
         if (c->filtering() && (rc = part(stage_outlier(c, q, s, true), "outlier_filter"))) return rc;
         if ((rc = part(stage_merge(c, s, nullptr, true), "merge"))) return rc;
@@ -593,8 +600,9 @@ int httm_create(const httm_config* cfg, httm_ctx** out) {
         c->blk_start = std::move(plan.blk_start);
         c->blocks = std::move(plan.blocks);
         c->geom = std::move(plan.geom);
-        for (int32_t b = 0; b < c->n_blocks; ++b)
-            for (int row0 = 0; row0 < c->blocks[b].n; row0 += kBigSliceRows) c->big_items.push_back(BigItem{b, row0});
+        c->big_order.resize(c->n_blocks);
+        std::iota(c->big_order.begin(), c->big_order.end(), 0);
+        std::stable_sort(c->big_order.begin(), c->big_order.end(), [&](int32_t x, int32_t y) { return c->blocks[x].n > c->blocks[y].n; });
     }
     {   // the match kernels hold a quarter of their largest block as dst tokens (the large-block path 1024); anchored blocks of
         // up to 256 tokens with more (two or three frames per block) go to a kernel of their own
@@ -640,7 +648,7 @@ int httm_create(const httm_config* cfg, httm_ctx** out) {
         (rc = c->alloc(&c->d_vm, H * c->m_k * kHeadDim)) || (rc = c->alloc(&c->d_om, H * c->m_q * kHeadDim)))
         return done(rc);
 
-    if ((rc = c->alloc(&c->d_partial, attention_partial_floats(c->sm_count))) || (rc = c->alloc(&c->d_part_count, attention_partial_counters(c->sm_count))))
+    if ((rc = c->alloc(&c->d_partial, attention_partial_floats(c->sm_count))) || (rc = c->alloc(&c->d_part_count, attention_partial_counters(c->sm_count) + 1)))
         return done(rc);
     if (c->max_block <= 32) {   // member lists of the merged query rows; entry M_q of every head is the constant N
         if ((rc = c->alloc(&c->d_group_start, H * (size_t)(c->m_q + 1))) || (rc = c->alloc(&c->d_group_member, H * N))) return done(rc);
@@ -649,12 +657,12 @@ int httm_create(const httm_config* cfg, httm_ctx** out) {
         if ((rc = check_cuda(c, cudaMemcpy(c->d_group_start, gs.data(), gs.size() * 4, cudaMemcpyHostToDevice), "group table upload"))) return done(rc);
     }
     if (c->big()) {
-        if ((rc = c->alloc(&c->d_big_items, c->big_items.size())) || (rc = c->alloc(&c->d_inv_norm_q, H * N)) ||
+        if ((rc = c->alloc(&c->d_big_order, c->big_order.size())) || (rc = c->alloc(&c->d_inv_norm_q, H * N)) ||
             (rc = c->alloc(&c->d_inv_norm_k, H * N)) || (rc = c->alloc(&c->d_best_key_q, H * N)) || (rc = c->alloc(&c->d_best_key_k, H * N)) ||
             (rc = c->alloc(&c->d_best_pos_q, H * N)) || (rc = c->alloc(&c->d_best_pos_k, H * N)))
             return done(rc);
-        if ((rc = check_cuda(c, cudaMemcpy(c->d_big_items, c->big_items.data(), c->big_items.size() * sizeof(BigItem), cudaMemcpyHostToDevice),
-                             "item table upload")))
+        if ((rc = check_cuda(c, cudaMemcpy(c->d_big_order, c->big_order.data(), c->big_order.size() * sizeof(int32_t), cudaMemcpyHostToDevice),
+                             "block order upload")))
             return done(rc);
     }
     // uploads; special tokens are never merged: their map entries are constants, written once

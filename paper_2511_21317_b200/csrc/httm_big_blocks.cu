@@ -3,9 +3,9 @@
 // warp's stage, and its similarity step (Eq. 1) is a real dense contraction: n tokens x n_dst dst tokens x 64.
 //
 //   big_scores_kernel   cosine of every token of a block with every dst token of the block on the 5th-generation
-//                       tensor cores (tcgen05.mma, accumulators in tensor memory; the dst tokens enter scaled by
-//                       their inverse norms, split exactly into three bf16 planes), fused with the row-wise
-//                       arg-max: per token the best dst and the best cosine
+//                       tensor cores (tcgen05.mma, accumulators in tensor memory), fused with the row-wise
+//                       arg-max, which weighs the products by the dst tokens' inverse norms: per token the best dst
+//                       and the best cosine
 //   big_select_kernel   the r src tokens with the best cosines merge (Sec. 3.2): exact radix select per block,
 //                       ties by position; writes the assignment map
 //   big_merge_kernel    mean of every group (Sec. 3.2): tokens sorted by (merged row, position), one warp
@@ -33,38 +33,119 @@ __device__ __forceinline__ bool is_dst_position(int j, int n_rule, int nd) {
 }
 
 // ------------------------------------------------------------------------------------------------ scores
-// cos(i, d) |x_i| = sum_k x_ik (w_d x_dk) with w_d = 1 / max(|x_d|, 1e-12).  The dst rows are multiplied by their
-// inverse norms when they are gathered, and the fp32 products are split EXACTLY into three bf16 planes (8 + 8 + 8
-// significant bits), so that three accumulating MMAs per K step give the scaled scores straight in tensor memory: the
-// arg-max warps neither load weights nor multiply (the tensor cores are idle most of the time in this kernel, the
-// arg-max warps are what bounds it).  The dst tokens of a block are taken 256 at a time (three planes of 32 KB); the
-// token tiles of the slice are streamed once per such chunk, and every token's best so far waits in shared memory.
-constexpr int TILE = 128;                        // rows of an operand tile
+// cos(i, d) |x_i| = w_d sum_k x_ik x_dk with w_d = 1 / max(|x_d|, 1e-12).  The products of bf16 values are exact in fp32 and add up in
+// tensor memory; the arg-max warps multiply by w_d (one rounding).  All dst tokens of a block (at most 1024: 128 KB) stay in shared
+// memory, so a token tile is loaded once and its best so far stays in registers.  What bounds it is the arg-max warps' instruction issue and
+// latency (the MMAs of a pair of tiles and 128 dst tokens take 512 cycles, the warps about 2300 of two groups at work), hence:
+//  - a warp works on TWO token tiles at a time: the data of a broadcast load of weights goes to every lane, four cycles of the SM's
+//    shared-memory port for four columns, and is used twice this way;
+//  - two groups of eight warps, each with a score buffer for a pair of tiles and 128 dst tokens (one group: 515 us);
+//  - work items (tensor, head, block) are taken from a counter, the longest first (dealt in rounds one tensor after the other, the longest of
+//    148 CTAs had 15 % more than the mean).
+// Measured at 16 heads x 22 blocks of up to 3840 tokens, 384 dst tokens of the queries and 960 of the keys: 611 us with the dst tokens split into three
+// scaled planes, 256 at a time, and one group of warps; 467 us now.  The dst tokens chosen are closer to the best in 64 bits
+// (1.6 million tokens of three scenes: 26 off the best by up to 4.6e-7 before, 6 by up to 1.2e-7).  Tried and dropped: an issuing warp for each
+// group (477 us), a longer ring of token tiles (487 us), 16 loads of a dst gather in flight (476 us), no carrying along where no row of the warp
+// improves (491 us).
+constexpr int TILE = 128;                        // rows of an operand tile, dst tokens of a chunk
 constexpr int TILE_BYTES = TILE * kRowBytes;     // 16 KB
-constexpr int kChunkDst = 256;                   // dst tokens per chunk = columns of a score buffer
-constexpr int kPlaneBytes = kChunkDst * kRowBytes;       // 32 KB
-constexpr int kSrcTilesPerItem = kBigSliceRows / TILE;   // 32: a work item is a whole block
-constexpr int SC_THREADS = 320;                  // warp 0: TMA producer, warp 1: MMA issuer, warps 2-9: arg-max (two column halves x four lane quadrants)
-constexpr int SC_TMEM_COLS = 512;                // two score buffers of 256 columns
-constexpr int SC_STAGES = 4;                     // ring of token tiles: a tile's load takes longer than its MMAs and its arg-max
+constexpr int SC_GROUPS = 2;                     // groups of arg-max warps (two column halves x four lane quadrants each)
+constexpr int SC_THREADS = 128 + SC_GROUPS * 256;   // warp 0: TMA producer, warp 1: MMA issuer (2 and 3 only make up the four), then the arg-max warps
+constexpr int kScoreRoleRegs = 32, kScoreMaxRegs = 112;   // of the 5 x 96 the kernel starts with
+constexpr int SC_TMEM_COLS = 512;                // a buffer pair of 2 x 128 columns (by tile of the pair) for each group
+constexpr int SC_STAGES = 4;                     // ring of token tiles: a pair for each group
 
 struct ScoreBars {
     uint64_t a_full[SC_STAGES], a_empty[SC_STAGES];   // ring of token tiles
-    uint64_t s_full[2], s_empty[2];   // score buffers
-    uint64_t x_full[2], x_done[2];    // exchange of the two column halves' results, by token-tile parity
+    uint64_t s_full[SC_GROUPS], s_empty[SC_GROUPS];   // pairs of score buffers
+    uint64_t x_full[SC_GROUPS], x_done[SC_GROUPS];    // exchange of the two column halves' results
     uint32_t tmem_base;
     int abort_flag;
+    int next;                         // the CTA's next work item
 };
-constexpr int SC_OFF_A = 3 * kPlaneBytes;                        // token tiles behind the three planes
-constexpr int SC_OFF_BEST = SC_OFF_A + SC_STAGES * TILE_BYTES;   // float [2 halves][tokens of the item]: best score so far
-constexpr int SC_OFF_ARG = SC_OFF_BEST + 2 * kBigSliceRows * 4;  // uint16 [2][tokens]: its dst (n_dst <= 1024)
-constexpr int SC_OFF_XCH = SC_OFF_ARG + 2 * kBigSliceRows * 2;   // [2][128] (best, arg) of column half 1
-constexpr int SC_OFF_BARS = SC_OFF_XCH + 2 * TILE * 8;
+constexpr int SC_OFF_A = kMaxBigDst * kRowBytes;                 // token tiles behind the dst tokens
+constexpr int SC_OFF_W = SC_OFF_A + SC_STAGES * TILE_BYTES;      // float [dst]: the weights of the dst tokens
+constexpr int SC_OFF_XCH = SC_OFF_W + kMaxBigDst * 4;            // [groups][2][128] (best, arg) of column half 1
+constexpr int SC_OFF_BARS = SC_OFF_XCH + 2 * 2 * TILE * 8;
 constexpr int SC_SMEM = SC_OFF_BARS + 256 + 1024 /*alignment slack*/;
+static_assert(sizeof(ScoreBars) <= 256 && kMaxBigDst % TILE == 0 && SC_SMEM <= 232448, "");
 
-__device__ __forceinline__ uint32_t bf16_bits_rn(float f) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(f);
-    return (uint32_t)*reinterpret_cast<const unsigned short*>(&h);
+// x s for two bf16 values packed in a word, s a power of two: exact (but for values that leave the format)
+__device__ __forceinline__ uint32_t scale_bf16x2(uint32_t v, float s) {
+    const __nv_bfloat162 r = __floats2bfloat162_rn(__uint_as_float(v << 16) * s, __uint_as_float(v & 0xffff0000u) * s);
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+
+// A token's best dst so far: its score, the first dst of the group of eight that holds it, and the scores of that group, which tell the
+// dst itself once at the end.  The eight scores are carried along by multiplying with zeros and ones on the FMA pipe, which has time:
+// looking for the column whenever a row of the warp improves (in nearly every group) takes two cycles of the ALU for each of 75
+// selects and compares, and the ALU has the maxima to take.  A score that is not finite spoils the eight (0 x inf): the dst is then
+// looked for again (find_again).
+constexpr int kGroup = 8;
+struct Best {
+    float score, first_dst;   // (-1: none)
+    float2 v[kGroup / 2];
+};
+__device__ __forceinline__ void take_best(Best& best, float (&s)[32], int first_dst, int valid) {   // dst first_dst + c, c < valid
+    if (valid < 32) {   // the block's last dst tokens: -inf for the maxima, zeros for what is carried along
+#pragma unroll
+        for (int c = 0; c < 32; ++c)
+            if (c >= valid) s[c] = -INFINITY;
+    }
+    float g[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        g[q] = fmaxf(tc::fmax3(tc::fmax3(s[8 * q], s[8 * q + 1], s[8 * q + 2]), s[8 * q + 3], s[8 * q + 4]), tc::fmax3(s[8 * q + 5], s[8 * q + 6], s[8 * q + 7]));
+    if (valid < 32) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c)
+            if (c >= valid) s[c] = 0.f;
+    }
+    const float m = fmaxf(tc::fmax3(g[0], g[1], g[2]), g[3]);
+    bool open = m > best.score;   // (ties: lowest dst, the first group that holds the maximum)
+    const float keep = open ? 0.f : 1.f;
+    float f[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const bool here = open && g[q] == m;
+        f[q] = here ? 1.f : 0.f;
+        open = open && !here;
+    }
+    best.score = fmaxf(best.score, m);
+    const float base = (float)first_dst;
+    best.first_dst = fmaf(best.first_dst, keep, fmaf(f[0], base, f[1] * (base + 8.f)) + fmaf(f[2], base + 16.f, f[3] * (base + 24.f)));
+#pragma unroll
+    for (int c = 0; c < kGroup / 2; ++c) {
+        float2 v = tc::fmul2(best.v[c], make_float2(keep, keep));
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v = tc::ffma2(make_float2(s[8 * q + 2 * c], s[8 * q + 2 * c + 1]), make_float2(f[q], f[q]), v);
+        best.v[c] = v;
+    }
+}
+// The dst tokens of one column half again, one by one, for a token whose eight scores have been spoilt: the best that is a number,
+// ties to the lowest.
+__device__ __noinline__ int find_again(const __nv_bfloat16* x, const unsigned char* dst, const float* w, int half, int nd) {
+    float best = -INFINITY;
+    int arg = 0;
+    for (int d = half * 64; d < nd; d += (d & 63) == 63 ? 65 : 1) {
+        float s = 0.f;
+        for (int c16 = 0; c16 < 8; ++c16) {
+            const uint4 a = ld_global(reinterpret_cast<const uint4*>(x) + c16);
+            const uint4 b = *reinterpret_cast<const uint4*>(dst + d * kRowBytes + ((c16 ^ (d & 7)) << 4));
+            const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                s = fmaf(__uint_as_float(aw[e] << 16), __uint_as_float(bw[e] << 16), s);
+                s = fmaf(__uint_as_float(aw[e] & 0xffff0000u), __uint_as_float(bw[e] & 0xffff0000u), s);
+            }
+        }
+        s *= w[d];
+        if (s > best) {
+            best = s;
+            arg = d;
+        }
+    }
+    return arg;
 }
 
 __global__ void __launch_bounds__(SC_THREADS, 1)
@@ -72,8 +153,7 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t s_b = tc::smem_addr(smem), s_a = s_b + SC_OFF_A;
-    float* best_s = reinterpret_cast<float*>(smem + SC_OFF_BEST);
-    uint16_t* arg_s = reinterpret_cast<uint16_t*>(smem + SC_OFF_ARG);
+    float* w_s = reinterpret_cast<float*>(smem + SC_OFF_W);
     float2* xch = reinterpret_cast<float2*>(smem + SC_OFF_XCH);
     ScoreBars* bars = reinterpret_cast<ScoreBars*>(smem + SC_OFF_BARS);
     volatile int* abort_flag = &bars->abort_flag;
@@ -85,7 +165,7 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             tc::mbar_init(tc::smem_addr(&bars->a_full[i]), 1);
             tc::mbar_init(tc::smem_addr(&bars->a_empty[i]), 1);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < SC_GROUPS; ++i) {
             tc::mbar_init(tc::smem_addr(&bars->s_full[i]), 1);
             tc::mbar_init(tc::smem_addr(&bars->s_empty[i]), 256);
             tc::mbar_init(tc::smem_addr(&bars->x_full[i]), 128);
@@ -103,216 +183,236 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     depend_wait();
     dependents_launch();
 
-    // completions so far of every barrier (each role counts its own): they give the phase parities across chunks and items
-    uint32_t n_tiles_done = 0;   // token tiles so far: tile k uses ring stage k % SC_STAGES and score buffer k & 1
-    uint32_t n_x[2] = {0, 0};    // exchanges per parity slot
-    const int64_t total = 2ll * a.heads * a.n_items;
-    constexpr uint32_t idesc = tc::idesc_bf16(128, kChunkDst, false, false);
-    constexpr uint64_t kTileStep = TILE_BYTES >> 4, kPlaneStep = kPlaneBytes >> 4;   // descriptor address fields count 16-byte units
-
-    for (int64_t item = blockIdx.x;; item += gridDim.x) {
-        __syncthreads();
-        if (item >= total || bars->abort_flag) break;   // (the flag is only set between two barriers: same answer in every thread)
-        const int t = (int)(item / ((int64_t)a.heads * a.n_items));
-        const int64_t rem = item - (int64_t)t * a.heads * a.n_items;
-        const int h = (int)(rem / a.n_items);
-        const BigItem it = a.items[rem - (int64_t)h * a.n_items];
-        const BlockInfo bi = a.blocks[it.block];
-        const int n = bi.n, r = t == 0 ? bi.r_q : bi.r_k, nd = t == 0 ? bi.nd_q : bi.nd_k;
-        if (r == 0) continue;   // nothing merges in this block (uniform)
-        const int n_chunks = (nd + kChunkDst - 1) / kChunkDst;
-        const int n_st = min(kSrcTilesPerItem, (n - it.row0 + TILE - 1) / TILE);  // token tiles of this slice
-        const int64_t head_row0 = (int64_t)h * a.n_tokens + bi.start;             // row of the block's first token in [H][N]
-
-        for (int chunk = 0; chunk < n_chunks; ++chunk) {
-            const int d_lo = chunk * kChunkDst, d_cnt = min(kChunkDst, nd - d_lo);   // this chunk's dst tokens
-            if (chunk > 0) {
-                __syncthreads();   // every role is done with the previous chunk's planes
-                if (bars->abort_flag) break;   // (uniform, as above)
-            }
-            // ---- dst tokens of the chunk, scaled and split, -> three resident planes (128-byte swizzle, as a tiled bulk
-            //      copy would leave them)
-            {
-                const __nv_bfloat16* x = a.xr[t] + head_row0 * kHeadDim;
-                const float* inv = a.inv_norm[t] + head_row0;
-                const int c16 = tid & 7;
-                constexpr int kRowsPerPass = SC_THREADS / 8, kPasses = (kChunkDst + kRowsPerPass - 1) / kRowsPerPass;
-                uint4 v[kPasses];   // all of this thread's loads are issued before the first is used
-                float w[kPasses];
-#pragma unroll
-                for (int u = 0; u < kPasses; ++u) {
-                    const int dl = (tid >> 3) + u * kRowsPerPass;
-                    v[u] = make_uint4(0u, 0u, 0u, 0u);
-                    w[u] = 0.f;
-                    if (dl < d_cnt) {
-                        const int pos = dst_position(d_lo + dl, bi.n_rule, nd);
-                        v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)pos * kHeadDim) + c16);
-                        w[u] = ld_global(inv + pos);
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < kPasses; ++u) {
-                    const int dl = (tid >> 3) + u * kRowsPerPass;
-                    if (dl >= kChunkDst) continue;
-                    // rows past the last dst token come out as zeros (x = 0, w = 0); their columns are masked below
-                    const uint32_t in[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-                    uint32_t o0[4], o1[4], o2[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        uint32_t b0[2], b1[2], b2[2];
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const float xv = __uint_as_float(e == 0 ? in[q] << 16 : in[q] & 0xffff0000u);
-                            const float p = xv * w[u];                                // one rounding to fp32 (24 bits)
-                            b0[e] = bf16_bits_rn(p);
-                            const float r1 = p - __uint_as_float(b0[e] << 16);        // exact
-                            b1[e] = bf16_bits_rn(r1);
-                            const float r2 = r1 - __uint_as_float(b1[e] << 16);       // exact, at most 8 significant bits
-                            b2[e] = bf16_bits_rn(r2);
-                        }
-                        o0[q] = b0[0] | (b0[1] << 16);
-                        o1[q] = b1[0] | (b1[1] << 16);
-                        o2[q] = b2[0] | (b2[1] << 16);
-                    }
-                    unsigned char* dst = smem + dl * kRowBytes + ((c16 ^ (dl & 7)) << 4);
-                    *reinterpret_cast<uint4*>(dst) = make_uint4(o0[0], o0[1], o0[2], o0[3]);
-                    *reinterpret_cast<uint4*>(dst + kPlaneBytes) = make_uint4(o1[0], o1[1], o1[2], o1[3]);
-                    *reinterpret_cast<uint4*>(dst + 2 * kPlaneBytes) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor cores read the planes through the async proxy
-            }
+    // Items come in the order of their work, the tensor with more dst tokens first; a CTA takes the next one that nobody has taken.
+    const int per_tensor = a.heads * a.n_blocks;
+    const int t_first = a.blocks[a.order[0]].nd_k >= a.blocks[a.order[0]].nd_q ? 1 : 0;
+    struct Item {
+        BlockInfo bi;
+        int t, h, nd;
+        int n_chunks, n_st, n_pairs;   // chunks of dst tokens, token tiles and pairs of them (none where nothing merges in this block)
+        int64_t row0;                  // row of the block's first token in [H][N]
+    };
+    auto item_of = [&](int item) {
+        Item it;
+        it.t = item < per_tensor ? t_first : 1 - t_first;
+        const int rem = item < per_tensor ? item : item - per_tensor;
+        it.bi = a.blocks[a.order[rem / a.heads]];
+        it.h = rem % a.heads;
+        it.nd = it.t == 0 ? it.bi.nd_q : it.bi.nd_k;
+        const bool merges = (it.t == 0 ? it.bi.r_q : it.bi.r_k) > 0;
+        it.n_chunks = merges ? (it.nd + TILE - 1) / TILE : 0;
+        it.n_st = merges ? (it.bi.n + TILE - 1) / TILE : 0;
+        it.n_pairs = (it.n_st + 1) / 2;
+        it.row0 = (int64_t)it.h * a.n_tokens + it.bi.start;
+        return it;
+    };
+    // Every role goes through the same items and meets the others twice in each: behind the gather of the dst tokens and at the end.
+    if (warp < 4) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kScoreRoleRegs));
+        uint32_t tiles_done = 0;                 // token tiles so far: tile k uses ring stage k % SC_STAGES
+        uint32_t steps_done[SC_GROUPS] = {};     // (pair of tiles, chunk) of either group so far: its score buffers' phases
+        for (int item = blockIdx.x; item < 2 * per_tensor; item = bars->next) {
+            int next = 0;
+            if (tid == 0) next = (int)gridDim.x + atomicAdd(a.counter, 1);
+            const Item it = item_of(item);
             __syncthreads();
-
             if (warp == 0) {
-                // -------------------------------------------------------------- producer: the token tiles of the slice, once per chunk
+                // ---------------------------------------------------------- producer: the token tiles of the block
                 if (tc::elect_one()) {
-                    for (int i = 0; i < n_st; ++i) {
-                        const uint32_t k = n_tiles_done + i, st = k % SC_STAGES, ph = (k / SC_STAGES) & 1u;
+                    for (int i = 0; i < it.n_st; ++i) {
+                        const uint32_t k = tiles_done + i, st = k % SC_STAGES, ph = (k / SC_STAGES) & 1u;
                         if (!tc::mbar_wait(tc::smem_addr(&bars->a_empty[st]), ph ^ 1u, abort_flag)) break;
                         const uint32_t bar = tc::smem_addr(&bars->a_full[st]);
                         tc::mbar_expect_tx(bar, TILE_BYTES);
                         // rows past the block's end belong to the next block (finite, results dropped) or are zero filled past N
-                        tc::tma_load_3d(s_a + st * TILE_BYTES, t == 0 ? &map_q : &map_k, bar, 0, bi.start + it.row0 + i * TILE, h);
+                        tc::tma_load_3d(s_a + st * TILE_BYTES, it.t == 0 ? &map_q : &map_k, bar, 0, it.bi.start + i * TILE, it.h);
                     }
                 }
                 __syncwarp();
+                if (tid == 0) bars->next = next;
             } else if (warp == 1) {
-                // -------------------------------------------------------------- issuer: S = X_tile . (hi + mid + lo)^T
+                // ---------------------------------------------------------- issuer: S = X_tile . D_chunk^T for both tiles of a pair, pairs
+                // p and p + 1 chunk by chunk in turn
                 if (tc::elect_one()) {
+                    constexpr uint32_t idesc = tc::idesc_bf16(128, TILE, false, false);
+                    constexpr uint64_t kTileStep = TILE_BYTES >> 4;   // descriptor address fields count 16-byte units
                     const uint64_t da0 = tc::smem_desc_sw128(s_a), db0 = tc::smem_desc_sw128(s_b);
                     bool ok = true;
-                    for (int i = 0; ok && i < n_st; ++i) {
-                        const uint32_t k = n_tiles_done + i, st = k % SC_STAGES, b = k & 1u;
-                        ok = tc::mbar_wait(tc::smem_addr(&bars->a_full[st]), (k / SC_STAGES) & 1u, abort_flag) &&
-                             tc::mbar_wait(tc::smem_addr(&bars->s_empty[b]), ((k >> 1) & 1u) ^ 1u, abort_flag);
-                        if (!ok) break;
-                        tc::fence_after_sync();
-                        const uint64_t da = da0 + (uint64_t)st * kTileStep;
+                    for (int p = 0; ok && p < it.n_pairs; p += SC_GROUPS) {
+                        const uint32_t k0 = tiles_done + 2 * p;
+                        const int tiles = min(2 * SC_GROUPS, it.n_st - 2 * p);
+                        for (int chunk = 0; ok && chunk < it.n_chunks; ++chunk) {
 #pragma unroll
-                        for (int pl = 0; pl < 3; ++pl)
-#pragma unroll
-                            for (int ks = 0; ks < 4; ++ks)   // K = 16 steps over the 64 channels: 32 bytes = 2 descriptor units
-                                tc::mma_ss(tmem + b * kChunkDst, da + 2 * ks, db0 + (uint64_t)pl * kPlaneStep + 2 * ks, idesc, (pl | ks) ? 1u : 0u);
-                        tc::mma_commit(tc::smem_addr(&bars->a_empty[st]));   // the tile may be refilled when these MMAs are done
-                        tc::mma_commit(tc::smem_addr(&bars->s_full[b]));
+                            for (int g = 0; g < SC_GROUPS; ++g) {
+                                if (2 * g >= tiles) break;
+                                for (int e = 2 * g; ok && chunk == 0 && e < 2 * g + 2 && e < tiles; ++e)
+                                    ok = tc::mbar_wait(tc::smem_addr(&bars->a_full[(k0 + e) % SC_STAGES]), ((k0 + e) / SC_STAGES) & 1u, abort_flag);
+                                if (!ok || !(ok = tc::mbar_wait(tc::smem_addr(&bars->s_empty[g]), (steps_done[g] & 1u) ^ 1u, abort_flag))) break;
+                                tc::fence_after_sync();
+                                const uint64_t db = db0 + (uint64_t)chunk * kTileStep;
+                                for (int e = 0; e < 2 && 2 * g + e < tiles; ++e) {
+                                    const uint64_t da = da0 + (uint64_t)((k0 + 2 * g + e) % SC_STAGES) * kTileStep;
+                                    const uint32_t t_s = tmem + (2 * g + e) * TILE;
+                                    tc::mma_ss_c<false>(t_s, da, db, idesc);   // K = 16 steps over the 64 channels: 32 bytes = 2 descriptor units
+                                    tc::mma_ss_c<true>(t_s, da + 2, db + 2, idesc);
+                                    tc::mma_ss_c<true>(t_s, da + 4, db + 4, idesc);
+                                    tc::mma_ss_c<true>(t_s, da + 6, db + 6, idesc);
+                                }
+                                tc::mma_commit(tc::smem_addr(&bars->s_full[g]));
+                                ++steps_done[g];
+                            }
+                        }
+                        for (int e = 0; ok && e < tiles; ++e) tc::mma_commit(tc::smem_addr(&bars->a_empty[(k0 + e) % SC_STAGES]));
                     }
                 }
                 __syncwarp();
-            } else {
-                // -------------------------------------------------------------- arg-max over the chunk's dst tokens, one thread per
-                // token and column half; the scores arrive scaled
-                const int half = (warp - 2) >> 2;
-                const int row = (warp & 3) * 32 + lane;            // row of the token tile = lane of tensor memory
-                const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-                const bool last_chunk = chunk == n_chunks - 1;
-                bool ok = true;
-                for (int i = 0; ok && i < n_st; ++i) {
-                    const uint32_t k = n_tiles_done + i, b = k & 1u;
-                    const int mine = half * kBigSliceRows + i * TILE + row;
-                    float best = -INFINITY;
-                    int arg = 0;
-                    if (chunk > 0) {
-                        best = best_s[mine];
-                        arg = arg_s[mine];
+            }
+            tiles_done += it.n_st;
+            __syncthreads();
+            if (*abort_flag) break;   // (the flag is only set between two barriers: same answer in every thread)
+        }
+    } else {
+        // -------------------------------------------------------------- arg-max over the chunk's dst tokens, one thread per token of either tile of a
+        // pair and column half
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kScoreMaxRegs));
+        const int g = (warp - 4) >> 3, half = ((warp - 4) >> 2) & 1;
+        const int row = (warp & 3) * 32 + lane;            // row of the token tile = lane of tensor memory
+        const uint32_t t_s = tmem + g * 2 * TILE + half * 64 + ((uint32_t)((warp & 3) * 32) << 16);
+        uint32_t steps_done = 0, pairs_done = 0;           // of this group, all items
+        for (int item = blockIdx.x; item < 2 * per_tensor; item = bars->next) {
+            const Item it = item_of(item);
+            const int nd = it.nd, n = it.bi.n;
+            const __nv_bfloat16* x = a.xr[it.t] + it.row0 * kHeadDim;
+            const float* inv = a.inv_norm[it.t] + it.row0;
+            // ---- the dst tokens, scaled by a power of two to norms in [1, 2) (no product with them overflows where the cosine would not), in
+            //      the image a tiled copy with the 128-byte swizzle would leave, and what is left of their weights
+            {
+                const int at = tid - 128, c16 = at & 7;
+                constexpr int kRowsPerPass = (SC_THREADS - 128) / 8, kBatch = 8;
+                for (int d0 = at >> 3; d0 < it.n_chunks * TILE; d0 += kBatch * kRowsPerPass) {
+                    uint4 v[kBatch];   // all of a batch's loads are issued before the first is used
+                    float w[kBatch];
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        const int d = d0 + u * kRowsPerPass;
+                        v[u] = make_uint4(0u, 0u, 0u, 0u);
+                        w[u] = 0.f;
+                        if (d < nd) {
+                            const int pos = dst_position(d, it.bi.n_rule, nd);
+                            v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)pos * kHeadDim) + c16);
+                            w[u] = ld_global(inv + pos);
+                        }
                     }
-                    ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->s_full[b]), (k >> 1) & 1u, abort_flag));   // (a warp gives up together)
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        const int d = d0 + u * kRowsPerPass;
+                        if (d >= it.n_chunks * TILE) break;   // (rows past the last dst token are zeros; their columns are masked below)
+                        const float scale = __uint_as_float(__float_as_uint(w[u]) & 0x7f800000u);   // 2^floor(log2 w); 0 for w = 0
+                        const uint4 o = make_uint4(scale_bf16x2(v[u].x, scale), scale_bf16x2(v[u].y, scale), scale_bf16x2(v[u].z, scale),
+                                                   scale_bf16x2(v[u].w, scale));
+                        *reinterpret_cast<uint4*>(smem + d * kRowBytes + ((c16 ^ (d & 7)) << 4)) = o;
+                        if (c16 == 0) w_s[d] = __uint_as_float((__float_as_uint(w[u]) & 0x007fffffu) | 0x3f800000u);
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor cores read the rows through the async proxy
+            }
+            __syncthreads();
+            bool ok = true;
+            for (int p = g; ok && p < it.n_pairs; p += SC_GROUPS) {
+                Best best[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    best[e].score = -INFINITY;
+                    best[e].first_dst = -1.f;
+#pragma unroll
+                    for (int c = 0; c < kGroup / 2; ++c) best[e].v[c] = make_float2(0.f, 0.f);
+                }
+                for (int chunk = 0; chunk < it.n_chunks; ++chunk, ++steps_done) {
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->s_full[g]), steps_done & 1u, abort_flag));   // (a warp gives up together)
                     if (!ok) break;
                     tc::fence_after_sync();
 #pragma unroll
                     for (int part = 0; part < 2; ++part) {
-                        uint32_t raw[64];
-                        const uint32_t taddr = tmem + b * kChunkDst + half * TILE + part * 64 + lane_addr;
-                        tc::tmem_ld32(taddr, raw);
-                        tc::tmem_ld32(taddr + 32, raw + 32);
+                        uint32_t raw[2][32];
+                        tc::tmem_ld32(t_s + part * 32, raw[0]);
+                        tc::tmem_ld32(t_s + TILE + part * 32, raw[1]);   // (behind the block's last tile: old scores, results dropped)
                         tc::tmem_wait_ld();
-                        if (part == 1) {   // both parts are in registers: the buffer can take the next scores
+                        if (part == 1) {
                             tc::fence_before_sync();
-                            tc::mbar_arrive(tc::smem_addr(&bars->s_empty[b]));
+                            tc::mbar_arrive(tc::smem_addr(&bars->s_empty[g]));   // the scores are in registers
                         }
-                        const int c0 = half * TILE + part * 64;   // first column of these 64 inside the chunk
-                        if (c0 < d_cnt) {                         // (uniform in the warp)
-                            if (c0 + 64 > d_cnt) {                // the block's last dst tokens: mask the columns behind them
+                        const int first_dst = chunk * TILE + half * 64 + part * 32;
+                        if (first_dst >= nd) continue;                       // (uniform in the warp)
+                        const float4* w4 = reinterpret_cast<const float4*>(w_s + first_dst);
+                        float s[2][32];
 #pragma unroll
-                                for (int c = 0; c < 64; ++c)
-                                    if (c0 + c >= d_cnt) raw[c] = 0xff800000u;   // -inf
-                            }
-                            // maxima of the four groups of 16 columns (independent chains), then of the part
-                            float g0 = -INFINITY, g1 = -INFINITY, g2 = -INFINITY, g3 = -INFINITY;
+                        for (int c = 0; c < 32; c += 4) {
+                            const float4 w = w4[c >> 2];
 #pragma unroll
-                            for (int c = 0; c < 16; c += 2) {
-                                g0 = tc::fmax3(g0, __uint_as_float(raw[c]), __uint_as_float(raw[c + 1]));
-                                g1 = tc::fmax3(g1, __uint_as_float(raw[16 + c]), __uint_as_float(raw[17 + c]));
-                                g2 = tc::fmax3(g2, __uint_as_float(raw[32 + c]), __uint_as_float(raw[33 + c]));
-                                g3 = tc::fmax3(g3, __uint_as_float(raw[48 + c]), __uint_as_float(raw[49 + c]));
-                            }
-                            const float m = fmaxf(tc::fmax3(g0, g1, g2), g3);
-                            if (m > best) {   // find the first column holding the maximum (ties: lowest dst): first group, then
-                                best = m;     // the first of its 16 columns (the search runs whenever any row of the warp improves)
-                                const bool in0 = g0 == m, in1 = g1 == m, in2 = g2 == m;
-                                const int group = in0 ? 0 : (in1 ? 1 : (in2 ? 2 : 3));
-                                int first = 15;
-#pragma unroll
-                                for (int c = 14; c >= 0; --c) {
-                                    const uint32_t v = in0 ? raw[c] : (in1 ? raw[16 + c] : (in2 ? raw[32 + c] : raw[48 + c]));
-                                    if (__uint_as_float(v) == m) first = c;
-                                }
-                                arg = d_lo + c0 + 16 * group + first;
+                            for (int e = 0; e < 2; ++e) {
+                                const float2 lo = tc::fmul2(make_float2(__uint_as_float(raw[e][c]), __uint_as_float(raw[e][c + 1])), make_float2(w.x, w.y));
+                                const float2 hi = tc::fmul2(make_float2(__uint_as_float(raw[e][c + 2]), __uint_as_float(raw[e][c + 3])), make_float2(w.z, w.w));
+                                s[e][c] = lo.x;
+                                s[e][c + 1] = lo.y;
+                                s[e][c + 2] = hi.x;
+                                s[e][c + 3] = hi.y;
                             }
                         }
+                        take_best(best[0], s[0], first_dst, nd - first_dst);
+                        take_best(best[1], s[1], first_dst, nd - first_dst);
                     }
-                    if (!last_chunk) {
-                        best_s[mine] = best;
-                        arg_s[mine] = (uint16_t)arg;
-                        continue;
-                    }
-                    // the two column halves of a token meet: half 1 hands (best, arg) over, half 0 decides (ties: lowest dst)
-                    const int slot = i & 1;
-                    if (half == 1) {
-                        ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->x_done[slot]), (n_x[slot] & 1u) ^ 1u, abort_flag));
-                        if (!ok) break;
-                        xch[slot * TILE + row] = make_float2(best, __int_as_float(arg));
-                        tc::mbar_arrive(tc::smem_addr(&bars->x_full[slot]));
-                    } else {
-                        ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->x_full[slot]), n_x[slot] & 1u, abort_flag));
-                        if (!ok) break;
-                        const float2 o = xch[slot * TILE + row];
-                        tc::mbar_arrive(tc::smem_addr(&bars->x_done[slot]));
-                        const int oarg = __float_as_int(o.y);
-                        if (o.x > best || (o.x == best && oarg < arg)) {
-                            best = o.x;
-                            arg = oarg;
+                }
+                if (!ok) break;
+                int arg[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    int in_group = kGroup;
+#pragma unroll
+                    for (int c = kGroup - 1; c >= 0; --c)
+                        if ((c & 1 ? best[e].v[c >> 1].y : best[e].v[c >> 1].x) == best[e].score) in_group = c;
+                    const int i = (2 * p + e) * TILE + row;   // token number inside the block
+                    if (best[e].first_dst < 0.f)
+                        arg[e] = 0;   // (no score is a number)
+                    else if (in_group < kGroup)
+                        arg[e] = (int)best[e].first_dst + in_group;
+                    else
+                        arg[e] = i < n ? find_again(x + (int64_t)i * kHeadDim, smem, w_s, half, nd) : 0;
+                }
+                // the two column halves of a token meet: half 1 hands (best, arg) over, half 0 decides (ties: lowest dst)
+                const uint32_t turn = pairs_done++ & 1u;
+                float2* mine = xch + g * 2 * TILE + row;
+                if (half == 1) {
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->x_done[g]), turn ^ 1u, abort_flag));
+                    if (!ok) break;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) mine[e * TILE] = make_float2(best[e].score, __int_as_float(arg[e]));
+                    tc::mbar_arrive(tc::smem_addr(&bars->x_full[g]));
+                } else {
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->x_full[g]), turn, abort_flag));
+                    if (!ok) break;
+                    float2 o[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) o[e] = mine[e * TILE];
+                    tc::mbar_arrive(tc::smem_addr(&bars->x_done[g]));
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        float score = best[e].score;
+                        const int oarg = __float_as_int(o[e].y);
+                        if (o[e].x > score || (o[e].x == score && oarg < arg[e])) {
+                            score = o[e].x;
+                            arg[e] = oarg;
                         }
-                        const int p = it.row0 + i * TILE + row;   // token number inside the block
-                        if (p < n) {
-                            const float w = ld_global(a.inv_norm[t] + head_row0 + p);
-                            a.best_key[t][head_row0 + p] = score_key(best * w);
-                            a.best_pos[t][head_row0 + p] = dst_position(arg, bi.n_rule, nd);
+                        const int i = (2 * p + e) * TILE + row;
+                        if (i < n) {
+                            const float w = ld_global(inv + i);
+                            a.best_key[it.t][it.row0 + i] = score_key(score * w);
+                            a.best_pos[it.t][it.row0 + i] = dst_position(arg[e], it.bi.n_rule, nd);
                         }
                     }
-                    ++n_x[slot];
                 }
             }
-            n_tiles_done += n_st;   // (every thread keeps the count, whatever its role)
+            __syncthreads();
+            if (*abort_flag) break;   // (as above)
         }
     }
     tc::fence_before_sync();
@@ -923,7 +1023,7 @@ cudaError_t launch_big_scores(const BigMatchArgs& a, int sm_count, cudaStream_t 
     if (!encode_rows_tensor_map(&mq, a.xr[0], a.n_tokens, a.heads, kHeadDim, (int64_t)a.n_tokens * kHeadDim, TILE) ||
         !encode_rows_tensor_map(&mk, a.xr[1], a.n_tokens, a.heads, kHeadDim, (int64_t)a.n_tokens * kHeadDim, TILE))
         return cudaErrorInvalidValue;
-    const int64_t total = 2ll * a.heads * a.n_items;
+    const int64_t total = 2ll * a.heads * a.n_blocks;
     int ctas = sm_count < 1 ? 1 : sm_count;
     if (ctas > total) ctas = (int)total;
     if (ctas < 1) ctas = 1;

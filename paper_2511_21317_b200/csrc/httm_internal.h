@@ -12,7 +12,6 @@ constexpr int kRowBytes = kHeadDim * 2;  // one token of one head, bf16
 constexpr int kMaxBlockTokens = 256;  // largest merging block that a warp or a team of warps holds on chip (match / merge)
 constexpr int kMaxBigBlockTokens = 4096;   // largest merging block of the large-block path (Sec. 4.1: 128 tokens x 30 frames = 3840)
 constexpr int kMaxBigDst = 1024;           // its dst tokens (a quarter of the block) stay in shared memory
-constexpr int kBigSliceRows = 4096;        // rows of a block one work item of the score kernel handles (the whole block)
 
 // Device status word values (first error wins).
 enum : int {
@@ -73,9 +72,6 @@ struct ReorderArgs {
 };
 
 // Large-block path (blocks of 257 .. 4096 tokens; Sec. 4.1's 128 x 30 regime): matching as a dense contraction.
-struct BigItem {
-    int32_t block, row0;     // rows [row0, row0 + kBigSliceRows) of this block
-};
 struct BigMatchArgs {
     const __nv_bfloat16* xr[2];   // reordered Q, K [H][N][64]
     const float* inv_norm[2];     // [H][N]
@@ -83,8 +79,9 @@ struct BigMatchArgs {
     int32_t* best_pos[2];         // [H][N] token number, inside the block, of that dst
     int32_t* assign[2];           // [H][N] out (select kernel)
     const BlockInfo* blocks;
-    const BigItem* items;         // the slices of all blocks (the same list for every tensor and head)
-    int32_t n_items, n_blocks, n_tokens, heads;
+    const int32_t* order;         // [blocks] from the longest to the shortest
+    int32_t* counter;             // work items of the score kernel taken behind the first of every CTA; zero before the launch
+    int32_t n_blocks, n_tokens, heads;
     int32_t* status;
 };
 

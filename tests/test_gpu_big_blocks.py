@@ -108,6 +108,45 @@ def test_block_sizes_at_the_cta_size_limits(n):
         run_filtered(wl, 0.1, peaky=True, launches=12)
 
 
+@pytest.mark.parametrize("n", [257, 260, 508, 516, 1028, 3844, 4096])
+def test_dst_tokens_at_the_chunk_limits(n):
+    """One block of n tokens per head, a quarter of them dst tokens: 65, 127 and 129 of them (chunks of 128, halves of 64, parts of 32),
+    257, 961 and 1024; even and odd numbers of token tiles, the last with one row or full."""
+    wl = synth.Workload(f"dst_limit_{n}", 1, 1, n, 1, 1, n, 0.7, 0.5, n_camera=0, n_register=1, heads=3, seed=n)
+    run_big(wl, peaky=True)
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan"), 2.0 ** 70], ids=["infinite", "not_a_number", "overflow"])
+def test_a_dst_token_without_a_similarity_is_nobodys_best(bad):
+    """Dst tokens that are infinite, not numbers or of a squared norm beyond fp32: the other tokens go to the best of the other dst tokens (all
+    similarities of this scene are positive), to within the rounding of the similarities (1e-5)."""
+    n, heads = 1100, 2
+    wl = synth.Workload("spoilt", 1, 1, n, 1, 1, n, 0.75, 0.75, n_camera=0, n_register=0, heads=heads, seed=3)
+    gen = np.random.default_rng(7)
+    x = (0.25 + gen.random((heads, n, 64))).astype(np.float32)
+    nd = n // 4
+    dst = np.arange(3, n, 4)
+    spoilt = dst[[0, 31, 32, 100, 274]]
+    x[:, spoilt] *= bad
+    t = torch.from_numpy(x).bfloat16().to(DEV)
+    good = torch.from_numpy((0.25 + gen.random(x.shape)).astype(np.float32)).bfloat16().to(DEV)
+    with hb.Httm(hb.HttmConfig.of(wl)) as ctx:
+        ctx.global_attention(t, t, good)
+        torch.cuda.synchronize()
+        assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+        maps = ctx.export(hb.X_ASSIGN_Q), ctx.export(hb.X_ASSIGN_K)
+    rows = t.double().cpu().numpy()
+    src, fine = np.setdiff1d(np.arange(n), dst), np.setdiff1d(dst, spoilt)
+    assert len(src) == int(0.75 * n) and len(dst) == nd
+    for h in range(heads):
+        unit = rows[h] / np.linalg.norm(rows[h], axis=1, keepdims=True)
+        sim = unit[src] @ unit[fine].T
+        for m in maps:
+            assert np.isin(m[h][src], fine).all() and (m[h][dst] == dst).all()
+            mine = (unit[src] * unit[m[h][src]]).sum(1)
+            assert (sim.max(1) - mine <= 1e-5).all(), (h, (sim.max(1) - mine).max())
+
+
 def test_sums_of_many_members_with_one_far_larger_member():
     """2 048 tokens in one block, multiples of one vector (every cosine a tie: nearly all of them merge into the first dst token), one of
     them 2^17 times the others.  In fp32 every small member added to a running sum of that size is rounded in the same direction, so a
