@@ -40,20 +40,23 @@ __device__ __forceinline__ bool is_dst_position(int j, int n_rule, int nd) {
 //  - a warp works on TWO token tiles at a time: the data of a broadcast load of weights goes to every lane, four cycles of the SM's
 //    shared-memory port for four columns, and is used twice this way;
 //  - two groups of eight warps, each with a score buffer for a pair of tiles and 128 dst tokens (one group: 515 us);
+//  - only the src tokens are rows of the contraction (a quarter of the keys are dst tokens), loaded by two warps with cp.async, the first tiles
+//    beside the dst tokens;
 //  - work items (tensor, head, block) are taken from a counter, the longest first (dealt in rounds one tensor after the other, the longest of
-//    148 CTAs had 15 % more than the mean).
+//    148 CTAs had 15 % more than the mean), and an issuing warp for each group (one for both kept them in step: 437 us).
+// The four warps of the roles run with 32 registers: nothing they run may be a function of its own, which would not know of that.
 // Measured at 16 heads x 22 blocks of up to 3840 tokens, 384 dst tokens of the queries and 960 of the keys: 611 us with the dst tokens split into three
-// scaled planes, 256 at a time, and one group of warps; 467 us now.  The dst tokens chosen are closer to the best in 64 bits
-// (1.6 million tokens of three scenes: 26 off the best by up to 4.6e-7 before, 6 by up to 1.2e-7).  Tried and dropped: an issuing warp for each
-// group (477 us), a longer ring of token tiles (487 us), 16 loads of a dst gather in flight (476 us), no carrying along where no row of the warp
-// improves (491 us).
+// scaled planes, 256 at a time, and one group of warps; 467 us with all tokens as rows; 426 us now.  The dst tokens chosen are closer to the best in 64 bits
+// (1.6 million tokens of three scenes: 26 off the best by up to 4.6e-7 before, 6 by up to 1.2e-7).  Tried and dropped: 64 and 104 registers (456 us),
+// no carrying along where no row of the warp improves (491 us at 467).
 constexpr int TILE = 128;                        // rows of an operand tile, dst tokens of a chunk
 constexpr int TILE_BYTES = TILE * kRowBytes;     // 16 KB
 constexpr int SC_GROUPS = 2;                     // groups of arg-max warps (two column halves x four lane quadrants each)
-constexpr int SC_THREADS = 128 + SC_GROUPS * 256;   // warp 0: TMA producer, warp 1: MMA issuer (2 and 3 only make up the four), then the arg-max warps
+constexpr int SC_THREADS = 128 + SC_GROUPS * 256;   // warps 0 and 1: MMA issuers of the groups, warps 2 and 3: loads of the token tiles and next work item, then the arg-max warps
+constexpr int SC_LOADERS = 64;
 constexpr int kScoreRoleRegs = 32, kScoreMaxRegs = 112;   // of the 5 x 96 the kernel starts with
 constexpr int SC_TMEM_COLS = 512;                // a buffer pair of 2 x 128 columns (by tile of the pair) for each group
-constexpr int SC_STAGES = 4;                     // ring of token tiles: a pair for each group
+constexpr int SC_STAGES = 10;                    // ring of token tiles behind the dst tokens: as many as there is room for, at least five
 
 struct ScoreBars {
     uint64_t a_full[SC_STAGES], a_empty[SC_STAGES];   // ring of token tiles
@@ -61,20 +64,72 @@ struct ScoreBars {
     uint64_t x_full[SC_GROUPS], x_done[SC_GROUPS];    // exchange of the two column halves' results
     uint32_t tmem_base;
     int abort_flag;
-    int next;                         // the CTA's next work item
 };
-constexpr int SC_OFF_A = kMaxBigDst * kRowBytes;                 // token tiles behind the dst tokens
-constexpr int SC_OFF_W = SC_OFF_A + SC_STAGES * TILE_BYTES;      // float [dst]: the weights of the dst tokens
+struct ScoreItem {
+    int t;                            // tensor (0: Q, 1: K); -1: no more items
+    int n_rule, even;                 // the block's dst rule; evenly spaced
+    int nd, n_src;                    // dst and src tokens
+    int n_chunks, n_st, n_pairs;      // chunks of dst tokens, tiles of src tokens and pairs of them (none where nothing merges in this block)
+    int stages, ring;                 // stages of the ring of token tiles and where it begins
+    int64_t row0;                     // row of the block's first token in [H][N]
+};
+constexpr int SC_AREA = kMaxBigDst * kRowBytes + 5 * TILE_BYTES + 8192;    // dst tokens and ring: 960 dst tokens leave six stages
+constexpr int SC_OFF_W = SC_AREA;                                // float [dst]: the weights of the dst tokens
 constexpr int SC_OFF_XCH = SC_OFF_W + kMaxBigDst * 4;            // [groups][2][128] (best, arg) of column half 1
 constexpr int SC_OFF_BARS = SC_OFF_XCH + 2 * 2 * TILE * 8;
-constexpr int SC_SMEM = SC_OFF_BARS + 256 + 1024 /*alignment slack*/;
-static_assert(sizeof(ScoreBars) <= 256 && kMaxBigDst % TILE == 0 && SC_SMEM <= 232448, "");
+constexpr int SC_OFF_ITEMS = SC_OFF_BARS + 384;                  // ScoreItem [2]: this one and the next
+constexpr int SC_SMEM = SC_OFF_ITEMS + 2 * 64 + 1024 /*alignment slack*/;
+static_assert(sizeof(ScoreBars) <= 384 && sizeof(ScoreItem) <= 64 && kMaxBigDst % TILE == 0 && SC_AREA % 1024 == 0 && SC_SMEM <= 232448, "");
 
+__device__ __forceinline__ void write_item(ScoreItem* to, const BigMatchArgs& a, int t_first, int item) {
+    const int per_tensor = a.heads * a.n_blocks;
+    if (item >= 2 * per_tensor) {
+        to->t = -1;
+        return;
+    }
+    const int t = item < per_tensor ? t_first : 1 - t_first, rem = item < per_tensor ? item : item - per_tensor;
+    const BlockInfo bi = a.blocks[a.order[rem / a.heads]];
+    const int nd = t == 0 ? bi.nd_q : bi.nd_k, n_src = bi.n - nd;
+    const bool merges = (t == 0 ? bi.r_q : bi.r_k) > 0;
+    const int n_st = merges ? (n_src + TILE - 1) / TILE : 0, ring = (nd + 7) / 8 * 8 * kRowBytes;   // (the last chunk's MMAs read into the ring: masked columns)
+    to->t = t;
+    to->n_rule = bi.n_rule;
+    to->nd = nd;
+    to->n_src = n_src;
+    to->even = bi.n_rule == bi.n;
+    to->n_chunks = merges ? (nd + TILE - 1) / TILE : 0;
+    to->n_st = n_st;
+    to->n_pairs = (n_st + 1) / 2;
+    to->ring = ring;
+    to->stages = min(SC_STAGES, (SC_AREA - ring) / TILE_BYTES);
+    to->row0 = (int64_t)(rem % a.heads) * a.n_tokens + bi.start;
+}
 // x s for two bf16 values packed in a word, s a power of two: exact (but for values that leave the format)
 __device__ __forceinline__ uint32_t scale_bf16x2(uint32_t v, float s) {
     const __nv_bfloat162 r = __floats2bfloat162_rn(__uint_as_float(v << 16) * s, __uint_as_float(v & 0xffff0000u) * s);
     return *reinterpret_cast<const uint32_t*>(&r);
 }
+__device__ __forceinline__ void load_async(uint32_t dst, const void* src) {   // 16 bytes
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// floor(x / den), floor((x + step) / den), ..
+struct Ramp {
+    int value, rest, den, step_value, step_rest;
+    __device__ __forceinline__ Ramp(int x, int step, int den_) : den(den_) {
+        value = x / den;
+        rest = x - value * den;
+        step_value = step / den;
+        step_rest = step - step_value * den;
+    }
+    __device__ __forceinline__ void next() {
+        value += step_value;
+        rest += step_rest;
+        if (rest >= den) {
+            rest -= den;
+            ++value;
+        }
+    }
+};
 
 // A token's best dst so far: its score, the first dst of the group of eight that holds it, and the scores of that group, which tell the
 // dst itself once at the end.  The eight scores are carried along by multiplying with zeros and ones on the FMA pipe, which has time:
@@ -149,10 +204,10 @@ __device__ __noinline__ int find_again(const __nv_bfloat16* x, const unsigned ch
 }
 
 __global__ void __launch_bounds__(SC_THREADS, 1)
-big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const BigMatchArgs a) {
+big_scores_kernel(const BigMatchArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const uint32_t s_b = tc::smem_addr(smem), s_a = s_b + SC_OFF_A;
+    const uint32_t s_b = tc::smem_addr(smem);   // dst tokens, behind them the ring of token tiles
     float* w_s = reinterpret_cast<float*>(smem + SC_OFF_W);
     float2* xch = reinterpret_cast<float2*>(smem + SC_OFF_XCH);
     ScoreBars* bars = reinterpret_cast<ScoreBars*>(smem + SC_OFF_BARS);
@@ -162,7 +217,7 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     if (tid == 0) {
         bars->abort_flag = 0;
         for (int i = 0; i < SC_STAGES; ++i) {
-            tc::mbar_init(tc::smem_addr(&bars->a_full[i]), 1);
+            tc::mbar_init(tc::smem_addr(&bars->a_full[i]), SC_LOADERS);
             tc::mbar_init(tc::smem_addr(&bars->a_empty[i]), 1);
         }
         for (int i = 0; i < SC_GROUPS; ++i) {
@@ -172,10 +227,13 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             tc::mbar_init(tc::smem_addr(&bars->x_done[i]), 128);
         }
         tc::fence_barrier_init();
-        tc::prefetch_tensormap(&map_q);
-        tc::prefetch_tensormap(&map_k);
     }
+    // Items come in the order of their work, the tensor with more dst tokens first; a CTA takes the next one that nobody has taken.  Warp 2 reads
+    // what there is to know about it while the others work on the one before (three dependent loads from memory).
+    const int t_first = a.blocks[a.order[0]].nd_k >= a.blocks[a.order[0]].nd_q ? 1 : 0;
+    ScoreItem* items = reinterpret_cast<ScoreItem*>(smem + SC_OFF_ITEMS);
     if (warp == 1) tc::tmem_alloc(tc::smem_addr(&bars->tmem_base), SC_TMEM_COLS);
+    if (tid == 64) write_item(items, a, t_first, blockIdx.x);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -183,91 +241,111 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     depend_wait();
     dependents_launch();
 
-    // Items come in the order of their work, the tensor with more dst tokens first; a CTA takes the next one that nobody has taken.
-    const int per_tensor = a.heads * a.n_blocks;
-    const int t_first = a.blocks[a.order[0]].nd_k >= a.blocks[a.order[0]].nd_q ? 1 : 0;
-    struct Item {
-        BlockInfo bi;
-        int t, h, nd;
-        int n_chunks, n_st, n_pairs;   // chunks of dst tokens, token tiles and pairs of them (none where nothing merges in this block)
-        int64_t row0;                  // row of the block's first token in [H][N]
-    };
-    auto item_of = [&](int item) {
-        Item it;
-        it.t = item < per_tensor ? t_first : 1 - t_first;
-        const int rem = item < per_tensor ? item : item - per_tensor;
-        it.bi = a.blocks[a.order[rem / a.heads]];
-        it.h = rem % a.heads;
-        it.nd = it.t == 0 ? it.bi.nd_q : it.bi.nd_k;
-        const bool merges = (it.t == 0 ? it.bi.r_q : it.bi.r_k) > 0;
-        it.n_chunks = merges ? (it.nd + TILE - 1) / TILE : 0;
-        it.n_st = merges ? (it.bi.n + TILE - 1) / TILE : 0;
-        it.n_pairs = (it.n_st + 1) / 2;
-        it.row0 = (int64_t)it.h * a.n_tokens + it.bi.start;
-        return it;
-    };
     // Every role goes through the same items and meets the others twice in each: behind the gather of the dst tokens and at the end.
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kScoreRoleRegs));
-        uint32_t tiles_done = 0;                 // token tiles so far: tile k uses ring stage k % SC_STAGES
-        uint32_t steps_done[SC_GROUPS] = {};     // (pair of tiles, chunk) of either group so far: its score buffers' phases
-        for (int item = blockIdx.x; item < 2 * per_tensor; item = bars->next) {
-            int next = 0;
-            if (tid == 0) next = (int)gridDim.x + atomicAdd(a.counter, 1);
-            const Item it = item_of(item);
-            __syncthreads();
-            if (warp == 0) {
-                // ---------------------------------------------------------- producer: the token tiles of the block
-                if (tc::elect_one()) {
-                    for (int i = 0; i < it.n_st; ++i) {
-                        const uint32_t k = tiles_done + i, st = k % SC_STAGES, ph = (k / SC_STAGES) & 1u;
-                        if (!tc::mbar_wait(tc::smem_addr(&bars->a_empty[st]), ph ^ 1u, abort_flag)) break;
-                        const uint32_t bar = tc::smem_addr(&bars->a_full[st]);
-                        tc::mbar_expect_tx(bar, TILE_BYTES);
-                        // rows past the block's end belong to the next block (finite, results dropped) or are zero filled past N
-                        tc::tma_load_3d(s_a + st * TILE_BYTES, it.t == 0 ? &map_q : &map_k, bar, 0, it.bi.start + i * TILE, it.h);
+        uint32_t fills = 0;                      // parity (bits) of the fills of every ring stage in the items so far
+        uint32_t steps_done = 0;                 // issuers: (pair of tiles, chunk) so far, the score buffers' phases
+        for (int n_items = 0;; ++n_items) {
+            const ScoreItem it = items[n_items & 1];
+            if (it.t < 0) break;
+            if (warp >= 2) {
+                // ---------------------------------------------------------- loads of the src tokens, 128 to a tile, in the image a tiled copy with
+                // the 128-byte swizzle would leave; a tile is handed over while the next one's loads are in flight, unless those have to wait for
+                // it.  The first tiles are loaded beside the dst tokens.
+                const __nv_bfloat16* x = a.xr[it.t] + it.row0 * kHeadDim;
+                const int at = tid - 64, c16 = at & 7;
+                // src token s is token s + (dst tokens before it): s + floor(s nd / (n - nd)), or s + nd where the first nd tokens are the dst tokens
+                Ramp before((at >> 3) * it.nd, SC_LOADERS / 8 * it.nd, max(it.n_src, 1));
+                int s = at >> 3, handed = 0, hand_st = 0;   // next src token of this thread; tiles handed over, stage of the next
+                uint32_t par = fills;
+                auto hand_over = [&]() {
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor cores read the rows through the async proxy
+                    tc::mbar_arrive(tc::smem_addr(&bars->a_full[hand_st]));
+                    ++handed;
+                    if (++hand_st == it.stages) hand_st = 0;
+                };
+                auto load_tile = [&](int st) {
+                    if (!__all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->a_empty[st]), (par >> st & 1u) ^ 1u, abort_flag))) return false;
+                    par ^= 1u << st;
+                    const uint32_t dst = s_b + it.ring + st * TILE_BYTES;
+#pragma unroll 4
+                    for (int row = at >> 3; row < TILE; row += SC_LOADERS / 8, s += SC_LOADERS / 8, before.next()) {
+                        const int pos = s < it.n_src ? s + (it.even ? before.value : it.nd) : 0;   // (behind the last src token: results dropped)
+                        load_async(dst + row * kRowBytes + ((c16 ^ (row & 7)) << 4), x + (int64_t)pos * kHeadDim + c16 * 8);
+                    }
+                    return true;
+                };
+                const int first = min(it.n_st, 4);
+                bool ok = true;
+                for (int st = 0; ok && st < first; ++st) ok = load_tile(st);
+                if (__syncthreads_or(0)) __syncthreads();
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                while (ok && handed < first) hand_over();
+                if (tid == 64) write_item(items + ((n_items + 1) & 1), a, t_first, (int)gridDim.x + atomicAdd(a.counter, 1));
+                __syncwarp();
+                for (int i = first, st = first; ok && i < it.n_st; ++i, st = st + 1 < it.stages ? st + 1 : 0) {
+                    if (handed < i && !__all_sync(0xffffffffu, tc::mbar_test(tc::smem_addr(&bars->a_empty[st]), (par >> st & 1u) ^ 1u))) {
+                        asm volatile("cp.async.wait_all;" ::: "memory");   // (the stage may be waiting for the tile before)
+                        hand_over();
+                    }
+                    if (!(ok = load_tile(st))) break;
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                    if (handed < i) {
+                        asm volatile("cp.async.wait_group 1;" ::: "memory");
+                        hand_over();
                     }
                 }
-                __syncwarp();
-                if (tid == 0) bars->next = next;
-            } else if (warp == 1) {
-                // ---------------------------------------------------------- issuer: S = X_tile . D_chunk^T for both tiles of a pair, pairs
-                // p and p + 1 chunk by chunk in turn
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                if (ok && handed < it.n_st) hand_over();
+            } else {
+                // ---------------------------------------------------------- issuer of a group: S = X_tile . D_chunk^T for both tiles of its pairs.
+                // (One warp for both groups keeps them in step, and both wait for their scores at the same time.)
+                if (__syncthreads_or(0)) __syncthreads();
                 if (tc::elect_one()) {
                     constexpr uint32_t idesc = tc::idesc_bf16(128, TILE, false, false);
                     constexpr uint64_t kTileStep = TILE_BYTES >> 4;   // descriptor address fields count 16-byte units
-                    const uint64_t da0 = tc::smem_desc_sw128(s_a), db0 = tc::smem_desc_sw128(s_b);
+                    const uint64_t da0 = tc::smem_desc_sw128(s_b + it.ring), db0 = tc::smem_desc_sw128(s_b);
+                    const int g = warp;
+                    const uint32_t t_s = tmem + 2 * g * TILE, full = tc::smem_addr(&bars->s_full[g]), empty = tc::smem_addr(&bars->s_empty[g]);
                     bool ok = true;
-                    for (int p = 0; ok && p < it.n_pairs; p += SC_GROUPS) {
-                        const uint32_t k0 = tiles_done + 2 * p;
-                        const int tiles = min(2 * SC_GROUPS, it.n_st - 2 * p);
-                        for (int chunk = 0; ok && chunk < it.n_chunks; ++chunk) {
-#pragma unroll
-                            for (int g = 0; g < SC_GROUPS; ++g) {
-                                if (2 * g >= tiles) break;
-                                for (int e = 2 * g; ok && chunk == 0 && e < 2 * g + 2 && e < tiles; ++e)
-                                    ok = tc::mbar_wait(tc::smem_addr(&bars->a_full[(k0 + e) % SC_STAGES]), ((k0 + e) / SC_STAGES) & 1u, abort_flag);
-                                if (!ok || !(ok = tc::mbar_wait(tc::smem_addr(&bars->s_empty[g]), (steps_done[g] & 1u) ^ 1u, abort_flag))) break;
-                                tc::fence_after_sync();
-                                const uint64_t db = db0 + (uint64_t)chunk * kTileStep;
-                                for (int e = 0; e < 2 && 2 * g + e < tiles; ++e) {
-                                    const uint64_t da = da0 + (uint64_t)((k0 + 2 * g + e) % SC_STAGES) * kTileStep;
-                                    const uint32_t t_s = tmem + (2 * g + e) * TILE;
-                                    tc::mma_ss_c<false>(t_s, da, db, idesc);   // K = 16 steps over the 64 channels: 32 bytes = 2 descriptor units
-                                    tc::mma_ss_c<true>(t_s, da + 2, db + 2, idesc);
-                                    tc::mma_ss_c<true>(t_s, da + 4, db + 4, idesc);
-                                    tc::mma_ss_c<true>(t_s, da + 6, db + 6, idesc);
-                                }
-                                tc::mma_commit(tc::smem_addr(&bars->s_full[g]));
-                                ++steps_done[g];
+                    int st = 2 * g;                                  // ring stage of the pair's first tile (there are at least five)
+                    uint32_t par = fills ^ ((1u << st) - 1u);        // parity (bits) of the fills that come next
+                    for (int p = g; ok && p < it.n_pairs; p += SC_GROUPS) {
+                        const bool two = 2 * p + 1 < it.n_st;
+                        const int st0 = st, st1 = st + 1 < it.stages ? st + 1 : 0;
+                        ok = tc::mbar_wait(tc::smem_addr(&bars->a_full[st0]), par >> st0 & 1u, abort_flag) &&
+                             (!two || tc::mbar_wait(tc::smem_addr(&bars->a_full[st1]), par >> st1 & 1u, abort_flag));
+                        const uint64_t da = da0 + (uint64_t)st0 * kTileStep, db = da0 + (uint64_t)st1 * kTileStep;
+                        uint64_t dd = db0;
+                        for (int chunk = 0; ok && chunk < it.n_chunks; ++chunk, ++steps_done, dd += kTileStep) {
+                            if (!(ok = tc::mbar_wait(empty, (steps_done & 1u) ^ 1u, abort_flag))) break;
+                            tc::fence_after_sync();
+                            tc::mma_ss_c<false>(t_s, da, dd, idesc);   // K = 16 steps over the 64 channels: 32 bytes = 2 descriptor units
+                            tc::mma_ss_c<true>(t_s, da + 2, dd + 2, idesc);
+                            tc::mma_ss_c<true>(t_s, da + 4, dd + 4, idesc);
+                            tc::mma_ss_c<true>(t_s, da + 6, dd + 6, idesc);
+                            if (two) {
+                                tc::mma_ss_c<false>(t_s + TILE, db, dd, idesc);
+                                tc::mma_ss_c<true>(t_s + TILE, db + 2, dd + 2, idesc);
+                                tc::mma_ss_c<true>(t_s + TILE, db + 4, dd + 4, idesc);
+                                tc::mma_ss_c<true>(t_s + TILE, db + 6, dd + 6, idesc);
                             }
+                            tc::mma_commit(full);
                         }
-                        for (int e = 0; ok && e < tiles; ++e) tc::mma_commit(tc::smem_addr(&bars->a_empty[(k0 + e) % SC_STAGES]));
+                        if (ok) {
+                            tc::mma_commit(tc::smem_addr(&bars->a_empty[st0]));
+                            if (two) tc::mma_commit(tc::smem_addr(&bars->a_empty[st1]));
+                        }
+                        for (int e = 0; e < 2 * SC_GROUPS; ++e) {   // the stages up to this group's next pair
+                            par ^= 1u << st;
+                            if (++st == it.stages) st = 0;
+                        }
                     }
                 }
                 __syncwarp();
             }
-            tiles_done += it.n_st;
+            for (int st = 0; st < it.stages; ++st) fills ^= (uint32_t)((it.n_st - st + it.stages - 1) / it.stages & 1) << st;
             __syncthreads();
             if (*abort_flag) break;   // (the flag is only set between two barriers: same answer in every thread)
         }
@@ -279,44 +357,50 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         const int row = (warp & 3) * 32 + lane;            // row of the token tile = lane of tensor memory
         const uint32_t t_s = tmem + g * 2 * TILE + half * 64 + ((uint32_t)((warp & 3) * 32) << 16);
         uint32_t steps_done = 0, pairs_done = 0;           // of this group, all items
-        for (int item = blockIdx.x; item < 2 * per_tensor; item = bars->next) {
-            const Item it = item_of(item);
-            const int nd = it.nd, n = it.bi.n;
+        for (int n_items = 0;; ++n_items) {
+            const ScoreItem& it = items[n_items & 1];
+            if (it.t < 0) break;
+            const int nd = it.nd, n_src = it.n_src;
+            auto src_position = [&](int s) { return s + (it.even ? s * nd / n_src : nd); };   // (see the loads of the tiles)
             const __nv_bfloat16* x = a.xr[it.t] + it.row0 * kHeadDim;
             const float* inv = a.inv_norm[it.t] + it.row0;
-            // ---- the dst tokens, scaled by a power of two to norms in [1, 2) (no product with them overflows where the cosine would not), in
-            //      the image a tiled copy with the 128-byte swizzle would leave, and what is left of their weights
+            // ---- the dst tokens, in the same image, and their weights
+            // (the last chunk's rows behind these belong to the ring of token tiles: columns that are masked)
+            const int rows = it.n_chunks > 0 ? nd : 0, at = tid - 128;
+            bool far = false;
+            for (int d = at; d < rows; d += SC_THREADS - 128) {   // (one or two weights per thread)
+                const float w = ld_global(inv + dst_position(d, it.n_rule, nd));
+                w_s[d] = w;
+                far |= !(w >= 0x1p-40f && w <= 0x1p40f);
+            }
             {
-                const int at = tid - 128, c16 = at & 7;
-                constexpr int kRowsPerPass = (SC_THREADS - 128) / 8, kBatch = 8;
-                for (int d0 = at >> 3; d0 < it.n_chunks * TILE; d0 += kBatch * kRowsPerPass) {
-                    uint4 v[kBatch];   // all of a batch's loads are issued before the first is used
-                    float w[kBatch];
-#pragma unroll
-                    for (int u = 0; u < kBatch; ++u) {
-                        const int d = d0 + u * kRowsPerPass;
-                        v[u] = make_uint4(0u, 0u, 0u, 0u);
-                        w[u] = 0.f;
-                        if (d < nd) {
-                            const int pos = dst_position(d, it.bi.n_rule, nd);
-                            v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)pos * kHeadDim) + c16);
-                            w[u] = ld_global(inv + pos);
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kBatch; ++u) {
-                        const int d = d0 + u * kRowsPerPass;
-                        if (d >= it.n_chunks * TILE) break;   // (rows past the last dst token are zeros; their columns are masked below)
-                        const float scale = __uint_as_float(__float_as_uint(w[u]) & 0x7f800000u);   // 2^floor(log2 w); 0 for w = 0
-                        const uint4 o = make_uint4(scale_bf16x2(v[u].x, scale), scale_bf16x2(v[u].y, scale), scale_bf16x2(v[u].z, scale),
-                                                   scale_bf16x2(v[u].w, scale));
-                        *reinterpret_cast<uint4*>(smem + d * kRowBytes + ((c16 ^ (d & 7)) << 4)) = o;
-                        if (c16 == 0) w_s[d] = __uint_as_float((__float_as_uint(w[u]) & 0x007fffffu) | 0x3f800000u);
+                const int c16 = at & 7;
+                constexpr int kRowsPerPass = (SC_THREADS - 128) / 8;
+                Ramp pos(((at >> 3) + 1) * it.n_rule - 1, kRowsPerPass * it.n_rule, nd);   // dst_position(d) = ceil((d + 1) n_rule / nd) - 1
+#pragma unroll 4
+                for (int d = at >> 3; d < rows; d += kRowsPerPass, pos.next())
+                    load_async(s_b + d * kRowBytes + ((c16 ^ (d & 7)) << 4), x + (int64_t)pos.value * kHeadDim + c16 * 8);
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor cores read the rows through the async proxy
+            if (__syncthreads_or(far)) {
+                // Somewhere a norm is far from one: such tokens are scaled by a power of two to norms in [1, 2), so that no product with them
+                // overflows where the cosine would not.
+                for (int d = at; d < rows; d += SC_THREADS - 128) {
+                    const float w = w_s[d];
+                    if (w >= 0x1p-40f && w <= 0x1p40f) continue;
+                    const float scale = __uint_as_float(__float_as_uint(w) & 0x7f800000u);   // 2^floor(log2 w); 0 for w = 0
+                    w_s[d] = __uint_as_float((__float_as_uint(w) & 0x007fffffu) | 0x3f800000u);
+#pragma unroll 1
+                    for (int c = 0; c < 8; ++c) {
+                        uint4* piece = reinterpret_cast<uint4*>(smem + d * kRowBytes) + c;
+                        const uint4 v = *piece;
+                        *piece = make_uint4(scale_bf16x2(v.x, scale), scale_bf16x2(v.y, scale), scale_bf16x2(v.z, scale), scale_bf16x2(v.w, scale));
                     }
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor cores read the rows through the async proxy
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncthreads();
             }
-            __syncthreads();
             bool ok = true;
             for (int p = g; ok && p < it.n_pairs; p += SC_GROUPS) {
                 Best best[2];
@@ -363,20 +447,21 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     }
                 }
                 if (!ok) break;
-                int arg[2];
+                int arg[2], own[2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
+                    const int s = (2 * p + e) * TILE + row;   // src token
+                    own[e] = s < n_src ? src_position(s) : -1;   // token number inside the block
                     int in_group = kGroup;
 #pragma unroll
                     for (int c = kGroup - 1; c >= 0; --c)
                         if ((c & 1 ? best[e].v[c >> 1].y : best[e].v[c >> 1].x) == best[e].score) in_group = c;
-                    const int i = (2 * p + e) * TILE + row;   // token number inside the block
                     if (best[e].first_dst < 0.f)
                         arg[e] = 0;   // (no score is a number)
                     else if (in_group < kGroup)
                         arg[e] = (int)best[e].first_dst + in_group;
                     else
-                        arg[e] = i < n ? find_again(x + (int64_t)i * kHeadDim, smem, w_s, half, nd) : 0;
+                        arg[e] = own[e] >= 0 ? find_again(x + (int64_t)own[e] * kHeadDim, smem, w_s, half, nd) : 0;
                 }
                 // the two column halves of a token meet: half 1 hands (best, arg) over, half 0 decides (ties: lowest dst)
                 const uint32_t turn = pairs_done++ & 1u;
@@ -394,6 +479,9 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 #pragma unroll
                     for (int e = 0; e < 2; ++e) o[e] = mine[e * TILE];
                     tc::mbar_arrive(tc::smem_addr(&bars->x_done[g]));
+                    float own_w[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) own_w[e] = own[e] >= 0 ? ld_global(inv + own[e]) : 0.f;
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         float score = best[e].score;
@@ -402,11 +490,9 @@ big_scores_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                             score = o[e].x;
                             arg[e] = oarg;
                         }
-                        const int i = (2 * p + e) * TILE + row;
-                        if (i < n) {
-                            const float w = ld_global(inv + i);
-                            a.best_key[it.t][it.row0 + i] = score_key(score * w);
-                            a.best_pos[it.t][it.row0 + i] = dst_position(arg[e], it.bi.n_rule, nd);
+                        if (own[e] >= 0) {
+                            a.best_key[it.t][it.row0 + own[e]] = score_key(score * own_w[e]);
+                            a.best_pos[it.t][it.row0 + own[e]] = dst_position(arg[e], it.n_rule, nd);
                         }
                     }
                 }
@@ -1019,15 +1105,11 @@ cudaError_t configure_big_blocks() {
 }
 
 cudaError_t launch_big_scores(const BigMatchArgs& a, int sm_count, cudaStream_t stream) {
-    CUtensorMap mq, mk;
-    if (!encode_rows_tensor_map(&mq, a.xr[0], a.n_tokens, a.heads, kHeadDim, (int64_t)a.n_tokens * kHeadDim, TILE) ||
-        !encode_rows_tensor_map(&mk, a.xr[1], a.n_tokens, a.heads, kHeadDim, (int64_t)a.n_tokens * kHeadDim, TILE))
-        return cudaErrorInvalidValue;
     const int64_t total = 2ll * a.heads * a.n_blocks;
     int ctas = sm_count < 1 ? 1 : sm_count;
     if (ctas > total) ctas = (int)total;
     if (ctas < 1) ctas = 1;
-    return launch_kernel(big_scores_kernel, ctas, SC_THREADS, SC_SMEM, stream, mq, mk, a);
+    return launch_kernel(big_scores_kernel, ctas, SC_THREADS, SC_SMEM, stream, a);
 }
 
 cudaError_t launch_big_select(const BigMatchArgs& a, cudaStream_t stream) {

@@ -139,12 +139,34 @@ def test_a_dst_token_without_a_similarity_is_nobodys_best(bad):
     src, fine = np.setdiff1d(np.arange(n), dst), np.setdiff1d(dst, spoilt)
     assert len(src) == int(0.75 * n) and len(dst) == nd
     for h in range(heads):
-        unit = rows[h] / np.linalg.norm(rows[h], axis=1, keepdims=True)
+        with np.errstate(all="ignore"):
+            unit = rows[h] / np.linalg.norm(rows[h], axis=1, keepdims=True)
         sim = unit[src] @ unit[fine].T
         for m in maps:
             assert np.isin(m[h][src], fine).all() and (m[h][dst] == dst).all()
             mine = (unit[src] * unit[m[h][src]]).sum(1)
             assert (sim.max(1) - mine <= 1e-5).all(), (h, (sim.max(1) - mine).max())
+
+
+def test_norms_far_from_one_change_no_map():
+    """Every token multiplied by a power of two of its own, 2^-30 .. 2^60 (squared norms stay inside fp32, norms above the clamp): products,
+    norms and weights scale exactly, so the maps are the same."""
+    n, heads = 1500, 2
+    wl = synth.Workload("scaled", 1, 1, n, 1, 1, n, 0.7, 0.4, n_camera=0, n_register=1, heads=heads, seed=4)
+    q, k, v = synth.make_qkv(wl)
+    gen = np.random.default_rng(9)
+    maps = []
+    for scaled in (False, True):
+        with hb.Httm(hb.HttmConfig.of(wl)) as ctx:
+            dq, dk, dv = (hb.bf16_from_bits(x, DEV) for x in (q, k, v))
+            if scaled:
+                dq, dk = (t * torch.exp2(torch.from_numpy(gen.integers(-30, 61, t.shape[:2])).float()).to(DEV).bfloat16()[..., None] for t in (dq, dk))
+            ctx.global_attention(dq, dk, dv)
+            torch.cuda.synchronize()
+            assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+            maps.append((ctx.export(hb.X_ASSIGN_Q), ctx.export(hb.X_ASSIGN_K)))
+    for a, b in zip(*maps):
+        assert np.array_equal(a, b)
 
 
 def test_sums_of_many_members_with_one_far_larger_member():
