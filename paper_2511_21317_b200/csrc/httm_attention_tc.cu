@@ -34,7 +34,9 @@ constexpr int NTHREADS = 320;   // producer warp, MMA warp, 2 x 4 softmax warps:
 constexpr int TMEM_COLS = 512;
 constexpr int kTableHeads = 256;   // head tables (per-head query lengths) of up to this many heads are kept in shared memory
 constexpr int kOutRowPitch = kRowBytes + 16;             // staged output rows: the pitch keeps 16-byte stores of a quarter warp on distinct banks
-constexpr int kOutStageBytes = 8 * 32 * kOutRowPitch;   // eight softmax warps x 32 output rows, staged for bulk stores
+constexpr int kTargetChunk = 128;                        // target tokens of a warp's 32 rows that are fetched ahead (on average about 100)
+constexpr int kOutWarpBytes = 32 * kOutRowPitch + kTargetChunk * 8;   // of each softmax warp: 32 output rows, (token, row) of their targets
+constexpr int kOutStageBytes = 8 * kOutWarpBytes;
 constexpr int SMEM_BYTES = (2 + 2 * KV_STAGES) * TILE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/ + 1024 /*row exchange*/ +
                            (2 * kTableHeads + 4) * 4 /*head tables*/ + kOutStageBytes;
 constexpr int kPColumn = 64;                  // P (bf16 pairs, 64 columns) lies over columns 64 .. 127 of its S
@@ -316,64 +318,93 @@ struct PassWalker {
 // once per score tile k with k mod 3 == b (2 n tiles in a pair pass, n in a single pass), n key tiles in the pass.
 __device__ __forceinline__ int count_mod3(int n, int r) { return (n - r + 2) / 3; }
 
-// Where the 32 output rows of a softmax warp go.  UNMERGE (Eq. 5-7 folded into the epilogue): row `grow` is the attention
-// output of a merged query and goes to every original token of its group, at the token's place in the final
-// [tokens][heads x 64] tensor; the first four members are fetched ahead of the epilogue, larger groups read the rest
-// of their list when they are stored.  Otherwise the row goes to row `grow` of the merged output.
+// Where the 32 output rows of a softmax warp go: row `grow` of a thread goes to row `grow` of the merged output.
+template <bool UNMERGE>
 struct RowTargets {
-    int count;      // tokens this thread's row is written to (0: the row does not exist)
-    int token[4];   // the first four of them
-    int first;      // index of the group's first member in the member list
+    int row;   // -1: the row does not exist
+};
+// UNMERGE (Eq. 5-7 folded into the epilogue): row `grow` is the attention output of a merged query and goes to every original token of its
+// group, at the token's place in the final [tokens][heads x 64] tensor.  The member lists of consecutive rows lie one behind the
+// other, so a warp's targets are one run of the list: every lane fetches some of them ahead of the epilogue, whatever rows they belong to.
+template <>
+struct RowTargets<true> {
+    int total;   // targets of the warp's rows
+    int start;   // first target of this lane's row (beyond all targets: the row does not exist)
+    int first;   // index of the warp's first target in the member list
+    int token[kTargetChunk / 32];   // targets lane, lane + 32, ..
 };
 template <bool UNMERGE>
-__device__ __forceinline__ RowTargets row_targets(const TcParams& p, int head, int grow, bool valid) {
-    RowTargets t{};
-    if (!valid) return t;
-    if (!UNMERGE) {
-        t.count = 1;
-        t.token[0] = grow;
-        return t;
-    }
-    const int32_t* gs = p.group_start + (int64_t)head * (p.m_q + 1) + grow;
-    const int32_t* member = p.group_member + (int64_t)head * p.n_tokens;
-    t.first = ld_global(gs);
-    t.count = ld_global(gs + 1) - t.first;
+__device__ __forceinline__ RowTargets<UNMERGE> row_targets(const TcParams& p, int head, int grow, bool valid, int lane) {
+    RowTargets<UNMERGE> t{};
+    if constexpr (!UNMERGE) {
+        t.row = valid ? grow : -1;
+    } else {
+        int first = 0, last = 0;
+        if (valid) {
+            const int32_t* gs = p.group_start + (int64_t)head * (p.m_q + 1) + grow;
+            first = ld_global(gs);
+            last = ld_global(gs + 1);
+        }
+        t.first = __shfl_sync(0xffffffffu, first, 0);
+        t.start = valid ? first - t.first : 0x7fffffff;
+        t.total = __reduce_max_sync(0xffffffffu, valid ? last - t.first : 0);
+        const int32_t* member = p.group_member + (int64_t)head * p.n_tokens + t.first;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) t.token[i] = i < t.count ? ld_global(member + t.first + i) : 0;
+        for (int i = 0; i < kTargetChunk / 32; ++i) t.token[i] = 32 * i + lane < t.total ? ld_global(member + 32 * i + lane) : 0;
+    }
     return t;
 }
-// Every lane hands in its row (eight 16-byte pieces) and its targets.  The row is staged in shared memory and leaves as
-// one 128-byte bulk copy per target token (whole lines, issued by the row's own thread: no loop over the warp's rows).
-// The copies are asynchronous: bulk_stores_done() must come before the stage is rewritten and before the kernel ends.
+// Every lane hands in its row (eight 16-byte pieces), which is staged in shared memory.  Without UNMERGE it leaves as one 128-byte bulk copy,
+// issued by the row's own thread; the copies are asynchronous: bulk_stores_done() must come before the stage is rewritten and
+// before the kernel ends.  With UNMERGE the warp stores its rows, eight lanes to a target token: whole lines, four targets per
+// instruction.  (One bulk copy per target took 6 200 cycles at the end of a pass with three targets per row: an SM issues a copy every eight cycles,
+// and the warp waits for that.  Measured, whole call, before / after: 1 044 tokens 20.2 / 18.9 us, 10 992 117.3 / 113.2, 32 976 616 / 609.  Where every
+// row has one target the bulk copies take 2 400 cycles of 570 000 in a pass over 258 key tiles, stores 1 200, and the kernel as a whole is
+// slower with them: the compiler schedules the exponentials differently, 4 690 / 4 885 us for 32 976 x 32 976 x 16 heads.)
 __device__ __forceinline__ void bulk_stores_done() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 template <bool UNMERGE>
-__device__ __forceinline__ void store_rows(const TcParams& p, int head, const uint4 (&v)[8], const RowTargets& t, unsigned char* stage, int lane) {
-    bulk_stores_done();   // (the copies of the previous pass have long left)
+__device__ __forceinline__ void store_rows(const TcParams& p, int head, const uint4 (&v)[8], const RowTargets<UNMERGE>& t, unsigned char* stage, int lane) {
+    if constexpr (!UNMERGE)
+        bulk_stores_done();   // (the copies of the previous pass have long left)
+    else
+        __syncwarp();         // (the stage of the previous pass has been read)
     unsigned char* row = stage + lane * kOutRowPitch;
 #pragma unroll
     for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(row + c * 16) = v[c];
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the staged row is visible to the bulk-copy engine
-    const uint32_t src = tc::smem_addr(row);
     __nv_bfloat16* base = p.out + (int64_t)head * p.out_stride_head;
-    const int32_t* member = UNMERGE ? p.group_member + (int64_t)head * p.n_tokens + t.first : nullptr;
-    auto send = [&](int token) {
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(base + (int64_t)token * p.out_stride_token), "r"(src),
-                     "n"(kRowBytes)
-                     : "memory");
-    };
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        if (q < t.count) send(t.token[q]);
+    if constexpr (!UNMERGE) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the staged row is visible to the bulk-copy engine
+        if (t.row >= 0)
+            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(base + (int64_t)t.row * p.out_stride_token),
+                         "r"(tc::smem_addr(row)), "n"(kRowBytes)
+                         : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    } else {
+        int2* list = reinterpret_cast<int2*>(stage + 32 * kOutRowPitch);
+        const int32_t* member = p.group_member + (int64_t)head * p.n_tokens + t.first;
+        const int sub = lane >> 3, piece = lane & 7;
 #pragma unroll 1
-    for (int q = 4; q < t.count; q += 4) {   // four loads in flight: one by one they took 0.5 us each (32 976 tokens 582 -> 580 us per call)
-        int token[4];
+        for (int c0 = 0; c0 < t.total; c0 += kTargetChunk) {
+            if (c0 > 0) __syncwarp();
 #pragma unroll
-        for (int i = 0; i < 4; ++i) token[i] = ld_global(member + min(q + i, t.count - 1));
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (q + i < t.count) send(token[i]);
+            for (int i = 0; i < kTargetChunk / 32; ++i) {
+                // the row of a target: the last one that starts at or before it (every row has at least one target)
+                const int e0 = c0 + 32 * i, at = t.start - e0;
+                const unsigned here = __reduce_or_sync(0xffffffffu, at >= 0 && at < 32 ? 1u << at : 0u);
+                const int before = __popc(__ballot_sync(0xffffffffu, at < 0));
+                const int token = c0 == 0 ? t.token[i] : (e0 + lane < t.total ? ld_global(member + e0 + lane) : 0);
+                list[32 * i + lane] = make_int2(token, before + __popc(here & (0xffffffffu >> (31 - lane))) - 1);
+            }
+            __syncwarp();
+            const int n = min(t.total - c0, kTargetChunk);
+#pragma unroll 4
+            for (int e = sub; e < n; e += 4) {
+                const int2 target = list[e];
+                reinterpret_cast<uint4*>(base + (int64_t)target.x * p.out_stride_token)[piece] =
+                    *reinterpret_cast<const uint4*>(stage + target.y * kOutRowPitch + piece * 16);
+            }
+        }
     }
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
 // The end of a pass over part of the keys (group A's four warps, thread = row of the tile): the combined but unnormalised
@@ -426,7 +457,7 @@ __device__ __noinline__ bool epilogue_part(const TcParams& p, const PartArgs& a,
         __threadfence();
     }
     if (!__shfl_sync(0xffffffffu, last, 0)) return true;
-    const RowTargets targets = row_targets<UNMERGE>(p, a.head, a.grow, a.grow < a.mq_rows);
+    const RowTargets<UNMERGE> targets = row_targets<UNMERGE>(p, a.head, a.grow, a.grow < a.mq_rows, lane);
     const float* other = p.partial + (int64_t)first * kPartFloats;
     float top = -INFINITY, sum = 0.f, o[kHeadDim];
 #pragma unroll 4
@@ -697,7 +728,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         uint32_t n_single = 0;                          // single passes so far (phase of x_full / x_done)
         float2* xch = reinterpret_cast<float2*>(smem + (2 + 2 * KV_STAGES) * TILE_BYTES + 256);   // [128 rows] (max, sum) of group B
         unsigned char* out_stage = smem + (2 + 2 * KV_STAGES) * TILE_BYTES + 256 + 1024 + (2 * kTableHeads + 4) * 4 +
-                                   (warp - 2) * 32 * kOutRowPitch;   // this warp's 32 output rows
+                                   (warp - 2) * kOutWarpBytes;   // this warp's 32 output rows and their targets
         bool ok = true;
         for (int pass = 0; ok && walker.next(&ps); ++pass) {
             const int n_score = ps.pair ? 2 * ps.n : ps.n;
@@ -811,7 +842,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                 }
                 if (ok && ps.pair) {
                     const int grow = (ps.tile + x) * BM + row;
-                    const RowTargets targets = row_targets<UNMERGE>(p, ps.head, grow, grow < mq_rows);   // (in flight during the wait)
+                    const RowTargets<UNMERGE> targets = row_targets<UNMERGE>(p, ps.head, grow, grow < mq_rows, lane);   // (in flight during the wait)
                     if ((ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->o_final), (uint32_t)pass & 1u, abort_flag)))) {
                         tc::fence_after_sync();
                         const float inv = 1.0f / l;
@@ -852,7 +883,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
                     // single pass, group A: combine the two partial softmaxes over disjoint keys
                     //   out = (O_A 2^(m_A - m) + O_B 2^(m_B - m)) / (l_A 2^(m_A - m) + l_B 2^(m_B - m)),  m = max(m_A, m_B)
                     const int grow = ps.tile * BM + row;
-                    const RowTargets targets = row_targets<UNMERGE>(p, ps.head, grow, grow < mq_rows);   // (in flight during the waits)
+                    const RowTargets<UNMERGE> targets = row_targets<UNMERGE>(p, ps.head, grow, grow < mq_rows, lane);   // (in flight during the waits)
                     ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->o_final), (uint32_t)pass & 1u, abort_flag) &&
                                                      tc::mbar_wait(tc::smem_addr(&bars->x_full), n_single & 1u, abort_flag));
                     if (ok) {
@@ -890,7 +921,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 #pragma unroll
             for (int b = 0; b < 3; ++b) sp_base[b] += (uint32_t)count_mod3(n_score, b);
         }
-        bulk_stores_done();
+        if constexpr (!UNMERGE) bulk_stores_done();
     }
     tc::fence_before_sync();
     __syncthreads();

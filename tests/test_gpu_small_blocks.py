@@ -32,3 +32,22 @@ def test_whole_units_and_split_units_agree(blk, ratio, specials, frames):
         one = run(hb.HttmConfig.of(wl.replace(heads=1)), (q[h:h + 1], k[h:h + 1], v[h:h + 1]))
         for name in ITEMS:
             assert np.array_equal(whole[name][h], one[name][0]), (name, h)
+
+
+@pytest.mark.parametrize("ratio", [0.0, 0.5, 0.72, 0.75, 0.8, 0.97])
+@pytest.mark.parametrize("strided", [False, True])
+def test_rows_with_many_target_tokens(ratio, strided):
+    """The epilogue that unmerges stores 32 rows to all their target tokens, 128 targets at a time: one target per row up to 32, lists just
+    below and above 128, 256 and more, tiles whose last rows do not exist, rows of a wider output too.  The same rows through the unmerge kernel."""
+    wl = synth.Workload("targets", 8, 20, 24, 2, 4, 4, ratio, 0.5, n_camera=1, n_register=2, heads=3, seed=6)
+    q, k, v = (hb.bf16_from_bits(x, DEV) for x in synth.make_qkv(wl))
+    n = wl.n_tokens
+    with hb.Httm(hb.HttmConfig.of(wl)) as ctx:
+        wide = wl.heads * 64 + (72 if strided else 0)   # (rows of a wider tensor)
+        outs = [torch.zeros(n, wide, dtype=torch.bfloat16, device=DEV)[:, :wl.heads * 64] for _ in range(2)]
+        ctx.global_attention(q, k, v, outs[0])
+        ctx.launch_stage(hb.STAGE_ATTENTION)
+        ctx.launch_stage(hb.STAGE_UNMERGE, out=outs[1])
+        torch.cuda.synchronize()
+        assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+        assert torch.equal(outs[0], outs[1])
