@@ -650,17 +650,14 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) big_select_kernel(const BigMat
 // They gather rows from DRAM and are bound by the loads in flight: several CTAs share an SM (1536 threads of at most 40
 // registers), so that one gathers while another sorts.
 constexpr int kSortedThreads = 1536;   // resident threads per SM the kernels are compiled for (40 registers)
+constexpr int kMergeThreads = 1024;    // .. and the merge kernel: at 64 registers nothing of its sums is spilled, and the fewer blocks gather no slower
+                                       // (3840-token blocks as below 241 -> 225 us, 64-token ones 36.9 -> 32.8, 128-token ones 71.7 -> 70; the
+                                       // deviation kernel, which reads its rows twice and computes more, is better at three CTAs: filter 178 against 195)
 __host__ __device__ constexpr int mg_smem_bytes(int N) { return N * 4 /*keys*/ + N * 2 /*row of kept token*/ + (N + 4) * 4 /*segments*/ + 256; }   // N = E T tokens
 __host__ __device__ constexpr int of_smem_bytes(int N) { return mg_smem_bytes(N) + N * 2 /*position of every row's kept token*/ + N /*outlier flags*/ + N * 2 /*new representative of every row*/; }
 
-__device__ __forceinline__ void unpack8f(const uint4& raw, float* f) {
-    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        f[2 * i] = __uint_as_float(w[i] << 16);
-        f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-    }
-}
+// two channels of a bf16 row
+__device__ __forceinline__ float2 unpack2(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)); }
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&v);
@@ -725,7 +722,7 @@ __device__ __forceinline__ void radix_places(const int (&digit)[E], int (&place)
 // The order comes from two stable counting passes over six bits of the row each (one if there are at most 64 rows), so
 // it does not depend on scheduling.  A bitonic sort of the keys took 28 us for 3840 tokens (78 rounds with a barrier each).
 // At 82 440 tokens x 16 heads in 3840-token blocks, one CTA of 1024 threads per SM: deviation 203 -> 153 us, filter 92 -> 40, merge
-// 310 -> 303; with three CTAs of 512 threads per SM, half of which gather while others sort: 144, 31 and 212 us.
+// 310 -> 303; with three CTAs of 512 threads per SM, half of which gather while others sort: 144 (now 101), 31 and 212 us.
 template <int T, int E>
 __device__ int build_groups(const int32_t* A, int block_start, int n, int limit, uint32_t* keys, int16_t* row_of, int* seg, int* warp_sum,
                             int16_t* rep_of_row, int32_t* status, int32_t* rank_out, int moff) {
@@ -817,33 +814,33 @@ __device__ int build_groups(const int32_t* A, int block_start, int n, int limit,
 // bound by load latency.  They are added in pairs of pairs, to one of two sums in turn: n / 8 + 4 roundings for n members.  (Added
 // one after the other they took n: with one member 2^17 times the others, 2 048 of them left the mean half a step of bf16 off; that
 // was a little faster, at 82 440 tokens x 16 heads in 3840-token blocks filter 216 / 221 us, merge 224 / 237 us.)
-__device__ __forceinline__ void sum_members(const __nv_bfloat16* x, int64_t stride, const uint32_t* keys, int i0, int i1, float (&sum)[8]) {
-    float other[8];
+__device__ __forceinline__ void sum_members(const __nv_bfloat16* x, const uint32_t* keys, int i0, int i1, float2 (&sum)[4]) {
+    float2 other[4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) sum[e] = other[e] = 0.f;
-    auto add_four = [&](int i, float (&to)[8]) {
+    for (int e = 0; e < 4; ++e) sum[e] = other[e] = make_float2(0.f, 0.f);
+    auto add_four = [&](int i, float2 (&to)[4]) {
         uint4 v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             v[u] = make_uint4(0u, 0u, 0u, 0u);
-            if (i + u < i1) v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)(keys[i + u] & 4095u) * stride));
+            if (i + u < i1) v[u] = ld_global(reinterpret_cast<const uint4*>(x + (keys[i + u] & 4095u) * kHeadDim));
         }
-        float f[4][8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) unpack8f(v[u], f[u]);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) to[e] += (f[0][e] + f[1][e]) + (f[2][e] + f[3][e]);
+        for (int e = 0; e < 4; ++e) {
+            auto word = [&](int u) { return unpack2(e == 0 ? v[u].x : e == 1 ? v[u].y : e == 2 ? v[u].z : v[u].w); };
+            to[e] = tc::fadd2(to[e], tc::fadd2(tc::fadd2(word(0), word(1)), tc::fadd2(word(2), word(3))));
+        }
     };
     for (int i = i0; i < i1; i += 8) {
         add_four(i, sum);
         if (i + 4 < i1) add_four(i + 4, other);
     }
 #pragma unroll
-    for (int e = 0; e < 8; ++e) sum[e] += other[e];
+    for (int e = 0; e < 4; ++e) sum[e] = tc::fadd2(sum[e], other[e]);
 }
 
 template <int T, int E>
-__global__ void __launch_bounds__(T, kSortedThreads / T) big_merge_kernel(const MergeArgs a, int sp_chunks) {
+__global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const MergeArgs a, int sp_chunks) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
     uint32_t* keys = reinterpret_cast<uint32_t*>(mg_smem);                                     // [P] (merged row << 12) | position
     int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (E * T) * 4);            // [n] merged row of a kept token, -1
@@ -886,18 +883,15 @@ __global__ void __launch_bounds__(T, kSortedThreads / T) big_merge_kernel(const 
         __nv_bfloat16* out = a.merged[t] + ((int64_t)h * m_len + moff) * kHeadDim;
         for (int row = warp * 4 + sub; row < n_kept; row += (T / 32) * 4) {
             const int i0 = seg[row], i1 = seg[row + 1];
-            float acc[8];
-            sum_members(x + 8 * ch, kHeadDim, keys, i0, i1, acc);
+            float2 acc[4];
+            sum_members(x + 8 * ch, keys, i0, i1, acc);
             if (i1 > i0) {
                 const float inv = 1.0f / (float)(i1 - i0);
-                float r8[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) r8[e] = acc[e] * inv;
                 uint4 o;
-                o.x = pack2(r8[0], r8[1]);
-                o.y = pack2(r8[2], r8[3]);
-                o.z = pack2(r8[4], r8[5]);
-                o.w = pack2(r8[6], r8[7]);
+                o.x = pack2(acc[0].x * inv, acc[0].y * inv);
+                o.y = pack2(acc[1].x * inv, acc[1].y * inv);
+                o.z = pack2(acc[2].x * inv, acc[2].y * inv);
+                o.w = pack2(acc[3].x * inv, acc[3].y * inv);
                 reinterpret_cast<uint4*>(out + (int64_t)row * kHeadDim)[ch] = o;
             }
         }
@@ -910,7 +904,10 @@ __global__ void __launch_bounds__(T, kSortedThreads / T) big_merge_kernel(const 
 // path, which work on the array of deviations), outliers leave their groups - on the sorted group structure of the merge
 // kernel.  One CTA per (head, block).
 
-// eps[h][p] = || q_p - mean of the group p was merged into ||_2 in fp32; 0 for a token on its own
+// eps[h][p] = || q_p - mean of the group p was merged into ||_2 in fp32; 0 for a token on its own.
+// Bound by the instructions issued (61 warp instructions per token): two channels per instruction, one exchange for the sums of four
+// members and one square root for them took the filter kernels together, at 82 440 tokens x 16 heads in 3840-token blocks, from 221 to 178 us
+// (32 976 tokens in 128-token blocks: 104.7 -> 92.2; 137 400 in 64-token blocks: 363 -> 302).
 template <int T, int E>
 __global__ void __launch_bounds__(T, kSortedThreads / T) big_deviation_kernel(const OutlierArgs a) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
@@ -932,50 +929,46 @@ __global__ void __launch_bounds__(T, kSortedThreads / T) big_deviation_kernel(co
         return;
     }
     const int n_kept = build_groups<T, E>(a.assign_q + base, bi.start, n, n, keys, row_of, seg, warp_sum, nullptr, a.status, nullptr, 0);
-    const __nv_bfloat16* x = a.src_q.ptr + (int64_t)h * a.src_q.stride_head + (int64_t)bi.start * a.src_q.stride_token;
-    const int64_t st = a.src_q.stride_token;
+    const __nv_bfloat16* x = a.src_q.ptr + base * kHeadDim + 8 * ch;   // the reordered copy
     // eight lanes per group (a lane owns 8 of the 64 channels), four groups per warp at a time
     for (int row = warp * 4 + sub; row < ((n_kept + 3) & ~3); row += (T / 32) * 4) {   // (whole sub-groups stay together for the shuffles)
         const bool live = row < n_kept;
         const int i0 = live ? seg[row] : 0, i1 = live ? seg[row + 1] : 0;
-        const int cnt = i1 - i0;
-        float mean[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) mean[e] = 0.f;
-        if (cnt >= 2) {
-            float acc[8];
-            sum_members(x + 8 * ch, st, keys, i0, i1, acc);
-            const float inv = 1.0f / (float)cnt;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) mean[e] = acc[e] * inv;   // kept in fp32
+        if (i1 - i0 < 2) {
+            if (i1 > i0 && ch == 0) eps[keys[i0] & 4095u] = 0.f;
+            continue;
         }
+        float2 mean[4];
+        sum_members(x, keys, i0, i1, mean);
+        const float inv = 1.0f / (float)(i1 - i0);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) mean[e] = make_float2(mean[e].x * inv, mean[e].y * inv);   // kept in fp32
         // (the eight lanes of a group walk its members together: the trip count is the same in all of them); four members
-        // at a time, so that four loads are in flight
+        // at a time, so that four loads are in flight; behind the last member, it again
         const unsigned group_mask = 0xffu << (8 * sub);
         for (int i = i0; i < i1; i += 4) {
             uint4 v[4];
-            int pos[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = ld_global(reinterpret_cast<const uint4*>(x + (keys[min(i + u, i1 - 1)] & 4095u) * kHeadDim));
+            float d2[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                pos[u] = i + u < i1 ? (int)(keys[i + u] & 4095u) : -1;
-                v[u] = make_uint4(0u, 0u, 0u, 0u);
-                if (cnt >= 2 && pos[u] >= 0) v[u] = ld_global(reinterpret_cast<const uint4*>(x + (int64_t)pos[u] * st) + ch);
-            }
+                float2 sq = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                float f[8];
-                unpack8f(v[u], f);
-                float d2 = 0.f;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const float d = f[e] - mean[e];
-                    d2 = fmaf(d, d, d2);
+                for (int e = 0; e < 4; ++e) {
+                    const float2 d = tc::fsub2(unpack2(e == 0 ? v[u].x : e == 1 ? v[u].y : e == 2 ? v[u].z : v[u].w), mean[e]);
+                    sq = tc::ffma2(d, d, sq);
                 }
-                d2 += __shfl_xor_sync(group_mask, d2, 1);
-                d2 += __shfl_xor_sync(group_mask, d2, 2);
-                d2 += __shfl_xor_sync(group_mask, d2, 4);
-                if (ch == 0 && pos[u] >= 0) eps[pos[u]] = cnt >= 2 ? sqrtf(d2) : 0.f;
+                d2[u] = sq.x + sq.y;
             }
+            // sums over the eight lanes, each lane ending with one member's: half of them change sides in the first two steps
+            const bool b0 = ch & 1, b1 = ch & 2;
+            const float o0 = __shfl_xor_sync(group_mask, b0 ? d2[0] : d2[2], 1), o1 = __shfl_xor_sync(group_mask, b0 ? d2[1] : d2[3], 1);
+            const float s0 = (b0 ? d2[2] : d2[0]) + o0, s1 = (b0 ? d2[3] : d2[1]) + o1;
+            float t = (b1 ? s1 : s0) + __shfl_xor_sync(group_mask, b1 ? s0 : s1, 2);
+            t += __shfl_xor_sync(group_mask, t, 4);
+            const int at = i + (b0 ? 2 : 0) + (b1 ? 1 : 0);
+            if (ch < 4 && at < i1) eps[keys[at] & 4095u] = sqrtf(t);
         }
     }
 }
