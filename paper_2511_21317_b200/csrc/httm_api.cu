@@ -187,7 +187,7 @@ float scale_log2() { return 1.4426950408889634f / std::sqrt((float)kHeadDim); }
 int32_t* item_counter(httm_ctx* c) { return c->d_part_count + attention_partial_counters(c->sm_count); }
 // What the first kernel of a call sets to zero for the kernels behind it
 void clear_state(httm_ctx* c, ClearRange (&clear)[2]) {
-    clear[0] = ClearRange{c->d_part_count, (int32_t)attention_partial_counters(c->sm_count) + 1};
+    clear[0] = ClearRange{c->d_part_count, (int32_t)attention_partial_counters(c->sm_count) + (c->big() ? 1 : 0)};
     if (c->filtering()) clear[1] = ClearRange{c->d_sel, kSelWords};
 }
 

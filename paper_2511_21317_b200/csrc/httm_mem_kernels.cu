@@ -466,6 +466,7 @@ __global__ void __launch_bounds__(256) select_level_kernel(const OutlierArgs a, 
 }
 
 constexpr int kRefineThreads = 256;
+static_assert(kRefineThreads == 256 && kDevWarps * 32 == 256, "select_level reads the histogram with 256 threads");
 // LEVEL 1: histogram of bits 20-10 of the deviations whose bits 31-21 equal the level-0 choice; LEVEL 2: of bits 9-0
 // of those whose bits 31-10 equal the choice so far.  LEVEL 0 (only where the deviation kernel does not build it on the
 // fly: the large-block path): histogram of bits 31-21 of all deviations.
