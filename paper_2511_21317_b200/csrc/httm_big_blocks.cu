@@ -367,12 +367,7 @@ big_scores_kernel(const BigMatchArgs a) {
             // ---- the dst tokens, in the same image, and their weights
             // (the last chunk's rows behind these belong to the ring of token tiles: columns that are masked)
             const int rows = it.n_chunks > 0 ? nd : 0, at = tid - 128;
-            bool far = false;
-            for (int d = at; d < rows; d += SC_THREADS - 128) {   // (one or two weights per thread)
-                const float w = ld_global(inv + dst_position(d, it.n_rule, nd));
-                w_s[d] = w;
-                far |= !(w >= 0x1p-40f && w <= 0x1p40f);
-            }
+            for (int d = at; d < rows; d += SC_THREADS - 128) w_s[d] = ld_global(inv + dst_position(d, it.n_rule, nd));   // (one or two per thread)
             {
                 const int c16 = at & 7;
                 constexpr int kRowsPerPass = (SC_THREADS - 128) / 8;
@@ -381,14 +376,22 @@ big_scores_kernel(const BigMatchArgs a) {
                 for (int d = at >> 3; d < rows; d += kRowsPerPass, pos.next())
                     load_async(s_b + d * kRowBytes + ((c16 ^ (d & 7)) << 4), x + (int64_t)pos.value * kHeadDim + c16 * 8);
             }
+            // Is any norm of the block, of a src or a dst token, outside 2^-39 .. 2^40?  (A weight is at most 1e12, just below 2^40; 0: the squared norm
+            // overflowed.)  Inside, every product lies in 2^+-80.
+            bool far = false;
+            const int n_all = rows > 0 ? nd + n_src : 0;
+#pragma unroll 4
+            for (int j = at; j < n_all; j += SC_THREADS - 128) {
+                const float w = ld_global(inv + j);
+                far |= !(w >= 0x1p-40f && w <= 0x1p39f);
+            }
             asm volatile("cp.async.wait_all;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor cores read the rows through the async proxy
             if (__syncthreads_or(far)) {
-                // Somewhere a norm is far from one: such tokens are scaled by a power of two to norms in [1, 2), so that no product with them
-                // overflows where the cosine would not.
+                // All dst tokens are scaled by a power of two to norms in (1/2, 1], those below the clamp by 2^39: no product with them is beyond the
+                // src token's own norm, and none is lost below fp32's range where the weighted one would not be.
                 for (int d = at; d < rows; d += SC_THREADS - 128) {
                     const float w = w_s[d];
-                    if (w >= 0x1p-40f && w <= 0x1p40f) continue;
                     const float scale = __uint_as_float(__float_as_uint(w) & 0x7f800000u);   // 2^floor(log2 w); 0 for w = 0
                     w_s[d] = __uint_as_float((__float_as_uint(w) & 0x007fffffu) | 0x3f800000u);
 #pragma unroll 1
@@ -491,6 +494,8 @@ big_scores_kernel(const BigMatchArgs a) {
                             arg[e] = oarg;
                         }
                         if (own[e] >= 0) {
+                            // (0 where the token's squared norm overflows.  An infinite token's is not a number, whose key orders above all numbers: it
+                            // merges first, as in the kernels of smaller blocks.)
                             a.best_key[it.t][it.row0 + own[e]] = score_key(score * own_w[e]);
                             a.best_pos[it.t][it.row0 + own[e]] = dst_position(arg[e], it.n_rule, nd);
                         }

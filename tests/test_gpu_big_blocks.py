@@ -205,3 +205,85 @@ def test_sums_of_many_members_with_one_far_larger_member():
         for got in (k_m[h][row], v_m[h][row]):   # within half a bf16 step of the mean, up to the same bound
             step = 2.0 ** (np.floor(np.log2(np.abs(mean))) - 7)
             assert (np.abs(got - mean) <= step / 2 + roundings * size).all(), (h, (np.abs(got - mean) / step).max())
+
+
+def similarities(x, src, dst):
+    """What a similarity is where fp32 cannot hold a square (x [n][64], values of bf16 in float64): weights 1 / max(norm, 1e-12) from the squared
+    norm in fp32 (0 where it overflows), the product of a src token with a weighted dst token, weighted by the src token's own weight.  Returns the weighted
+    products [src][dst] and the weights of the src tokens."""
+    with np.errstate(all="ignore"):
+        w = np.minimum(1.0 / np.sqrt((x * x).sum(1).astype(np.float32).astype(np.float64)), 1e12)
+        return x[src] @ (x[dst] * w[dst, None]).T, w[src]
+
+
+@pytest.mark.parametrize("dst_scale", [0, 27, -74])
+@pytest.mark.parametrize("src_scale", [-74, 68, 98, 120])
+def test_products_that_fp32_does_not_hold(src_scale, dst_scale):
+    """Every third src token times 2^src_scale, every dst token times 2^dst_scale (rows of norms around 5): their products leave fp32's range, but the
+    products with dst tokens of norm one do not.  A src token goes to the dst token of the largest weighted product; one whose squared
+    norm overflows has weight 0 and similarity 0: it merges behind the others, such tokens in position order."""
+    n, heads = 900, 2
+    r = int(0.7 * n)
+    wl = synth.Workload("range", 1, 1, n, 1, 1, n, 0.7, 0.7, n_camera=0, n_register=0, heads=heads, seed=3)
+    gen = np.random.default_rng(21)
+    x = (0.25 + gen.random((heads, n, 64))).astype(np.float32)
+    nd = n // 4
+    dst = np.array([j for j in range(n) if (j + 1) * nd // n > j * nd // n])
+    src = np.setdiff1d(np.arange(n), dst)
+    far = src[::3]
+    assert len(src) - len(far) < r < len(src)   # some of the scaled tokens merge, some do not
+    x[:, far] *= 2.0 ** src_scale
+    x[:, dst] *= 2.0 ** dst_scale
+    t = torch.from_numpy(x).bfloat16().to(DEV)
+    good = torch.from_numpy((0.25 + gen.random(x.shape)).astype(np.float32)).bfloat16().to(DEV)
+    with hb.Httm(hb.HttmConfig.of(wl)) as ctx:
+        ctx.global_attention(t, t, good)
+        torch.cuda.synchronize()
+        assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+        maps = ctx.export(hb.X_ASSIGN_Q), ctx.export(hb.X_ASSIGN_K)
+    rows = t.double().cpu().numpy()
+    for h in range(heads):
+        prod, w = similarities(rows[h], src, dst)
+        best, key = prod.max(1), prod.max(1) * w
+        for m in maps:
+            to = m[h][src]
+            merged = to != src
+            assert merged.sum() == r and (m[h][dst] == dst).all() and np.isin(to[merged], dst).all()
+            mine = prod[np.flatnonzero(merged), np.searchsorted(dst, to[merged])]
+            assert (mine >= best[merged] * (1 - 1e-5)).all(), (h, (1 - mine / best[merged]).max())
+            assert key[merged].min() >= key[~merged].max() - 1e-5 * abs(key).max()
+            if src_scale > 64:   # weight 0: equal similarities, the lowest positions merge
+                tied = np.flatnonzero(w == 0)
+                assert len(tied) == len(far) and (np.diff(merged[tied].astype(int)) <= 0).all()
+
+
+@pytest.mark.parametrize("dst_scale", [0, 27])
+def test_infinite_src_tokens_merge_first(dst_scale):
+    """An infinite src token: its weight is 0, its similarity 0 x infinity, whose key orders above all numbers, as in the kernels of smaller blocks.
+    All its products are infinite here: the lowest dst token."""
+    n, heads = 900, 2
+    wl = synth.Workload("infinite", 1, 1, n, 1, 1, n, 0.5, 0.5, n_camera=0, n_register=0, heads=heads, seed=3)
+    gen = np.random.default_rng(22)
+    x = (0.25 + gen.random((heads, n, 64))).astype(np.float32)
+    nd = n // 4
+    dst = np.array([j for j in range(n) if (j + 1) * nd // n > j * nd // n])
+    src = np.setdiff1d(np.arange(n), dst)
+    far, near = src[5::7], np.setdiff1d(src, src[5::7])
+    x[:, dst] *= 2.0 ** dst_scale
+    x[:, far] = np.inf
+    t = torch.from_numpy(x).bfloat16().to(DEV)
+    good = torch.from_numpy((0.25 + gen.random(x.shape)).astype(np.float32)).bfloat16().to(DEV)
+    with hb.Httm(hb.HttmConfig.of(wl)) as ctx:
+        ctx.global_attention(t, t, good)
+        torch.cuda.synchronize()
+        assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+        maps = ctx.export(hb.X_ASSIGN_Q), ctx.export(hb.X_ASSIGN_K)
+    rows = t.double().cpu().numpy()
+    for h in range(heads):
+        prod, w = similarities(rows[h], near, dst)
+        key = prod.max(1) * w
+        for m in maps:
+            assert (m[h][far] == dst[0]).all()
+            merged = m[h][near] != near
+            assert merged.sum() == n // 2 - len(far)
+            assert key[merged].min() >= key[~merged].max() - 1e-5
