@@ -11,6 +11,8 @@
 //   big_merge_kernel    mean of every group (Sec. 3.2): tokens sorted by (merged row, position), one warp
 //                       gathers the members of a row in that order; writes merged Q / K / V and rank_q
 // All three read the reordered copies (a block is a contiguous run of rows there).
+#include <cfloat>
+
 #include "httm_internal.h"
 #include "httm_launch.cuh"
 #include "tc_sm100.cuh"
@@ -109,6 +111,14 @@ __device__ __forceinline__ uint32_t scale_bf16x2(uint32_t v, float s) {
     const __nv_bfloat162 r = __floats2bfloat162_rn(__uint_as_float(v << 16) * s, __uint_as_float(v & 0xffff0000u) * s);
     return *reinterpret_cast<const uint32_t*>(&r);
 }
+__device__ __forceinline__ bool zero_row(const __nv_bfloat16* x) {
+    uint32_t any = 0;
+    for (int c = 0; c < 8; ++c) {
+        const uint4 v = ld_global(reinterpret_cast<const uint4*>(x) + c);
+        any |= v.x | v.y | v.z | v.w;
+    }
+    return (any & 0x7fff7fffu) == 0;
+}
 __device__ __forceinline__ void load_async(uint32_t dst, const void* src) {   // 16 bytes
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
@@ -134,13 +144,14 @@ struct Ramp {
 // A token's best dst so far: its score, the first dst of the group of eight that holds it, and the scores of that group, which tell the
 // dst itself once at the end.  The eight scores are carried along by multiplying with zeros and ones on the FMA pipe, which has time:
 // looking for the column whenever a row of the warp improves (in nearly every group) takes two cycles of the ALU for each of 75
-// selects and compares, and the ALU has the maxima to take.  A score that is not finite spoils the eight (0 x inf): the dst is then
-// looked for again (find_again).
+// selects and compares, and the ALU has the maxima to take.  A score that is not finite would spoil its place among the
+// eight for good (0 x inf): in blocks that can have such scores they are brought inside fp32's range first (finite_score).
 constexpr int kGroup = 8;
 struct Best {
     float score, first_dst;   // (-1: none)
     float2 v[kGroup / 2];
 };
+__device__ __forceinline__ float finite_score(float s) { return fminf(fmaxf(s, -FLT_MAX), FLT_MAX); }   // -FLT_MAX where s is not a number
 __device__ __forceinline__ void take_best(Best& best, float (&s)[32], int first_dst, int valid) {   // dst first_dst + c, c < valid
     if (valid < 32) {   // the block's last dst tokens: -inf for the maxima, zeros for what is carried along
 #pragma unroll
@@ -177,32 +188,6 @@ __device__ __forceinline__ void take_best(Best& best, float (&s)[32], int first_
         best.v[c] = v;
     }
 }
-// The dst tokens of one column half again, one by one, for a token whose eight scores have been spoilt: the best that is a number,
-// ties to the lowest.
-__device__ __noinline__ int find_again(const __nv_bfloat16* x, const unsigned char* dst, const float* w, int half, int nd) {
-    float best = -INFINITY;
-    int arg = 0;
-    for (int d = half * 64; d < nd; d += (d & 63) == 63 ? 65 : 1) {
-        float s = 0.f;
-        for (int c16 = 0; c16 < 8; ++c16) {
-            const uint4 a = ld_global(reinterpret_cast<const uint4*>(x) + c16);
-            const uint4 b = *reinterpret_cast<const uint4*>(dst + d * kRowBytes + ((c16 ^ (d & 7)) << 4));
-            const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                s = fmaf(__uint_as_float(aw[e] << 16), __uint_as_float(bw[e] << 16), s);
-                s = fmaf(__uint_as_float(aw[e] & 0xffff0000u), __uint_as_float(bw[e] & 0xffff0000u), s);
-            }
-        }
-        s *= w[d];
-        if (s > best) {
-            best = s;
-            arg = d;
-        }
-    }
-    return arg;
-}
-
 __global__ void __launch_bounds__(SC_THREADS, 1)
 big_scores_kernel(const BigMatchArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -376,18 +361,19 @@ big_scores_kernel(const BigMatchArgs a) {
                 for (int d = at >> 3; d < rows; d += kRowsPerPass, pos.next())
                     load_async(s_b + d * kRowBytes + ((c16 ^ (d & 7)) << 4), x + (int64_t)pos.value * kHeadDim + c16 * 8);
             }
-            // Is any norm of the block, of a src or a dst token, outside 2^-39 .. 2^40?  (A weight is at most 1e12, just below 2^40; 0: the squared norm
-            // overflowed.)  Inside, every product lies in 2^+-80.
+            // Is any norm of the block, of a src or a dst token, outside 2^-39 .. 2^40 and not zero?  (A weight is at most 1e12, just below 2^40, where the
+            // token is zero, tiny or not a number; 0: the squared norm overflowed.)  Inside, every product lies in 2^+-80.
             bool far = false;
             const int n_all = rows > 0 ? nd + n_src : 0;
 #pragma unroll 4
             for (int j = at; j < n_all; j += SC_THREADS - 128) {
                 const float w = ld_global(inv + j);
-                far |= !(w >= 0x1p-40f && w <= 0x1p39f);
+                far |= w < 0x1p-40f || (w > 0x1p39f && !zero_row(x + (int64_t)j * kHeadDim));
             }
             asm volatile("cp.async.wait_all;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor cores read the rows through the async proxy
-            if (__syncthreads_or(far)) {
+            const bool any_far = __syncthreads_or(far);
+            if (any_far) {
                 // All dst tokens are scaled by a power of two to norms in (1/2, 1], those below the clamp by 2^39: no product with them is beyond the
                 // src token's own norm, and none is lost below fp32's range where the weighted one would not be.
                 for (int d = at; d < rows; d += SC_THREADS - 128) {
@@ -445,6 +431,12 @@ big_scores_kernel(const BigMatchArgs a) {
                                 s[e][c + 3] = hi.y;
                             }
                         }
+                        if (any_far) {   // (such blocks only: 64 more instructions of the ALU, 7 % of the call at 82 440 tokens if it is all of them)
+#pragma unroll
+                            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                                for (int c = 0; c < 32; ++c) s[e][c] = finite_score(s[e][c]);
+                        }
                         take_best(best[0], s[0], first_dst, nd - first_dst);
                         take_best(best[1], s[1], first_dst, nd - first_dst);
                     }
@@ -455,16 +447,16 @@ big_scores_kernel(const BigMatchArgs a) {
                 for (int e = 0; e < 2; ++e) {
                     const int s = (2 * p + e) * TILE + row;   // src token
                     own[e] = s < n_src ? src_position(s) : -1;   // token number inside the block
-                    int in_group = kGroup;
+                    int in_group = 0;
 #pragma unroll
                     for (int c = kGroup - 1; c >= 0; --c)
                         if ((c & 1 ? best[e].v[c >> 1].y : best[e].v[c >> 1].x) == best[e].score) in_group = c;
-                    if (best[e].first_dst < 0.f)
-                        arg[e] = 0;   // (no score is a number)
-                    else if (in_group < kGroup)
-                        arg[e] = (int)best[e].first_dst + in_group;
-                    else
-                        arg[e] = own[e] >= 0 ? find_again(x + (int64_t)own[e] * kHeadDim, smem, w_s, half, nd) : 0;
+                    arg[e] = (int)best[e].first_dst + in_group;
+                    if (best[e].score == FLT_MAX) best[e].score = INFINITY;   // (see finite_score)
+                    if (best[e].score <= -FLT_MAX) {   // no score is a number
+                        best[e].score = -INFINITY;
+                        arg[e] = 0;
+                    }
                 }
                 // the two column halves of a token meet: half 1 hands (best, arg) over, half 0 decides (ties: lowest dst)
                 const uint32_t turn = pairs_done++ & 1u;

@@ -287,3 +287,32 @@ def test_infinite_src_tokens_merge_first(dst_scale):
             merged = m[h][near] != near
             assert merged.sum() == n // 2 - len(far)
             assert key[merged].min() >= key[~merged].max() - 1e-5
+
+
+@pytest.mark.parametrize("column", [0, 5])
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")], ids=["infinite", "not_a_number"])
+@pytest.mark.parametrize("first", [16, 72, 200], ids=["same_part", "other_half", "later_chunk"])
+def test_equal_best_dst_tokens_beside_one_without_a_similarity(first, bad, column):
+    """Src tokens equal to two dst tokens among eight neighbours, and a dst token without a similarity at the first one's place among
+    eight others: they go to the first of the two."""
+    n, heads = 1100, 2
+    wl = synth.Workload("spoilt_ties", 1, 1, n, 1, 1, n, 0.75, 0.75, n_camera=0, n_register=0, heads=heads, seed=3)
+    gen = np.random.default_rng(23)
+    x = gen.standard_normal((heads, n, 64)).astype(np.float32)
+    nd = n // 4
+    dst = np.array([j for j in range(n) if (j + 1) * nd // n > j * nd // n])
+    src = np.setdiff1d(np.arange(n), dst)
+    low, high = dst[first + column], dst[first + 7]
+    same = src[::5]
+    x[:, high] = x[:, low]
+    x[:, same] = x[:, low][:, None]
+    x[:, dst[column + (64 if first > 64 else 0)]] = bad
+    t = torch.from_numpy(x).bfloat16().to(DEV)
+    good = torch.from_numpy(gen.standard_normal(x.shape).astype(np.float32)).bfloat16().to(DEV)
+    with hb.Httm(hb.HttmConfig.of(wl)) as ctx:
+        ctx.global_attention(t, t, good)
+        torch.cuda.synchronize()
+        assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+        maps = ctx.export(hb.X_ASSIGN_Q), ctx.export(hb.X_ASSIGN_K)
+    for m in maps:
+        assert (m[:, same] == low).all()
