@@ -8,6 +8,7 @@ has no dependency on torch's copy.
 from __future__ import annotations
 
 import os
+import re
 import subprocess
 import sys
 from concurrent.futures import ThreadPoolExecutor
@@ -23,6 +24,16 @@ NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
 ]
+
+# Their kernels change the registers of their warps as they run (setmaxnreg).  A function that is called does not know how many its caller has
+# left: in such a file everything has to be inlined.
+NO_CALLS = ("httm_big_blocks.cu",)
+
+
+def called_functions(ptxas_log: str) -> list[str]:
+    """The device functions, other than kernels, for which ptxas -v lists properties: those that were not inlined everywhere."""
+    kernels = set(re.findall(r"Compiling entry function '([^']+)'", ptxas_log))
+    return [name for name in re.findall(r"Function properties for (\S+)", ptxas_log) if name not in kernels]
 
 
 def _nvcc() -> str:
@@ -42,16 +53,16 @@ def build(force: bool = False, verbose: bool = False) -> str:
         return LIB
     os.makedirs(OBJ_DIR, exist_ok=True)
     nvcc = _nvcc()
-    extra = ["-Xptxas", "-v"] if verbose else []
-
     def compile_one(src: str) -> str:
         obj = os.path.join(OBJ_DIR, src.replace(".cu", ".o"))
-        cmd = [nvcc, *NVCC_FLAGS, *extra, "-I", INCLUDE, "-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [nvcc, *NVCC_FLAGS, "-Xptxas", "-v", "-I", INCLUDE, "-c", os.path.join(CSRC, src), "-o", obj]
         res = subprocess.run(cmd, capture_output=True, text=True)
         if verbose or res.returncode != 0:
             sys.stderr.write(res.stdout + res.stderr)
         if res.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}")
+        if src in NO_CALLS and called_functions(res.stdout + res.stderr):
+            raise RuntimeError(f"{src}: not inlined: {called_functions(res.stdout + res.stderr)}")
         return obj
 
     with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:

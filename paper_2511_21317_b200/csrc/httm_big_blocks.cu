@@ -46,7 +46,8 @@ __device__ __forceinline__ bool is_dst_position(int j, int n_rule, int nd) {
 //    beside the dst tokens;
 //  - work items (tensor, head, block) are taken from a counter, the longest first (dealt in rounds one tensor after the other, the longest of
 //    148 CTAs had 15 % more than the mean), and an issuing warp for each group (one for both kept them in step: 437 us).
-// The four warps of the roles run with 32 registers: nothing they run may be a function of its own, which would not know of that.
+// The four warps of the roles run with 32 registers: nothing they run may be a function of its own, which would not know of that (build.py fails
+// where the compiler has made one).
 // Measured at 16 heads x 22 blocks of up to 3840 tokens, 384 dst tokens of the queries and 960 of the keys: 611 us with the dst tokens split into three
 // scaled planes, 256 at a time, and one group of warps; 467 us with all tokens as rows; 426 us now.  The dst tokens chosen are closer to the best in 64 bits
 // (1.6 million tokens of three scenes: 26 off the best by up to 4.6e-7 before, 6 by up to 1.2e-7).  Tried and dropped: 64 and 104 registers (456 us),
@@ -244,13 +245,13 @@ big_scores_kernel(const BigMatchArgs a) {
                 Ramp before((at >> 3) * it.nd, SC_LOADERS / 8 * it.nd, max(it.n_src, 1));
                 int s = at >> 3, handed = 0, hand_st = 0;   // next src token of this thread; tiles handed over, stage of the next
                 uint32_t par = fills;
-                auto hand_over = [&]() {
+                auto hand_over = [&]() __attribute__((always_inline)) {
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor cores read the rows through the async proxy
                     tc::mbar_arrive(tc::smem_addr(&bars->a_full[hand_st]));
                     ++handed;
                     if (++hand_st == it.stages) hand_st = 0;
                 };
-                auto load_tile = [&](int st) {
+                auto load_tile = [&](int st) __attribute__((always_inline)) {
                     if (!__all_sync(0xffffffffu, tc::mbar_wait(tc::smem_addr(&bars->a_empty[st]), (par >> st & 1u) ^ 1u, abort_flag))) return false;
                     par ^= 1u << st;
                     const uint32_t dst = s_b + it.ring + st * TILE_BYTES;
@@ -1085,7 +1086,11 @@ cudaError_t configure_sorted_group_kernels() {
 }
 
 cudaError_t configure_big_blocks() {
-    cudaError_t e = cudaFuncSetAttribute(big_scores_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM);
+    // setmaxnreg.inc takes registers from those the CTA was launched with, and waits without limit for more than there are
+    cudaFuncAttributes launched;
+    cudaError_t e = cudaFuncGetAttributes(&launched, big_scores_kernel);
+    if (e == cudaSuccess && launched.numRegs * SC_THREADS < 128 * kScoreRoleRegs + (SC_THREADS - 128) * kScoreMaxRegs) e = cudaErrorInvalidConfiguration;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(big_scores_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM);
     if (e == cudaSuccess) e = configure_sorted_group_kernels<64, 4>();
     if (e == cudaSuccess) e = configure_sorted_group_kernels<128, 4>();
     if (e == cudaSuccess) e = configure_sorted_group_kernels<256, 4>();
