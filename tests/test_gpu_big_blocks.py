@@ -1,5 +1,7 @@
 """Parity of the large-block path (merging blocks of 257 .. 4096 tokens: the paper's runs of 128 tokens over 30
 frames, Sec. 3.3 / 4.1) with the CPU oracle.  All tests here need a B200."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -316,3 +318,26 @@ def test_equal_best_dst_tokens_beside_one_without_a_similarity(first, bad, colum
         maps = ctx.export(hb.X_ASSIGN_Q), ctx.export(hb.X_ASSIGN_K)
     for m in maps:
         assert (m[:, same] == low).all()
+
+
+@pytest.mark.parametrize("ratio_q,ratio_kv,anchor", [(0.9, 0.7, 0), (0.0, 0.5, 0), (0.6, 0.7, 1)], ids=["five_stages", "queries_not_merged", "anchored"])
+def test_several_blocks_per_cta_agree_with_one(ratio_q, ratio_kv, anchor):
+    """The score kernel's CTAs take blocks from a counter and carry the state of their rings and buffers from one to the next: 18 blocks (ten of 4096 tokens, of up to
+    1024 dst tokens; two of 96, five of 128, one of 3) x 16 heads x 2 tensors are four per CTA.  One head at a time every CTA takes at most one: the same maps."""
+    wl = synth.Workload("several", 65, 1, 643, 32, 1, 128, ratio_q, ratio_kv, n_camera=1, n_register=0, heads=16, seed=3)
+    gen = torch.Generator(device=DEV).manual_seed(5)
+    q, k, v = (torch.randn(wl.heads, wl.n_tokens, 64, generator=gen, device=DEV).bfloat16() for _ in range(3))
+
+    def maps(*tensors):
+        ctx.global_attention(*tensors)
+        torch.cuda.synchronize()
+        assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+        return ctx.export(hb.X_ASSIGN_Q), ctx.export(hb.X_ASSIGN_K)
+
+    with hb.Httm(dataclasses.replace(hb.HttmConfig.of(wl), anchor_first_frame=anchor)) as ctx:
+        together = maps(q, k, v)
+    with hb.Httm(dataclasses.replace(hb.HttmConfig.of(wl.replace(heads=1)), anchor_first_frame=anchor)) as ctx:
+        for h in range(wl.heads):
+            alone = maps(q[h:h + 1], k[h:h + 1], v[h:h + 1])
+            for m, one in zip(together, alone):
+                assert np.array_equal(m[h], one[0]), h
