@@ -194,7 +194,7 @@ __device__ __noinline__ RedoneTile redo_score_tile(const __nv_bfloat16* q_row, c
 // into P = G / e parts of the keys, one per CTA: a part is a single pass over n / P key tiles that leaves its unnormalised
 // output, maxima and sums in a workspace, and the warp whose part of its rows arrives last adds them up (nobody waits).  A part
 // costs about kPartCost key tiles besides its own, and single passes for all CTAs and then parts kPassCost more than a round
-// of pairs, hence the rule (3.03 tiles per SM of 28 key tiles: whole 127 us, split 143).  Where the tiles are not split and more than G remain they
+// of pairs, hence the rule (3.03 tiles per SM of 28 key tiles: whole 113 us a call, split 121).  Where the tiles are not split and more than G remain they
 // go as one more (partial) round of pairs, which takes the same time as two rounds of single passes.
 // Measured (whole call, before / after): 9.19 tiles per SM of 83 key tiles 732 / 698 us, 14.05 of 195 3038 / 2922 us.
 constexpr int kPartCost = 14, kPassCost = 10, kMinPart = 8;
@@ -321,7 +321,7 @@ __device__ __forceinline__ int count_mod3(int n, int r) { return (n - r + 2) / 3
 // Where the 32 output rows of a softmax warp go: row `grow` of a thread goes to row `grow` of the merged output.
 template <bool UNMERGE>
 struct RowTargets {
-    bool valid;   // (a flag of its own: with row -1 in place of it 7 898 tokens x 16 heads took 93.0 us a call, so 92.7)
+    bool valid;
     int row;
 };
 // UNMERGE (Eq. 5-7 folded into the epilogue): row `grow` is the attention output of a merged query and goes to every original token of its

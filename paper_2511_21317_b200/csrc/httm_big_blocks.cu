@@ -2,10 +2,10 @@
 // n_s = 128 tokens over n_t = 30 frames, 3840 tokens per block (Sec. 3.3, Sec. 4.1).  A block no longer fits one
 // warp's stage, and its similarity step (Eq. 1) is a real dense contraction: n tokens x n_dst dst tokens x 64.
 //
-//   big_scores_kernel   cosine of every token of a block with every dst token of the block on the 5th-generation
+//   big_scores_kernel   cosine of every src token of a block with every dst token of the block on the 5th-generation
 //                       tensor cores (tcgen05.mma, accumulators in tensor memory), fused with the row-wise
-//                       arg-max, which weighs the products by the dst tokens' inverse norms: per token the best dst
-//                       and the best cosine
+//                       arg-max, which weighs the products by the dst tokens' inverse norms: per src token the best dst
+//                       and the best cosine (nothing is written for dst tokens and for blocks in which nothing merges)
 //   big_select_kernel   the r src tokens with the best cosines merge (Sec. 3.2): exact radix select per block,
 //                       ties by position; writes the assignment map
 //   big_merge_kernel    mean of every group (Sec. 3.2): tokens sorted by (merged row, position), one warp
@@ -38,7 +38,7 @@ __device__ __forceinline__ bool is_dst_position(int j, int n_rule, int nd) {
 // cos(i, d) |x_i| = w_d sum_k x_ik x_dk with w_d = 1 / max(|x_d|, 1e-12).  The products of bf16 values are exact in fp32 and add up in
 // tensor memory; the arg-max warps multiply by w_d (one rounding).  All dst tokens of a block (at most 1024: 128 KB) stay in shared
 // memory, so a token tile is loaded once and its best so far stays in registers.  What bounds it is the arg-max warps' instruction issue and
-// latency (the MMAs of a pair of tiles and 128 dst tokens take 512 cycles, the warps about 2300 of two groups at work), hence:
+// latency (a pair of tiles and 128 dst tokens takes an SM about 2500 cycles, 512 of them MMAs: 46 656 such steps on 148 SMs in 407 us at 1.96 GHz), hence:
 //  - a warp works on TWO token tiles at a time: the data of a broadcast load of weights goes to every lane, four cycles of the SM's
 //    shared-memory port for four columns, and is used twice this way;
 //  - two groups of eight warps, each with a score buffer for a pair of tiles and 128 dst tokens (one group: 515 us);
@@ -49,7 +49,9 @@ __device__ __forceinline__ bool is_dst_position(int j, int n_rule, int nd) {
 // The four warps of the roles run with 32 registers: nothing they run may be a function of its own, which would not know of that (build.py fails
 // where the compiler has made one).
 // Measured at 16 heads x 22 blocks of up to 3840 tokens, 384 dst tokens of the queries and 960 of the keys: 611 us with the dst tokens split into three
-// scaled planes, 256 at a time, and one group of warps; 467 us with all tokens as rows; 426 us now.  The dst tokens chosen are closer to the best in 64 bits
+// scaled planes, 256 at a time, and one group of warps; 467 us with all tokens as rows; 426 us with a function for scores that had been spoilt; 407 us now.
+// It spills all the same: ptxas gives the kernel the 96 registers of its launch, and the scores of two tiles with two Best do not fit (254 bytes stored, 368
+// loaded per thread).  The dst tokens chosen are closer to the best in 64 bits
 // (1.6 million tokens of three scenes: 26 off the best by up to 4.6e-7 before, 6 by up to 1.2e-7).  Tried and dropped: 64 and 104 registers (456 us),
 // no carrying along where no row of the warp improves (491 us at 467).
 constexpr int TILE = 128;                        // rows of an operand tile, dst tokens of a chunk
@@ -903,7 +905,8 @@ __global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const M
 // kernel.  One CTA per (head, block).
 
 // eps[h][p] = || q_p - mean of the group p was merged into ||_2 in fp32; 0 for a token on its own.
-// Bound by the instructions issued (61 warp instructions per token): two channels per instruction, one exchange for the sums of four
+// Bound by the instructions issued and by the gathers (39 warp instructions per token, 61 before; at 40 registers 92 bytes per thread are spilled
+// with 8 tokens per thread): two channels per instruction, one exchange for the sums of four
 // members and one square root for them took the filter kernels together, at 82 440 tokens x 16 heads in 3840-token blocks, from 221 to 178 us
 // (32 976 tokens in 128-token blocks: 104.7 -> 92.2; 137 400 in 64-token blocks: 363 -> 302).
 template <int T, int E>

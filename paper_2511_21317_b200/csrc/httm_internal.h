@@ -75,8 +75,9 @@ struct ReorderArgs {
 struct BigMatchArgs {
     const __nv_bfloat16* xr[2];   // reordered Q, K [H][N][64]
     const float* inv_norm[2];     // [H][N]
-    uint32_t* best_key[2];        // [H][N] order-preserving key of every token's best cosine to a dst token
-    int32_t* best_pos[2];         // [H][N] token number, inside the block, of that dst
+    uint32_t* best_key[2];        // [H][N] order-preserving key of a src token's best cosine to a dst token; the score kernel writes the src tokens of
+                                  // blocks in which something merges, all other entries are undefined
+    int32_t* best_pos[2];         // [H][N] token number, inside the block, of that dst; written and undefined alike
     int32_t* assign[2];           // [H][N] out (select kernel)
     const BlockInfo* blocks;
     const int32_t* order;         // [blocks] from the longest to the shortest
