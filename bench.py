@@ -404,14 +404,14 @@ def run_ours(args, wl):
         attn_flops = 4.0 * H * Mq * Mk * D
         alg["match_direct"], alg["merge_direct"] = alg["match"], alg["merge"]
         alg["big_select"] = 2 * H * N * (4 + 4 + 4)   # keys and best dst read, map written
-        # the large-block score kernel is a contraction: every token of a block against the block's dst tokens
+        # the large-block score kernel is a contraction: every src token of a block against the block's dst tokens
         big_flops = 0.0
         if big:
             for n in np.diff(ctx.export(hb.X_BLOCK_START).astype(np.int64)):
                 for ratio in (wl.ratio_q, wl.ratio_kv):
                     r = min(int(np.floor(ratio * n + 1e-9)), n - 1)
                     nd = min(-(-n // 4), n - r)
-                    big_flops += 2.0 * H * n * nd * D if r > 0 else 0.0
+                    big_flops += 2.0 * H * (n - nd) * nd * D if r > 0 else 0.0
         kernels = {}
         for st in order:
             name, ms = hb.STAGE_NAMES[st], float(stage_ms[st])
