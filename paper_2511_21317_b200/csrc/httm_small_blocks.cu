@@ -10,7 +10,8 @@
 //   - K's groups serve V, and the maps are read once per unit;
 //   - results leave through the stage as whole rows instead of 4 bytes per lane.
 // Measured at 32 976 tokens x 16 heads, 32-token blocks: match 53 -> 39.6 us, merge 69.6 -> 62.4 us (both
-// with the interval between two events).
+// with the interval between two events).  What is left is the latency of a warp's instruction stream, hence as few instructions as possible
+// (match: one token per lane from the arg-max on) and as many warps as fit (merge: two stages and 80 registers, 24 warps per SM).
 #include "httm_blocks.cuh"
 #include "httm_launch.cuh"
 
@@ -28,7 +29,9 @@ constexpr uint32_t kStage = 32 * kRowBytes;   // one block of one tensor, 128-by
 // merge; ties go to the lowest dst and the lowest src position.  The dot products and the squared norms (diagonals of a tile
 // against itself) are m16n8k16 MMAs on ldmatrix fragments of the swizzled stage; the dst rows are gathered by giving
 // ldmatrix their addresses.  Products of bf16 values are exact in fp32.
-// Row rho of the stage is owned, from the arg-max on, by lane (rho & 7) * 4 + ((rho >> 3) & 1), slot rho >> 4.
+// (Every lane owns one token when the r best are chosen.  With two tokens in every other lane a tensor took 518 instructions, now 441, and the kernel alone, one launch
+// at a time, 39.3 -> 34.8 us at 32 976 tokens; between the other kernels of a call 40.8 -> 40.4, 65 952 tokens 82.9 -> 72.7.)
+// Row rho of the stage is owned, from the arg-max on, by lane (rho & 7) * 4 + (rho >> 3).
 constexpr int kMatchSmem = kWarps * (2 * (int)kStage + 16) + 1024 /*alignment slack*/;
 
 // SPLIT: fewer units than warps: a warp has one tensor of one unit
@@ -38,7 +41,8 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + align_pad(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 2, tq = lane & 3, odd = tq & 1;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
+    const int g = lane >> 2, tq = lane & 3;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
+    const int rho = 8 * tq + g;                // the stage row this lane owns
     const uint32_t stage0 = smem_u32(smem + (size_t)warp * 2 * kStage);
     const uint32_t bar0 = smem_u32(smem + (size_t)kWarps * 2 * kStage + warp * 16);
     if (lane == 0) {
@@ -95,8 +99,8 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     int shape_a = -1, shape_b = -1;
     uint32_t d_off[2] = {0, 0};   // ldmatrix offsets of dst row lane & 7
     int d_pos = 0;                // token number of dst lane & 7
-    int tok[2] = {-1, -1};        // tokens owned (-1: none)
-    bool is_src[2] = {false, false};
+    int tok = -1;                 // token owned (-1: none)
+    bool is_src = false;
 
     int it = 0;
     bool failed = false;
@@ -135,13 +139,8 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     const int row = DIRECT ? row_of_token(box, bg, d_pos) : d_pos;
 #pragma unroll
                     for (int kp = 0; kp < 2; ++kp) d_off[kp] = row * kRowBytes + (((4 * kp + (lane >> 3)) ^ (row & 7)) << 4);
-#pragma unroll
-                    for (int mt = 0; mt < 2; ++mt) {
-                        const int rho = mt * 16 + odd * 8 + g;
-                        const int j = DIRECT ? token_of_row(box, bg, rho) : (rho < n ? rho : -1);
-                        tok[mt] = tq < 2 ? j : -1;
-                        is_src[mt] = tok[mt] >= 0 && !(j < n_rule && small_div((j + 1) * nd, n_rule) > small_div(j * nd, n_rule));
-                    }
+                    tok = DIRECT ? token_of_row(box, bg, rho) : (rho < n ? rho : -1);
+                    is_src = tok >= 0 && !(tok < n_rule && small_div((tok + 1) * nd, n_rule) > small_div(tok * nd, n_rule));
                 }
             }
             const uint32_t blk = stage0 + t * kStage;
@@ -169,11 +168,24 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             float w0 = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq)), w1 = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq + 4));
             if (2 * tq >= nd) w0 = CUDART_NAN_F;
             if (2 * tq + 1 >= nd) w1 = CUDART_NAN_F;
-            // ---- best dst of every row
-            uint32_t key[2] = {0u, 0u};
-            int best[2] = {0, 0};
+            // ---- best dst of every row.  The four lanes of a row meet: an exchange with lane ^ 1 leaves a lane one of a tile's rows g and g + 8, one with
+            // lane ^ 2 one of the two tiles
+            const bool odd = tq & 1, high = tq & 2;
+            auto meet = [](float& top, int& arg, float send, int send_arg, int with) {
+                const float ov = __shfl_xor_sync(0xffffffffu, send, with);
+                const int oa = __shfl_xor_sync(0xffffffffu, send_arg, with);
+                if (ov > top || (ov == top && oa < arg)) {   // (ties: the lower dst)
+                    top = ov;
+                    arg = oa;
+                }
+            };
+            float top[2], norm[2];
+            int arg[2];
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt) {
+                top[mt] = -INFINITY;
+                norm[mt] = 0.f;
+                arg[mt] = 0;
                 if (mt * 16 < n_rows) {   // warp-uniform
                     float c[4], lo[4], hi[4];
 #pragma unroll
@@ -190,69 +202,50 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                             mma_bf16_16816(hi, af, af[1], af[3]);
                         }
                     }
-                    // rows g and g + 8, this lane's two dst tokens (ties: the lower one)
+                    // this lane's two dst tokens first
                     // (the maximum with -infinity drops what is not a number: a place without a dst token, tokens whose norm overflows)
                     const float s00 = fmaxf(c[0] * w0, -INFINITY), s01 = fmaxf(c[1] * w1, -INFINITY);
                     const float s10 = fmaxf(c[2] * w0, -INFINITY), s11 = fmaxf(c[3] * w1, -INFINITY);
                     const float t0 = fmaxf(s00, s01), t1 = fmaxf(s10, s11);
                     const int d0 = 2 * tq + (s01 > s00 ? 1 : 0), d1 = 2 * tq + (s11 > s10 ? 1 : 0);
-                    // lanes 0, 1 of a row's four split the two rows, then meet lanes 2, 3
-                    float top = odd ? t1 : t0;
-                    int arg = odd ? d1 : d0;
-                    {
-                        const float ov = __shfl_xor_sync(0xffffffffu, odd ? t0 : t1, 1);
-                        const int oa = __shfl_xor_sync(0xffffffffu, odd ? d0 : d1, 1);
-                        if (ov > top || (ov == top && oa < arg)) {
-                            top = ov;
-                            arg = oa;
-                        }
-                    }
-                    {
-                        const float ov = __shfl_xor_sync(0xffffffffu, top, 2);
-                        const int oa = __shfl_xor_sync(0xffffffffu, arg, 2);
-                        if (ov > top || (ov == top && oa < arg)) {
-                            top = ov;
-                            arg = oa;
-                        }
-                    }
+                    top[mt] = odd ? t1 : t0;
+                    arg[mt] = odd ? d1 : d0;
+                    meet(top[mt], arg[mt], odd ? t0 : t1, odd ? d0 : d1, 1);
                     const int diag = 4 * g + (g >> 1);   // the lane that holds the squared norms of rows g and g + 8
                     const float nl = __shfl_sync(0xffffffffu, (g & 1) ? lo[1] : lo[0], diag), nh = __shfl_sync(0xffffffffu, (g & 1) ? hi[3] : hi[2], diag);
-                    key[mt] = score_key(top * inv_norm(odd ? nh : nl));
-                    best[mt] = arg;
+                    norm[mt] = odd ? nh : nl;
                 }
             }
+            float best_score = high ? top[1] : top[0];
+            int best = high ? arg[1] : arg[0];
+            meet(best_score, best, high ? top[0] : top[1], high ? arg[0] : arg[1], 2);
+            best_score *= inv_norm(high ? norm[1] : norm[0]);
+            const uint32_t key = score_key(best_score);
             __syncwarp();   // every lane has read the stage
             if (more && lane == 0) issue(t, bg_next, bi_next.start, h_next);
 
             // ---- the r src with the best scores merge (ties: lowest position first)
             const int n_out = n - nd - r;
-            bool merged[2];
-            const int rho0 = odd * 8 + g, rho1 = rho0 + 16;
+            bool merged;
             if (r <= n_out) {
-                merged[0] = merged[1] = false;
+                merged = false;
                 for (int round = 0; round < r; ++round) {
-                    const uint32_t k0 = is_src[0] && !merged[0] ? key[0] : 0u, k1 = is_src[1] && !merged[1] ? key[1] : 0u;
-                    const uint32_t m = __reduce_max_sync(0xffffffffu, max(k0, k1));
-                    const int win = __reduce_min_sync(0xffffffffu, k0 == m ? rho0 : (k1 == m ? rho1 : 0x7fffffff));   // lowest position holding it
-                    merged[0] = merged[0] || (is_src[0] && win == rho0);
-                    merged[1] = merged[1] || (is_src[1] && win == rho1);
+                    const uint32_t k = is_src && !merged ? key : 0u;
+                    const uint32_t m = __reduce_max_sync(0xffffffffu, k);
+                    const unsigned win = __reduce_min_sync(0xffffffffu, k == m ? (unsigned)rho : 0xffffffffu);   // lowest position holding it
+                    merged = merged || (is_src && win == (unsigned)rho);
                 }
             } else {
-                merged[0] = is_src[0];
-                merged[1] = is_src[1];
+                merged = is_src;
                 for (int round = 0; round < n_out; ++round) {
-                    const uint32_t k0 = merged[0] ? key[0] : 0xffffffffu, k1 = merged[1] ? key[1] : 0xffffffffu;
-                    const uint32_t m = __reduce_min_sync(0xffffffffu, min(k0, k1));
-                    const int win = __reduce_max_sync(0xffffffffu, merged[1] && k1 == m ? rho1 : (merged[0] && k0 == m ? rho0 : -1));   // highest position
-                    if (win == rho0) merged[0] = merged[0] && tq >= 2;
-                    if (win == rho1) merged[1] = merged[1] && tq >= 2;
+                    const uint32_t k = merged ? key : 0xffffffffu;
+                    const uint32_t m = __reduce_min_sync(0xffffffffu, k);
+                    const int win = __reduce_max_sync(0xffffffffu, merged && k == m ? rho : -1);   // highest position
+                    merged = merged && win != rho;
                 }
             }
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-                const int target = __shfl_sync(0xffffffffu, d_pos, best[mt]);
-                if (tok[mt] >= 0) A[tok[mt]] = bi.start + (merged[mt] ? target : tok[mt]);
-            }
+            const int target = __shfl_sync(0xffffffffu, d_pos, best);
+            if (tok >= 0) A[tok] = bi.start + (merged ? target : tok);
         }
         if (failed) break;
     }
@@ -265,28 +258,31 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 // The group sums of a block are one small dense contraction: merged_sum[kept row][channel] = sum_token W[row][token] x[token][channel]
 // with the 0/1 assignment matrix W (exact in bf16, built in registers from the map), fp32 accumulation, times the reciprocal
 // of the group size, one rounding to bf16.  Kept tokens are compacted in reordered order.  The rows go through the stage they came
-// from (its fragments are in registers by then) and leave 16 bytes per lane, whole rows; then the stage is refilled.
+// from, 16 channels at a time (whose fragments are in registers by then), and leave 16 bytes per lane, whole rows; then the stage is refilled.
+// Tensor i of the warp's sequence Q K V Q K V .. lies in stage i & 1.  With a stage for each tensor and all 64 channels in registers (128) 16 warps
+// fit on an SM: 61.4 -> 57.3 us at 32 976 tokens, 132 -> 115 at 65 952 (two stages and 16 warps: 66.6).
 constexpr int kMergeAux = 32 * 4 + 32 * 4 + 32 + 64;   // reciprocal group sizes, group sizes, 3 mbarriers, merged rows of the tokens
-constexpr int kMergeSmem = kWarps * (3 * (int)kStage + kMergeAux) + 1024 /*alignment slack*/;
+constexpr int kMergeStages = 2;
+constexpr int kMergeSmem = kWarps * (kMergeStages * (int)kStage + kMergeAux) + 1024 /*alignment slack*/;
 
 __device__ __forceinline__ void stmatrix_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
     asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
 }
 template <bool DIRECT, bool SPLIT>
-__global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __grid_constant__ MergeMaps maps, const __grid_constant__ MergeArgs a) {
+__global__ void __launch_bounds__(kWarps * 32, 3) merge_small_kernel(const __grid_constant__ MergeMaps maps, const __grid_constant__ MergeArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + align_pad(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tq = lane & 3;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
-    unsigned char* stage = smem + (size_t)warp * 3 * kStage;
-    unsigned char* aux = smem + (size_t)kWarps * 3 * kStage + (size_t)warp * kMergeAux;
+    unsigned char* stage = smem + warp * (kMergeStages * kStage);
+    unsigned char* aux = smem + kWarps * kMergeStages * kStage + warp * kMergeAux;
     float* rcnt = reinterpret_cast<float*>(aux);             // [32] 1 / group size of kept row
     int* gsz = reinterpret_cast<int*>(aux + 32 * 4);         // [32] size of kept row
     const uint32_t stage0 = smem_u32(stage), bar0 = smem_u32(aux + 2 * 32 * 4);
     __nv_bfloat16* rows_of = reinterpret_cast<__nv_bfloat16*>(aux + 2 * 32 * 4 + 32);   // [32] merged rows of the tokens, in fragment order
     if (lane == 0) {
 #pragma unroll
-        for (int t = 0; t < 3; ++t) mbar_init(bar0 + 8 * t, 1);
+        for (int st = 0; st < kMergeStages; ++st) mbar_init(bar0 + 8 * st, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     Box box{};
@@ -295,7 +291,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
     if (DIRECT)   // stage rows that no block load writes enter the MMAs with weight 0: they must hold finite values
         for (int q = box.rows * 8 + lane; q < 32 * 8; q += 32)
 #pragma unroll
-            for (int t = 0; t < 3; ++t) *reinterpret_cast<uint4*>(stage + t * kStage + q * 16) = make_uint4(0u, 0u, 0u, 0u);
+            for (int st = 0; st < kMergeStages; ++st) *reinterpret_cast<uint4*>(stage + st * kStage + q * 16) = make_uint4(0u, 0u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
 
@@ -339,8 +335,8 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
     auto fetch_offset = [&](Meta* m) {   // with outlier filtering the heads' rows start elsewhere
         if (a.moff_q_var && next.u < a.n_blocks) m->moff_q = ld_global(a.moff_q_var + (int64_t)m->h * a.n_blocks + next.u);
     };
-    auto issue = [&](int t, const Meta& m) {   // lane 0 only
-        const uint32_t mb = bar0 + 8 * t, dst = stage0 + t * kStage;
+    auto issue = [&](int t, uint32_t st, const Meta& m) {   // lane 0 only
+        const uint32_t mb = bar0 + 8 * st, dst = stage0 + st * kStage;
         if (!DIRECT) {
             mbar_expect_tx(mb, kStage);   // (rows past the head's end are zero filled)
             tma_rows_load(dst, &maps.block[t], mb, m.start, m.h);
@@ -370,8 +366,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
     auto issue_first = [&]() {
         if (first < n_units && lane == 0)
 #pragma unroll
-            for (int t = 0; t < 3; ++t)
-                if (!SPLIT || t == t_first) issue(t, meta_next);
+            for (int i = 0; i < (SPLIT ? 1 : 2); ++i) issue(t_first + i, i, meta_next);
     };
     if (a.early) issue_first();
     depend_wait();
@@ -386,9 +381,9 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
 
     const float recip = 1.0f / (float)(lane + 1);   // lane i holds 1 / (i + 1)
 
-    int it = 0;
-    bool failed = false;
-    for (int64_t unit = first; unit < n_units; unit += stride, ++it) {
+    uint32_t seq = 0;   // tensors so far: in stage seq & 1
+    bool failed = false, ahead = false;   // ahead: the next tensor's load is in flight too
+    for (int64_t unit = first; unit < n_units; unit += stride) {
         const Meta m = meta_next;
         const int target[2] = {target_next[0], target_next[1]};
         const bool more = unit + stride < n_units;
@@ -403,11 +398,12 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
         int row_of = -1, n_kept = 0;
         uint2 rw[2];
 #pragma unroll 1
-        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 2); ++t) {
+        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 2); ++t, ++seq) {
+            const uint32_t st = seq & 1u;
             const int r = m.r(t), moff = t == 0 ? m.moff_q : m.moff_k, m_len = t == 0 ? a.m_q : a.m_k;
             uint4* out = reinterpret_cast<uint4*>(a.merged[t] + ((int64_t)m.h * m_len + moff) * kHeadDim);
-            const uint32_t blk = stage0 + t * kStage;
-            const unsigned char* rows = stage + t * kStage;
+            const uint32_t blk = stage0 + st * kStage;
+            const unsigned char* rows = stage + st * kStage;
             int n_out = n;   // rows that leave
             if (r > 0 && (SPLIT || t < 2)) {   // the groups of this map (V follows K)
                 int rep = t == 0 ? target[0] : target[1];
@@ -459,8 +455,9 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
                     w_fragment(af0[ks], rw[ks], row_pair(g), row_pair(g + 8));
                 }
             }
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8 * t, it & 1, a.status, kDevTimeoutMatchLoad))) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8 * st, seq >> 1 & 1u, a.status, kDevTimeoutMatchLoad))) {
                 failed = true;
+                ahead = !SPLIT && (t < 2 || more);
                 break;
             }
             if (r == 0) {   // nothing merges here: the rows leave as they are
@@ -472,50 +469,39 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
                     }
                 }
             } else {
-                // x fragments: for k step ks (16 tokens) and channel tile pair np, one ldmatrix.x4.trans gives
-                // b0, b1 of channel tile 2 np and b0, b1 of channel tile 2 np + 1
-                uint32_t bf[2][4][4];
-#pragma unroll
-                for (int ks = 0; ks < 2; ++ks) {
-                    if (ks < n_ks) {
-                        const int j = 16 * ks + (lane & 15);
-#pragma unroll
-                        for (int np = 0; np < 4; ++np) ldmatrix_x4_trans(bf[ks][np], blk + j * kRowBytes + (((2 * np + (lane >> 4)) ^ (j & 7)) << 4));
-                    }
-                }
-                __syncwarp();   // every lane has its fragments: the stage takes the merged rows
+                // x fragments of 16 channels: for k step ks (16 tokens) one ldmatrix.x4.trans gives b0, b1 of channel tile 2 np and b0, b1 of
+                // channel tile 2 np + 1.  The merged rows take the same channels of the stage, so 16 channels at a time are in registers.
                 const int n_mt = n_kept > 16 ? 2 : 1;
-#pragma unroll 1
-                for (int mt = 0; mt < n_mt; ++mt) {
-                    const int r0 = 16 * mt + g, r1 = r0 + 8;   // this lane's two accumulator rows
-                    if (n_mt == 2) {   // (with one tile the fragments stay as they are)
-                        w_fragment(af0[0], rw[0], row_pair(r0), row_pair(r1));
-                        w_fragment(af0[1], rw[1], row_pair(r0), row_pair(r1));
-                    }
-                    float c[8][4];
+                const uint32_t from = blk + (lane & 15) * kRowBytes;
+                const float i0 = g < n_kept ? rcnt[g] : 0.f, i1 = g + 8 < n_kept ? rcnt[g + 8] : 0.f;
+                const int j = (lane & 7) + ((lane >> 4) << 3);   // row whose address this lane gives (matrices: rows 0-7 x two tiles, rows 8-15 x two)
 #pragma unroll
-                    for (int ks = 0; ks < 2; ++ks) {
-                        if (ks < n_ks) {
-                            uint32_t* af = af0[ks];
-#pragma unroll
-                            for (int nt = 0; nt < 8; ++nt) {
-                                if (ks == 0)
-                                    mma_first(c[nt], af, bf[ks][nt >> 1][2 * (nt & 1)], bf[ks][nt >> 1][2 * (nt & 1) + 1]);
-                                else
-                                    mma_bf16_16816(c[nt], af, bf[ks][nt >> 1][2 * (nt & 1)], bf[ks][nt >> 1][2 * (nt & 1) + 1]);
-                            }
+                for (int np = 0; np < 4; ++np) {
+                    uint32_t bf[2][4];
+                    const uint32_t chunk = ((2 * np + (lane >> 4)) ^ (lane & 7)) << 4, to = blk + j * kRowBytes + (((2 * np + ((lane >> 3) & 1)) ^ (lane & 7)) << 4);
+                    ldmatrix_x4_trans(bf[0], from + chunk);
+                    if (n_ks > 1) ldmatrix_x4_trans(bf[1], from + 16 * kRowBytes + chunk);
+                    __syncwarp();   // every lane has its fragments
+                    auto rows_out = [&](const uint32_t (&w)[2][4], int mt, float i0, float i1) {
+                        float p[2][4];
+                        mma_first(p[0], w[0], bf[0][0], bf[0][1]);
+                        mma_first(p[1], w[0], bf[0][2], bf[0][3]);
+                        if (n_ks > 1) {
+                            mma_bf16_16816(p[0], w[1], bf[1][0], bf[1][1]);
+                            mma_bf16_16816(p[1], w[1], bf[1][2], bf[1][3]);
                         }
-                    }
-                    // rows past the last kept one become zeros (not 0 x something: the stage must stay finite)
-                    const bool w0 = r0 < n_kept, w1 = r1 < n_kept;
-                    const float i0 = w0 ? rcnt[r0] : 0.f, i1 = w1 ? rcnt[r1] : 0.f;
-                    const int j = 16 * mt + (lane & 7) + ((lane >> 4) << 3);   // row whose address this lane gives (matrices: rows 0-7 x two tiles, rows 8-15 x two)
-#pragma unroll
-                    for (int np = 0; np < 4; ++np) {
-                        const float(*p)[4] = &c[2 * np];
-                        stmatrix_x4(blk + j * kRowBytes + (((2 * np + ((lane >> 3) & 1)) ^ (j & 7)) << 4), w0 ? pack2_bf16(p[0][0] * i0, p[0][1] * i0) : 0u,
+                        // rows past the last kept one become zeros (not 0 x something: the stage must stay finite)
+                        const bool w0 = 16 * mt + g < n_kept, w1 = 16 * mt + g + 8 < n_kept;
+                        stmatrix_x4(to + mt * 16 * kRowBytes, w0 ? pack2_bf16(p[0][0] * i0, p[0][1] * i0) : 0u,
                                     w0 ? pack2_bf16(p[1][0] * i0, p[1][1] * i0) : 0u, w1 ? pack2_bf16(p[0][2] * i1, p[0][3] * i1) : 0u,
                                     w1 ? pack2_bf16(p[1][2] * i1, p[1][3] * i1) : 0u);
+                    };
+                    rows_out(af0, 0, i0, i1);
+                    if (n_mt == 2) {
+                        uint32_t w[2][4];
+                        w_fragment(w[0], rw[0], row_pair(g + 16), row_pair(g + 24));
+                        w_fragment(w[1], rw[1], row_pair(g + 16), row_pair(g + 24));
+                        rows_out(w, 1, g + 16 < n_kept ? rcnt[g + 16] : 0.f, g + 24 < n_kept ? rcnt[g + 24] : 0.f);
                     }
                 }
                 __syncwarp();
@@ -541,13 +527,20 @@ __global__ void __launch_bounds__(kWarps * 32, 2) merge_small_kernel(const __gri
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the merged rows were written by ordinary stores, the refill is not
             __syncwarp();
-            if (more && lane == 0) issue(t, meta_next);
+            if (lane == 0) {   // the tensor after the next one takes this stage: V behind Q, then Q and K of the next unit
+                if (SPLIT) {
+                    if (more) issue(t, st, meta_next);
+                } else if (t == 0) {
+                    issue(2, st, m);
+                } else if (more) {
+                    issue(t - 1, st, meta_next);
+                }
+            }
         }
         if (failed) break;
     }
-    if (failed) {
-        for (int t = SPLIT ? t_first : 0; t <= t_last; ++t) mbar_wait_bounded(bar0 + 8 * t, it & 1, a.status, kDevTimeoutMatchLoad);
-    }
+    if (failed)   // give copies that may still be in flight a bounded chance to land before the shared memory is released
+        for (uint32_t i = seq; i <= seq + (ahead ? 1 : 0); ++i) mbar_wait_bounded(bar0 + 8 * (i & 1u), i >> 1 & 1u, a.status, kDevTimeoutMatchLoad);
 }
 
 int small_grid(int64_t units, int sm_count, int ctas_per_sm) {
@@ -583,7 +576,7 @@ cudaError_t launch_merge_small(const MergeArgs& a, int sm_count, cudaStream_t st
     if (!encode_merge_maps(&m, a, 32)) return cudaErrorInvalidValue;
     const int sp_units = direct ? (a.layout.n_special > 0 ? a.layout.frames : 0) : (a.n_special_total + 31) / 32;
     const int64_t units = (int64_t)a.heads * (a.n_blocks + sp_units);
-    const int parts = 3 * units <= 2ll * kWarps * sm_count ? 3 : 1, grid = small_grid(units * parts, sm_count, 2);
+    const int parts = 3 * units <= 3ll * kWarps * sm_count ? 3 : 1, grid = small_grid(units * parts, sm_count, 3);
     const bool split = parts > 1;
     auto kernel = direct ? (split ? merge_small_kernel<true, true> : merge_small_kernel<true, false>)
                          : (split ? merge_small_kernel<false, true> : merge_small_kernel<false, false>);

@@ -6,6 +6,7 @@ import torch
 
 from paper_2511_21317_b200 import binding as hb
 from paper_2511_21317_b200 import synth
+from tests.test_gpu_parity import run_case
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -32,6 +33,16 @@ def test_whole_units_and_split_units_agree(blk, ratio, specials, frames):
         one = run(hb.HttmConfig.of(wl.replace(heads=1)), (q[h:h + 1], k[h:h + 1], v[h:h + 1]))
         for name in ITEMS:
             assert np.array_equal(whole[name][h], one[name][0]), (name, h)
+
+
+@pytest.mark.parametrize("blk,ratio", [((2, 4, 4), 0.04), ((2, 4, 4), 0.46), ((2, 4, 4), 0.5), ((2, 4, 4), 0.53), ((2, 4, 4), 0.97), ((1, 4, 4), 0.07), ((1, 4, 4), 0.94),
+                                       ((1, 1, 17), 0.06), ((3, 3, 3), 0.4), ((1, 1, 2), 0.5)])
+def test_numbers_of_kept_rows_and_tokens(blk, ratio):
+    """One and two 16-row tiles of merged rows (31, 18, 16, 15 and 1 kept of 32 tokens), one and two 16-token steps (15 and 1 kept of 16, 16 of 17), against the
+    oracle; the blocks at the edges of the grid are clipped."""
+    wl = synth.Workload("kept", 5, 9, 18, *blk, ratio, ratio, n_camera=1, n_register=2, heads=2, seed=7)
+    stats = run_case(wl, peaky=True)
+    assert stats["peaky_needed"] <= 0.001 * stats["out_elements"]
 
 
 @pytest.mark.parametrize("ratio", [0.0, 0.5, 0.72, 0.75, 0.8, 0.97])
