@@ -206,7 +206,7 @@ cudaError_t launch_match(const MatchArgs& a, int max_block_tokens, int sm_count,
 cudaError_t launch_match_anchor(const MatchArgs& a, const TensorView& src_q, const TensorView& src_k, const int32_t* pi, int n_anchor,
                                 int main_capacity, int max_block_tokens, cudaStream_t stream);
 cudaError_t launch_merge(const MergeArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream);
-cudaError_t launch_match_small(const MatchArgs& a, int sm_count, cudaStream_t stream);   // blocks of at most 32 tokens
+cudaError_t launch_match_small(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream);   // blocks of at most 64 tokens
 cudaError_t launch_merge_small(const MergeArgs& a, int sm_count, cudaStream_t stream);
 cudaError_t configure_small_blocks();
 cudaError_t launch_match_mid(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream);   // blocks of 33 .. 256 tokens

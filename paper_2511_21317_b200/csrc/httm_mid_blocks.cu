@@ -1,6 +1,7 @@
 // Matching and merging for merging blocks of 33 .. 256 tokens (Eq. 1, Sec. 3.2).  A TEAM of W warps, a CTA of its own, works
 // off a UNIT = one (head, block) with all its tensors; a thread owns P rows of the stage, so that a team takes blocks of
 // 32 W P tokens: (W, P) = (1, 2), (4, 1) and (8, 1) for blocks of up to 64, 128 and 256 tokens.
+// (Blocks of up to 64 tokens are matched by the small-block kernel where there are many of them: launch_match.)
 //
 // What bounds them is instructions and their latency, not memory (2 - 3.3 of 6.5 TB/s).  With one warp per (tensor, head, block) and
 // all of its tokens (16 / 12 / 6 warps per SM, as many blocks as shared memory takes) a 128-token block kept its warp busy for

@@ -1,5 +1,6 @@
 // Matching and merging for merging blocks of at most 32 tokens (Eq. 1, Sec. 3.2), one warp per UNIT = one (head, block) with all
 // its tensors: the match kernel works off Q and K of a block, the merge kernel Q, K and V (V follows K's map).
+// Many blocks of up to 64 tokens are matched here too.
 //
 // A block is 4 KB and 5 KFLOP per tensor, so what bounds these kernels is not the arithmetic but the instructions around it:
 // table entries, block geometry, dst positions, the next load.  With one task per (tensor, head, block) the match kernel
@@ -32,17 +33,25 @@ constexpr uint32_t kStage = 32 * kRowBytes;   // one block of one tensor, 128-by
 // (Every lane owns one token when the r best are chosen.  With two tokens in every other lane a tensor took 518 instructions, now 441, and the kernel alone, one launch
 // at a time, 39.3 -> 34.8 us at 32 976 tokens; between the other kernels of a call 40.8 -> 40.4, 65 952 tokens 82.9 -> 72.7.)
 // Row rho of the stage is owned, from the arg-max on, by lane (rho & 7) * 4 + (rho >> 3).
-constexpr int kMatchSmem = kWarps * (2 * (int)kStage + 16) + 1024 /*alignment slack*/;
+constexpr int kMatchSmem = kWarps * (2 * (int)kStage + 16) + 1024 /*alignment slack*/;   // two blocks of 32 rows or one of 64 per warp
 
+constexpr int match_ctas(int tiles) { return tiles == 2 ? 3 : 2; }   // per SM: 80 and 128 registers
+// TILES: blocks of up to 32 tokens, 8 dst tokens (2), a stage for either tensor; or up to 64 tokens, 16 dst tokens (4): one stage for Q and K in turn, so that 16 warps
+// fit on an SM (the team of one warp of httm_mid_blocks.cu has two and 12 warps).  K is on its way while the tokens of Q are chosen, so this needs more units than warps
+// to pay: 137 400 tokens in 64-token blocks 161.8 -> 137.5 us, a call 4098 -> 4037; 7 898 tokens in 48-token blocks, 1.3 units per warp, a call 93.5 -> 92.6; 0.6 units
+// per warp 101.8 -> 102.3.  (24 warps with 80 registers spill: 159 us.)
 // SPLIT: fewer units than warps: a warp has one tensor of one unit
-template <bool DIRECT, bool SPLIT>
-__global__ void __launch_bounds__(kWarps * 32, 3)
+template <int TILES, bool DIRECT, bool SPLIT>
+__global__ void __launch_bounds__(kWarps * 32, match_ctas(TILES))
 match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ MatchArgs a) {
+    constexpr int ND = TILES / 2, SLOTS = TILES / 2;   // groups of eight dst tokens; tokens per lane
+    constexpr int STAGES = TILES == 2 ? 2 : 1;
+    constexpr uint32_t STAGE = TILES * 16 * kRowBytes;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + align_pad(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tq = lane & 3;   // accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
-    const int rho = 8 * tq + g;                // the stage row this lane owns
+    const int rho0 = 8 * tq + g;               // the stage rows this lane owns: rho0 + 32 i
     const uint32_t stage0 = smem_u32(smem + (size_t)warp * 2 * kStage);
     const uint32_t bar0 = smem_u32(smem + (size_t)kWarps * 2 * kStage + warp * 16);
     if (lane == 0) {
@@ -66,14 +75,14 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     next.init(first, stride, a.n_blocks);
     auto issue = [&](int t, const int4& geom, int start, int h) {   // lane 0 only
         const Geometry bg = unpack_geometry(geom);
-        const uint32_t mb = bar0 + 8 * t;
+        const uint32_t st = STAGES == 2 ? t : 0, mb = bar0 + 8 * st;
         const CUtensorMap* m = t == 0 ? &map_q : &map_k;
         if (DIRECT) {
             mbar_expect_tx(mb, (uint32_t)box.rows * kRowBytes);
-            tma_block_load(stage0 + t * kStage, m, mb, bg.x0, bg.y0, bg.s0, h);
+            tma_block_load(stage0 + st * STAGE, m, mb, bg.x0, bg.y0, bg.s0, h);
         } else {
-            mbar_expect_tx(mb, kStage);
-            tma_rows_load(stage0 + t * kStage, m, mb, start, h);
+            mbar_expect_tx(mb, STAGE);
+            tma_rows_load(stage0 + st * STAGE, m, mb, start, h);
         }
     };
     BlockInfo bi_next{};
@@ -89,7 +98,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     dependents_launch();
     clear_words(a.clear, blockIdx.x, gridDim.x);
     if (first < n_units && lane == 0)
-        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t) issue(t, bg_next, bi_next.start, h_next);
+        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : STAGES - 1); ++t) issue(t, bg_next, bi_next.start, h_next);
 
     // ldmatrix offsets of a 16-row tile: rows 0-7 / 8-15 (lane bit 3), k chunk 2 ks / 2 ks + 1 (lane bit 4); chunk c of row j sits at c ^ (j & 7)
     uint32_t a_off[4];
@@ -97,14 +106,20 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     for (int ks = 0; ks < 4; ++ks) a_off[ks] = ((lane & 7) + ((lane >> 3) & 1) * 8) * kRowBytes + (((2 * ks + (lane >> 4)) ^ (lane & 7)) << 4);
     // what this lane knows about the shape of the blocks at hand
     int shape_a = -1, shape_b = -1;
-    uint32_t d_off[2] = {0, 0};   // ldmatrix offsets of dst row lane & 7
-    int d_pos = 0;                // token number of dst lane & 7
-    int tok = -1;                 // token owned (-1: none)
-    bool is_src = false;
+    uint32_t d_off[ND][2];        // ldmatrix offsets of dst rows 8 d + (lane & 7)
+    int d_pos = 0;                // token number of dst lane & (8 ND - 1)
+    int tok[SLOTS];               // tokens owned (-1: none)
+    bool is_src[SLOTS];
+#pragma unroll
+    for (int i = 0; i < SLOTS; ++i) {
+        d_off[i][0] = d_off[i][1] = 0;
+        tok[i] = -1;
+        is_src[i] = false;
+    }
 
-    int it = 0;
+    int it = 0;   // loads of a stage so far (TILES 4: tensors, else units)
     bool failed = false;
-    for (int64_t unit = first; unit < n_units; unit += stride, ++it) {
+    for (int64_t unit = first; unit < n_units; unit += stride, it += STAGES == 2) {
         const BlockInfo bi = bi_next;
         const int4 geom = bg_next;
         const int h = h_next, n = bi.n;
@@ -114,60 +129,83 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             fetch();   // in flight while this unit is worked off
         }
 #pragma unroll 1
-        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t) {
+        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t, it += STAGES == 1) {
+            // the next tensor of this stage: this one of the next unit or, with one stage, K behind Q
+            auto refill = [&]() {   // lane 0 only
+                if (STAGES == 1 && t == 0)
+                    issue(1, geom, bi.start, h);
+                else if (more)
+                    issue(STAGES == 1 ? 0 : t, bg_next, bi_next.start, h_next);
+            };
             const int r = t == 0 ? bi.r_q : bi.r_k, nd = t == 0 ? bi.nd_q : bi.nd_k;
             int32_t* A = a.assign[t] + (int64_t)h * a.n_tokens + bi.start;
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8 * t, it & 1, a.status, kDevTimeoutMatchLoad))) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + (STAGES == 2 ? 8 * t : 0), it & 1, a.status, kDevTimeoutMatchLoad))) {
                 failed = true;
                 break;
             }
-            if (r == 0 || nd > 8) {   // nothing merges, or an anchored block with more dst tokens (match_anchor_kernel)
-                if (r == 0 && lane < n) A[lane] = bi.start + lane;
+            if (r == 0 || nd > 8 * ND) {   // nothing merges, or an anchored block with more dst tokens (match_anchor_kernel)
+                if (r == 0)
+                    for (int j = lane; j < n; j += 32) A[j] = bi.start + j;
                 __syncwarp();
-                if (more && lane == 0) issue(t, bg_next, bi_next.start, h_next);
+                if (lane == 0) refill();
                 continue;
             }
             const int n_rows = DIRECT ? box.rows : n;   // rows of the stage that may hold tokens
             {
-                const int sa = n | (nd << 8) | (bi.n_rule << 16), sb = DIRECT ? shape_key(geom) : 0;
+                const int sa = n | (nd << 8) | (bi.n_rule << 16), sb = DIRECT ? shape_key(geom) : 0;   // (n and n_rule at most 64)
                 if (sa != shape_a || sb != shape_b) {
                     const Geometry bg = unpack_geometry(geom);
                     shape_a = sa;
                     shape_b = sb;
                     const int n_rule = bi.n_rule;   // n (evenly spaced dst tokens) or n_dst (the first n_dst tokens: first-frame anchoring)
-                    d_pos = small_div((min(lane & 7, nd - 1) + 1) * n_rule + nd - 1, nd) - 1;
-                    const int row = DIRECT ? row_of_token(box, bg, d_pos) : d_pos;
+                    d_pos = small_div((min(lane & (8 * ND - 1), nd - 1) + 1) * n_rule + nd - 1, nd) - 1;
 #pragma unroll
-                    for (int kp = 0; kp < 2; ++kp) d_off[kp] = row * kRowBytes + (((4 * kp + (lane >> 3)) ^ (row & 7)) << 4);
-                    tok = DIRECT ? token_of_row(box, bg, rho) : (rho < n ? rho : -1);
-                    is_src = tok >= 0 && !(tok < n_rule && small_div((tok + 1) * nd, n_rule) > small_div(tok * nd, n_rule));
+                    for (int d = 0; d < ND; ++d) {
+                        const int pos = ND == 1 ? d_pos : __shfl_sync(0xffffffffu, d_pos, 8 * d + (lane & 7)), row = DIRECT ? row_of_token(box, bg, pos) : pos;
+#pragma unroll
+                        for (int kp = 0; kp < 2; ++kp) d_off[d][kp] = row * kRowBytes + (((4 * kp + (lane >> 3)) ^ (row & 7)) << 4);
+                    }
+#pragma unroll
+                    for (int i = 0; i < SLOTS; ++i) {
+                        const int rho = rho0 + 32 * i, j = DIRECT ? token_of_row(box, bg, rho) : (rho < n ? rho : -1);
+                        tok[i] = j;
+                        is_src[i] = j >= 0 && !(j < n_rule && small_div((j + 1) * nd, n_rule) > small_div(j * nd, n_rule));
+                    }
                 }
             }
-            const uint32_t blk = stage0 + t * kStage;
+            const uint32_t blk = stage0 + (STAGES == 2 ? t * STAGE : 0);
             // ---- dst fragments (k steps 2 kp, 2 kp + 1 per ldmatrix.x4) and their norms: lane 9 tq holds that of dst 2 tq, 9 tq + 4 of 2 tq + 1
-            uint32_t bf[4][2];
+            uint32_t bf[ND][4][2];
+            float w0[ND], w1[ND];
 #pragma unroll
-            for (int kp = 0; kp < 2; ++kp) {
-                uint32_t rr[4];
-                ldmatrix_x4(rr, blk + d_off[kp]);
-                bf[2 * kp][0] = rr[0];
-                bf[2 * kp][1] = rr[1];
-                bf[2 * kp + 1][0] = rr[2];
-                bf[2 * kp + 1][1] = rr[3];
-            }
-            float dn[4];
+            for (int d = 0; d < ND; ++d) {
+                w0[d] = w1[d] = CUDART_NAN_F;
+                if (d == 0 || 8 * d < nd) {   // (uniform)
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                const uint32_t ad[4] = {bf[ks][0], bf[ks][0], bf[ks][1], bf[ks][1]};
-                if (ks == 0)
-                    mma_first(dn, ad, bf[ks][0], bf[ks][1]);
-                else
-                    mma_bf16_16816(dn, ad, bf[ks][0], bf[ks][1]);
+                    for (int kp = 0; kp < 2; ++kp) {
+                        uint32_t rr[4];
+                        ldmatrix_x4(rr, blk + d_off[d][kp]);
+                        bf[d][2 * kp][0] = rr[0];
+                        bf[d][2 * kp][1] = rr[1];
+                        bf[d][2 * kp + 1][0] = rr[2];
+                        bf[d][2 * kp + 1][1] = rr[3];
+                    }
+                    float dn[4];
+#pragma unroll
+                    for (int ks = 0; ks < 4; ++ks) {
+                        const uint32_t ad[4] = {bf[d][ks][0], bf[d][ks][0], bf[d][ks][1], bf[d][ks][1]};
+                        if (ks == 0)
+                            mma_first(dn, ad, bf[d][ks][0], bf[d][ks][1]);
+                        else
+                            mma_bf16_16816(dn, ad, bf[d][ks][0], bf[d][ks][1]);
+                    }
+                    const float dsel = (g & 1) ? dn[1] : dn[0];
+                    w0[d] = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq));
+                    w1[d] = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq + 4));
+                    if (8 * d + 2 * tq >= nd) w0[d] = CUDART_NAN_F;
+                    if (8 * d + 2 * tq + 1 >= nd) w1[d] = CUDART_NAN_F;
+                }
             }
-            const float dsel = (g & 1) ? dn[1] : dn[0];
-            float w0 = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq)), w1 = inv_norm(__shfl_sync(0xffffffffu, dsel, 9 * tq + 4));
-            if (2 * tq >= nd) w0 = CUDART_NAN_F;
-            if (2 * tq + 1 >= nd) w1 = CUDART_NAN_F;
             // ---- best dst of every row.  The four lanes of a row meet: an exchange with lane ^ 1 leaves a lane one of a tile's rows g and g + 8, one with
             // lane ^ 2 one of the two tiles
             const bool odd = tq & 1, high = tq & 2;
@@ -179,35 +217,54 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     arg = oa;
                 }
             };
-            float top[2], norm[2];
-            int arg[2];
+            float top[TILES], norm[TILES];
+            int arg[TILES];
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
+            for (int mt = 0; mt < TILES; ++mt) {
                 top[mt] = -INFINITY;
                 norm[mt] = 0.f;
                 arg[mt] = 0;
                 if (mt * 16 < n_rows) {   // warp-uniform
-                    float c[4], lo[4], hi[4];
+                    float c[ND][4], lo[4], hi[4];
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks) {
                         uint32_t af[4];
                         ldmatrix_x4(af, blk + mt * 16 * kRowBytes + a_off[ks]);
                         if (ks == 0) {
-                            mma_first(c, af, bf[ks][0], bf[ks][1]);
+#pragma unroll
+                            for (int d = 0; d < ND; ++d)
+                                if (d == 0 || 8 * d < nd) mma_first(c[d], af, bf[d][ks][0], bf[d][ks][1]);
                             mma_first(lo, af, af[0], af[2]);   // against rows 0-7 of the tile
                             mma_first(hi, af, af[1], af[3]);   // against rows 8-15
                         } else {
-                            mma_bf16_16816(c, af, bf[ks][0], bf[ks][1]);
+#pragma unroll
+                            for (int d = 0; d < ND; ++d)
+                                if (d == 0 || 8 * d < nd) mma_bf16_16816(c[d], af, bf[d][ks][0], bf[d][ks][1]);
                             mma_bf16_16816(lo, af, af[0], af[2]);
                             mma_bf16_16816(hi, af, af[1], af[3]);
                         }
                     }
-                    // this lane's two dst tokens first
+                    // this lane's dst tokens first, for rows g and g + 8
                     // (the maximum with -infinity drops what is not a number: a place without a dst token, tokens whose norm overflows)
-                    const float s00 = fmaxf(c[0] * w0, -INFINITY), s01 = fmaxf(c[1] * w1, -INFINITY);
-                    const float s10 = fmaxf(c[2] * w0, -INFINITY), s11 = fmaxf(c[3] * w1, -INFINITY);
-                    const float t0 = fmaxf(s00, s01), t1 = fmaxf(s10, s11);
-                    const int d0 = 2 * tq + (s01 > s00 ? 1 : 0), d1 = 2 * tq + (s11 > s10 ? 1 : 0);
+                    float t0 = 0.f, t1 = 0.f;
+                    int d0 = 0, d1 = 0;
+#pragma unroll
+                    for (int d = 0; d < ND; ++d) {
+                        if (d == 0 || 8 * d < nd) {
+                            const float s00 = fmaxf(c[d][0] * w0[d], -INFINITY), s01 = fmaxf(c[d][1] * w1[d], -INFINITY);
+                            const float s10 = fmaxf(c[d][2] * w0[d], -INFINITY), s11 = fmaxf(c[d][3] * w1[d], -INFINITY);
+                            const float u0 = fmaxf(s00, s01), u1 = fmaxf(s10, s11);
+                            const int e0 = 8 * d + 2 * tq + (s01 > s00 ? 1 : 0), e1 = 8 * d + 2 * tq + (s11 > s10 ? 1 : 0);
+                            if (d == 0 || u0 > t0) {
+                                t0 = u0;
+                                d0 = e0;
+                            }
+                            if (d == 0 || u1 > t1) {
+                                t1 = u1;
+                                d1 = e1;
+                            }
+                        }
+                    }
                     top[mt] = odd ? t1 : t0;
                     arg[mt] = odd ? d1 : d0;
                     meet(top[mt], arg[mt], odd ? t0 : t1, odd ? d0 : d1, 1);
@@ -216,41 +273,67 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     norm[mt] = odd ? nh : nl;
                 }
             }
-            float best_score = high ? top[1] : top[0];
-            int best = high ? arg[1] : arg[0];
-            meet(best_score, best, high ? top[0] : top[1], high ? arg[0] : arg[1], 2);
-            best_score *= inv_norm(high ? norm[1] : norm[0]);
-            const uint32_t key = score_key(best_score);
+            uint32_t key[SLOTS];   // 0: not a src token
+            int best[SLOTS];
+#pragma unroll
+            for (int i = 0; i < SLOTS; ++i) {
+                float best_score = high ? top[2 * i + 1] : top[2 * i];
+                best[i] = high ? arg[2 * i + 1] : arg[2 * i];
+                meet(best_score, best[i], high ? top[2 * i] : top[2 * i + 1], high ? arg[2 * i] : arg[2 * i + 1], 2);
+                key[i] = is_src[i] ? score_key(best_score * inv_norm(high ? norm[2 * i + 1] : norm[2 * i])) : 0u;
+            }
             __syncwarp();   // every lane has read the stage
-            if (more && lane == 0) issue(t, bg_next, bi_next.start, h_next);
+            if (lane == 0) refill();
 
             // ---- the r src with the best scores merge (ties: lowest position first)
             const int n_out = n - nd - r;
-            bool merged;
+            bool merged[SLOTS];
             if (r <= n_out) {
-                merged = false;
+#pragma unroll
+                for (int i = 0; i < SLOTS; ++i) merged[i] = false;
                 for (int round = 0; round < r; ++round) {
-                    const uint32_t k = is_src && !merged ? key : 0u;
-                    const uint32_t m = __reduce_max_sync(0xffffffffu, k);
-                    const unsigned win = __reduce_min_sync(0xffffffffu, k == m ? (unsigned)rho : 0xffffffffu);   // lowest position holding it
-                    merged = merged || (is_src && win == (unsigned)rho);
+                    uint32_t k[SLOTS], top_key = 0u;
+#pragma unroll
+                    for (int i = 0; i < SLOTS; ++i) {
+                        k[i] = merged[i] ? 0u : key[i];
+                        top_key = max(top_key, k[i]);
+                    }
+                    top_key = __reduce_max_sync(0xffffffffu, top_key);
+                    unsigned at = 0xffffffffu;
+#pragma unroll
+                    for (int i = SLOTS - 1; i >= 0; --i)
+                        if (k[i] == top_key) at = rho0 + 32 * i;
+                    const unsigned win = __reduce_min_sync(0xffffffffu, at);   // lowest position holding it
+#pragma unroll
+                    for (int i = 0; i < SLOTS; ++i) merged[i] = merged[i] || (is_src[i] && win == (unsigned)(rho0 + 32 * i));
                 }
             } else {
-                merged = is_src;
+#pragma unroll
+                for (int i = 0; i < SLOTS; ++i) merged[i] = is_src[i];
                 for (int round = 0; round < n_out; ++round) {
-                    const uint32_t k = merged ? key : 0xffffffffu;
-                    const uint32_t m = __reduce_min_sync(0xffffffffu, k);
-                    const int win = __reduce_max_sync(0xffffffffu, merged && k == m ? rho : -1);   // highest position
-                    merged = merged && win != rho;
+                    uint32_t low = 0xffffffffu;
+#pragma unroll
+                    for (int i = 0; i < SLOTS; ++i) low = min(low, merged[i] ? key[i] : 0xffffffffu);
+                    low = __reduce_min_sync(0xffffffffu, low);
+                    int at = -1;
+#pragma unroll
+                    for (int i = 0; i < SLOTS; ++i)
+                        if (merged[i] && key[i] == low) at = rho0 + 32 * i;
+                    const int win = __reduce_max_sync(0xffffffffu, at);   // highest position
+#pragma unroll
+                    for (int i = 0; i < SLOTS; ++i) merged[i] = merged[i] && win != rho0 + 32 * i;
                 }
             }
-            const int target = __shfl_sync(0xffffffffu, d_pos, best);
-            if (tok >= 0) A[tok] = bi.start + (merged ? target : tok);
+#pragma unroll
+            for (int i = 0; i < SLOTS; ++i) {
+                const int target = __shfl_sync(0xffffffffu, d_pos, best[i]);
+                if (tok[i] >= 0) A[tok[i]] = bi.start + (merged[i] ? target : tok[i]);
+            }
         }
         if (failed) break;
     }
     if (failed) {   // give copies that may still be in flight a bounded chance to land before the shared memory is released
-        for (int t = SPLIT ? t_first : 0; t <= t_last; ++t) mbar_wait_bounded(bar0 + 8 * t, it & 1, a.status, kDevTimeoutMatchLoad);
+        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : STAGES - 1); ++t) mbar_wait_bounded(bar0 + (STAGES == 2 ? 8 * t : 0), it & 1, a.status, kDevTimeoutMatchLoad);
     }
 }
 
@@ -550,24 +633,31 @@ int small_grid(int64_t units, int sm_count, int ctas_per_sm) {
 
 }  // namespace
 
-cudaError_t launch_match_small(const MatchArgs& a, int sm_count, cudaStream_t stream) {
+namespace {
+template <int TILES>
+cudaError_t launch_match_tiles(const MatchArgs& a, int sm_count, cudaStream_t stream) {
     CUtensorMap mq, mk;
     const int64_t N = a.n_tokens;
     const bool direct = a.geom != nullptr;
     if (direct) {
         if (!encode_block_map(&mq, a.src[0], a.layout, a.heads) || !encode_block_map(&mk, a.src[1], a.layout, a.heads)) return cudaErrorInvalidValue;
-    } else if (!encode_rows_tensor_map(&mq, a.xr[0], N, a.heads, kHeadDim, N * kHeadDim, 32) ||
-               !encode_rows_tensor_map(&mk, a.xr[1], N, a.heads, kHeadDim, N * kHeadDim, 32)) {
+    } else if (!encode_rows_tensor_map(&mq, a.xr[0], N, a.heads, kHeadDim, N * kHeadDim, 16 * TILES) ||
+               !encode_rows_tensor_map(&mk, a.xr[1], N, a.heads, kHeadDim, N * kHeadDim, 16 * TILES)) {
         return cudaErrorInvalidValue;
     }
+    const int64_t units = (int64_t)a.heads * a.n_blocks;
+    auto launch = [&](auto kernel, int parts) {
+        return launch_kernel(kernel, small_grid(units * parts, sm_count, match_ctas(TILES)), kWarps * 32, kMatchSmem, stream, mq, mk, a);
+    };
     // With no more than one tensor per warp the tensors of a unit go to different warps: the call then waits for one, not two
     // (512 units: 11.3 -> 9.4 us, in the merge kernel below 13.1 -> 9.0).
-    const int64_t units = (int64_t)a.heads * a.n_blocks;
-    const int parts = 2 * units <= 3ll * kWarps * sm_count ? 2 : 1, grid = small_grid(units * parts, sm_count, 3);
-    const bool split = parts > 1;
-    auto kernel = direct ? (split ? match_small_kernel<true, true> : match_small_kernel<true, false>)
-                         : (split ? match_small_kernel<false, true> : match_small_kernel<false, false>);
-    return launch_kernel(kernel, grid, kWarps * 32, kMatchSmem, stream, mq, mk, a);
+    if constexpr (TILES == 2)
+        if (2 * units <= (int64_t)match_ctas(TILES) * kWarps * sm_count) return launch(direct ? match_small_kernel<TILES, true, true> : match_small_kernel<TILES, false, true>, 2);
+    return launch(direct ? match_small_kernel<TILES, true, false> : match_small_kernel<TILES, false, false>, 1);
+}
+}  // namespace
+cudaError_t launch_match_small(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
+    return max_block_tokens <= 32 ? launch_match_tiles<2>(a, sm_count, stream) : launch_match_tiles<4>(a, sm_count, stream);
 }
 
 cudaError_t launch_merge_small(const MergeArgs& a, int sm_count, cudaStream_t stream) {
@@ -588,10 +678,12 @@ cudaError_t configure_small_blocks() {
     auto set = [&](auto kernel, int bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
-    set(match_small_kernel<false, false>, kMatchSmem);
-    set(match_small_kernel<false, true>, kMatchSmem);
-    set(match_small_kernel<true, false>, kMatchSmem);
-    set(match_small_kernel<true, true>, kMatchSmem);
+    set(match_small_kernel<2, false, false>, kMatchSmem);
+    set(match_small_kernel<4, false, false>, kMatchSmem);
+    set(match_small_kernel<2, false, true>, kMatchSmem);
+    set(match_small_kernel<2, true, false>, kMatchSmem);
+    set(match_small_kernel<4, true, false>, kMatchSmem);
+    set(match_small_kernel<2, true, true>, kMatchSmem);
     set(merge_small_kernel<false, false>, kMergeSmem);
     set(merge_small_kernel<false, true>, kMergeSmem);
     set(merge_small_kernel<true, false>, kMergeSmem);
