@@ -12,7 +12,7 @@
 //   - results leave through the stage as whole rows instead of 4 bytes per lane.
 // Measured at 32 976 tokens x 16 heads, 32-token blocks: match 53 -> 39.6 us, merge 69.6 -> 62.4 us (both
 // with the interval between two events).  What is left is the latency of a warp's instruction stream, hence as few instructions as possible
-// (match: one token per lane from the arg-max on) and as many warps as fit (merge: two stages and 80 registers, 24 warps per SM).
+// (match: one token per lane from the arg-max on) and as many warps as fit (merge: two stages).
 #include "httm_blocks.cuh"
 #include "httm_launch.cuh"
 
@@ -342,8 +342,8 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 // with the 0/1 assignment matrix W (exact in bf16, built in registers from the map), fp32 accumulation, times the reciprocal
 // of the group size, one rounding to bf16.  Kept tokens are compacted in reordered order.  The rows go through the stage they came
 // from, 16 channels at a time (whose fragments are in registers by then), and leave 16 bytes per lane, whole rows; then the stage is refilled.
-// Tensor i of the warp's sequence Q K V Q K V .. lies in stage i & 1.  With a stage for each tensor and all 64 channels in registers (128) 16 warps
-// fit on an SM: 61.4 -> 57.3 us at 32 976 tokens, 132 -> 115 at 65 952 (two stages and 16 warps: 66.6).
+// Tensor i of the warp's sequence Q K V Q K V .. lies in stage i & 1.  With a stage for each tensor and all 64 channels in registers at a time (128 of them) 16 warps
+// were all that fits on an SM: 61.4 -> 57.3 us at 32 976 tokens, 132 -> 115 at 65 952, 19.5 -> 17.5 at 5 516 (launch_merge_small).
 constexpr int kMergeAux = 32 * 4 + 32 * 4 + 32 + 64;   // reciprocal group sizes, group sizes, 3 mbarriers, merged rows of the tokens
 constexpr int kMergeStages = 2;
 constexpr int kMergeSmem = kWarps * (kMergeStages * (int)kStage + kMergeAux) + 1024 /*alignment slack*/;
@@ -351,8 +351,8 @@ constexpr int kMergeSmem = kWarps * (kMergeStages * (int)kStage + kMergeAux) + 1
 __device__ __forceinline__ void stmatrix_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
     asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
 }
-template <bool DIRECT, bool SPLIT>
-__global__ void __launch_bounds__(kWarps * 32, 3) merge_small_kernel(const __grid_constant__ MergeMaps maps, const __grid_constant__ MergeArgs a) {
+template <int CTAS, bool DIRECT, bool SPLIT>   // CTAS: per SM
+__global__ void __launch_bounds__(kWarps * 32, CTAS) merge_small_kernel(const __grid_constant__ MergeMaps maps, const __grid_constant__ MergeArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + align_pad(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -666,11 +666,12 @@ cudaError_t launch_merge_small(const MergeArgs& a, int sm_count, cudaStream_t st
     if (!encode_merge_maps(&m, a, 32)) return cudaErrorInvalidValue;
     const int sp_units = direct ? (a.layout.n_special > 0 ? a.layout.frames : 0) : (a.n_special_total + 31) / 32;
     const int64_t units = (int64_t)a.heads * (a.n_blocks + sp_units);
-    const int parts = 3 * units <= 3ll * kWarps * sm_count ? 3 : 1, grid = small_grid(units * parts, sm_count, 3);
-    const bool split = parts > 1;
-    auto kernel = direct ? (split ? merge_small_kernel<true, true> : merge_small_kernel<true, false>)
-                         : (split ? merge_small_kernel<false, true> : merge_small_kernel<false, false>);
-    return launch_kernel(kernel, grid, kWarps * 32, kMergeSmem, stream, m, a);
+    auto launch = [&](auto kernel, int parts, int ctas) { return launch_kernel(kernel, small_grid(units * parts, sm_count, ctas), kWarps * 32, kMergeSmem, stream, m, a); };
+    if (3 * units <= 2ll * kWarps * sm_count) return launch(direct ? merge_small_kernel<2, true, true> : merge_small_kernel<2, false, true>, 3, 2);
+    // A round of units takes 24 warps per SM (80 registers) 1.4 times as long as 16 (111), so the third CTA pays in the long run: merge at 65 952 tokens x 16 heads (11 rounds of
+    // 24 warps) 115 us with it, 122 without, 32 976 (5.5) 57.3 and 58.4, 10 992 (1.8) 24.5 and 23.6, 5 516 (1.04, two either way) 19.5 and 17.5.
+    if (units > 5 * 3ll * kWarps * sm_count) return launch(direct ? merge_small_kernel<3, true, false> : merge_small_kernel<3, false, false>, 1, 3);
+    return launch(direct ? merge_small_kernel<2, true, false> : merge_small_kernel<2, false, false>, 1, 2);
 }
 
 cudaError_t configure_small_blocks() {
@@ -684,10 +685,12 @@ cudaError_t configure_small_blocks() {
     set(match_small_kernel<2, true, false>, kMatchSmem);
     set(match_small_kernel<4, true, false>, kMatchSmem);
     set(match_small_kernel<2, true, true>, kMatchSmem);
-    set(merge_small_kernel<false, false>, kMergeSmem);
-    set(merge_small_kernel<false, true>, kMergeSmem);
-    set(merge_small_kernel<true, false>, kMergeSmem);
-    set(merge_small_kernel<true, true>, kMergeSmem);
+    set(merge_small_kernel<2, false, false>, kMergeSmem);
+    set(merge_small_kernel<2, false, true>, kMergeSmem);
+    set(merge_small_kernel<2, true, false>, kMergeSmem);
+    set(merge_small_kernel<2, true, true>, kMergeSmem);
+    set(merge_small_kernel<3, false, false>, kMergeSmem);
+    set(merge_small_kernel<3, true, false>, kMergeSmem);
     return e;
 }
 
