@@ -38,6 +38,8 @@ struct httm_ctx {
     int32_t n_special = 0, tokens_per_frame = 0, n_tokens = 0, n_blocks = 0, max_block = 0;
     int32_t m_q = 0, m_k = 0;
     int sm_count = 148;
+    CUtensorMap merged_maps[3] = {};   // of Q_m, K_m, V_m as the attention kernel reads them: the workspace stays where it is
+    bool have_merged_maps = false;
     std::vector<int32_t> pi, pi_inv, blk_start;
     std::vector<BlockInfo> blocks;
     std::vector<BlockGeom> geom;
@@ -353,6 +355,7 @@ int stage_attention(httm_ctx* c, cudaStream_t s, const httm_tensor* final_out = 
     a.q = view(c->filtering() ? c->d_qm_var : c->d_qm, c->q_rows());
     a.k = view(c->d_km, c->m_k);
     a.v = view(c->d_vm, c->m_k);
+    for (int i = c->filtering() ? 1 : 0; c->have_merged_maps && i < 3; ++i) a.maps[i] = &c->merged_maps[i];   // (with outlier filtering Q_m is another tensor)
     if (final_out) {
         if (!fused_unmerge(c)) return c->fail(HTTM_ERR_UNSUPPORTED, "unmerge in the attention epilogue needs blocks of at most 32 tokens and no outlier filtering");
         a.out = reinterpret_cast<__nv_bfloat16*>(final_out->ptr);
@@ -648,6 +651,9 @@ int httm_create(const httm_config* cfg, httm_ctx** out) {
         (rc = c->alloc(&c->d_vm, H * c->m_k * kHeadDim)) || (rc = c->alloc(&c->d_om, H * c->m_q * kHeadDim)))
         return done(rc);
 
+    c->have_merged_maps = encode_attention_map(&c->merged_maps[0], view(c->d_qm, c->m_q), c->m_q, cfg->heads) &&
+                          encode_attention_map(&c->merged_maps[1], view(c->d_km, c->m_k), c->m_k, cfg->heads) &&
+                          encode_attention_map(&c->merged_maps[2], view(c->d_vm, c->m_k), c->m_k, cfg->heads);
     if ((rc = c->alloc(&c->d_partial, attention_partial_floats(c->sm_count))) || (rc = c->alloc(&c->d_part_count, attention_partial_counters(c->sm_count) + 1)))
         return done(rc);
     if (c->max_block <= 32) {   // member lists of the merged query rows; entry M_q of every head is the constant N

@@ -946,13 +946,20 @@ cudaError_t configure_attention() {
     return cudaFuncSetAttribute(attention_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
 }
 
+static_assert(BM == BN, "one kind of tile");
+bool encode_attention_map(CUtensorMap* map, const TensorView& t, int32_t rows, int32_t heads) {
+    return encode_rows_tensor_map(map, t.ptr, rows, heads, t.stride_token, t.stride_head, BM);
+}
 // Returns cudaErrorInvalidValue if a tensor map cannot be encoded.
 cudaError_t launch_attention(const AttentionArgs& a, int sm_count, cudaStream_t stream) {
-    CUtensorMap mq, mk, mv;
-    if (!encode_rows_tensor_map(&mq, a.q.ptr, a.m_q, a.heads, a.q.stride_token, a.q.stride_head, BM) ||
-        !encode_rows_tensor_map(&mk, a.k.ptr, a.m_k, a.heads, a.k.stride_token, a.k.stride_head, BN) ||
-        !encode_rows_tensor_map(&mv, a.v.ptr, a.m_k, a.heads, a.v.stride_token, a.v.stride_head, BN))
-        return cudaErrorInvalidValue;
+    CUtensorMap made[3];
+    const CUtensorMap* maps[3];
+    const TensorView* views[3] = {&a.q, &a.k, &a.v};
+    for (int i = 0; i < 3; ++i) {
+        maps[i] = a.maps[i] ? a.maps[i] : &made[i];
+        if (!a.maps[i] && !encode_attention_map(&made[i], *views[i], i == 0 ? a.m_q : a.m_k, a.heads)) return cudaErrorInvalidValue;
+    }
+    const CUtensorMap &mq = *maps[0], &mk = *maps[1], &mv = *maps[2];
     const int tiles_per_head = (a.m_q + BM - 1) / BM, total = tiles_per_head * a.heads;
     // one CTA per SM (fewer when there are fewer tiles, unless they are split)
     int ctas = sm_count < 1 ? 1 : sm_count;

@@ -1,6 +1,7 @@
 // Internal declarations shared by the translation units of libhttm (not part of the ABI).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -184,6 +185,7 @@ struct AttentionArgs {
     const int32_t* group_start;
     const int32_t* group_member;
     int32_t n_tokens;
+    const CUtensorMap* maps[3];   // optional: those of q, k and v (encode_attention_map), where the caller keeps them
     // optional: workspace for query tiles that are split over CTAs (attention_partial_floats / _counters; the counters are zero
     // before every launch); null: tiles are dealt whole.  Launches that share it run in order.
     float* partial;
@@ -228,6 +230,7 @@ cudaError_t launch_big_merge(const MergeArgs& a, int max_block_tokens, cudaStrea
 cudaError_t configure_big_blocks();
 cudaError_t launch_linear(const LinearArgs& a, int sm_count, cudaStream_t stream);   // tcgen05 GEMM for the projections
 cudaError_t configure_linear();
+bool encode_attention_map(CUtensorMap* map, const TensorView& t, int32_t rows, int32_t heads);   // of q, k or v
 cudaError_t launch_attention(const AttentionArgs& a, int sm_count, cudaStream_t stream);   // tcgen05 / TMEM kernel
 cudaError_t configure_attention();
 size_t attention_partial_floats(int sm_count);
