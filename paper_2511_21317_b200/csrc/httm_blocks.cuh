@@ -174,6 +174,15 @@ struct UnitCursor {
     }
 };
 
+// Host: CTAs of eight warps per SM, 2 or 3, for kernels whose warps work off a unit at a time.  A round of units takes 24 warps about 1.4 times as long as 16, so the
+// third CTA pays where it saves more than a third of the rounds, and in the long run.  Merge of 32-token blocks, 16 heads: 65 952 tokens (11 rounds of 24 warps) 115 us with it,
+// 122 without, 32 976 (5.5 rounds) 57.3 and 58.4, 10 992 (2 rounds or 3) 24.5 and 23.6, 5 516 (2 either way) 19.5 and 17.5; 10 374 tokens x 8 heads (1 or 2)
+// a call of 50.8 us with it, 52.8 without.
+inline int unit_ctas(int64_t units, int sm_count) {
+    const int64_t warps = 8ll * (sm_count < 1 ? 1 : sm_count), rounds2 = (units + 2 * warps - 1) / (2 * warps), rounds3 = (units + 3 * warps - 1) / (3 * warps);
+    return rounds3 > 5 || 3 * rounds3 < 2 * rounds2 ? 3 : 2;
+}
+
 struct Geometry {   // BlockGeom in registers
     int s0, y0, x0, frames, rows, cols;
 };

@@ -343,7 +343,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 // of the group size, one rounding to bf16.  Kept tokens are compacted in reordered order.  The rows go through the stage they came
 // from, 16 channels at a time (whose fragments are in registers by then), and leave 16 bytes per lane, whole rows; then the stage is refilled.
 // Tensor i of the warp's sequence Q K V Q K V .. lies in stage i & 1.  With a stage for each tensor and all 64 channels in registers at a time (128 of them) 16 warps
-// were all that fits on an SM: 61.4 -> 57.3 us at 32 976 tokens, 132 -> 115 at 65 952, 19.5 -> 17.5 at 5 516 (launch_merge_small).
+// were all that fits on an SM: 61.4 -> 57.3 us at 32 976 tokens, 132 -> 115 at 65 952, 19.5 -> 17.5 at 5 516 (unit_ctas).
 constexpr int kMergeAux = 32 * 4 + 32 * 4 + 32 + 64;   // reciprocal group sizes, group sizes, 3 mbarriers, merged rows of the tokens
 constexpr int kMergeStages = 2;
 constexpr int kMergeSmem = kWarps * (kMergeStages * (int)kStage + kMergeAux) + 1024 /*alignment slack*/;
@@ -668,9 +668,7 @@ cudaError_t launch_merge_small(const MergeArgs& a, int sm_count, cudaStream_t st
     const int64_t units = (int64_t)a.heads * (a.n_blocks + sp_units);
     auto launch = [&](auto kernel, int parts, int ctas) { return launch_kernel(kernel, small_grid(units * parts, sm_count, ctas), kWarps * 32, kMergeSmem, stream, m, a); };
     if (3 * units <= 2ll * kWarps * sm_count) return launch(direct ? merge_small_kernel<2, true, true> : merge_small_kernel<2, false, true>, 3, 2);
-    // A round of units takes 24 warps per SM (80 registers) 1.4 times as long as 16 (111), so the third CTA pays in the long run: merge at 65 952 tokens x 16 heads (11 rounds of
-    // 24 warps) 115 us with it, 122 without, 32 976 (5.5) 57.3 and 58.4, 10 992 (1.8) 24.5 and 23.6, 5 516 (1.04, two either way) 19.5 and 17.5.
-    if (units > 5 * 3ll * kWarps * sm_count) return launch(direct ? merge_small_kernel<3, true, false> : merge_small_kernel<3, false, false>, 1, 3);
+    if (unit_ctas(units, sm_count) == 3) return launch(direct ? merge_small_kernel<3, true, false> : merge_small_kernel<3, false, false>, 1, 3);   // 80 registers, else 111
     return launch(direct ? merge_small_kernel<2, true, false> : merge_small_kernel<2, false, false>, 1, 2);
 }
 
