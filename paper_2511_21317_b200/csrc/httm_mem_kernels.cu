@@ -176,32 +176,33 @@ cudaError_t launch_merge(const MergeArgs& a, int max_block_tokens, int sm_count,
 //                      merged length, and the head's first 128-row query tile (for the attention kernel)
 // ------------------------------------------------------------------------------------
 __device__ void finish_level(const OutlierArgs& a, int level, int* hist);   // (threshold selection, below)
-// Latency of the warps' instruction streams and bytes in flight bound the deviation kernel: 16 warps per SM with two stages each rather than
-// 12 with three, and the means read back 16 bytes at a time (32 976 tokens: all five kernels of the filter 72 -> 65.5 us, the call 685 -> 679 us).
-constexpr int kDevWarps = 8;     // 8 x 12.6 KB of shared memory: two CTAs per SM
-constexpr int kDevStages = 2;    // block loads in flight per warp
+// Latency of the warps' instruction streams and bytes in flight bound the deviation kernel: as many warps as fit.  With one stage per warp (refilled while the
+// distances are computed: a lane keeps its token in registers), 16 channels of the means at a time and a histogram of the 1024 bins that occur three CTAs fit on an SM; two
+// stages and two CTAs, before: the five kernels of the filter 59.4 us at 32 976 tokens, now 55.3; the call 697.9 -> 693.8.
+constexpr int kDevWarps = 8;     // 8 x 8.5 KB of shared memory: three CTAs per SM
 constexpr int kCentStride = 68;  // floats per mean: 16-byte reads of eight different means fall on distinct banks
 constexpr int kDevAux = 16 * kCentStride * 4 + 16 * 4 + 32 + 64;   // means of the groups of two or more (at most 16 in 32 tokens), reciprocal sizes, mbarriers, rows
-constexpr int kDevSmem = kDevWarps * (kDevStages * 32 * kRowBytes + kDevAux) + 2048 * 4 /*histogram*/ + 1024 /*alignment slack*/;
+constexpr int kDevBins = 1024;   // of level 0: the sign bit of a deviation is 0
+constexpr int kDevSmem = kDevWarps * (32 * kRowBytes + kDevAux) + kDevBins * 4 /*histogram*/ + 1024 /*alignment slack*/;
 
-__global__ void __launch_bounds__(kDevWarps * 32, 2)
+__global__ void __launch_bounds__(kDevWarps * 32, 3)
 deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a) {
     constexpr uint32_t STAGE_BYTES = 32 * kRowBytes;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + align_pad(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tq = lane & 3;   // MMA accumulator layout: rows g, g + 8; columns 2 tq, 2 tq + 1
-    unsigned char* stage = smem + (size_t)warp * kDevStages * STAGE_BYTES;
-    unsigned char* aux = smem + (size_t)kDevWarps * kDevStages * STAGE_BYTES + (size_t)warp * kDevAux;
+    unsigned char* stage = smem + warp * STAGE_BYTES;
+    unsigned char* aux = smem + kDevWarps * STAGE_BYTES + warp * kDevAux;
     float* cent = reinterpret_cast<float*>(aux);                   // [16][68] group means
     float* rcnt = cent + 16 * kCentStride;                         // [16] 1 / group size
-    int* hist = reinterpret_cast<int*>(smem + (size_t)kDevWarps * (kDevStages * STAGE_BYTES + kDevAux));   // [2048] bits 31-21 of this CTA's deviations
-    for (int i = threadIdx.x; i < 2048; i += kDevWarps * 32) hist[i] = 0;
+    int* hist = reinterpret_cast<int*>(smem + kDevWarps * (STAGE_BYTES + kDevAux));   // [1024] bits 30-21 of this CTA's deviations
+    for (int i = threadIdx.x; i < kDevBins; i += kDevWarps * 32) hist[i] = 0;
     __syncthreads();
-    const uint32_t mbar0 = smem_u32(aux + 16 * kCentStride * 4 + 16 * 4), stage0 = smem_u32(stage);
+    const uint32_t mbar = smem_u32(aux + 16 * kCentStride * 4 + 16 * 4), blk = smem_u32(stage);
     __nv_bfloat16* rows_of = reinterpret_cast<__nv_bfloat16*>(aux + 16 * kCentStride * 4 + 16 * 4 + 32);   // [32] mean of each token, in fragment order
     if (lane == 0) {
-        for (int st = 0; st < kDevStages; ++st) mbar_init(mbar0 + 8 * st, 1);
+        mbar_init(mbar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -211,7 +212,7 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
     const int box_rows = box_f * box_h * box_w;
     const int own_t = lane / (box_h * box_w), own_y = (lane / box_w) % box_h, own_x = lane % box_w;
     for (int q = box_rows * 8 + lane; q < 32 * 8; q += 32)   // rows no load ever writes enter the MMAs with weight 0: keep them finite
-        for (int st = 0; st < kDevStages; ++st) *reinterpret_cast<uint4*>(stage + st * STAGE_BYTES + q * 16) = make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(stage + q * 16) = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
     BoxMap bm;
     bm.clipped = false;
@@ -222,26 +223,21 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
     TaskCursor cur, nxt;
     cur.init(first, stride, a.heads, a.n_blocks);   // one "tensor": t stays 0 while the task index is in range
     nxt = cur;
-    auto issue = [&](const TaskCursor& c, int buf) {   // lane 0 only
-        const BlockGeom bg = a.geom[c.u];
-        const uint32_t mb = mbar0 + 8 * buf;
-        mbar_expect_tx(mb, (uint32_t)box_rows * kRowBytes);
-        tma_block_load(stage0 + buf * STAGE_BYTES, &map_q, mb, bg.x0, bg.y0, bg.s0, c.h);
+    auto issue = [&]() {   // lane 0 only
+        const BlockGeom bg = a.geom[nxt.u];
+        mbar_expect_tx(mbar, (uint32_t)box_rows * kRowBytes);
+        tma_block_load(blk, &map_q, mbar, bg.x0, bg.y0, bg.s0, nxt.h);
     };
     if (!a.early) depend_wait();
-#pragma unroll
-    for (int st = 0; st < kDevStages; ++st) {
-        if (first + st * stride < n_tasks && lane == 0) issue(nxt, st);
-        nxt.advance();
-    }
+    if (first < n_tasks && lane == 0) issue();
+    nxt.advance();
     if (a.early) depend_wait();
     dependents_launch();
 
-    int buf = 0;
     uint32_t parity = 0;
     bool failed = false;
-    for (int64_t task = first; task < n_tasks; task += stride, cur.advance(), nxt.advance()) {
-        const bool more = task + kDevStages * stride < n_tasks;
+    for (int64_t task = first; task < n_tasks; task += stride, cur.advance(), nxt.advance(), parity ^= 1u) {
+        const bool more = task + stride < n_tasks;
         const int h = cur.h;
         const BlockInfo bi = a.blocks[cur.u];
         const BlockGeom bg = a.geom[cur.u];
@@ -258,14 +254,15 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
             }
             rep = bm.row_of_token(rep);
         }
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(mbar0 + 8 * buf, parity, a.status, kDevTimeoutMatchLoad))) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(mbar, parity, a.status, kDevTimeoutMatchLoad))) {
             failed = true;
             break;
         }
         if (r == 0) {   // nothing merged in this block: every deviation is 0
             if (tok >= 0) eps[tok] = 0.f;
+            __syncwarp();
+            if (more && lane == 0) issue();
         } else {
-            const uint32_t blk = stage0 + buf * STAGE_BYTES;
             // groups of two or more tokens get a mean; row of the mean = rank of the group's representative among them
             const unsigned group = __match_any_sync(0xffffffffu, rep);   // (lanes without a token share rep = -1: ignored below)
             const int group_size = rep >= 0 ? __popc(group) : 0;
@@ -273,53 +270,45 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
             const int row_of = group_size >= 2 ? __popc(multi & ((1u << rep) - 1u)) : -1;
             if (rep == lane && group_size >= 2) rcnt[row_of] = 1.0f / (float)group_size;
             rows_of[fragment_order(lane)] = __float2bfloat16_rn((float)row_of);
-            // group sums = W x on the tensor cores, as in merge_small_kernel: W [16 means][32 tokens] of zeros and ones
-            uint32_t bf[2][4][4];
-            const int n_ks = box_rows > 16 ? 2 : 1;
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-                if (ks < n_ks) {
-                    const int row = 16 * ks + (lane & 7) + ((lane >> 3) & 1) * 8;
-                    const uint32_t rowaddr = blk + row * kRowBytes;
-#pragma unroll
-                    for (int np = 0; np < 4; ++np) ldmatrix_x4_trans(bf[ks][np], rowaddr + (((2 * np + (lane >> 4)) ^ (row & 7)) << 4));
-                }
-            }
             __syncwarp();   // rows and reciprocal group sizes visible
-            float c[8][4];
-            const int r0 = g, r1 = g + 8;
+            // group sums = W x on the tensor cores, as in merge_small_kernel: W [16 means][32 tokens] of zeros and ones, 16 channels at a time; the means stay in
+            // fp32 (no rounding to bf16 before the distance)
+            const int n_ks = box_rows > 16 ? 2 : 1, n_cent = __popc(multi);
+            uint32_t af[2][4];
 #pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-                if (ks < n_ks) {
-                    uint32_t af[4];
-                    w_fragment(af, *reinterpret_cast<const uint2*>(rows_of + 16 * ks + 4 * tq), row_pair(r0), row_pair(r1));
+            for (int ks = 0; ks < 2; ++ks) w_fragment(af[ks], *reinterpret_cast<const uint2*>(rows_of + 16 * ks + 4 * tq), row_pair(g), row_pair(g + 8));
+            const float i0 = g < n_cent ? rcnt[g] : 0.f, i1 = g + 8 < n_cent ? rcnt[g + 8] : 0.f;
+            const uint32_t from = blk + (lane & 15) * kRowBytes;
 #pragma unroll
-                    for (int nt = 0; nt < 8; ++nt) {
-                        if (ks == 0)
-                            mma_first(c[nt], af, bf[ks][nt >> 1][2 * (nt & 1)], bf[ks][nt >> 1][2 * (nt & 1) + 1]);
-                        else
-                            mma_bf16_16816(c[nt], af, bf[ks][nt >> 1][2 * (nt & 1)], bf[ks][nt >> 1][2 * (nt & 1) + 1]);
-                    }
+            for (int np = 0; np < 4; ++np) {
+                const uint32_t chunk = ((2 * np + (lane >> 4)) ^ (lane & 7)) << 4;
+                uint32_t bf[2][4];
+                float c[2][4];
+                ldmatrix_x4_trans(bf[0], from + chunk);
+                if (n_ks > 1) ldmatrix_x4_trans(bf[1], from + 16 * kRowBytes + chunk);
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    mma_first(c[nt], af[0], bf[0][2 * nt], bf[0][2 * nt + 1]);
+                    if (n_ks > 1) mma_bf16_16816(c[nt], af[1], bf[1][2 * nt], bf[1][2 * nt + 1]);
+                    float* to = cent + (2 * np + nt) * 8 + 2 * tq;
+                    if (g < n_cent) *reinterpret_cast<float2*>(to + g * kCentStride) = make_float2(c[nt][0] * i0, c[nt][1] * i0);
+                    if (g + 8 < n_cent) *reinterpret_cast<float2*>(to + (g + 8) * kCentStride) = make_float2(c[nt][2] * i1, c[nt][3] * i1);
                 }
             }
-            const int n_cent = __popc(multi);
-            const float i0 = r0 < n_cent ? rcnt[r0] : 0.f, i1 = r1 < n_cent ? rcnt[r1] : 0.f;
+            uint4 x8[8];   // this lane's token (stage row `lane`)
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt) {   // the means stay in fp32 (no rounding to bf16 before the distance)
-                if (r0 < n_cent) *reinterpret_cast<float2*>(cent + r0 * kCentStride + nt * 8 + 2 * tq) = make_float2(c[nt][0] * i0, c[nt][1] * i0);
-                if (r1 < n_cent) *reinterpret_cast<float2*>(cent + r1 * kCentStride + nt * 8 + 2 * tq) = make_float2(c[nt][2] * i1, c[nt][3] * i1);
-            }
-            __syncwarp();   // means visible
+            for (int ch = 0; ch < 8; ++ch) x8[ch] = *reinterpret_cast<const uint4*>(stage + lane * kRowBytes + ((ch ^ (lane & 7)) << 4));
+            __syncwarp();   // means visible, every lane has read the stage
+            if (more && lane == 0) issue();
             float dev = 0.f;
             if (tok >= 0) {
                 float2 d2 = make_float2(0.f, 0.f);   // even and odd channels
-                if (row_of >= 0) {   // distance of this lane's token (stage row `lane`) to its group's mean
-                    const unsigned char* row = stage + buf * STAGE_BYTES + lane * kRowBytes;
+                if (row_of >= 0) {   // distance of this lane's token to its group's mean
                     const float* cr = cent + row_of * kCentStride;
 #pragma unroll
                     for (int ch = 0; ch < 8; ++ch) {
                         float x[8];
-                        unpack8(*reinterpret_cast<const uint4*>(row + ((ch ^ (lane & 7)) << 4)), x);
+                        unpack8(x8[ch], x);
                         const float4 lo = *reinterpret_cast<const float4*>(cr + ch * 8), hi = *reinterpret_cast<const float4*>(cr + ch * 8 + 4);
                         const float2 m[4] = {make_float2(lo.x, lo.y), make_float2(lo.z, lo.w), make_float2(hi.x, hi.y), make_float2(hi.z, hi.w)};
 #pragma unroll
@@ -333,29 +322,19 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
                 eps[tok] = dev;
             }
             // level 0 of the threshold selection: histogram of the top 11 bits (zeros are not counted), one atomic per distinct bin
-            const int bin = (int)(__float_as_uint(dev) >> 21);
+            const int bin = (int)(__float_as_uint(dev) >> 21) & (kDevBins - 1);
             const unsigned peers = __match_any_sync(0xffffffffu, bin);
             if (bin > 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], __popc(peers));
         }
-        __syncwarp();   // every lane is done with the stage and the tables
-        if (more && lane == 0) issue(nxt, buf);
-        if (++buf == kDevStages) {
-            buf = 0;
-            parity ^= 1u;
-        }
+        __syncwarp();   // every lane is done with the tables
     }
-    if (failed) {   // give copies that may still be in flight a bounded chance to land before the shared memory is released
-        for (int st = 0; st < kDevStages; ++st) {
-            mbar_wait_bounded(mbar0 + 8 * st, parity, a.status, kDevTimeoutMatchLoad);
-            mbar_wait_bounded(mbar0 + 8 * st, parity ^ 1u, a.status, kDevTimeoutMatchLoad);
-        }
-    }
+    if (failed) mbar_wait_bounded(mbar, parity, a.status, kDevTimeoutMatchLoad);   // give the copy in flight a bounded chance to land before the shared memory is released
     __syncthreads();
-    for (int i = threadIdx.x; i < 2048; i += kDevWarps * 32) {
+    for (int i = threadIdx.x; i < kDevBins; i += kDevWarps * 32) {
         const int c = hist[i];
         if (c) atomicAdd(a.sel + kSelHist + i, c);
     }
-    finish_level(a, 0, hist);
+    finish_level(a, 0, reinterpret_cast<int*>(smem));   // (the stages, which nothing is copied to any more)
 }
 
 // ---- tau = the (K+1)-th largest deviation over all heads (K = the budget): radix select on the bit patterns of the
@@ -622,7 +601,7 @@ cudaError_t launch_deviation(const OutlierArgs& a, int sm_count, cudaStream_t st
     if (!encode_block_map(&mq, a.src_q, a.layout, a.heads)) return cudaErrorInvalidValue;
     const int64_t n_tasks = (int64_t)a.heads * a.n_blocks;
     int64_t grid = (n_tasks + kDevWarps - 1) / kDevWarps;
-    if (grid > 2ll * sm_count) grid = 2ll * sm_count;
+    if (grid > 3ll * sm_count) grid = 3ll * sm_count;
     if (grid < 1) grid = 1;
     return launch_kernel(deviation_kernel, (unsigned)grid, kDevWarps * 32, kDevSmem, stream, mq, a);
 }
