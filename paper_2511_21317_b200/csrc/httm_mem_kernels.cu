@@ -234,9 +234,9 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
     if (a.early) depend_wait();
     dependents_launch();
 
-    uint32_t parity = 0;
+    int buf = 0;   // phase of the stage's barrier
     bool failed = false;
-    for (int64_t task = first; task < n_tasks; task += stride, cur.advance(), nxt.advance(), parity ^= 1u) {
+    for (int64_t task = first; task < n_tasks; task += stride, cur.advance(), nxt.advance(), buf ^= 1) {
         const bool more = task + stride < n_tasks;
         const int h = cur.h;
         const BlockInfo bi = a.blocks[cur.u];
@@ -254,7 +254,7 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
             }
             rep = bm.row_of_token(rep);
         }
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(mbar, parity, a.status, kDevTimeoutMatchLoad))) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(mbar, buf, a.status, kDevTimeoutMatchLoad))) {
             failed = true;
             break;
         }
@@ -328,7 +328,7 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
         }
         __syncwarp();   // every lane is done with the tables
     }
-    if (failed) mbar_wait_bounded(mbar, parity, a.status, kDevTimeoutMatchLoad);   // give the copy in flight a bounded chance to land before the shared memory is released
+    if (failed) mbar_wait_bounded(mbar, buf, a.status, kDevTimeoutMatchLoad);   // give the copy in flight a bounded chance to land before the shared memory is released
     __syncthreads();
     for (int i = threadIdx.x; i < kDevBins; i += kDevWarps * 32) {
         const int c = hist[i];
