@@ -37,8 +37,9 @@ __device__ __forceinline__ bool team_any(bool x) {
 // Per tensor: squared norms of the team's rows (diagonals of a 16-row tile against itself), then the cosines of a warp's 32 rows
 // with every dst token, 8 dst tokens at a time gathered by giving ldmatrix their row addresses (m16n8k16, exact bf16
 // products, fp32 accumulation), best dst per row (ties: lowest).  The r src with the best scores merge (ties: lowest position
-// first): every thread counts the keys before its own; where a single warp has at most kMaxRounds to leave out (all blocks
-// from ratio 0.5 on) it strikes them one by one with warp minima instead (48-token blocks, ratio 0.6: 20 instead of 27 us).
+// first): a single warp strikes the ones to leave out one by one with warp minima where there are at most kMaxRounds (all blocks from ratio 0.5 on; 48-token blocks,
+// ratio 0.6: 20 us instead of 27), else every thread counts the keys before its own; the warps of a
+// larger team look for the line between them (choose).
 constexpr int kMaxRounds = 16;
 struct MatchAux {   // shared memory behind the two stages
     int inv, keys, best, dst_row, dst_pos, src, bars, bytes;
@@ -79,6 +80,48 @@ constexpr int team_smem(int w, int p) {
 constexpr int team_ctas(int w, int p) {   // CTAs per SM: all of a persistent grid have to be resident
     const int by_warps = (p == 1 ? 24 : 12) / w, by_smem = 228 * 1024 / (team_smem(w, p) + 1024);
     return by_warps < by_smem ? by_warps : by_smem;
+}
+
+// Is this thread's key (row 32 warp + lane, 0: no src token) one of the r largest of n_rows stage rows, equal ones at the lowest rows first?  (Fewer than all merge.)
+// Every warp of the team looks for a value with r keys above it, by bisection between the smallest and the largest key: with distinct keys about as many steps as the
+// logarithm of their number, 32 at most.  Every thread counting the keys that come before its own took a warp of a 128-token block 400 instructions, this 150: 32 976 tokens x 16 heads,
+// ratio 0.6 a call 1021 -> 980 us, 0.7 655 -> 615; 52 318 tokens x 8 heads, ratios 0.56 and 0.74, match 87 -> 57 us.
+template <int NK>
+__device__ __forceinline__ bool choose(const uint32_t* keys, int n_rows, int r, uint32_t mine, int warp, int lane) {
+    uint32_t k[NK], hi = 0u, lo = 0xffffffffu;
+#pragma unroll
+    for (int j = 0; j < NK; ++j) {
+        k[j] = 32 * j + lane < n_rows ? keys[32 * j + lane] : 0u;
+        hi = max(hi, k[j]);
+        lo = min(lo, k[j] - 1u);   // (0 becomes the largest)
+    }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_min_sync(0xffffffffu, lo);   // at most r keys above hi, at least r above lo
+    int above = 0;                             // keys above hi
+#pragma unroll 1
+    while (hi - lo > 1u) {
+        const uint32_t bar = lo + (hi - lo) / 2;
+        int c = 0;
+#pragma unroll
+        for (int j = 0; j < NK; ++j) c += k[j] > bar ? 1 : 0;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (c > r) {
+            lo = bar;
+        } else {
+            hi = bar;
+            above = c;
+            if (c == r) break;
+        }
+    }
+    if (above == r) return mine > hi;
+    // more keys equal to hi than are wanted of them: those at the lowest rows
+    int before = 0;
+#pragma unroll
+    for (int j = 0; j < NK; ++j) {
+        const unsigned equal = __ballot_sync(0xffffffffu, k[j] == hi);
+        before += j < warp ? __popc(equal) : (j == warp ? __popc(equal & ((1u << lane) - 1u)) : 0);
+    }
+    return mine > hi || (mine == hi && before < r - above);
 }
 
 template <int W, int P, bool DIRECT>
@@ -323,6 +366,8 @@ match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 #pragma unroll
                     for (int p = 0; p < P; ++p) merged[p] = merged[p] && out != 32 * p + lane;
                 }
+            } else if (W > 1) {
+                merged[0] = choose<NMAX / 32>(keys, (n_rows + 15) & ~15, r, key[0], warp, lane);
             } else {   // count the src tokens that come before each
 #pragma unroll
                 for (int p = 0; p < P; ++p) {

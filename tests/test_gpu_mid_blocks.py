@@ -50,3 +50,15 @@ def test_a_block_per_warp_and_per_team_agree(blk, ratio_q, ratio_kv):
         one = run(hb.HttmConfig.of(wl.replace(heads=1)), (q[h:h + 1], k[h:h + 1], v[h:h + 1]))
         for name in ITEMS:
             assert np.array_equal(whole[name][h], one[name][0]), (name, h)
+
+
+@pytest.mark.parametrize("blk,ratio", [((2, 8, 8), 0.5), ((2, 8, 8), 0.7), ((1, 5, 13), 0.3), ((4, 8, 8), 0.6), ((4, 4, 4), 0.5), ((2, 4, 4), 0.5), ((2, 4, 4), 0.3)])
+def test_some_scores_are_equal(blk, ratio):
+    """Tokens that are one of a few vectors: the line between those that merge and the others runs through equal scores, of which the lowest positions merge."""
+    wl = synth.Workload("equal", 3, blk[1] + 3, 2 * blk[2] + 1, *blk, ratio, ratio, n_camera=1, n_register=1, heads=3, seed=8)
+    q, k, v = synth.make_qkv(wl)
+    rng = np.random.default_rng(9)
+    for h in range(wl.heads):
+        kinds = q[h, rng.integers(0, wl.n_tokens, size=3 + 3 * h)]
+        q[h] = kinds[rng.integers(0, len(kinds), size=wl.n_tokens)]
+    report_peaky("equal", run_case(wl, q, q, v, peaky=True))
