@@ -343,7 +343,7 @@ int stage_merge(httm_ctx* c, cudaStream_t s, const httm_tensor* src = nullptr, b
     a.status = c->d_status;
     a.early = chained;
     c->launches++;
-    if (c->big() || sorted_filter(c)) return check_cuda(c, launch_big_merge(a, c->max_block, s), "sorted-group merge launch");
+    if (c->big() || sorted_filter(c)) return check_cuda(c, launch_big_merge(a, c->max_block, c->sm_count, s), "sorted-group merge launch");
     return check_cuda(c, launch_merge(a, c->max_block, c->sm_count, s), "merge launch");
 }
 
@@ -442,7 +442,7 @@ int stage_outlier(httm_ctx* c, const httm_tensor& q, cudaStream_t s, bool chaine
         const bool sorted = sorted_filter(c);
         if (sorted) {
             a.src_q = view(c->d_qr, c->n_tokens);
-            if ((rc = check_cuda(c, launch_big_deviation(a, c->max_block, s), "large-block deviation launch"))) return rc;
+            if ((rc = check_cuda(c, launch_big_deviation(a, c->max_block, c->sm_count, s), "large-block deviation launch"))) return rc;
             if ((rc = check_cuda(c, launch_refine_level(a, 0, c->sm_count, s), "threshold launch"))) return rc;
             c->launches += 2;
         } else {
@@ -468,7 +468,7 @@ int stage_outlier(httm_ctx* c, const httm_tensor& q, cudaStream_t s, bool chaine
     }
     if (sorted_filter(c)) {   // the blocks are runs of rows of the reordered copy; six kernels
         a.src_q = view(c->d_qr, c->n_tokens);
-        if ((rc = check_cuda(c, launch_big_deviation(a, c->max_block, s), "large-block deviation launch"))) return rc;
+        if ((rc = check_cuda(c, launch_big_deviation(a, c->max_block, c->sm_count, s), "large-block deviation launch"))) return rc;
         if ((rc = check_cuda(c, launch_threshold0(a, c->sm_count, s), "threshold launch"))) return rc;
         if ((rc = check_cuda(c, launch_big_filter(a, c->max_block, s), "large-block filter launch"))) return rc;
         c->launches += 6;

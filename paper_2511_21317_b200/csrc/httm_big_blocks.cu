@@ -74,7 +74,7 @@ struct ScoreItem {
     int t;                            // tensor (0: Q, 1: K); -1: no more items
     int n_rule, even;                 // the block's dst rule; evenly spaced
     int nd, n_src;                    // dst and src tokens
-    int n_chunks, n_st, n_pairs;      // chunks of dst tokens, tiles of src tokens and pairs of them (none where nothing merges in this block)
+    int n_chunks, st0, n_st, n_pairs; // chunks of dst tokens, the item's tiles of src tokens and pairs of them (none where nothing merges in this block)
     int stages, ring;                 // stages of the ring of token tiles and where it begins
     int64_t row0;                     // row of the block's first token in [H][N]
 };
@@ -87,22 +87,25 @@ constexpr int SC_SMEM = SC_OFF_ITEMS + 2 * 64 + 1024 /*alignment slack*/;
 static_assert(sizeof(ScoreBars) <= 384 && sizeof(ScoreItem) <= 64 && kMaxBigDst % TILE == 0 && SC_AREA % 1024 == 0 && SC_SMEM <= 232448, "");
 
 __device__ __forceinline__ void write_item(ScoreItem* to, const BigMatchArgs& a, int t_first, int item) {
-    const int per_tensor = a.heads * a.n_blocks;
+    const int per_tensor = a.heads * a.n_blocks * a.parts;
     if (item >= 2 * per_tensor) {
         to->t = -1;
         return;
     }
-    const int t = item < per_tensor ? t_first : 1 - t_first, rem = item < per_tensor ? item : item - per_tensor;
+    const int t = item < per_tensor ? t_first : 1 - t_first, at = item < per_tensor ? item : item - per_tensor;
+    const int rem = at / a.parts, part = at - rem * a.parts;
     const BlockInfo bi = a.blocks[a.order[rem / a.heads]];
     const int nd = t == 0 ? bi.nd_q : bi.nd_k, n_src = bi.n - nd;
     const bool merges = (t == 0 ? bi.r_q : bi.r_k) > 0;
-    const int n_st = merges ? (n_src + TILE - 1) / TILE : 0, ring = (nd + 7) / 8 * 8 * kRowBytes;   // (the last chunk's MMAs read into the ring: masked columns)
+    const int tiles = merges ? (n_src + TILE - 1) / TILE : 0, st0 = tiles * part / a.parts, n_st = tiles * (part + 1) / a.parts - st0;
+    const int ring = (nd + 7) / 8 * 8 * kRowBytes;   // (the last chunk's MMAs read into the ring: masked columns)
     to->t = t;
     to->n_rule = bi.n_rule;
     to->nd = nd;
     to->n_src = n_src;
     to->even = bi.n_rule == bi.n;
-    to->n_chunks = merges ? (nd + TILE - 1) / TILE : 0;
+    to->n_chunks = n_st > 0 ? (nd + TILE - 1) / TILE : 0;
+    to->st0 = st0;
     to->n_st = n_st;
     to->n_pairs = (n_st + 1) / 2;
     to->ring = ring;
@@ -244,8 +247,8 @@ big_scores_kernel(const BigMatchArgs a) {
                 const __nv_bfloat16* x = a.xr[it.t] + it.row0 * kHeadDim;
                 const int at = tid - 64, c16 = at & 7;
                 // src token s is token s + (dst tokens before it): s + floor(s nd / (n - nd)), or s + nd where the first nd tokens are the dst tokens
-                Ramp before((at >> 3) * it.nd, SC_LOADERS / 8 * it.nd, max(it.n_src, 1));
-                int s = at >> 3, handed = 0, hand_st = 0;   // next src token of this thread; tiles handed over, stage of the next
+                Ramp before((it.st0 * TILE + (at >> 3)) * it.nd, SC_LOADERS / 8 * it.nd, max(it.n_src, 1));
+                int s = it.st0 * TILE + (at >> 3), handed = 0, hand_st = 0;   // next src token of this thread; tiles handed over, stage of the next
                 uint32_t par = fills;
                 auto hand_over = [&]() __attribute__((always_inline)) {
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor cores read the rows through the async proxy
@@ -448,8 +451,8 @@ big_scores_kernel(const BigMatchArgs a) {
                 int arg[2], own[2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const int s = (2 * p + e) * TILE + row;   // src token
-                    own[e] = s < n_src ? src_position(s) : -1;   // token number inside the block
+                    const int s = (it.st0 + 2 * p + e) * TILE + row;   // src token
+                    own[e] = 2 * p + e < it.n_st && s < n_src ? src_position(s) : -1;   // token number inside the block (behind an odd last tile: another item's)
                     int in_group = 0;
 #pragma unroll
                     for (int c = kGroup - 1; c >= 0; --c)
@@ -840,7 +843,7 @@ __device__ __forceinline__ void sum_members(const __nv_bfloat16* x, const uint32
 }
 
 template <int T, int E>
-__global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const MergeArgs a, int sp_chunks) {
+__global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const MergeArgs a, int sp_chunks, int shares) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
     uint32_t* keys = reinterpret_cast<uint32_t*>(mg_smem);                                     // [P] (merged row << 12) | position
     int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (E * T) * 4);            // [n] merged row of a kept token, -1
@@ -849,7 +852,7 @@ __global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const M
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     depend_wait();
     dependents_launch();
-    const int n_block_ctas = 2 * a.heads * a.n_blocks;
+    const int n_block_ctas = 2 * a.heads * a.n_blocks * shares;
     const int ch = lane & 7, sub = lane >> 3;   // 16-byte chunk of a row; which of four rows in flight
 
     if ((int)blockIdx.x >= n_block_ctas) {
@@ -864,9 +867,9 @@ __global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const M
         }
         return;
     }
-    const int per_map = a.heads * a.n_blocks;
+    const int per_map = a.heads * a.n_blocks, cta = blockIdx.x / shares, share = blockIdx.x - cta * shares;
     // (the K map, which also merges V, first: its CTAs take longer)
-    const int m = 1 - blockIdx.x / per_map, h = (blockIdx.x % per_map) / a.n_blocks, b = blockIdx.x % a.n_blocks;
+    const int m = 1 - cta / per_map, h = (cta % per_map) / a.n_blocks, b = cta % a.n_blocks;
     const BlockInfo bi = a.blocks[b];
     const int n = bi.n, r = m == 0 ? bi.r_q : bi.r_k, m_len = m == 0 ? a.m_q : a.m_k;
     const bool variable = m == 0 && a.moff_q_var != nullptr;   // after outlier filtering the kept count of a block varies by head
@@ -881,7 +884,7 @@ __global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const M
     for (int t = (m == 0 ? 0 : 1); t <= (m == 0 ? 0 : 2); ++t) {
         const __nv_bfloat16* x = a.xr[t] + base * kHeadDim;
         __nv_bfloat16* out = a.merged[t] + ((int64_t)h * m_len + moff) * kHeadDim;
-        for (int row = warp * 4 + sub; row < n_kept; row += (T / 32) * 4) {
+        for (int row = share * (T / 8) + warp * 4 + sub; row < n_kept; row += shares * (T / 8)) {
             const int i0 = seg[row], i1 = seg[row + 1];
             float2 acc[4];
             sum_members(x + 8 * ch, keys, i0, i1, acc);
@@ -910,7 +913,7 @@ __global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const M
 // members and one square root for them took the filter kernels together, at 82 440 tokens x 16 heads in 3840-token blocks, from 221 to 178 us
 // (32 976 tokens in 128-token blocks: 104.7 -> 92.2; 137 400 in 64-token blocks: 363 -> 302).
 template <int T, int E>
-__global__ void __launch_bounds__(T, kSortedThreads / T) big_deviation_kernel(const OutlierArgs a) {
+__global__ void __launch_bounds__(T, kSortedThreads / T) big_deviation_kernel(const OutlierArgs a, int shares) {
     extern __shared__ __align__(16) unsigned char mg_smem[];
     uint32_t* keys = reinterpret_cast<uint32_t*>(mg_smem);
     int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (E * T) * 4);
@@ -918,7 +921,7 @@ __global__ void __launch_bounds__(T, kSortedThreads / T) big_deviation_kernel(co
     int* warp_sum = seg + (E * T) + 4;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ch = lane & 7, sub = lane >> 3;
-    const int h = blockIdx.x / a.n_blocks, b = blockIdx.x % a.n_blocks;
+    const int cta = blockIdx.x / shares, share = blockIdx.x - cta * shares, h = cta / a.n_blocks, b = cta % a.n_blocks;
     const BlockInfo bi = a.blocks[b];
     const int n = bi.n;
     const int64_t base = (int64_t)h * a.n_tokens + bi.start;
@@ -932,7 +935,7 @@ __global__ void __launch_bounds__(T, kSortedThreads / T) big_deviation_kernel(co
     const int n_kept = build_groups<T, E>(a.assign_q + base, bi.start, n, n, keys, row_of, seg, warp_sum, nullptr, a.status, nullptr, 0);
     const __nv_bfloat16* x = a.src_q.ptr + base * kHeadDim + 8 * ch;   // the reordered copy
     // eight lanes per group (a lane owns 8 of the 64 channels), four groups per warp at a time
-    for (int row = warp * 4 + sub; row < ((n_kept + 3) & ~3); row += (T / 32) * 4) {   // (whole sub-groups stay together for the shuffles)
+    for (int row = share * (T / 8) + warp * 4 + sub; row < ((n_kept + 3) & ~3); row += shares * (T / 8)) {   // (whole sub-groups stay together for the shuffles)
         const bool live = row < n_kept;
         const int i0 = live ? seg[row] : 0, i1 = live ? seg[row + 1] : 0;
         if (i1 - i0 < 2) {
@@ -1065,10 +1068,19 @@ cudaError_t with_cta_size(int max_block, F&& f) {
     return f(std::integral_constant<int, 512>{}, std::integral_constant<int, 8>{});
 }
 
-cudaError_t launch_big_deviation(const OutlierArgs& a, int max_block, cudaStream_t stream) {
+// CTAs for a block of the kernels that sort its tokens and then gather the rows of its groups, where blocks alone would leave SMs without: each sorts all tokens and
+// gathers a share of the rows: merge of 64 maps of up to 1408 tokens 23.6 -> 17.4 us, of 96 of up to 1024 29.7 -> 19.5.  (With more of them than fit at once every
+// sort is paid for: two CTAs for each of 704 maps of 3840 tokens 225 -> 250 us.)
+int row_shares(int64_t blocks, int64_t resident) {
+    const int64_t s = resident / (blocks > 0 ? blocks : 1);
+    return (int)(s < 1 ? 1 : s > 4 ? 4 : s);
+}
+
+cudaError_t launch_big_deviation(const OutlierArgs& a, int max_block, int sm_count, cudaStream_t stream) {
     return with_cta_size(max_block, [&](auto t, auto e) {
         constexpr int T = decltype(t)::value, E = decltype(e)::value;
-        return launch_kernel(big_deviation_kernel<T, E>, a.heads * a.n_blocks, T, mg_smem_bytes(E * T), stream, a);
+        const int shares = row_shares((int64_t)a.heads * a.n_blocks, (int64_t)(kSortedThreads / T) * sm_count);
+        return launch_kernel(big_deviation_kernel<T, E>, a.heads * a.n_blocks * shares, T, mg_smem_bytes(E * T), stream, a, shares);
     });
 }
 
@@ -1102,11 +1114,15 @@ cudaError_t configure_big_blocks() {
     return e;
 }
 
-cudaError_t launch_big_scores(const BigMatchArgs& a, int sm_count, cudaStream_t stream) {
-    const int64_t total = 2ll * a.heads * a.n_blocks;
-    int ctas = sm_count < 1 ? 1 : sm_count;
-    if (ctas > total) ctas = (int)total;
-    if (ctas < 1) ctas = 1;
+cudaError_t launch_big_scores(const BigMatchArgs& args, int sm_count, cudaStream_t stream) {
+    // Where there are fewer blocks than SMs their src tokens are shared out: every part copies all dst tokens (about 6 us), so only for SMs that have nothing else to do.
+    // 64 items of up to 1408 tokens 31.6 -> 25.5 us.
+    BigMatchArgs a = args;
+    const int64_t blocks = 2ll * a.heads * a.n_blocks;
+    const int sms = sm_count < 1 ? 1 : sm_count;
+    a.parts = (int)(blocks < 1 || blocks > sms ? 1 : sms / blocks > 4 ? 4 : sms / blocks);
+    const int64_t total = blocks * a.parts;
+    const int ctas = (int)(total > sms ? sms : total < 1 ? 1 : total);
     return launch_kernel(big_scores_kernel, ctas, SC_THREADS, SC_SMEM, stream, a);
 }
 
@@ -1114,11 +1130,12 @@ cudaError_t launch_big_select(const BigMatchArgs& a, cudaStream_t stream) {
     return launch_kernel(big_select_kernel, 2 * a.heads * a.n_blocks, SEL_THREADS, 0, stream, a);
 }
 
-cudaError_t launch_big_merge(const MergeArgs& a, int max_block, cudaStream_t stream) {
+cudaError_t launch_big_merge(const MergeArgs& a, int max_block, int sm_count, cudaStream_t stream) {
     return with_cta_size(max_block, [&](auto t, auto e) {
         constexpr int T = decltype(t)::value, E = decltype(e)::value;
         const int sp_chunks = (a.n_special_total + T / 8 - 1) / (T / 8);
-        return launch_kernel(big_merge_kernel<T, E>, 2 * a.heads * a.n_blocks + a.heads * sp_chunks, T, mg_smem_bytes(E * T), stream, a, sp_chunks);
+        const int shares = row_shares(2ll * a.heads * a.n_blocks, (int64_t)(kMergeThreads / T) * sm_count);
+        return launch_kernel(big_merge_kernel<T, E>, 2 * a.heads * a.n_blocks * shares + a.heads * sp_chunks, T, mg_smem_bytes(E * T), stream, a, sp_chunks, shares);
     });
 }
 

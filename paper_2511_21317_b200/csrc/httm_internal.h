@@ -84,6 +84,7 @@ struct BigMatchArgs {
     const int32_t* order;         // [blocks] from the longest to the shortest
     int32_t* counter;             // work items of the score kernel taken behind the first of every CTA; zero before the launch
     int32_t n_blocks, n_tokens, heads;
+    int32_t parts;                // work items a block's src tokens are shared out to (launch_big_scores)
     int32_t* status;
 };
 
@@ -222,11 +223,11 @@ cudaError_t launch_offsets(const OutlierArgs& a, cudaStream_t stream);  // per-h
 cudaError_t launch_threshold0(const OutlierArgs& a, int sm_count, cudaStream_t stream);   // threshold with the level-0 histogram taken from the deviations (three kernels)
 cudaError_t launch_refine_level(const OutlierArgs& a, int level, int sm_count, cudaStream_t stream);   // histogram of one level alone (0, 1, 2)
 cudaError_t launch_select_level(const OutlierArgs& a, int level, cudaStream_t stream);                 // choose the bin of one level from its (summed) histogram
-cudaError_t launch_big_deviation(const OutlierArgs& a, int max_block_tokens, cudaStream_t stream);   // large blocks: deviations
+cudaError_t launch_big_deviation(const OutlierArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream);   // large blocks: deviations
 cudaError_t launch_big_filter(const OutlierArgs& a, int max_block_tokens, cudaStream_t stream);      // large blocks: map rewrite + kept counts
 cudaError_t launch_big_scores(const BigMatchArgs& a, int sm_count, cudaStream_t stream);   // tcgen05 contraction + row argmax
 cudaError_t launch_big_select(const BigMatchArgs& a, cudaStream_t stream);                  // top-r per (tensor, head, block)
-cudaError_t launch_big_merge(const MergeArgs& a, int max_block_tokens, cudaStream_t stream);                      // sort by merged row + gather means
+cudaError_t launch_big_merge(const MergeArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream);                      // sort by merged row + gather means
 cudaError_t configure_big_blocks();
 cudaError_t launch_linear(const LinearArgs& a, int sm_count, cudaStream_t stream);   // tcgen05 GEMM for the projections
 cudaError_t configure_linear();
