@@ -212,7 +212,7 @@ cudaError_t launch_merge(const MergeArgs& a, int max_block_tokens, int sm_count,
 cudaError_t launch_match_small(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream);   // blocks of at most 64 tokens
 cudaError_t launch_merge_small(const MergeArgs& a, int sm_count, cudaStream_t stream);
 cudaError_t configure_small_blocks();
-cudaError_t launch_match_mid(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream);   // blocks of 33 .. 256 tokens
+cudaError_t launch_match_mid(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream);   // blocks of 65 .. 256 tokens
 cudaError_t launch_merge_mid(const MergeArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream);
 cudaError_t configure_mid_blocks();
 cudaError_t launch_unmerge(const UnmergeArgs& a, cudaStream_t stream);

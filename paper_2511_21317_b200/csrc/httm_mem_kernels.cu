@@ -158,9 +158,7 @@ cudaError_t launch_match_anchor(const MatchArgs& a, const TensorView& src_q, con
 }
 
 cudaError_t launch_match(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
-    // 33 .. 64 tokens: a unit per warp of the small-block kernel where there are more units than it has warps (measured there)
-    const bool many = (int64_t)a.heads * a.n_blocks > 16ll * sm_count;
-    return max_block_tokens <= (many ? 64 : 32) ? launch_match_small(a, max_block_tokens, sm_count, stream) : launch_match_mid(a, max_block_tokens, sm_count, stream);
+    return max_block_tokens <= 64 ? launch_match_small(a, max_block_tokens, sm_count, stream) : launch_match_mid(a, max_block_tokens, sm_count, stream);
 }
 cudaError_t launch_merge(const MergeArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
     return max_block_tokens <= 32 ? launch_merge_small(a, sm_count, stream) : launch_merge_mid(a, max_block_tokens, sm_count, stream);

@@ -1,7 +1,7 @@
-// Matching and merging for merging blocks of 33 .. 256 tokens (Eq. 1, Sec. 3.2).  A TEAM of W warps, a CTA of its own, works
+// Matching (65 .. 256 tokens) and merging (33 .. 256) of merging blocks (Eq. 1, Sec. 3.2).  A TEAM of W warps, a CTA of its own, works
 // off a UNIT = one (head, block) with all its tensors; a thread owns P rows of the stage, so that a team takes blocks of
 // 32 W P tokens: (W, P) = (1, 2), (4, 1) and (8, 1) for blocks of up to 64, 128 and 256 tokens.
-// (Blocks of up to 64 tokens are matched by the small-block kernel where there are many of them: launch_match.)
+// (Blocks of up to 64 tokens are matched by the small-block kernel.)
 //
 // What bounds them is instructions and their latency, not memory (2 - 3.3 of 6.5 TB/s).  With one warp per (tensor, head, block) and
 // all of its tokens (16 / 12 / 6 warps per SM, as many blocks as shared memory takes) a 128-token block kept its warp busy for
@@ -37,10 +37,7 @@ __device__ __forceinline__ bool team_any(bool x) {
 // Per tensor: squared norms of the team's rows (diagonals of a 16-row tile against itself), then the cosines of a warp's 32 rows
 // with every dst token, 8 dst tokens at a time gathered by giving ldmatrix their row addresses (m16n8k16, exact bf16
 // products, fp32 accumulation), best dst per row (ties: lowest).  The r src with the best scores merge (ties: lowest position
-// first): a single warp strikes the ones to leave out one by one with warp minima where there are at most kMaxRounds (all blocks from ratio 0.5 on; 48-token blocks,
-// ratio 0.6: 20 us instead of 27), else every thread counts the keys before its own; the warps of a
-// larger team look for the line between them (choose).
-constexpr int kMaxRounds = 16;
+// first): the warps of the team look for the line between them and the others (choose).
 struct MatchAux {   // shared memory behind the two stages
     int inv, keys, best, dst_row, dst_pos, src, bars, bytes;
 };
@@ -127,6 +124,7 @@ __device__ __forceinline__ bool choose(const uint32_t* keys, int n_rows, int r, 
 template <int W, int P, bool DIRECT>
 __global__ void __launch_bounds__(32 * W, team_ctas(W, P))
 match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ MatchArgs a) {
+    static_assert(W > 1 && P == 1, "a thread has one token, a team several warps");
     constexpr int NMAX = team_tokens(W, P), MT = 2 * P, MAX_DST = NMAX / 4;   // MT: 16-row tiles per warp
     constexpr uint32_t STAGE = NMAX * kRowBytes;
     constexpr MatchAux X = match_aux(NMAX);
@@ -342,63 +340,10 @@ match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (more && tid == 0) issue(t, geom_next, bi_next.start, h_next);
             // ---- the r src with the best scores merge (ties: lowest position first; rows are in token order)
             const int n_out = n - nd - r;
-            uint32_t key[P];
-            bool merged[P];
-#pragma unroll
-            for (int p = 0; p < P; ++p) {
-                key[p] = tok[p] >= 0 ? keys[own + 32 * p] : 0u;   // (0: not a src token)
-                merged[p] = key[p] != 0;
-            }
-            if (n_out <= 0) {
-                // all of them
-            } else if (W == 1 && n_out <= kMaxRounds) {   // strike the worst one n_out times (ties: highest position first)
-                for (int round = 0; round < n_out; ++round) {
-                    uint32_t low = 0xffffffffu;
-#pragma unroll
-                    for (int p = 0; p < P; ++p) low = min(low, merged[p] ? key[p] : 0xffffffffu);
-                    low = __reduce_min_sync(0xffffffffu, low);
-                    int out = 0;
-#pragma unroll
-                    for (int p = 0; p < P; ++p) {
-                        const unsigned at = __ballot_sync(0xffffffffu, merged[p] && key[p] == low);
-                        if (at) out = 32 * p + 31 - __clz(at);
-                    }
-#pragma unroll
-                    for (int p = 0; p < P; ++p) merged[p] = merged[p] && out != 32 * p + lane;
-                }
-            } else if (W > 1) {
-                merged[0] = choose<NMAX / 32>(keys, (n_rows + 15) & ~15, r, key[0], warp, lane);
-            } else {   // count the src tokens that come before each
-#pragma unroll
-                for (int p = 0; p < P; ++p) {
-                    if (!merged[p]) continue;
-                    int rank = 0;
-#pragma unroll 1
-                    for (int w = 0; w * 32 < n_rows; ++w) {
-                        // src at higher positions come before this one with a better score, those at lower positions with as good a score too
-                        const bool same = w == warp * P + p;
-                        const uint32_t bar = w < warp * P + p ? key[p] - 1 : key[p];
-                        const int n32 = min(32, ((n_rows + 15) & ~15) - 32 * w);
-                        for (int i = 0; i < n32; i += 4) {
-                            const uint4 k4 = *reinterpret_cast<const uint4*>(keys + 32 * w + i);   // (the same four for every thread: a broadcast)
-                            rank += k4.x > bar ? 1 : 0;
-                            rank += k4.y > bar ? 1 : 0;
-                            rank += k4.z > bar ? 1 : 0;
-                            rank += k4.w > bar ? 1 : 0;
-                            if (same) {
-                                rank += k4.x == key[p] && i < lane ? 1 : 0;
-                                rank += k4.y == key[p] && i + 1 < lane ? 1 : 0;
-                                rank += k4.z == key[p] && i + 2 < lane ? 1 : 0;
-                                rank += k4.w == key[p] && i + 3 < lane ? 1 : 0;
-                            }
-                        }
-                    }
-                    merged[p] = rank < r;
-                }
-            }
-#pragma unroll
-            for (int p = 0; p < P; ++p)
-                if (tok[p] >= 0) A[tok[p]] = bi.start + (merged[p] ? dst_pos[best[own + 32 * p]] : tok[p]);
+            const uint32_t key = tok[0] >= 0 ? keys[own] : 0u;   // (0: not a src token)
+            bool merged = key != 0;
+            if (n_out > 0) merged = choose<NMAX / 32>(keys, (n_rows + 15) & ~15, r, key, warp, lane);
+            if (tok[0] >= 0) A[tok[0]] = bi.start + (merged ? dst_pos[best[own]] : tok[0]);
         }
         if (failed >= 0) break;
     }
@@ -723,8 +668,10 @@ cudaError_t configure_t() {
     auto set = [&](auto kernel, int bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
-    set(match_team_kernel<W, P, false>, team_smem(W, P));
-    set(match_team_kernel<W, P, true>, team_smem(W, P));
+    if constexpr (W > 1) {
+        set(match_team_kernel<W, P, false>, team_smem(W, P));
+        set(match_team_kernel<W, P, true>, team_smem(W, P));
+    }
     set(merge_team_kernel<W, P, false>, team_smem(W, P));
     set(merge_team_kernel<W, P, true>, team_smem(W, P));
     return e;
@@ -733,7 +680,6 @@ cudaError_t configure_t() {
 }  // namespace
 
 cudaError_t launch_match_mid(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
-    if (max_block_tokens <= 64) return launch_match_t<1, 2>(a, sm_count, stream);
     if (max_block_tokens <= 128) return launch_match_t<4, 1>(a, sm_count, stream);
     return launch_match_t<8, 1>(a, sm_count, stream);
 }

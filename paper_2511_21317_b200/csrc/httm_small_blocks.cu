@@ -1,6 +1,6 @@
 // Matching and merging for merging blocks of at most 32 tokens (Eq. 1, Sec. 3.2), one warp per UNIT = one (head, block) with all
 // its tensors: the match kernel works off Q and K of a block, the merge kernel Q, K and V (V follows K's map).
-// Many blocks of up to 64 tokens are matched here too.
+// Blocks of up to 64 tokens are matched here too.
 //
 // A block is 4 KB and 5 KFLOP per tensor, so what bounds these kernels is not the arithmetic but the instructions around it:
 // table entries, block geometry, dst positions, the next load.  With one task per (tensor, head, block) the match kernel
@@ -37,9 +37,9 @@ constexpr int kMatchSmem = kWarps * (2 * (int)kStage + 16) + 1024 /*alignment sl
 
 constexpr int match_ctas(int tiles) { return tiles == 2 ? 3 : 2; }   // per SM: 80 and 128 registers
 // TILES: blocks of up to 32 tokens, 8 dst tokens (2), a stage for either tensor; or up to 64 tokens, 16 dst tokens (4): one stage for Q and K in turn, so that 16 warps
-// fit on an SM (the team of one warp of httm_mid_blocks.cu has two and 12 warps).  K is on its way while the tokens of Q are chosen, so this needs more units than warps
-// to pay: 137 400 tokens in 64-token blocks 161.8 -> 137.5 us, a call 4098 -> 4037; 7 898 tokens in 48-token blocks, 1.3 units per warp, a call 93.5 -> 92.6; 0.6 units
-// per warp 101.8 -> 102.3.  (24 warps with 80 registers spill: 159 us.)
+// fit on an SM.  A team of one warp that kept all its fragments and had two stages, of which 10 fitted, against this: 137 400 tokens in 64-token blocks 161.8 / 137.5 us, a
+// call 4098 / 4037; 7 898 tokens in 48-token blocks 93.5 / 92.6; 4 067 .. 5 229 tokens x 16 heads in 48-token blocks, two rounds against one, calls 8 - 9 % less; 1 743 tokens,
+// a tensor per warp here, 22.5 / 20.8.  (24 warps with 80 registers spill: 159 us.)
 // SPLIT: fewer units than warps: a warp has one tensor of one unit
 template <int TILES, bool DIRECT, bool SPLIT>
 __global__ void __launch_bounds__(kWarps * 32, match_ctas(TILES))
@@ -132,10 +132,10 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t, it += STAGES == 1) {
             // the next tensor of this stage: this one of the next unit or, with one stage, K behind Q
             auto refill = [&]() {   // lane 0 only
-                if (STAGES == 1 && t == 0)
+                if (STAGES == 1 && !SPLIT && t == 0)
                     issue(1, geom, bi.start, h);
                 else if (more)
-                    issue(STAGES == 1 ? 0 : t, bg_next, bi_next.start, h_next);
+                    issue(STAGES == 1 && !SPLIT ? 0 : t, bg_next, bi_next.start, h_next);
             };
             const int r = t == 0 ? bi.r_q : bi.r_k, nd = t == 0 ? bi.nd_q : bi.nd_k;
             int32_t* A = a.assign[t] + (int64_t)h * a.n_tokens + bi.start;
@@ -651,8 +651,8 @@ cudaError_t launch_match_tiles(const MatchArgs& a, int sm_count, cudaStream_t st
     };
     // With no more than one tensor per warp the tensors of a unit go to different warps: the call then waits for one, not two
     // (512 units: 11.3 -> 9.4 us, in the merge kernel below 13.1 -> 9.0).
-    if constexpr (TILES == 2)
-        if (2 * units <= (int64_t)match_ctas(TILES) * kWarps * sm_count) return launch(direct ? match_small_kernel<TILES, true, true> : match_small_kernel<TILES, false, true>, 2);
+    if (2 * units <= (int64_t)match_ctas(TILES) * kWarps * sm_count)
+        return launch(direct ? match_small_kernel<TILES, true, true> : match_small_kernel<TILES, false, true>, 2);
     return launch(direct ? match_small_kernel<TILES, true, false> : match_small_kernel<TILES, false, false>, 1);
 }
 }  // namespace
@@ -679,6 +679,8 @@ cudaError_t configure_small_blocks() {
     };
     set(match_small_kernel<2, false, false>, kMatchSmem);
     set(match_small_kernel<4, false, false>, kMatchSmem);
+    set(match_small_kernel<4, false, true>, kMatchSmem);
+    set(match_small_kernel<4, true, true>, kMatchSmem);
     set(match_small_kernel<2, false, true>, kMatchSmem);
     set(match_small_kernel<2, true, false>, kMatchSmem);
     set(match_small_kernel<4, true, false>, kMatchSmem);
