@@ -73,9 +73,9 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     }
     UnitCursor next;   // the unit whose loads are issued next
     next.init(first, stride, a.n_blocks);
-    auto issue = [&](int t, const int4& geom, int start, int h) {   // lane 0 only
+    auto issue = [&](int t, uint32_t st, const int4& geom, int start, int h) {   // lane 0 only
         const Geometry bg = unpack_geometry(geom);
-        const uint32_t st = STAGES == 2 ? t : 0, mb = bar0 + 8 * st;
+        const uint32_t mb = bar0 + 8 * st;
         const CUtensorMap* m = t == 0 ? &map_q : &map_k;
         if (DIRECT) {
             mbar_expect_tx(mb, (uint32_t)box.rows * kRowBytes);
@@ -98,7 +98,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     dependents_launch();
     clear_words(a.clear, blockIdx.x, gridDim.x);
     if (first < n_units && lane == 0)
-        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : STAGES - 1); ++t) issue(t, bg_next, bi_next.start, h_next);
+        for (int st = 0; st < (SPLIT ? 1 : STAGES); ++st) issue(t_first + st, st, bg_next, bi_next.start, h_next);
 
     // ldmatrix offsets of a 16-row tile: rows 0-7 / 8-15 (lane bit 3), k chunk 2 ks / 2 ks + 1 (lane bit 4); chunk c of row j sits at c ^ (j & 7)
     uint32_t a_off[4];
@@ -117,9 +117,9 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         is_src[i] = false;
     }
 
-    int it = 0;   // loads of a stage so far (TILES 4: tensors, else units)
-    bool failed = false;
-    for (int64_t unit = first; unit < n_units; unit += stride, it += STAGES == 2) {
+    uint32_t seq = 0;   // tensors so far: in stage seq % STAGES
+    bool failed = false, ahead = false;   // ahead: the next tensor's load is in flight too
+    for (int64_t unit = first; unit < n_units; unit += stride) {
         const BlockInfo bi = bi_next;
         const int4 geom = bg_next;
         const int h = h_next, n = bi.n;
@@ -129,18 +129,20 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             fetch();   // in flight while this unit is worked off
         }
 #pragma unroll 1
-        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t, it += STAGES == 1) {
+        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t, ++seq) {
+            const uint32_t st = seq % STAGES;
             // the next tensor of this stage: this one of the next unit or, with one stage, K behind Q
             auto refill = [&]() {   // lane 0 only
                 if (STAGES == 1 && !SPLIT && t == 0)
-                    issue(1, geom, bi.start, h);
+                    issue(1, st, geom, bi.start, h);
                 else if (more)
-                    issue(STAGES == 1 && !SPLIT ? 0 : t, bg_next, bi_next.start, h_next);
+                    issue(STAGES == 1 && !SPLIT ? 0 : t, st, bg_next, bi_next.start, h_next);
             };
             const int r = t == 0 ? bi.r_q : bi.r_k, nd = t == 0 ? bi.nd_q : bi.nd_k;
             int32_t* A = a.assign[t] + (int64_t)h * a.n_tokens + bi.start;
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + (STAGES == 2 ? 8 * t : 0), it & 1, a.status, kDevTimeoutMatchLoad))) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8 * st, seq / STAGES & 1u, a.status, kDevTimeoutMatchLoad))) {
                 failed = true;
+                ahead = STAGES == 2 && !SPLIT && (t < 1 || more);
                 break;
             }
             if (r == 0 || nd > 8 * ND) {   // nothing merges, or an anchored block with more dst tokens (match_anchor_kernel)
@@ -173,7 +175,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     }
                 }
             }
-            const uint32_t blk = stage0 + (STAGES == 2 ? t * STAGE : 0);
+            const uint32_t blk = stage0 + st * STAGE;
             // ---- dst fragments (k steps 2 kp, 2 kp + 1 per ldmatrix.x4) and their norms: lane 9 tq holds that of dst 2 tq, 9 tq + 4 of 2 tq + 1
             uint32_t bf[ND][4][2];
             float w0[ND], w1[ND];
@@ -332,9 +334,8 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         if (failed) break;
     }
-    if (failed) {   // give copies that may still be in flight a bounded chance to land before the shared memory is released
-        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : STAGES - 1); ++t) mbar_wait_bounded(bar0 + (STAGES == 2 ? 8 * t : 0), it & 1, a.status, kDevTimeoutMatchLoad);
-    }
+    if (failed)   // give copies that may still be in flight a bounded chance to land before the shared memory is released
+        for (uint32_t i = seq; i <= seq + (ahead ? 1 : 0); ++i) mbar_wait_bounded(bar0 + 8 * (i % STAGES), i / STAGES & 1u, a.status, kDevTimeoutMatchLoad);
 }
 
 // ------------------------------------------------------------------------------------ merge

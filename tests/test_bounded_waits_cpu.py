@@ -26,7 +26,7 @@ WARP_ROLES = [
     ("httm_big_blocks.cu", "arg-max over the chunk's dst tokens", "tmem_dealloc"),
     ("httm_linear.cu", "epilogue: lane = row", "tcgen05.dealloc"),
     ("httm_mem_kernels.cu", "int buf = 0;", "if (failed)"),
-    ("httm_small_blocks.cu", "int it = 0;", "if (failed) break;"),
+    ("httm_small_blocks.cu", "uint32_t seq = 0;", "if (failed) break;"),
 ]
 
 
@@ -42,3 +42,25 @@ def test_a_warp_gives_up_as_a_whole(name, start, end):
     for at in waits:
         statement = code[max(code.rfind(c, 0, at) for c in ";{}") + 1:at]
         assert "__all_sync(0xffffffffu," in statement, code[at - 60:at + 60]
+
+
+@pytest.mark.parametrize("kernel,tensors", [("match_small_kernel", 2), ("merge_small_kernel", 3)])
+def test_a_warp_that_gives_up_waits_for_every_load_in_flight(kernel, tensors):
+    """The loads of a warp are numbered in the order in which they are issued and awaited.  With two stages the first two are issued ahead and another behind
+    every one that has arrived, so all that is in flight when number `seq` does not arrive is that one and, unless it is the last, the next.  Checked
+    on the kernel's own expressions."""
+    code = open(os.path.join(CSRC, "httm_small_blocks.cu")).read()
+    begin = code.index(kernel + "(const __grid_constant__")
+    code = re.sub(r"//.*", "", code[begin:code.index("\n}\n", begin)])
+    ahead = re.search(r"failed = true;\s*ahead = ([^;]*);", code).group(1).replace("&&", " and ").replace("||", " or ").replace("!", " not ")
+    for units in (1, 2, 3):
+        for seq in range(tensors * units):
+            unit, t = divmod(seq, tensors)
+            issued = min(2 + seq, tensors * units)
+            assert eval(ahead, {"STAGES": 2, "SPLIT": False, "t": t, "more": unit + 1 < units}) == (issued > seq + 1), (unit, t)
+    assert not eval(ahead, {"STAGES": 2, "SPLIT": True, "t": 0, "more": False})   # (a warp with one tensor)
+    # and it waits for them where and in the phase in which the loop would
+    stage = re.search(r"uint32_t st = ([^;]*);", code).group(1)
+    waits = [re.sub(r"\bst\b", "(" + stage + ")", w) for w in re.findall(r"mbar_wait_bounded\((.*?), a\.status", code)]
+    assert len(waits) == 2 and "i <= seq + (ahead ? 1 : 0)" in code
+    assert re.sub(r"\bi\b", "seq", waits[1]) == waits[0], waits
