@@ -36,16 +36,17 @@ constexpr uint32_t kStage = 32 * kRowBytes;   // one block of one tensor, 128-by
 constexpr int kMatchSmem = kWarps * (2 * (int)kStage + 16) + 1024 /*alignment slack*/;   // two blocks of 32 rows or one of 64 per warp
 
 constexpr int match_ctas(int tiles) { return tiles == 2 ? 3 : 2; }   // per SM: 80 and 128 registers
-// TILES: blocks of up to 32 tokens, 8 dst tokens (2), a stage for either tensor; or up to 64 tokens, 16 dst tokens (4): one stage for Q and K in turn, so that 16 warps
-// fit on an SM.  A team of one warp that kept all its fragments and had two stages, of which 10 fitted, against this: 137 400 tokens in 64-token blocks 161.8 / 137.5 us, a
-// call 4098 / 4037; 7 898 tokens in 48-token blocks 93.5 / 92.6; 4 067 .. 5 229 tokens x 16 heads in 48-token blocks, two rounds against one, calls 8 - 9 % less; 1 743 tokens,
-// a tensor per warp here, 22.5 / 20.8.  (24 warps with 80 registers spill: 159 us.)
-// SPLIT: fewer units than warps: a warp has one tensor of one unit
-template <int TILES, bool DIRECT, bool SPLIT>
+// TILES: blocks of up to 32 tokens, 8 dst tokens (2); or up to 64 tokens, 16 dst tokens (4), where a warp has room for one tensor, so that 16 warps fit on an SM.
+// UNITS: a task is a unit, both its tensors in a stage each; else one tensor of it.
+// A team of one warp that kept all fragments of a 64-token block and had two stages, of which 10 fitted on an SM, both tensors of a unit in turn through one stage, and a
+// tensor at a time: 137 400 tokens x 16 heads in 64-token blocks, ratio 0.8, match 166.2 / 137.5 / 131.5 us; calls on 16 488 tokens 113.7 / 115.7 / 111.4 (4800 units on 2368
+// warps: three rounds of units, five of tensors), on 10 992 tokens 67.1 / 68.2 / 64.6; 7 898 tokens in 48-token blocks 93.1 / 92.7 / 90.7.  (24 warps with 80 registers spill.)
+template <int TILES, bool DIRECT, bool UNITS>
 __global__ void __launch_bounds__(kWarps * 32, match_ctas(TILES))
 match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ MatchArgs a) {
     constexpr int ND = TILES / 2, SLOTS = TILES / 2;   // groups of eight dst tokens; tokens per lane
-    constexpr int STAGES = TILES == 2 ? 2 : 1;
+    constexpr int STAGES = UNITS ? 2 : 1;
+    static_assert(TILES == 2 || !UNITS, "a warp has room for two tensors of 32 tokens");
     constexpr uint32_t STAGE = TILES * 16 * kRowBytes;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + align_pad(smem_raw);
@@ -64,14 +65,9 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 
     Box box{};
     if (DIRECT) box.set(a.layout);
-    const int64_t n_units = (int64_t)a.heads * a.n_blocks;
-    int stride = gridDim.x * kWarps, first = blockIdx.x * kWarps + warp, t_first = 0, t_last = 1;
-    if (SPLIT) {
-        t_first = t_last = first >= n_units ? 1 : 0;
-        first = (int)min(n_units, first - t_first * n_units);
-        stride = (int)n_units;
-    }
-    UnitCursor next;   // the unit whose loads are issued next
+    const int64_t n_tasks = (UNITS ? 1ll : 2ll) * a.heads * a.n_blocks;
+    const int stride = gridDim.x * kWarps, first = blockIdx.x * kWarps + warp;
+    UnitCursor next;   // the task whose loads are issued next; a tensor at a time: K's heads follow Q's
     next.init(first, stride, a.n_blocks);
     auto issue = [&](int t, uint32_t st, const int4& geom, int start, int h) {   // lane 0 only
         const Geometry bg = unpack_geometry(geom);
@@ -87,18 +83,19 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     };
     BlockInfo bi_next{};
     int4 bg_next{};
-    int h_next = 0;
+    int h_next = 0, t_next = 0;   // (t_next: first tensor of the task)
     auto fetch = [&]() {
         bi_next = a.blocks[next.u];
         if (DIRECT) bg_next = load_geometry(a.geom, next.u);
-        h_next = next.h;
+        t_next = !UNITS && next.h >= a.heads ? 1 : 0;
+        h_next = next.h - t_next * a.heads;
     };
-    if (first < n_units) fetch();
+    if (first < n_tasks) fetch();
     depend_wait();
     dependents_launch();
     clear_words(a.clear, blockIdx.x, gridDim.x);
-    if (first < n_units && lane == 0)
-        for (int st = 0; st < (SPLIT ? 1 : STAGES); ++st) issue(t_first + st, st, bg_next, bi_next.start, h_next);
+    if (first < n_tasks && lane == 0)
+        for (int st = 0; st < STAGES; ++st) issue(t_next + st, st, bg_next, bi_next.start, h_next);
 
     // ldmatrix offsets of a 16-row tile: rows 0-7 / 8-15 (lane bit 3), k chunk 2 ks / 2 ks + 1 (lane bit 4); chunk c of row j sits at c ^ (j & 7)
     uint32_t a_off[4];
@@ -119,30 +116,26 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 
     uint32_t seq = 0;   // tensors so far: in stage seq % STAGES
     bool failed = false, ahead = false;   // ahead: the next tensor's load is in flight too
-    for (int64_t unit = first; unit < n_units; unit += stride) {
+    for (int64_t task = first; task < n_tasks; task += stride) {
         const BlockInfo bi = bi_next;
         const int4 geom = bg_next;
-        const int h = h_next, n = bi.n;
-        const bool more = unit + stride < n_units;
+        const int h = h_next, t0 = t_next, n = bi.n;
+        const bool more = task + stride < n_tasks;
         if (more) {
             next.advance();
-            fetch();   // in flight while this unit is worked off
+            fetch();   // in flight while this task is worked off
         }
 #pragma unroll 1
-        for (int t = SPLIT ? t_first : 0; t <= (SPLIT ? t_last : 1); ++t, ++seq) {
+        for (int t = t0; t < t0 + STAGES; ++t, ++seq) {
             const uint32_t st = seq % STAGES;
-            // the next tensor of this stage: this one of the next unit or, with one stage, K behind Q
-            auto refill = [&]() {   // lane 0 only
-                if (STAGES == 1 && !SPLIT && t == 0)
-                    issue(1, st, geom, bi.start, h);
-                else if (more)
-                    issue(STAGES == 1 && !SPLIT ? 0 : t, st, bg_next, bi_next.start, h_next);
+            auto refill = [&]() {   // the tensor that takes this stage next (lane 0 only)
+                if (more) issue(UNITS ? t : t_next, st, bg_next, bi_next.start, h_next);
             };
             const int r = t == 0 ? bi.r_q : bi.r_k, nd = t == 0 ? bi.nd_q : bi.nd_k;
             int32_t* A = a.assign[t] + (int64_t)h * a.n_tokens + bi.start;
             if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8 * st, seq / STAGES & 1u, a.status, kDevTimeoutMatchLoad))) {
                 failed = true;
-                ahead = STAGES == 2 && !SPLIT && (t < 1 || more);
+                ahead = UNITS && (t < 1 || more);
                 break;
             }
             if (r == 0 || nd > 8 * ND) {   // nothing merges, or an anchored block with more dst tokens (match_anchor_kernel)
@@ -648,13 +641,19 @@ cudaError_t launch_match_tiles(const MatchArgs& a, int sm_count, cudaStream_t st
     }
     const int64_t units = (int64_t)a.heads * a.n_blocks;
     auto launch = [&](auto kernel, int parts) {
-        return launch_kernel(kernel, small_grid(units * parts, sm_count, match_ctas(TILES)), kWarps * 32, kMatchSmem, stream, mq, mk, a);
+        // Tasks of one tensor are dealt out evenly where there are few rounds of them, so that the last is no nearly empty one and the merge kernel's CTAs find room
+        // earlier.  64-token blocks, ratio 0.8, calls with all warps / evenly dealt: 1.4 rounds 39.2 / 38.1 us, 2.7 65.1 / 64.6, 4.1 112.7 / 111.4, 5.4 166.2 / 166.6, 8.1
+        // 172.1 / 173.0.
+        const int64_t tasks = units * parts, warps = (int64_t)match_ctas(TILES) * kWarps * sm_count, rounds = (tasks + warps - 1) / warps;
+        const int64_t dealt = parts == 2 && rounds > 1 && rounds <= 5 ? (tasks + rounds - 1) / rounds : tasks;
+        return launch_kernel(kernel, small_grid(dealt, sm_count, match_ctas(TILES)), kWarps * 32, kMatchSmem, stream, mq, mk, a);
     };
     // With no more than one tensor per warp the tensors of a unit go to different warps: the call then waits for one, not two
     // (512 units: 11.3 -> 9.4 us, in the merge kernel below 13.1 -> 9.0).
-    if (2 * units <= (int64_t)match_ctas(TILES) * kWarps * sm_count)
-        return launch(direct ? match_small_kernel<TILES, true, true> : match_small_kernel<TILES, false, true>, 2);
-    return launch(direct ? match_small_kernel<TILES, true, false> : match_small_kernel<TILES, false, false>, 1);
+    if constexpr (TILES == 2)
+        if (2 * units > (int64_t)match_ctas(TILES) * kWarps * sm_count)
+            return launch(direct ? match_small_kernel<TILES, true, true> : match_small_kernel<TILES, false, true>, 1);
+    return launch(direct ? match_small_kernel<TILES, true, false> : match_small_kernel<TILES, false, false>, 2);
 }
 }  // namespace
 cudaError_t launch_match_small(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
@@ -679,13 +678,11 @@ cudaError_t configure_small_blocks() {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
     set(match_small_kernel<2, false, false>, kMatchSmem);
-    set(match_small_kernel<4, false, false>, kMatchSmem);
-    set(match_small_kernel<4, false, true>, kMatchSmem);
-    set(match_small_kernel<4, true, true>, kMatchSmem);
     set(match_small_kernel<2, false, true>, kMatchSmem);
     set(match_small_kernel<2, true, false>, kMatchSmem);
-    set(match_small_kernel<4, true, false>, kMatchSmem);
     set(match_small_kernel<2, true, true>, kMatchSmem);
+    set(match_small_kernel<4, false, false>, kMatchSmem);
+    set(match_small_kernel<4, true, false>, kMatchSmem);
     set(merge_small_kernel<2, false, false>, kMergeSmem);
     set(merge_small_kernel<2, false, true>, kMergeSmem);
     set(merge_small_kernel<2, true, false>, kMergeSmem);

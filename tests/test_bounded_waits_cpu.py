@@ -57,8 +57,8 @@ def test_a_warp_that_gives_up_waits_for_every_load_in_flight(kernel, tensors):
         for seq in range(tensors * units):
             unit, t = divmod(seq, tensors)
             issued = min(2 + seq, tensors * units)
-            assert eval(ahead, {"STAGES": 2, "SPLIT": False, "t": t, "more": unit + 1 < units}) == (issued > seq + 1), (unit, t)
-    assert not eval(ahead, {"STAGES": 2, "SPLIT": True, "t": 0, "more": False})   # (a warp with one tensor)
+            assert eval(ahead, {"UNITS": True, "SPLIT": False, "t": t, "more": unit + 1 < units}) == (issued > seq + 1), (unit, t)
+    assert not eval(ahead, {"UNITS": False, "SPLIT": True, "t": 0, "more": True})   # (a tensor at a time, through one stage)
     # and it waits for them where and in the phase in which the loop would
     stage = re.search(r"uint32_t st = ([^;]*);", code).group(1)
     waits = [re.sub(r"\bst\b", "(" + stage + ")", w) for w in re.findall(r"mbar_wait_bounded\((.*?), a\.status", code)]
