@@ -50,8 +50,8 @@ __device__ __forceinline__ bool is_dst_position(int j, int n_rule, int nd) {
 // where the compiler has made one).
 // Measured at 16 heads x 22 blocks of up to 3840 tokens, 384 dst tokens of the queries and 960 of the keys: 611 us with the dst tokens split into three
 // scaled planes, 256 at a time, and one group of warps; 467 us with all tokens as rows; 426 us with a function for scores that had been spoilt; 407 us now.
-// It spills all the same: ptxas gives the kernel the 96 registers of its launch, and the scores of two tiles with two Best do not fit (254 bytes stored, 368
-// loaded per thread).  The dst tokens chosen are closer to the best in 64 bits
+// It spills all the same: ptxas gives the kernel the 96 registers of its launch, and the scores of two tiles with two Best do not fit (234 bytes stored, 360
+// loaded per thread; 278 and 404 with PARTS).  The dst tokens chosen are closer to the best in 64 bits
 // (1.6 million tokens of three scenes: 26 off the best by up to 4.6e-7 before, 6 by up to 1.2e-7).  Tried and dropped: 64 and 104 registers (456 us),
 // no carrying along where no row of the warp improves (491 us at 467).
 constexpr int TILE = 128;                        // rows of an operand tile, dst tokens of a chunk
@@ -86,18 +86,19 @@ constexpr int SC_OFF_ITEMS = SC_OFF_BARS + 384;                  // ScoreItem [2
 constexpr int SC_SMEM = SC_OFF_ITEMS + 2 * 64 + 1024 /*alignment slack*/;
 static_assert(sizeof(ScoreBars) <= 384 && sizeof(ScoreItem) <= 64 && kMaxBigDst % TILE == 0 && SC_AREA % 1024 == 0 && SC_SMEM <= 232448, "");
 
+template <bool PARTS>
 __device__ __forceinline__ void write_item(ScoreItem* to, const BigMatchArgs& a, int t_first, int item) {
-    const int per_tensor = a.heads * a.n_blocks * a.parts;
+    const int parts = PARTS ? a.parts : 1, per_tensor = a.heads * a.n_blocks * parts;
     if (item >= 2 * per_tensor) {
         to->t = -1;
         return;
     }
     const int t = item < per_tensor ? t_first : 1 - t_first, at = item < per_tensor ? item : item - per_tensor;
-    const int rem = at / a.parts, part = at - rem * a.parts;
+    const int rem = at / parts, part = at - rem * parts;
     const BlockInfo bi = a.blocks[a.order[rem / a.heads]];
     const int nd = t == 0 ? bi.nd_q : bi.nd_k, n_src = bi.n - nd;
     const bool merges = (t == 0 ? bi.r_q : bi.r_k) > 0;
-    const int tiles = merges ? (n_src + TILE - 1) / TILE : 0, st0 = tiles * part / a.parts, n_st = tiles * (part + 1) / a.parts - st0;
+    const int tiles = merges ? (n_src + TILE - 1) / TILE : 0, st0 = tiles * part / parts, n_st = tiles * (part + 1) / parts - st0;
     const int ring = (nd + 7) / 8 * 8 * kRowBytes;   // (the last chunk's MMAs read into the ring: masked columns)
     to->t = t;
     to->n_rule = bi.n_rule;
@@ -194,6 +195,9 @@ __device__ __forceinline__ void take_best(Best& best, float (&s)[32], int first_
         best.v[c] = v;
     }
 }
+// PARTS: blocks shared out to several items (launch_big_scores).  Items that begin at a tile of their own cost more spills: in a call with many blocks, 32 976 tokens x 16 heads in
+// blocks of up to 1152 tokens, the kernel took 147.5 us, without 145.4.
+template <bool PARTS>
 __global__ void __launch_bounds__(SC_THREADS, 1)
 big_scores_kernel(const BigMatchArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -224,7 +228,7 @@ big_scores_kernel(const BigMatchArgs a) {
     const int t_first = a.blocks[a.order[0]].nd_k >= a.blocks[a.order[0]].nd_q ? 1 : 0;
     ScoreItem* items = reinterpret_cast<ScoreItem*>(smem + SC_OFF_ITEMS);
     if (warp == 1) tc::tmem_alloc(tc::smem_addr(&bars->tmem_base), SC_TMEM_COLS);
-    if (tid == 64) write_item(items, a, t_first, blockIdx.x);
+    if (tid == 64) write_item<PARTS>(items, a, t_first, blockIdx.x);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -247,8 +251,9 @@ big_scores_kernel(const BigMatchArgs a) {
                 const __nv_bfloat16* x = a.xr[it.t] + it.row0 * kHeadDim;
                 const int at = tid - 64, c16 = at & 7;
                 // src token s is token s + (dst tokens before it): s + floor(s nd / (n - nd)), or s + nd where the first nd tokens are the dst tokens
-                Ramp before((it.st0 * TILE + (at >> 3)) * it.nd, SC_LOADERS / 8 * it.nd, max(it.n_src, 1));
-                int s = it.st0 * TILE + (at >> 3), handed = 0, hand_st = 0;   // next src token of this thread; tiles handed over, stage of the next
+                const int s0 = PARTS ? it.st0 * TILE : 0;
+                Ramp before((s0 + (at >> 3)) * it.nd, SC_LOADERS / 8 * it.nd, max(it.n_src, 1));
+                int s = s0 + (at >> 3), handed = 0, hand_st = 0;   // next src token of this thread; tiles handed over, stage of the next
                 uint32_t par = fills;
                 auto hand_over = [&]() __attribute__((always_inline)) {
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tensor cores read the rows through the async proxy
@@ -273,7 +278,7 @@ big_scores_kernel(const BigMatchArgs a) {
                 if (__syncthreads_or(0)) __syncthreads();
                 asm volatile("cp.async.wait_all;" ::: "memory");
                 while (ok && handed < first) hand_over();
-                if (tid == 64) write_item(items + ((n_items + 1) & 1), a, t_first, (int)gridDim.x + atomicAdd(a.counter, 1));
+                if (tid == 64) write_item<PARTS>(items + ((n_items + 1) & 1), a, t_first, (int)gridDim.x + atomicAdd(a.counter, 1));
                 __syncwarp();
                 for (int i = first, st = first; ok && i < it.n_st; ++i, st = st + 1 < it.stages ? st + 1 : 0) {
                     if (handed < i && !__all_sync(0xffffffffu, tc::mbar_test(tc::smem_addr(&bars->a_empty[st]), (par >> st & 1u) ^ 1u))) {
@@ -451,8 +456,8 @@ big_scores_kernel(const BigMatchArgs a) {
                 int arg[2], own[2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const int s = (it.st0 + 2 * p + e) * TILE + row;   // src token
-                    own[e] = 2 * p + e < it.n_st && s < n_src ? src_position(s) : -1;   // token number inside the block (behind an odd last tile: another item's)
+                    const int s = ((PARTS ? it.st0 : 0) + 2 * p + e) * TILE + row;   // src token
+                    own[e] = (!PARTS || 2 * p + e < it.n_st) && s < n_src ? src_position(s) : -1;   // token number inside the block (behind an odd last tile: another item's)
                     int in_group = 0;
 #pragma unroll
                     for (int c = kGroup - 1; c >= 0; --c)
@@ -1102,10 +1107,13 @@ cudaError_t configure_sorted_group_kernels() {
 
 cudaError_t configure_big_blocks() {
     // setmaxnreg.inc takes registers from those the CTA was launched with, and waits without limit for more than there are
-    cudaFuncAttributes launched;
-    cudaError_t e = cudaFuncGetAttributes(&launched, big_scores_kernel);
-    if (e == cudaSuccess && launched.numRegs * SC_THREADS < 128 * kScoreRoleRegs + (SC_THREADS - 128) * kScoreMaxRegs) e = cudaErrorInvalidConfiguration;
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(big_scores_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM);
+    cudaError_t e = cudaSuccess;
+    for (auto scores : {big_scores_kernel<false>, big_scores_kernel<true>}) {
+        cudaFuncAttributes launched;
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&launched, scores);
+        if (e == cudaSuccess && launched.numRegs * SC_THREADS < 128 * kScoreRoleRegs + (SC_THREADS - 128) * kScoreMaxRegs) e = cudaErrorInvalidConfiguration;
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(scores, cudaFuncAttributeMaxDynamicSharedMemorySize, SC_SMEM);
+    }
     if (e == cudaSuccess) e = configure_sorted_group_kernels<64, 4>();
     if (e == cudaSuccess) e = configure_sorted_group_kernels<128, 4>();
     if (e == cudaSuccess) e = configure_sorted_group_kernels<256, 4>();
@@ -1123,7 +1131,7 @@ cudaError_t launch_big_scores(const BigMatchArgs& args, int sm_count, cudaStream
     a.parts = (int)(blocks < 1 || blocks > sms ? 1 : sms / blocks > 4 ? 4 : sms / blocks);
     const int64_t total = blocks * a.parts;
     const int ctas = (int)(total > sms ? sms : total < 1 ? 1 : total);
-    return launch_kernel(big_scores_kernel, ctas, SC_THREADS, SC_SMEM, stream, a);
+    return launch_kernel(a.parts > 1 ? big_scores_kernel<true> : big_scores_kernel<false>, ctas, SC_THREADS, SC_SMEM, stream, a);
 }
 
 cudaError_t launch_big_select(const BigMatchArgs& a, cudaStream_t stream) {

@@ -41,6 +41,11 @@ def test_nothing_is_called_and_the_registers_were_there(tmp_path, src):
     code = open(os.path.join(CSRC, src)).read()
     role, most = map(int, re.search(r"kScoreRoleRegs = (\d+), kScoreMaxRegs = (\d+)", code).groups())
     groups = int(re.search(r"SC_GROUPS = (\d+)", code).group(1))
-    at = log.index("big_scores_kernel")
-    used = int(re.search(r"Used (\d+) registers", log[at:]).group(1))
-    assert used * (128 + groups * 256) >= 128 * role + groups * 256 * most
+    kernels = [m.end() for m in re.finditer(r"Compiling entry function '[^']*big_scores_kernel", log)]
+    spills = []
+    for at in kernels:
+        used = int(re.search(r"Used (\d+) registers", log[at:]).group(1))
+        assert used * (128 + groups * 256) >= 128 * role + groups * 256 * most
+        spills.append(int(re.search(r"(\d+) bytes spill loads", log[at:]).group(1)))
+    # what blocks shared out to several items need is not paid for by calls with many blocks
+    assert len(spills) == 2 and min(spills) <= 368
