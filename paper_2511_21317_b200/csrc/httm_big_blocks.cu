@@ -847,8 +847,11 @@ __device__ __forceinline__ void sum_members(const __nv_bfloat16* x, const uint32
     for (int e = 0; e < 4; ++e) sum[e] = tc::fadd2(sum[e], other[e]);
 }
 
-template <int T, int E>
-__global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const MergeArgs a, int sp_chunks, int shares) {
+// SHARED: several CTAs for a block (row_shares).  With the distance between a warp's rows known only at run time a call with many blocks, 32 976 tokens x 16 heads in blocks of
+// up to 1152 tokens, took 512.2 us, without 510.8.
+template <int T, int E, bool SHARED>
+__global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const MergeArgs a, int sp_chunks, int n_shares) {
+    const int shares = SHARED ? n_shares : 1;
     extern __shared__ __align__(16) unsigned char mg_smem[];
     uint32_t* keys = reinterpret_cast<uint32_t*>(mg_smem);                                     // [P] (merged row << 12) | position
     int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (E * T) * 4);            // [n] merged row of a kept token, -1
@@ -917,8 +920,9 @@ __global__ void __launch_bounds__(T, kMergeThreads / T) big_merge_kernel(const M
 // with 8 tokens per thread): two channels per instruction, one exchange for the sums of four
 // members and one square root for them took the filter kernels together, at 82 440 tokens x 16 heads in 3840-token blocks, from 221 to 178 us
 // (32 976 tokens in 128-token blocks: 104.7 -> 92.2; 137 400 in 64-token blocks: 363 -> 302).
-template <int T, int E>
-__global__ void __launch_bounds__(T, kSortedThreads / T) big_deviation_kernel(const OutlierArgs a, int shares) {
+template <int T, int E, bool SHARED>
+__global__ void __launch_bounds__(T, kSortedThreads / T) big_deviation_kernel(const OutlierArgs a, int n_shares) {
+    const int shares = SHARED ? n_shares : 1;
     extern __shared__ __align__(16) unsigned char mg_smem[];
     uint32_t* keys = reinterpret_cast<uint32_t*>(mg_smem);
     int16_t* row_of = reinterpret_cast<int16_t*>(mg_smem + (E * T) * 4);
@@ -1085,7 +1089,7 @@ cudaError_t launch_big_deviation(const OutlierArgs& a, int max_block, int sm_cou
     return with_cta_size(max_block, [&](auto t, auto e) {
         constexpr int T = decltype(t)::value, E = decltype(e)::value;
         const int shares = row_shares((int64_t)a.heads * a.n_blocks, (int64_t)(kSortedThreads / T) * sm_count);
-        return launch_kernel(big_deviation_kernel<T, E>, a.heads * a.n_blocks * shares, T, mg_smem_bytes(E * T), stream, a, shares);
+        return launch_kernel(shares > 1 ? big_deviation_kernel<T, E, true> : big_deviation_kernel<T, E, false>, a.heads * a.n_blocks * shares, T, mg_smem_bytes(E * T), stream, a, shares);
     });
 }
 
@@ -1098,11 +1102,16 @@ cudaError_t launch_big_filter(const OutlierArgs& a, int max_block, cudaStream_t 
 
 template <int T, int E>
 cudaError_t configure_sorted_group_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(big_merge_kernel<T, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, mg_smem_bytes(E * T));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(big_deviation_kernel<T, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, mg_smem_bytes(E * T));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(big_filter_kernel<T, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, of_smem_bytes(E * T));
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto kernel, int bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    set(big_merge_kernel<T, E, false>, mg_smem_bytes(E * T));
+    set(big_merge_kernel<T, E, true>, mg_smem_bytes(E * T));
+    set(big_deviation_kernel<T, E, false>, mg_smem_bytes(E * T));
+    set(big_deviation_kernel<T, E, true>, mg_smem_bytes(E * T));
+    set(big_filter_kernel<T, E>, of_smem_bytes(E * T));
+    return e;
 }
 
 cudaError_t configure_big_blocks() {
@@ -1143,7 +1152,7 @@ cudaError_t launch_big_merge(const MergeArgs& a, int max_block, int sm_count, cu
         constexpr int T = decltype(t)::value, E = decltype(e)::value;
         const int sp_chunks = (a.n_special_total + T / 8 - 1) / (T / 8);
         const int shares = row_shares(2ll * a.heads * a.n_blocks, (int64_t)(kMergeThreads / T) * sm_count);
-        return launch_kernel(big_merge_kernel<T, E>, 2 * a.heads * a.n_blocks * shares + a.heads * sp_chunks, T, mg_smem_bytes(E * T), stream, a, sp_chunks, shares);
+        return launch_kernel(shares > 1 ? big_merge_kernel<T, E, true> : big_merge_kernel<T, E, false>, 2 * a.heads * a.n_blocks * shares + a.heads * sp_chunks, T, mg_smem_bytes(E * T), stream, a, sp_chunks, shares);
     });
 }
 
