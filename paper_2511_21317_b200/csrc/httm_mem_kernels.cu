@@ -179,7 +179,7 @@ __device__ void finish_level(const OutlierArgs& a, int level, int* hist);   // (
 // stages and two CTAs, before: the five kernels of the filter 59.4 us at 32 976 tokens, now 55.3; the call 697.9 -> 693.8.
 constexpr int kDevWarps = 8;     // 8 x 8.5 KB of shared memory: three CTAs per SM
 constexpr int kCentStride = 68;  // floats per mean: 16-byte reads of eight different means fall on distinct banks
-constexpr int kDevAux = 16 * kCentStride * 4 + 16 * 4 + 32 + 64;   // means of the groups of two or more (at most 16 in 32 tokens), reciprocal sizes, mbarriers, rows
+constexpr int kDevAux = 16 * kCentStride * 4 + 16 * 4 + 32 + 64;   // means of the groups of two or more (at most 16 in 32 tokens), reciprocal sizes, an mbarrier, rows
 constexpr int kDevBins = 1024;   // of level 0: the sign bit of a deviation is 0
 constexpr int kDevSmem = kDevWarps * (32 * kRowBytes + kDevAux) + kDevBins * 4 /*histogram*/ + 1024 /*alignment slack*/;
 
@@ -232,9 +232,9 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
     if (a.early) depend_wait();
     dependents_launch();
 
-    int buf = 0;   // phase of the stage's barrier
+    uint32_t phase = 0;   // of the stage's barrier
     bool failed = false;
-    for (int64_t task = first; task < n_tasks; task += stride, cur.advance(), nxt.advance(), buf ^= 1) {
+    for (int64_t task = first; task < n_tasks; task += stride, cur.advance(), nxt.advance(), phase ^= 1u) {
         const bool more = task + stride < n_tasks;
         const int h = cur.h;
         const BlockInfo bi = a.blocks[cur.u];
@@ -252,7 +252,7 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
             }
             rep = bm.row_of_token(rep);
         }
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(mbar, buf, a.status, kDevTimeoutMatchLoad))) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(mbar, phase, a.status, kDevTimeoutMatchLoad))) {
             failed = true;
             break;
         }
@@ -326,7 +326,7 @@ deviation_kernel(const __grid_constant__ CUtensorMap map_q, const OutlierArgs a)
         }
         __syncwarp();   // every lane is done with the tables
     }
-    if (failed) mbar_wait_bounded(mbar, buf, a.status, kDevTimeoutMatchLoad);   // give the copy in flight a bounded chance to land before the shared memory is released
+    if (failed) mbar_wait_bounded(mbar, phase, a.status, kDevTimeoutMatchLoad);   // give the copy in flight a bounded chance to land before the shared memory is released
     __syncthreads();
     for (int i = threadIdx.x; i < kDevBins; i += kDevWarps * 32) {
         const int c = hist[i];

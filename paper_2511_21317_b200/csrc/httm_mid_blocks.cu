@@ -121,11 +121,11 @@ __device__ __forceinline__ bool choose(const uint32_t* keys, int n_rows, int r, 
     return mine > hi || (mine == hi && before < r - above);
 }
 
-template <int W, int P, bool DIRECT>
-__global__ void __launch_bounds__(32 * W, team_ctas(W, P))
+template <int W, bool DIRECT>
+__global__ void __launch_bounds__(32 * W, team_ctas(W, 1))
 match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ MatchArgs a) {
-    static_assert(W > 1 && P == 1, "a thread has one token, a team several warps");
-    constexpr int NMAX = team_tokens(W, P), MT = 2 * P, MAX_DST = NMAX / 4;   // MT: 16-row tiles per warp
+    static_assert(W > 1, "a team has several warps, a thread one token");
+    constexpr int NMAX = team_tokens(W, 1), MT = 2, MAX_DST = NMAX / 4;   // MT: 16-row tiles per warp
     constexpr uint32_t STAGE = NMAX * kRowBytes;
     constexpr MatchAux X = match_aux(NMAX);
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -184,12 +184,10 @@ match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     // ldmatrix offsets of a 16-row tile: rows 0-7 / 8-15 (lane bit 3), k chunk 2 ks / 2 ks + 1 (lane bit 4); chunk c of row j sits at c ^ (j & 7)
     uint32_t a_off[4];
 #pragma unroll
-    for (int ks = 0; ks < 4; ++ks) a_off[ks] = (warp * 32 * P + (lane & 15)) * kRowBytes + (((2 * ks + (lane >> 4)) ^ (lane & 7)) << 4);
+    for (int ks = 0; ks < 4; ++ks) a_off[ks] = (warp * 32 + (lane & 15)) * kRowBytes + (((2 * ks + (lane >> 4)) ^ (lane & 7)) << 4);
     int shape_a = -1, shape_b = -1;   // shape of the blocks at hand: the tables and tok are made for it
-    int tok[P];                       // tokens in this thread's stage rows own + 32 p
-    const int row0 = warp * 32 * P, own = row0 + lane;
-#pragma unroll
-    for (int p = 0; p < P; ++p) tok[p] = -1;
+    int tok = -1;                     // token in this thread's stage row
+    const int row0 = warp * 32, own = row0 + lane;
     int it = 0;
     int failed = -1;   // tensor whose load did not arrive
     for (int64_t unit = blockIdx.x; unit < n_units; unit += gridDim.x, ++it) {
@@ -230,12 +228,8 @@ match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                         dst_pos[tid] = pos;
                         dst_row[tid] = DIRECT ? row_of_token(box, bg, pos) : pos;
                     }
-#pragma unroll
-                    for (int p = 0; p < P; ++p) {
-                        const int rho = own + 32 * p, j = DIRECT ? token_of_row(box, bg, rho) : (rho < n ? rho : -1);
-                        tok[p] = j;
-                        src[rho] = j >= 0 && !(j < n_rule && small_div((j + 1) * nd, n_rule) > small_div(j * nd, n_rule)) ? 1 : 0;
-                    }
+                    tok = DIRECT ? token_of_row(box, bg, own) : (own < n ? own : -1);
+                    src[own] = tok >= 0 && !(tok < n_rule && small_div((tok + 1) * nd, n_rule) > small_div(tok * nd, n_rule)) ? 1 : 0;
                 }
             }
             const uint32_t blk = stage0 + t * STAGE;
@@ -340,10 +334,10 @@ match_team_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (more && tid == 0) issue(t, geom_next, bi_next.start, h_next);
             // ---- the r src with the best scores merge (ties: lowest position first; rows are in token order)
             const int n_out = n - nd - r;
-            const uint32_t key = tok[0] >= 0 ? keys[own] : 0u;   // (0: not a src token)
+            const uint32_t key = tok >= 0 ? keys[own] : 0u;   // (0: not a src token)
             bool merged = key != 0;
             if (n_out > 0) merged = choose<NMAX / 32>(keys, (n_rows + 15) & ~15, r, key, warp, lane);
-            if (tok[0] >= 0) A[tok[0]] = bi.start + (merged ? dst_pos[best[own]] : tok[0]);
+            if (tok >= 0) A[tok] = bi.start + (merged ? dst_pos[best[own]] : tok);
         }
         if (failed >= 0) break;
     }
@@ -638,19 +632,19 @@ int team_grid(int64_t units, int sm_count, int ctas) {
     return (int)(units > cap ? cap : (units < 1 ? 1 : units));
 }
 
-template <int W, int P>
+template <int W>
 cudaError_t launch_match_t(const MatchArgs& a, int sm_count, cudaStream_t stream) {
     CUtensorMap mq, mk;
     const int64_t N = a.n_tokens;
     const bool direct = a.geom != nullptr;
     if (direct) {
         if (!encode_block_map(&mq, a.src[0], a.layout, a.heads) || !encode_block_map(&mk, a.src[1], a.layout, a.heads)) return cudaErrorInvalidValue;
-    } else if (!encode_rows_tensor_map(&mq, a.xr[0], N, a.heads, kHeadDim, N * kHeadDim, team_tokens(W, P)) ||
-               !encode_rows_tensor_map(&mk, a.xr[1], N, a.heads, kHeadDim, N * kHeadDim, team_tokens(W, P))) {
+    } else if (!encode_rows_tensor_map(&mq, a.xr[0], N, a.heads, kHeadDim, N * kHeadDim, team_tokens(W, 1)) ||
+               !encode_rows_tensor_map(&mk, a.xr[1], N, a.heads, kHeadDim, N * kHeadDim, team_tokens(W, 1))) {
         return cudaErrorInvalidValue;
     }
-    auto kernel = direct ? match_team_kernel<W, P, true> : match_team_kernel<W, P, false>;
-    return launch_kernel(kernel, team_grid((int64_t)a.heads * a.n_blocks, sm_count, team_ctas(W, P)), 32 * W, team_smem(W, P), stream, mq, mk, a);
+    auto kernel = direct ? match_team_kernel<W, true> : match_team_kernel<W, false>;
+    return launch_kernel(kernel, team_grid((int64_t)a.heads * a.n_blocks, sm_count, team_ctas(W, 1)), 32 * W, team_smem(W, 1), stream, mq, mk, a);
 }
 template <int W, int P>
 cudaError_t launch_merge_t(const MergeArgs& a, int sm_count, cudaStream_t stream) {
@@ -669,8 +663,8 @@ cudaError_t configure_t() {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
     if constexpr (W > 1) {
-        set(match_team_kernel<W, P, false>, team_smem(W, P));
-        set(match_team_kernel<W, P, true>, team_smem(W, P));
+        set(match_team_kernel<W, false>, team_smem(W, 1));
+        set(match_team_kernel<W, true>, team_smem(W, 1));
     }
     set(merge_team_kernel<W, P, false>, team_smem(W, P));
     set(merge_team_kernel<W, P, true>, team_smem(W, P));
@@ -680,8 +674,8 @@ cudaError_t configure_t() {
 }  // namespace
 
 cudaError_t launch_match_mid(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
-    if (max_block_tokens <= 128) return launch_match_t<4, 1>(a, sm_count, stream);
-    return launch_match_t<8, 1>(a, sm_count, stream);
+    if (max_block_tokens <= 128) return launch_match_t<4>(a, sm_count, stream);
+    return launch_match_t<8>(a, sm_count, stream);
 }
 cudaError_t launch_merge_mid(const MergeArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
     if (max_block_tokens <= 64) return launch_merge_t<1, 2>(a, sm_count, stream);

@@ -338,7 +338,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 // from, 16 channels at a time (whose fragments are in registers by then), and leave 16 bytes per lane, whole rows; then the stage is refilled.
 // Tensor i of the warp's sequence Q K V Q K V .. lies in stage i & 1.  With a stage for each tensor and all 64 channels in registers at a time (128 of them) 16 warps
 // were all that fits on an SM: 61.4 -> 57.3 us at 32 976 tokens, 132 -> 115 at 65 952, 19.5 -> 17.5 at 5 516 (unit_ctas).
-constexpr int kMergeAux = 32 * 4 + 32 * 4 + 32 + 64;   // reciprocal group sizes, group sizes, 3 mbarriers, merged rows of the tokens
+constexpr int kMergeAux = 32 * 4 + 32 * 4 + 16 + 64;   // reciprocal group sizes, group sizes, 2 mbarriers, merged rows of the tokens
 constexpr int kMergeStages = 2;
 constexpr int kMergeSmem = kWarps * (kMergeStages * (int)kStage + kMergeAux) + 1024 /*alignment slack*/;
 
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kWarps * 32, CTAS) merge_small_kernel(const __
     float* rcnt = reinterpret_cast<float*>(aux);             // [32] 1 / group size of kept row
     int* gsz = reinterpret_cast<int*>(aux + 32 * 4);         // [32] size of kept row
     const uint32_t stage0 = smem_u32(stage), bar0 = smem_u32(aux + 2 * 32 * 4);
-    __nv_bfloat16* rows_of = reinterpret_cast<__nv_bfloat16*>(aux + 2 * 32 * 4 + 32);   // [32] merged rows of the tokens, in fragment order
+    __nv_bfloat16* rows_of = reinterpret_cast<__nv_bfloat16*>(aux + 2 * 32 * 4 + 16);   // [32] merged rows of the tokens, in fragment order
     if (lane == 0) {
 #pragma unroll
         for (int st = 0; st < kMergeStages; ++st) mbar_init(bar0 + 8 * st, 1);
@@ -604,14 +604,11 @@ __global__ void __launch_bounds__(kWarps * 32, CTAS) merge_small_kernel(const __
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the merged rows were written by ordinary stores, the refill is not
             __syncwarp();
-            if (lane == 0) {   // the tensor after the next one takes this stage: V behind Q, then Q and K of the next unit
-                if (SPLIT) {
-                    if (more) issue(t, st, meta_next);
-                } else if (t == 0) {
+            if (!SPLIT && lane == 0) {   // the tensor after the next one takes this stage: V behind Q, then Q and K of the next unit
+                if (t == 0)
                     issue(2, st, m);
-                } else if (more) {
+                else if (more)
                     issue(t - 1, st, meta_next);
-                }
             }
         }
         if (failed) break;

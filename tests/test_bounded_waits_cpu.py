@@ -25,12 +25,13 @@ WARP_ROLES = [
     ("httm_attention_tc.cu", "softmax + epilogue", "tmem_dealloc"),
     ("httm_big_blocks.cu", "arg-max over the chunk's dst tokens", "tmem_dealloc"),
     ("httm_linear.cu", "epilogue: lane = row", "tcgen05.dealloc"),
-    ("httm_mem_kernels.cu", "int buf = 0;", "if (failed)"),
-    ("httm_small_blocks.cu", "uint32_t seq = 0;", "if (failed) break;"),
+    ("httm_mem_kernels.cu", "for (int64_t task = first; task < n_tasks; task += stride, cur.advance()", "if (failed)"),
+    ("httm_small_blocks.cu", "for (int64_t task = first; task < n_tasks; task += stride)", "if (failed) break;"),
+    ("httm_small_blocks.cu", "for (int64_t unit = first; unit < n_units; unit += stride)", "if (failed) break;"),
 ]
 
 
-@pytest.mark.parametrize("name,start,end", WARP_ROLES, ids=["parts", "softmax", "scores", "linear", "deviation", "match_small"])
+@pytest.mark.parametrize("name,start,end", WARP_ROLES, ids=["parts", "softmax", "scores", "linear", "deviation", "match_small", "merge_small"])
 def test_a_warp_gives_up_as_a_whole(name, start, end):
     """The lanes of a warp poll a barrier each for itself, and one may see the time-out where the next still sees the barrier complete.  The
     loads from tensor memory, votes and shuffles behind the wait need all lanes, so the outcome of every wait is a vote of the warp."""
@@ -42,6 +43,18 @@ def test_a_warp_gives_up_as_a_whole(name, start, end):
     for at in waits:
         statement = code[max(code.rfind(c, 0, at) for c in ";{}") + 1:at]
         assert "__all_sync(0xffffffffu," in statement, code[at - 60:at + 60]
+
+
+@pytest.mark.parametrize("kernel", ["match_team_kernel", "merge_team_kernel"])
+def test_a_team_gives_up_as_a_whole(kernel):
+    """In the kernels with a team of warps per block a thread only notes that its wait ran out; the team leaves after a vote of all its threads."""
+    code = open(os.path.join(CSRC, "httm_mid_blocks.cu")).read()
+    begin = code.index("for (int64_t unit = blockIdx.x;", code.index(kernel + "(const __grid_constant__"))
+    code = re.sub(r"//.*", "", code[begin:code.index("\n    }\n", begin)])
+    waits = [code[code.rfind(";", 0, m.start()) + 1:m.start()].strip() for m in re.finditer(r"mbar_wait\w*\(", code)]
+    assert waits == ["const bool arrived ="] and "return" not in code
+    leaves = re.findall(r"if \(([^{;]*)\) (?:\{\s*failed = \w+;\s*)?break;", code)
+    assert len(leaves) == code.count("break;") and set(leaves) <= {"team_any<W>(!arrived)", "failed", "failed >= 0"}, leaves
 
 
 @pytest.mark.parametrize("kernel,tensors", [("match_small_kernel", 2), ("merge_small_kernel", 3)])
