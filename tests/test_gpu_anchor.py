@@ -56,6 +56,9 @@ GEOMS = [
     ("two_frames_32", 4, 8, 8, (2, 4, 4), 0.7, 0.7, 1, 4, 2),              # 16 of 32 tokens are dst
     ("two_frames_32_clipped", 5, 9, 10, (2, 4, 4), 0.5, 0.9, 1, 4, 2),
     ("three_frames_48", 6, 8, 8, (3, 4, 4), 0.6, 0.8, 1, 4, 2),            # 16 of 48
+    ("two_frames_50", 5, 12, 13, (2, 5, 5), 0.6, 0.9, 1, 4, 2),             # 25 of 50 and, in clipped blocks, 10 of 20 or 6 of 12
+    ("two_frames_64", 6, 8, 16, (2, 4, 8), 0.7, 0.4, 1, 4, 2),             # 32 of 64
+    ("two_frames_64_reordered_copies", 4, 9, 9, (2, 4, 8), 0.5, 0.5, 1, 44, 2),
     ("two_frames_128", 4, 17, 19, (2, 8, 8), 0.7, 0.9, 1, 4, 2),           # 64 of 128, clipped windows
     ("two_frames_256", 4, 16, 16, (2, 8, 16), 0.8, 0.4, 1, 4, 1),          # 128 of 256
     ("one_frame_blocks", 3, 8, 8, (1, 4, 4), 0.7, 0.7, 1, 4, 2),           # every token of the first group is a dst token: nothing merges there
@@ -68,6 +71,15 @@ def test_anchored_geometries(case):
     name, S, h, w, blk, rq, rkv, ncam, nreg, H = case
     wl = synth.Workload(name, S, h, w, blk[0], blk[1], blk[2], rq, rkv, n_camera=ncam, n_register=nreg, heads=H, seed=7)
     run_anchored(wl, peaky=True)
+
+
+@pytest.mark.parametrize("n_register", [4, 44], ids=["direct", "over_reordered_copies"])
+def test_blocks_left_out_beside_matched_ones(n_register):
+    """Blocks of 50 tokens of which 25 are dst tokens go to the first frame group's own kernel.  With 24 heads a warp of the other one has several tensors in turn, some of which
+    it leaves out: maps and merged tensors on all tokens."""
+    wl = synth.Workload("left_out", 7, 33, 28, 2, 5, 5, 0.6, 0.8, n_camera=1, n_register=n_register, heads=24, seed=8)
+    assert 2 * wl.heads * 4 * 7 * 6 > 3 * 16 * 148   # (tensors of blocks against warps)
+    run_anchored(wl, sample=np.array([0, 5, 6, 1000, wl.n_tokens - 1]), peaky=True)
 
 
 def test_anchoring_changes_only_the_first_frame_group():

@@ -3,6 +3,7 @@ tables and groups run one block ahead, against the same head alone, bit for bit.
 import numpy as np
 import pytest
 
+from oracle import httm_oracle as orc
 from paper_2511_21317_b200 import binding as hb
 from paper_2511_21317_b200 import synth
 from tests.test_gpu_parity import report_peaky, run_case
@@ -55,7 +56,7 @@ def test_several_tensors_per_warp_and_one_agree(blk, ratio_q, ratio_kv, heads):
 
 @pytest.mark.parametrize("blk,ratio", [((2, 8, 8), 0.5), ((2, 8, 8), 0.7), ((1, 5, 13), 0.3), ((4, 8, 8), 0.6), ((4, 4, 4), 0.5), ((2, 4, 4), 0.5), ((2, 4, 4), 0.3)])
 def test_some_scores_are_equal(blk, ratio):
-    """Tokens that are one of a few vectors: the line between those that merge and the others runs through equal scores, of which the lowest positions merge."""
+    """Tokens that are one of a few vectors: the line between those that merge and the others runs through scores that are equal but for their rounding."""
     wl = synth.Workload("equal", 3, blk[1] + 3, 2 * blk[2] + 1, *blk, ratio, ratio, n_camera=1, n_register=1, heads=3, seed=8)
     q, k, v = synth.make_qkv(wl)
     rng = np.random.default_rng(9)
@@ -63,3 +64,25 @@ def test_some_scores_are_equal(blk, ratio):
         kinds = q[h, rng.integers(0, wl.n_tokens, size=3 + 3 * h)]
         q[h] = kinds[rng.integers(0, len(kinds), size=wl.n_tokens)]
     report_peaky("equal", run_case(wl, q, q, v, peaky=True))
+
+
+def signs(wl, seed):
+    """Vectors of 64 ones and minus ones: norms of 8 and products that are small whole numbers, so that similarities are either equal or differ by 1/32, in fp32 and
+    in the oracle's arithmetic alike."""
+    rng = np.random.default_rng(seed)
+    return np.where(rng.integers(0, 2, size=(wl.heads, wl.n_tokens, 64)) > 0, 0x3f80, 0xbf80).astype(np.uint16)
+
+
+@pytest.mark.parametrize("heads,frames", [(2, 3), (24, 23)], ids=["few", "many"])
+@pytest.mark.parametrize("blk,ratio_q,ratio_kv", [((1, 3, 5), 0.5, 0.2), ((2, 4, 4), 0.3, 0.6), ((3, 4, 4), 0.6, 0.25), ((4, 4, 4), 0.5, 0.7), ((2, 5, 6), 0.1, 0.6),
+                                                  ((2, 8, 8), 0.5, 0.7), ((1, 5, 13), 0.3, 0.5), ((4, 8, 8), 0.6, 0.2), ((4, 8, 9), 0.4, 0.6)],
+                         ids=["15", "32", "48", "64", "60", "128", "65", "256", "288"])
+def test_equal_similarities_go_by_position(blk, ratio_q, ratio_kv, heads, frames):
+    """Exactly equal similarities: the best dst token is the first of them, and of the src tokens on the line between those that merge and the others those at the
+    lowest positions merge.  The maps are the oracle's, token by token."""
+    wl = synth.Workload("signs", frames, 2 * blk[1] + 3, 2 * blk[2] + 1, *blk, ratio_q, ratio_kv, n_camera=1, n_register=1, heads=heads, seed=1)
+    q, k, v = (signs(wl, seed) for seed in (3, 4, 5))
+    want = orc.global_attention(orc.Geometry.of(wl), ratio_q, ratio_kv, q, k, v, attend=False)
+    assert (want.margin_sel_q == 0).any() and (want.margin_sel_k == 0).any() and (want.margin_best_q == 0).any()
+    got = run(hb.HttmConfig.of(wl), [hb.bf16_from_bits(x, "cuda:0") for x in (q, k, v)])
+    assert np.array_equal(got["assign_q"], want.assign_q) and np.array_equal(got["assign_k"], want.assign_k)
