@@ -346,28 +346,46 @@ def test_several_blocks_per_cta_agree_with_one(ratio_q, ratio_kv, anchor):
 @pytest.mark.parametrize("heads,frames,width,run", [(1, 11, 700, 128), (2, 9, 300, 64), (1, 5, 131, 131), (3, 30, 257, 96), (5, 7, 520, 128)])
 def test_blocks_shared_out_to_several_ctas(heads, frames, width, run):
     """Few blocks: their src tokens go to several score CTAs, their groups to several merge CTAs (one to four, with odd numbers of tiles), and the
-    same heads among so many others that there is one of each for a block: the same maps, ranks and merged tensors, bit for bit.  Again with outlier filtering, whose
-    threshold depends on all heads: the deviations, which are of the map before, and what K's map gives."""
+    same heads among many others to one score CTA and one or two merge CTAs: the same maps, ranks and merged tensors, bit for bit."""
+    wl = synth.Workload("shares", frames, 1, width, frames, 1, run, 0.8, 0.6, n_camera=1, n_register=2, heads=heads, seed=11)
+    many = wl.replace(heads=148)
+    reps = -(-148 // heads)
+    q, k, v = (np.tile(x, (reps, 1, 1))[:148] for x in synth.make_qkv(wl))
+    items = {"assign_q": hb.X_ASSIGN_Q, "assign_k": hb.X_ASSIGN_K, "rank_q": hb.X_RANK_Q, "q_m": hb.X_Q_MERGED, "k_m": hb.X_K_MERGED, "v_m": hb.X_V_MERGED}
+    got = {}
+    for name, w, n in (("few", wl, heads), ("many", many, 148)):
+        with hb.Httm(hb.HttmConfig.of(w)) as ctx:
+            ctx.global_attention(*(hb.bf16_from_bits(x[:n], DEV) for x in (q, k, v)))
+            torch.cuda.synchronize()
+            assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+            got[name] = {i: ctx.export(x) for i, x in items.items()}
+    for i in items:
+        assert np.array_equal(got["few"][i], got["many"][i][:heads]), i
+        assert np.array_equal(got["few"][i][0], got["many"][i][heads * (reps - 1)]), i
+
+
+@pytest.mark.parametrize("heads,frames,width,run", [(1, 11, 700, 128), (2, 9, 300, 64), (1, 5, 131, 131), (3, 30, 257, 96), (5, 7, 520, 128)])
+@pytest.mark.parametrize("fraction", [0.0, 0.1])
+def test_heads_among_others_that_leave_one_cta_per_block(heads, frames, width, run, fraction):
+    """So many other heads that every block has one CTA in all kernels, without outlier filtering and with it.  The threshold of the filter depends on all heads, so
+    with it the deviations, which are of the map before, and what K's map gives are compared."""
     wl = synth.Workload("shares", frames, 1, width, frames, 1, run, 0.8, 0.6, n_camera=1, n_register=2, heads=heads, seed=11)
     blocks = -(-width // run)
     reps = -(-450 // (heads * blocks)) + 1   # (blocks of all heads; 888 CTAs of 256 threads that fold deviations fit at once, fewer of the others)
     n_many = heads * (reps - 1) + 1
-    x = synth.make_qkv(wl)
-    many = tuple(hb.bf16_from_bits(np.tile(t, (reps, 1, 1))[:n_many], DEV) for t in x)
-    plain = {"assign_q": hb.X_ASSIGN_Q, "assign_k": hb.X_ASSIGN_K, "rank_q": hb.X_RANK_Q, "q_m": hb.X_Q_MERGED, "k_m": hb.X_K_MERGED, "v_m": hb.X_V_MERGED}
-    filtered = {"eps": hb.X_DEVIATION, "assign_q0": hb.X_ASSIGN_Q_INITIAL, "assign_k": hb.X_ASSIGN_K, "k_m": hb.X_K_MERGED, "v_m": hb.X_V_MERGED}
-    for fraction, items in ((0.0, plain), (0.1, filtered)):
-        got = {}
-        for name, n in (("few", heads), ("many", n_many)):
-            with hb.Httm(hb.HttmConfig.of(wl.replace(heads=n))) as ctx:
-                if fraction:
-                    ctx.set_outlier_fraction(fraction)
-                ctx.global_attention(*(t[:n] for t in many))
-                torch.cuda.synchronize()
-                assert ctx.query(hb.Q_DEVICE_STATUS) == 0
-                got[name] = {i: ctx.export(what) for i, what in items.items()}
-        for i in items:
-            assert np.array_equal(got["few"][i], got["many"][i][:heads]), i
-            assert np.array_equal(got["few"][i][0], got["many"][i][heads * (reps - 1)]), i
-        if fraction:
-            assert (got["few"]["eps"] > 0).any()
+    many = tuple(hb.bf16_from_bits(np.tile(t, (reps, 1, 1))[:n_many], DEV) for t in synth.make_qkv(wl))
+    items = {"assign_k": hb.X_ASSIGN_K, "k_m": hb.X_K_MERGED, "v_m": hb.X_V_MERGED}
+    items.update({"eps": hb.X_DEVIATION, "assign_q0": hb.X_ASSIGN_Q_INITIAL} if fraction else {"assign_q": hb.X_ASSIGN_Q, "rank_q": hb.X_RANK_Q, "q_m": hb.X_Q_MERGED})
+    got = {}
+    for name, n in (("few", heads), ("many", n_many)):
+        with hb.Httm(hb.HttmConfig.of(wl.replace(heads=n))) as ctx:
+            if fraction:
+                ctx.set_outlier_fraction(fraction)
+            ctx.global_attention(*(t[:n] for t in many))
+            torch.cuda.synchronize()
+            assert ctx.query(hb.Q_DEVICE_STATUS) == 0
+            got[name] = {i: ctx.export(what) for i, what in items.items()}
+    for i in items:
+        assert np.array_equal(got["few"][i], got["many"][i][:heads]), i
+        assert np.array_equal(got["few"][i][0], got["many"][i][heads * (reps - 1)]), i
+    assert not fraction or (got["few"]["eps"] > 0).any()

@@ -36,19 +36,34 @@ def test_many_blocks_per_team(blk, frames, specials):
             assert np.array_equal(whole[name][h], one[name][0]), (name, h)
 
 
-@pytest.mark.parametrize("blk,ratio_q,ratio_kv,heads", [((1, 3, 11), 0.1, 0.95, 16), ((3, 4, 4), 0.75, 0.0, 24), ((3, 3, 5), 0.3, 0.86, 16), ((1, 7, 7), 0.5, 0.9, 24),
-                                                        ((4, 4, 4), 0.25, 0.97, 16), ((4, 4, 4), 0.25, 0.97, 24)], ids=["33", "48", "45", "49", "64", "64_24_heads"])
-def test_several_tensors_per_warp_and_one_agree(blk, ratio_q, ratio_kv, heads):
-    """A warp of the small-block kernel matches a tensor of a block of 33 .. 64 tokens at a time, five in turn with 16 heads (dealt out evenly), six or seven
-    with 24, those of Q first: few merge and nearly all, eight dst tokens and sixteen, clipped blocks, equal similarities.  The same head alone has one for every warp."""
-    wl = synth.Workload("many", 12 * blk[0] + 1, 5 * blk[1] + 2, 3 * blk[2] + 1, *blk, ratio_q, ratio_kv, n_camera=1, n_register=4, heads=heads, seed=4)
-    tasks, warps = 2 * 13 * 6 * 4 * heads, 16 * 148
-    assert -(-tasks // warps) == (5 if heads == 16 else 7) and 2 * 13 * 6 * 4 <= warps
+@pytest.mark.parametrize("blk,ratio_q,ratio_kv", [((1, 3, 11), 0.1, 0.95), ((3, 4, 4), 0.75, 0.0), ((3, 3, 5), 0.3, 0.86), ((1, 7, 7), 0.5, 0.9), ((4, 4, 4), 0.25, 0.97)],
+                         ids=["33", "48", "45", "49", "64"])
+def test_whole_units_and_split_units_of_33_to_64_tokens_agree(blk, ratio_q, ratio_kv):
+    """Blocks of 33 .. 64 tokens go to one warp of the small-block kernel, several tensors of them in turn where there are many: few merge and nearly all, eight dst tokens
+    and sixteen, clipped blocks, equal similarities.  Those of the same head alone go to a warp each."""
+    wl = synth.Workload("many", 12 * blk[0] + 1, 5 * blk[1] + 2, 3 * blk[2] + 1, *blk, ratio_q, ratio_kv, n_camera=1, n_register=4, heads=16, seed=4)
+    assert 13 * 6 * 4 * wl.heads > 16 * 148 >= 13 * 6 * 4   # (units against warps)
     q, k, v = synth.make_qkv(wl)
     q[3] = synth.make_identical_block_tokens(wl, seed=6)[3]
     q, k, v = (hb.bf16_from_bits(x, "cuda:0") for x in (q, k, v))
     whole = run(hb.HttmConfig.of(wl), (q, k, v))
-    for h in (0, 3, heads - 1):
+    for h in (0, 3, 15):
+        one = run(hb.HttmConfig.of(wl.replace(heads=1)), (q[h:h + 1], k[h:h + 1], v[h:h + 1]))
+        for name in ITEMS:
+            assert np.array_equal(whole[name][h], one[name][0]), (name, h)
+
+
+@pytest.mark.parametrize("blk,ratio_q,ratio_kv", [((3, 4, 4), 0.75, 0.0), ((1, 7, 7), 0.5, 0.9), ((4, 4, 4), 0.25, 0.97)], ids=["48", "49", "64"])
+def test_several_tensors_per_warp_and_one_agree(blk, ratio_q, ratio_kv):
+    """The same with 24 heads: six or seven tensors in turn, those of Q first (with 16 heads five, dealt out evenly)."""
+    wl = synth.Workload("many", 12 * blk[0] + 1, 5 * blk[1] + 2, 3 * blk[2] + 1, *blk, ratio_q, ratio_kv, n_camera=1, n_register=4, heads=24, seed=4)
+    tasks, warps = 2 * 13 * 6 * 4 * wl.heads, 16 * 148
+    assert -(-tasks // warps) == 7 and 2 * 13 * 6 * 4 <= warps
+    q, k, v = synth.make_qkv(wl)
+    q[3] = synth.make_identical_block_tokens(wl, seed=6)[3]
+    q, k, v = (hb.bf16_from_bits(x, "cuda:0") for x in (q, k, v))
+    whole = run(hb.HttmConfig.of(wl), (q, k, v))
+    for h in (0, 3, 23):
         one = run(hb.HttmConfig.of(wl.replace(heads=1)), (q[h:h + 1], k[h:h + 1], v[h:h + 1]))
         for name in ITEMS:
             assert np.array_equal(whole[name][h], one[name][0]), (name, h)

@@ -41,11 +41,21 @@ def test_nothing_is_called_and_the_registers_were_there(tmp_path, src):
     code = open(os.path.join(CSRC, src)).read()
     role, most = map(int, re.search(r"kScoreRoleRegs = (\d+), kScoreMaxRegs = (\d+)", code).groups())
     groups = int(re.search(r"SC_GROUPS = (\d+)", code).group(1))
+    at = log.index("big_scores_kernel")
+    used = int(re.search(r"Used (\d+) registers", log[at:]).group(1))
+    assert used * (128 + groups * 256) >= 128 * role + groups * 256 * most
+
+
+def test_calls_with_many_blocks_do_not_pay_for_blocks_shared_out(tmp_path):
+    """Both kinds of the score kernel have the registers their split needs, and the kind for many blocks spills no more than the kernel did before there was another."""
+    src = os.path.join(CSRC, "httm_big_blocks.cu")
+    res = subprocess.run([httm_build._nvcc(), *httm_build.NVCC_FLAGS, "-Xptxas", "-v", "-I", httm_build.INCLUDE, "-c", src, "-o", str(tmp_path / "f.o")],
+                         capture_output=True, text=True, check=True)
+    log, code = res.stdout + res.stderr, open(src).read()
+    role, most = map(int, re.search(r"kScoreRoleRegs = (\d+), kScoreMaxRegs = (\d+)", code).groups())
+    groups = int(re.search(r"SC_GROUPS = (\d+)", code).group(1))
     kernels = [m.end() for m in re.finditer(r"Compiling entry function '[^']*big_scores_kernel", log)]
-    spills = []
-    for at in kernels:
-        used = int(re.search(r"Used (\d+) registers", log[at:]).group(1))
-        assert used * (128 + groups * 256) >= 128 * role + groups * 256 * most
-        spills.append(int(re.search(r"(\d+) bytes spill loads", log[at:]).group(1)))
-    # what blocks shared out to several items need is not paid for by calls with many blocks
-    assert len(spills) == 2 and min(spills) <= 368
+    used = [int(re.search(r"Used (\d+) registers", log[at:]).group(1)) for at in kernels]
+    spills = [int(re.search(r"(\d+) bytes spill loads", log[at:]).group(1)) for at in kernels]
+    assert len(kernels) == 2 and min(used) * (128 + groups * 256) >= 128 * role + groups * 256 * most
+    assert min(spills) <= 368, spills
