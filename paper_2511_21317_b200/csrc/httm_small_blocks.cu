@@ -37,16 +37,17 @@ constexpr int kMatchSmem = kWarps * (2 * (int)kStage + 16) + 1024 /*alignment sl
 
 constexpr int match_ctas(int tiles) { return tiles == 2 ? 3 : 2; }   // per SM: 80 and 128 registers
 // TILES: blocks of up to 32 tokens, 8 dst tokens (2); or up to 64 tokens, 16 dst tokens (4), where a warp has room for one tensor, so that 16 warps fit on an SM.
-// UNITS: a task is a unit, both its tensors in a stage each; else one tensor of it.
+// UNITS: a task is a unit, both its tensors in a stage each; else one tensor of it.  ONE: no warp has a second task, and nothing for the next one is kept or looked up:
+// calls in 32-token blocks on 1 044 tokens x 16 heads 18.0 -> 17.6 us, 2 219 x 16 23.6 -> 23.1, 2 219 x 8 21.4 -> 20.4; 48-token blocks, 1 167 x 8 20.4 -> 20.2.
 // A team of one warp that kept all fragments of a 64-token block and had two stages, of which 10 fitted on an SM, both tensors of a unit in turn through one stage, and a
 // tensor at a time: 137 400 tokens x 16 heads in 64-token blocks, ratio 0.8, match 166.2 / 137.5 / 131.5 us; calls on 16 488 tokens 113.7 / 115.7 / 111.4 (4800 units on 2368
 // warps: three rounds of units, five of tensors), on 10 992 tokens 67.1 / 68.2 / 64.6; 7 898 tokens in 48-token blocks 93.1 / 92.7 / 90.7.  (24 warps with 80 registers spill.)
-template <int TILES, bool DIRECT, bool UNITS>
+template <int TILES, bool DIRECT, bool UNITS, bool ONE>
 __global__ void __launch_bounds__(kWarps * 32, match_ctas(TILES))
 match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ MatchArgs a) {
     constexpr int ND = TILES / 2, SLOTS = TILES / 2;   // groups of eight dst tokens; tokens per lane
     constexpr int STAGES = UNITS ? 2 : 1;
-    static_assert(TILES == 2 || !UNITS, "a warp has room for two tensors of 32 tokens");
+    static_assert(!UNITS || (TILES == 2 && !ONE), "a warp has room for two tensors of 32 tokens; few units are dealt out as tensors");
     constexpr uint32_t STAGE = TILES * 16 * kRowBytes;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + align_pad(smem_raw);
@@ -120,7 +121,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         const BlockInfo bi = bi_next;
         const int4 geom = bg_next;
         const int h = h_next, t0 = t_next, n = bi.n;
-        const bool more = task + stride < n_tasks;
+        const bool more = !ONE && task + stride < n_tasks;
         if (more) {
             next.advance();
             fetch();   // in flight while this task is worked off
@@ -326,6 +327,7 @@ match_small_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
         }
         if (failed) break;
+        if (ONE) break;
     }
     if (failed)   // give copies that may still be in flight a bounded chance to land before the shared memory is released
         for (uint32_t i = seq; i <= seq + (ahead ? 1 : 0); ++i) mbar_wait_bounded(bar0 + 8 * (i % STAGES), i / STAGES & 1u, a.status, kDevTimeoutMatchLoad);
@@ -647,10 +649,10 @@ cudaError_t launch_match_tiles(const MatchArgs& a, int sm_count, cudaStream_t st
     };
     // With no more than one tensor per warp the tensors of a unit go to different warps: the call then waits for one, not two
     // (512 units: 11.3 -> 9.4 us, in the merge kernel below 13.1 -> 9.0).
-    if constexpr (TILES == 2)
-        if (2 * units > (int64_t)match_ctas(TILES) * kWarps * sm_count)
-            return launch(direct ? match_small_kernel<TILES, true, true> : match_small_kernel<TILES, false, true>, 1);
-    return launch(direct ? match_small_kernel<TILES, true, false> : match_small_kernel<TILES, false, false>, 2);
+    if (2 * units <= (int64_t)match_ctas(TILES) * kWarps * sm_count)
+        return launch(direct ? match_small_kernel<TILES, true, false, true> : match_small_kernel<TILES, false, false, true>, 2);
+    constexpr bool UNITS = TILES == 2;
+    return launch(direct ? match_small_kernel<TILES, true, UNITS, false> : match_small_kernel<TILES, false, UNITS, false>, UNITS ? 1 : 2);
 }
 }  // namespace
 cudaError_t launch_match_small(const MatchArgs& a, int max_block_tokens, int sm_count, cudaStream_t stream) {
@@ -674,12 +676,14 @@ cudaError_t configure_small_blocks() {
     auto set = [&](auto kernel, int bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     };
-    set(match_small_kernel<2, false, false>, kMatchSmem);
-    set(match_small_kernel<2, false, true>, kMatchSmem);
-    set(match_small_kernel<2, true, false>, kMatchSmem);
-    set(match_small_kernel<2, true, true>, kMatchSmem);
-    set(match_small_kernel<4, false, false>, kMatchSmem);
-    set(match_small_kernel<4, true, false>, kMatchSmem);
+    set(match_small_kernel<2, false, true, false>, kMatchSmem);
+    set(match_small_kernel<2, true, true, false>, kMatchSmem);
+    set(match_small_kernel<2, false, false, true>, kMatchSmem);
+    set(match_small_kernel<2, true, false, true>, kMatchSmem);
+    set(match_small_kernel<4, false, false, false>, kMatchSmem);
+    set(match_small_kernel<4, true, false, false>, kMatchSmem);
+    set(match_small_kernel<4, false, false, true>, kMatchSmem);
+    set(match_small_kernel<4, true, false, true>, kMatchSmem);
     set(merge_small_kernel<2, false, false>, kMergeSmem);
     set(merge_small_kernel<2, false, true>, kMergeSmem);
     set(merge_small_kernel<2, true, false>, kMergeSmem);

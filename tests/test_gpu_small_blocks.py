@@ -35,6 +35,22 @@ def test_whole_units_and_split_units_agree(blk, ratio, specials, frames):
             assert np.array_equal(whole[name][h], one[name][0]), (name, h)
 
 
+@pytest.mark.parametrize("blk,frames,columns", [((1, 4, 8), 3, 37), ((1, 4, 8), 3, 38), ((1, 4, 16), 2, 37), ((1, 4, 16), 2, 38)],
+                         ids=["32_as_many_as_warps", "32_more", "64_as_many_as_warps", "64_more"])
+@pytest.mark.parametrize("specials", [4, 44], ids=["direct", "over_reordered_copies"])
+def test_as_many_tensors_of_blocks_as_warps(blk, frames, columns, specials):
+    """One tensor for each warp that fits on the chip (24 or 16 of them on each of 148 SMs), and a few more than that, against the same heads alone."""
+    wl = synth.Workload("limit", frames, 4, columns * blk[2], *blk, 0.5, 0.7, n_camera=1, n_register=specials, heads=16, seed=5)
+    tensors, warps = 2 * wl.heads * frames * columns, (24 if blk[2] == 8 else 16) * 148
+    assert (tensors == warps) == (columns == 37) and tensors >= warps
+    q, k, v = (hb.bf16_from_bits(x, DEV) for x in synth.make_qkv(wl))
+    whole = run(hb.HttmConfig.of(wl), (q, k, v))
+    for h in (0, 7, 15):
+        one = run(hb.HttmConfig.of(wl.replace(heads=1)), (q[h:h + 1], k[h:h + 1], v[h:h + 1]))
+        for name in ITEMS:
+            assert np.array_equal(whole[name][h], one[name][0]), (name, h)
+
+
 @pytest.mark.parametrize("blk,ratio", [((2, 4, 4), 0.04), ((2, 4, 4), 0.46), ((2, 4, 4), 0.5), ((2, 4, 4), 0.53), ((2, 4, 4), 0.97), ((1, 4, 4), 0.07), ((1, 4, 4), 0.94),
                                        ((1, 1, 17), 0.06), ((3, 3, 3), 0.4), ((1, 1, 2), 0.5)])
 def test_numbers_of_kept_rows_and_tokens(blk, ratio):
