@@ -174,10 +174,11 @@ struct UnitCursor {
     }
 };
 
-// Host: CTAs of eight warps per SM, 2 or 3, for kernels whose warps work off a unit at a time.  A round of units takes 24 warps about 1.4 times as long as 16, so the
-// third CTA pays where it saves more than a third of the rounds, and in the long run.  Merge of 32-token blocks, 16 heads: 65 952 tokens (11 rounds of 24 warps) 115 us with it,
-// 122 without, 32 976 (5.5 rounds) 57.3 and 58.4, 10 992 (2 rounds or 3) 24.5 and 23.6, 5 516 (2 either way) 19.5 and 17.5; 10 374 tokens x 8 heads (1 or 2)
-// a call of 50.8 us with it, 52.8 without.
+// Host: CTAs of eight warps per SM, 2 or 3, for kernels whose warps work off a unit at a time.  The third pays where it saves more than a third of the rounds.  Calls on 32-token
+// blocks, 16 heads, ratio 0.9, with two CTAs / three (rounds in brackets): 5 496 tokens (2 / 1) 34.6 / 32.1 us, 16 488 (5 / 3) 80.3 / 78.6; where it saves less, 10 992 (3 / 2) 56.1 / 57.0,
+// 13 740 (4 / 3) 69.1 / 69.8, 19 236 (5 / 4) 112.3 / 117.5, 27 480 (7 / 5) 158.9 / 161.2.  From six rounds of 24 warps on the merge kernel takes 2 - 4 % less with three (32 976 tokens
+// 56.3 / 54.1, 65 952 105.5 / 103.4), the calls are within 1 % either way: 30 228 (8 / 6) 175.2 / 177.0, 32 976 (9 / 6) 190.7 / 189.5, at ratio 0.7 578 / 566, 43 968 (12 / 8) 280.1 / 281.7,
+// 65 952 (17 / 12) 516 / 518.
 inline int unit_ctas(int64_t units, int sm_count) {
     const int64_t warps = 8ll * (sm_count < 1 ? 1 : sm_count), rounds2 = (units + 2 * warps - 1) / (2 * warps), rounds3 = (units + 3 * warps - 1) / (3 * warps);
     return rounds3 > 5 || 3 * rounds3 < 2 * rounds2 ? 3 : 2;

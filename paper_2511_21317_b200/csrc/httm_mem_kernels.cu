@@ -176,7 +176,8 @@ cudaError_t launch_merge(const MergeArgs& a, int max_block_tokens, int sm_count,
 __device__ void finish_level(const OutlierArgs& a, int level, int* hist);   // (threshold selection, below)
 // Latency of the warps' instruction streams and bytes in flight bound the deviation kernel: as many warps as fit.  With one stage per warp (refilled while the
 // distances are computed: a lane keeps its token in registers), 16 channels of the means at a time and a histogram of the 1024 bins that occur three CTAs fit on an SM; two
-// stages and two CTAs, before: the five kernels of the filter 59.4 us at 32 976 tokens, now 55.3; the call 697.9 -> 693.8.
+// stages and two CTAs, before: the five kernels of the filter 59.4 us at 32 976 tokens, now 55.3; the call 697.9 -> 693.8.  A grid of two CTAs per SM is never better, also where the third saves
+// no round: calls at ratio 0.9 with two / three 61.5 / 59.2 us at 5 496 tokens, 96.6 / 94.4 at 10 992, 218.9 / 213.2 at 27 480, 371.6 / 362.5 at 43 968; 49.9 / 50.0 at 2 748.
 constexpr int kDevWarps = 8;     // 8 x 8.5 KB of shared memory: three CTAs per SM
 constexpr int kCentStride = 68;  // floats per mean: 16-byte reads of eight different means fall on distinct banks
 constexpr int kDevAux = 16 * kCentStride * 4 + 16 * 4 + 32 + 64;   // means of the groups of two or more (at most 16 in 32 tokens), reciprocal sizes, an mbarrier, rows

@@ -10,8 +10,8 @@
 // warp: two of them spend as many instructions again on what every warp of a team does for itself.
 // Measured, before / after (a call: back to back with others, so with what the kernels do to their neighbours):
 //   128-token blocks, 32 976 tokens x 16 heads, ratio 0.9: match 79 / 44 us, merge 70 / 50 us, call 227 / 166 us; (2, 2): 47, 51, 168;
-//   64-token blocks, 137 400 tokens, ratio 0.8: match 197 / 150 us, merge 200 / 180 us, call 3 606 / 3 546 us; (2, 1): 172, 215, 3 568;
-//   48-token blocks, clipped, 7 898 tokens, ratio 0.6: call 102 / 94 us; (2, 1): 106 us.
+//   64-token blocks, 137 400 tokens, ratio 0.8: merge 200 / 180 us, (2, 1): 215;
+//   48-token blocks, clipped, 7 898 tokens, ratio 0.6, with a team that matched them too: call 102 / 94 us; (2, 1): 106 us.
 #include "httm_blocks.cuh"
 #include "httm_launch.cuh"
 
@@ -67,9 +67,12 @@ __host__ __device__ constexpr MergeAux merge_aux(int tokens) {
     a.bytes = a.bars + 16;
     return a;
 }
-// Both kernels ask for the same shared memory.  The merge CTAs move in one by one as match CTAs of the kernel before end
+// Match and merge teams of a size ask for the same shared memory.  The merge CTAs move in one by one as match CTAs of the kernel before end
 // (launch ahead of the predecessor's end), and a hole of another size than theirs stays partly unused: with 19 408 and 20 320
-// bytes a third of the merge CTAs found no place until others had finished (137 344 tokens, 64-token blocks: 100 us).
+// bytes a third of the merge CTAs found no place until others had finished (137 344 tokens, 64-token blocks, when a team matched those: 100 us).
+// Teams of one warp now follow the small-block kernel's match CTAs of 66 688 bytes, and how large these are counts too: asking for 73 984 a call on 32 976 tokens in 64-token
+// blocks, ratio 0.8, takes 312 us instead of 297.  For blocks of at most 32 tokens it does not: match and merge with 73 984 bytes each, the deviation kernel's, instead of 66 688 and
+// 69 248 make no difference of more than 0.2 % in calls on 1 044 .. 65 952 tokens, with outlier filtering or without.
 constexpr int team_smem(int w, int p) {
     const int x = match_aux(team_tokens(w, p)).bytes, y = merge_aux(team_tokens(w, p)).bytes;
     return 2 * team_tokens(w, p) * kRowBytes + (x > y ? x : y) + 1024 /*alignment slack*/;

@@ -35,7 +35,7 @@ constexpr uint32_t kStage = 32 * kRowBytes;   // one block of one tensor, 128-by
 // Row rho of the stage is owned, from the arg-max on, by lane (rho & 7) * 4 + (rho >> 3).
 constexpr int kMatchSmem = kWarps * (2 * (int)kStage + 16) + 1024 /*alignment slack*/;   // two blocks of 32 rows or one of 64 per warp
 
-constexpr int match_ctas(int tiles) { return tiles == 2 ? 3 : 2; }   // per SM: 80 and 128 registers
+constexpr int match_ctas(int tiles) { return tiles == 2 ? 3 : 2; }   // per SM: 80 registers (with whole units 72 bytes of them spilled) and 120
 // TILES: blocks of up to 32 tokens, 8 dst tokens (2); or up to 64 tokens, 16 dst tokens (4), where a warp has room for one tensor, so that 16 warps fit on an SM.
 // UNITS: a task is a unit, both its tensors in a stage each; else one tensor of it.  ONE: no warp has a second task, and nothing for the next one is kept or looked up:
 // calls in 32-token blocks on 1 044 tokens x 16 heads 18.0 -> 17.6 us, 2 219 x 16 23.6 -> 23.1, 2 219 x 8 21.4 -> 20.4; 48-token blocks, 1 167 x 8 20.4 -> 20.2.
