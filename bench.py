@@ -31,7 +31,7 @@ from paper_2511_21317_b200 import synth  # noqa: E402
 # dram__bytes_read.sum + dram__bytes_write.sum of one attention launch (one ncu capture, summary under profiles/), with
 # the digest of the kernel's sources at the time of the capture: the figure is reported only while the sources still
 # have that digest (null for workloads that were not captured and once the kernel has changed).
-ATTENTION_DRAM_TRAFFIC = {"medium": (86675712 + 37901312, "5418a1e83a914051")}   # profiles/ncu_medium_call_kernels.txt
+ATTENTION_DRAM_TRAFFIC = {"medium": (87392512 + 37929728, "5418a1e83a914051")}   # profiles/ncu_medium_call_kernels.txt
 ATTENTION_SOURCES = ("paper_2511_21317_b200/csrc/httm_attention_tc.cu", "paper_2511_21317_b200/csrc/tc_sm100.cuh")
 METRIC = "httm_global_attention_layer_throughput"
 UNIT = "tokens/s"
