@@ -74,9 +74,9 @@ __host__ __device__ constexpr MergeAux merge_aux(int tokens) {
 // blocks, ratio 0.8, takes 312 us instead of 297.  For blocks of at most 32 tokens it does not: match and merge with 73 984 bytes each, the deviation kernel's, instead of 66 688 and
 // 69 248 make no difference of more than 0.2 % in calls on 1 044 .. 65 952 tokens, with outlier filtering or without.
 constexpr int team_smem(int w, int p) {
-    const int x = match_aux(team_tokens(w, p)).bytes, y = merge_aux(team_tokens(w, p)).bytes;
-    return 2 * team_tokens(w, p) * kRowBytes + (x > y ? x : y) + 1024 /*alignment slack*/;
+    return 2 * team_tokens(w, p) * kRowBytes + merge_aux(team_tokens(w, p)).bytes + 1024 /*alignment slack*/;
 }
+static_assert(match_aux(128).bytes <= merge_aux(128).bytes && match_aux(256).bytes <= merge_aux(256).bytes, "a match team fits in what the merge team needs");
 constexpr int team_ctas(int w, int p) {   // CTAs per SM: all of a persistent grid have to be resident
     const int by_warps = (p == 1 ? 24 : 12) / w, by_smem = 228 * 1024 / (team_smem(w, p) + 1024);
     return by_warps < by_smem ? by_warps : by_smem;
